@@ -13,6 +13,7 @@
 // host-side stand-in); make that first call before any stream capture.
 // Calls share the array: calls that overlap on the GPU (different streams,
 // or different host threads) race and must not be issued.
+#include <algorithm>
 #include <cfloat>
 #include <cmath>
 #include <mutex>
@@ -25,12 +26,16 @@
 namespace {
 
 constexpr int kBlock = 256;
-constexpr int kMaxBlocks = RICH_NOALLOC_MAX_CELLS / kBlock;
+// cells a thread takes per pass of its block, and the largest grid: eight
+// blocks on each of 152 SMs
+constexpr int kCells = 4;
+constexpr int kMaxBlocks = 8 * 152;
 
 // scratch: per-block minima of the cell time step as bit patterns (the
 // integer order of non-negative doubles is their numeric order; kBad marks
 // a block that met a cell whose time step is not a finite non-negative
-// number), then the number of blocks that have finished
+// number), then the number of blocks that have finished, which wraps back to
+// zero with the last one
 static __device__ __align__(256) unsigned long long g_courant_scratch[kMaxBlocks + 1];
 
 constexpr unsigned long long kBad = ~0ull;
@@ -53,23 +58,106 @@ __device__ __forceinline__ unsigned long long key_min(unsigned long long a, unsi
     return a < b ? a : b;
 }
 
-__global__ void k_courant_noalloc(int32_t n, double gamma, double cfl, int32_t motion_static,
-                                  const double *__restrict__ area, const double *__restrict__ rho,
-                                  const double *__restrict__ vx, const double *__restrict__ vy,
-                                  const double *__restrict__ p, const double *__restrict__ wx,
-                                  const double *__restrict__ wy, unsigned long long *scratch, double *dt_out)
+// |v| with its mantissa cut to 24 bits, for an exponent field in [1023 -
+// span, 1023 + span] (span <= 100): two shifts on the integer pipe.  FP64 to
+// FP32 conversions issue on the FP64 pipe.
+__device__ __forceinline__ float cut(double v)
 {
-    int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+    const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
+    return __uint_as_float(__funnelshift_l(lo, hi, 3) - 0xc0000000u);
+}
+// v positive with an exponent within 2^-span .. 2^span
+__device__ __forceinline__ bool in_span(double v, unsigned span)
+{
+    return ((unsigned)__double2hiint(v) >> 20) - (1023u - span) <= 2u * span;
+}
+__device__ __forceinline__ float root(float v)
+{
+    float r;
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
+    return r;
+}
+__device__ __forceinline__ float inverse(float v)
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
+    return r;
+}
+
+// Bound by DRAM (56 B per cell of a moving mesh) where evaluating every cell
+// in FP64 was bound by the FP64 pipe, which issues one warp instruction per
+// 16 clocks per SM: about 110 of them per cell step (three square roots and
+// two divides).  Each cell's time step is first estimated in FP32 within
+// 1e-6, and only cells whose estimate is within 4e-6 of the smallest so far
+// in their block, which the smallest time step's cell always is, are
+// evaluated in FP64 with the formula of the sweep: the result's bits are
+// those of evaluating every cell.  Cells outside the estimate's range
+// (gamma of 2^20 and above, density or pressure beyond 2^+-30, area beyond
+// 2^+-100, speeds above 2^60, and everything negative or not finite) always are.
+__global__ void __launch_bounds__(kBlock) k_courant_noalloc(
+    int32_t n, double gamma, float gamma_f, double cfl, int32_t motion_static, const double *__restrict__ area,
+    const double *__restrict__ rho, const double *__restrict__ vx, const double *__restrict__ vy,
+    const double *__restrict__ p, const double *__restrict__ wx, const double *__restrict__ wy,
+    unsigned long long *scratch, double *dt_out)
+{
     // kMax: the bits of +inf, above every finite non-negative time step
     const unsigned long long kMax = 0x7ff0000000000000ull;
+    constexpr unsigned kNone = 0x7f800000u;  // estimate of no cell
     unsigned long long k = kMax;
     bool bad = false;
-    if (i < n) {
-        const double cs = sqrt(gamma * p[i] / rho[i]);
-        const double R = sqrt(area[i] * (1.0 / M_PI));
-        const double ux = motion_static ? vx[i] : vx[i] - wx[i];
-        const double uy = motion_static ? vy[i] : vy[i] - wy[i];
-        k = step_key(R / (cs + sqrt(ux * ux + uy * uy)), bad);
+    __shared__ unsigned smallest;
+    if (threadIdx.x == 0) smallest = kNone;
+    __syncthreads();
+    for (int32_t base = blockIdx.x * kBlock * kCells; base < n; base += gridDim.x * kBlock * kCells) {
+        double A[kCells], r[kCells], P[kCells], ux[kCells], uy[kCells];
+        float est[kCells];
+#pragma unroll
+        for (int c = 0; c < kCells; c++) {
+            const int32_t i = base + c * kBlock + threadIdx.x;
+            if (i < n) {
+                A[c] = __ldcs(area + i);
+                r[c] = __ldcs(rho + i);
+                P[c] = __ldcs(p + i);
+                ux[c] = __ldcs(vx + i);
+                uy[c] = __ldcs(vy + i);
+                if (!motion_static) {
+                    ux[c] -= __ldcs(wx + i);
+                    uy[c] -= __ldcs(wy + i);
+                }
+            }
+        }
+        unsigned least = kNone;
+#pragma unroll
+        for (int c = 0; c < kCells; c++) {
+            est[c] = __uint_as_float(kNone);
+            if (base + c * kBlock + (int32_t)threadIdx.x >= n) continue;
+            const unsigned ex = ((unsigned)__double2hiint(ux[c]) >> 20) & 0x7ffu;
+            const unsigned ey = ((unsigned)__double2hiint(uy[c]) >> 20) & 0x7ffu;
+            if (!(gamma_f < 1048576.0f && in_span(r[c], 30) && in_span(P[c], 30) && in_span(A[c], 100) && ex <= 1083u && ey <= 1083u)) {
+                est[c] = 0.0f;  // always evaluated
+                continue;
+            }
+            // (a speed below 2^-100 vanishes beside c_s > 2^-31)
+            const float fx = ex < 923u ? 0.0f : cut(ux[c]), fy = ey < 923u ? 0.0f : cut(uy[c]);
+            const float cs = root(gamma_f * cut(P[c]) * inverse(cut(r[c])));
+            est[c] = root(cut(A[c]) * 0.318309886f) * inverse(cs + root(fx * fx + fy * fy));
+            least = min(least, __float_as_uint(est[c]));
+        }
+        least = __reduce_min_sync(0xffffffffu, least);
+        if ((threadIdx.x & 31) == 0 && least < kNone) atomicMin(&smallest, least);
+        __syncthreads();
+        // (another warp may lower it meanwhile, from cells of its next pass:
+        // any of the values does)
+        const float limit = __uint_as_float(*(volatile unsigned *)&smallest) * 1.000004f;
+#pragma unroll
+        for (int c = 0; c < kCells; c++) {
+            const int32_t i = base + c * kBlock + threadIdx.x;
+            if (i < n && est[c] <= limit) {
+                const double cs = sqrt(gamma * P[c] / r[c]);
+                const double R = sqrt(A[c] * (1.0 / M_PI));
+                k = key_min(k, step_key(R / (cs + sqrt(ux[c] * ux[c] + uy[c] * uy[c])), bad));
+            }
+        }
     }
     bad = __any_sync(0xffffffffu, bad);
     for (int o = 16; o > 0; o >>= 1) k = key_min(k, __shfl_down_sync(0xffffffffu, k, o));
@@ -89,8 +177,7 @@ __global__ void k_courant_noalloc(int32_t n, double gamma, double cfl, int32_t m
         for (int q = 1; q < kBlock / 32; q++) m = key_min(m, red[q]);
         scratch[blockIdx.x] = bad_block ? kBad : m;
         __threadfence();
-        unsigned long long done = atomicAdd(&scratch[kMaxBlocks], 1ull);
-        last = done == gridDim.x - 1;
+        last = atomicInc(reinterpret_cast<unsigned *>(&scratch[kMaxBlocks]), gridDim.x - 1) == gridDim.x - 1;
     }
     __syncthreads();
     if (!last) return;
@@ -150,11 +237,9 @@ extern "C" int rich_courant_dt_noalloc(const rich_config *cfg, int64_t n, const 
         scratch = g_scratch_addr[dev];
     }
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    const int blocks = (int)((n + kBlock - 1) / kBlock);
-    // the completion counter must start at zero on every call
-    if (cudaMemsetAsync(scratch + kMaxBlocks, 0, sizeof(unsigned long long), st) != cudaSuccess)
-        return rich::set_error(RICH_ECUDA, "cudaMemsetAsync failed");
-    k_courant_noalloc<<<blocks, kBlock, 0, st>>>((int32_t)n, cfg->gamma, cfg->cfl,
+    const int64_t tile = (int64_t)kBlock * kCells;
+    const int blocks = (int)std::min<int64_t>((n + tile - 1) / tile, kMaxBlocks);
+    k_courant_noalloc<<<blocks, kBlock, 0, st>>>((int32_t)n, cfg->gamma, (float)cfg->gamma, cfg->cfl,
                                                  cfg->motion == RICH_MESH_EULERIAN ? 1 : 0, area, rho, vx, vy, p,
                                                  wx, wy, scratch, dt_out);
     return cudaGetLastError() == cudaSuccess ? RICH_OK : rich::set_error(RICH_ECUDA, "launch failed");

@@ -99,3 +99,48 @@ def test_noalloc_bad_cell_gives_nan():
     rich.rich_courant_dt_noalloc(cfg, n, *[t.data_ptr() for t in bad], 0, 0, out.data_ptr())
     torch.cuda.synchronize()
     assert math.isnan(float(out.item()))
+
+
+@pytest.mark.parametrize("n", [1, 31, 255, 1023, 1024, 1025, 1216 * 1024 + 1, 3000001])
+@pytest.mark.parametrize("case", ["smooth", "equal", "wide", "huge_gamma", "still"])
+def test_noalloc_minimum_over_all_cells(n, case):
+    """The FP32 estimate that picks the cells to evaluate never loses the
+    smallest time step: sizes around a thread's, block's and grid's share;
+    cells all but equal; values far beyond the estimate's range; a fluid at
+    rest.  Against the same formula over every cell in FP64: a square root
+    or division is rounded once on both sides, and the sums under the second
+    root differ by a fused multiply-add, so 4 ulps cover the quotient."""
+    import torch
+    rich = _lib()
+    g = torch.Generator(device="cuda").manual_seed(n + len(case))
+
+    def u(lo, hi):
+        return torch.empty(n, dtype=torch.float64, device="cuda").uniform_(lo, hi, generator=g)
+
+    a = {"area": u(0.5, 1.5) / n, "rho": u(0.5, 2.0), "vx": u(-1, 1), "vy": u(-1, 1), "p": u(0.5, 2.0),
+         "wx": u(-1, 1), "wy": u(-1, 1)}
+    gamma = 5.0 / 3.0
+    if case == "equal":
+        # time steps within 1e-9 of each other
+        for k in FIELDS:
+            a[k] = torch.ones_like(a[k]) * (1.0 + 0.1 * len(k))
+        a["area"] = a["area"] * (1.0 + 1e-9 * u(0, 1))
+    elif case == "wide":
+        for k in ("area", "rho", "p"):
+            a[k] = torch.exp2(u(-300, 300))
+        a["vx"] = a["vx"] * torch.exp2(u(-200, 200))
+    elif case == "huge_gamma":
+        gamma = 1e30
+    elif case == "still":
+        a["wx"], a["wy"] = a["vx"].clone(), a["vy"].clone()
+        a["wx"][: n // 2] += 1e-300
+    out = torch.full((1,), -1.0, dtype=torch.float64, device="cuda")
+    cfg = W.default_cfg(gamma=gamma)
+    for _ in range(2):
+        rich.rich_courant_dt_noalloc(cfg, n, *[a[k].data_ptr() for k in FIELDS], out.data_ptr(),
+                                     torch.cuda.current_stream().cuda_stream)
+    ux, uy = a["vx"] - a["wx"], a["vy"] - a["wy"]
+    dt = torch.sqrt(a["area"] * (1.0 / math.pi)) / (torch.sqrt(gamma * a["p"] / a["rho"]) + torch.sqrt(ux * ux + uy * uy))
+    dt = dt[torch.isfinite(dt)]
+    want = cfg["cfl"] * float(dt.min())
+    assert abs(float(out.item()) - want) <= 4 * 2.0 ** -52 * want
