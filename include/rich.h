@@ -6,8 +6,9 @@
  * (arXiv:1410.3219), Section 2, with the "extrapolated fluxes" time
  * advancement of Section 2.3:
  *
- *   a0  host: ghost images + Delaunay triangulation by point insertion with
- *       exact, tie-broken in-circle predicates (Section 2.1)
+ *   a0  ghost images + Delaunay triangulation with exact, tie-broken in-circle
+ *       predicates (Section 2.1): a simulation's first mesh by point insertion
+ *       on the host, each later one as an update of the last on the device
  *   a1  Voronoi geometry: circumcentres, areas, centres of mass, edge lengths,
  *       midpoints, normals, c_ij (quantities defined under Eq. 1)
  *   a2  primitive variables rho, v, p and sound speed (ideal gas)
@@ -20,7 +21,9 @@
  *   a8  conservative update U_i -= dt * sum_j L_ij F_ij (Section 5)
  *   a9  advance the mesh-generating points
  *
- * Steps a1-a9 run as CUDA kernels on the device (sm_103a); a0 runs on the host.
+ * Steps a1-a9 and the mesh updates run as CUDA kernels on the device (sm_103a).
+ * The triangulation is unique, so the host and the device build the same mesh;
+ * a mesh that the update cannot make (see rich_tessellate) is built on the host.
  *
  * Conventions
  *  - All arrays passed in or out are HOST arrays unless a name says "device".
@@ -101,7 +104,8 @@ typedef struct {
     double t;           /* simulation time after the call */
     double dt_last;     /* last time step */
     double sweep_ms;    /* device time of steps a1-a9 summed over the call (CUDA events) */
-    double tess_ms;     /* host time of a0 summed over the call */
+    double tess_ms;     /* time of a0 summed over the call: host builds (wall), updates on the device (their checks
+                           by CUDA events, and the host's time to enqueue the rest) */
     double copy_ms;     /* host time spent in host<->device copies and waits */
     int64_t n_ghost, n_tri, n_edges, n_slots; /* size of the last tessellation */
 } rich_step_info;
@@ -122,16 +126,14 @@ int rich_init_mesh(const rich_config *cfg, int64_t n, const double *x, const dou
                    const double *vx, const double *vy, const double *p, rich_sim **out);
 
 /* Advance up to max_steps steps, stopping early once the time reaches t_end
-   (the last step is shortened to land on t_end).  Each step: a0 on the host
-   for the current points, then a1-a9 on the device (twice, with a0 for the
-   half-step points in between, in the time-centred scheme).  The points'
-   motion (a9) needs only the mesh velocity and dt, known after the geometry
-   stage, so each sweep writes the moved points first; the call reads them
-   back then and runs a0 for them on the host while the device computes the
-   gradients, fluxes and update.  A step that does not land on t_end thus
-   leaves the mesh of its points built, and the next step or call starts
-   with the sweep.  Results equal those of rich_tessellate / rich_sweep /
-   rich_sync in turn, bit for bit.  info may be NULL.
+   (the last step is shortened to land on t_end).  Each step: a1-a9 on the
+   device for the current points and mesh, then a0 for the moved points
+   (twice, with a0 for the half-step points in between, in the time-centred
+   scheme).  A step that does not land on t_end thus leaves the mesh of its
+   points built, and the next step or call starts with the sweep; the device
+   may still be writing that mesh when the call returns, and later calls wait
+   for it.  Results equal those of rich_tessellate / rich_sweep / rich_sync in
+   turn, bit for bit.  info may be NULL.
    Errors: RICH_ENEGATIVE / RICH_ENAN (state left at the last good step),
    RICH_ETESS, RICH_EDUPLICATE, RICH_ECUDA. */
 int rich_step(rich_sim *s, int32_t max_steps, double t_end, rich_step_info *info);
@@ -178,10 +180,14 @@ const char *rich_last_error(void);
    the handle's own stream).  The caller keeps the stream alive. */
 int rich_set_stream(rich_sim *s, void *cuda_stream);
 
-/* a0 for the current points: copy points device->host, tessellate on the
-   host, upload the rings (with each cell's first owned triangle and edge)
-   and build the triangle and edge lists from them on the device.
-   Synchronous.  RICH_ETESS if the device lists do not close. */
+/* a0 for the current points: the mesh on the device, of whichever points it
+   is, updated for them, with its triangle and edge lists.  The update leaves
+   a mesh to the host (the points are copied there, tessellated, and the rings
+   uploaded) for fewer than 64 cells, when a Voronoi circumdisk of a real cell
+   reaches 0.98 of the ghost band or, in a periodic box, a quarter of it, when
+   a cell has more than 32 neighbours, when points coincide, and when
+   coordinates that decide an exact predicate spread over more than 72 binary
+   orders of magnitude.  Synchronous.  RICH_ETESS if the lists do not close. */
 int rich_tessellate(rich_sim *s, rich_step_info *info);
 
 /* Enqueue a1-a9 for one step on the current connectivity (asynchronous; no
@@ -220,7 +226,8 @@ int rich_set_profiling(rich_sim *s, int32_t on);
 int rich_kernel_times(rich_sim *s, int32_t cap, double *ms, int32_t *count);
 const char *rich_kernel_name(int32_t stage);
 
-/* Wall time (ms) of the phases of the handle's last host tessellation (a0):
+/* Wall time (ms) of the phases of the handle's last host tessellation (the
+   first mesh of a simulation, unless the device's update left one to the host):
    ms[0] ghost images, point copies, bounding box and bucket grid; ms[1] the
    tiles (triangulation or in-place update, star checks, rings); ms[2]
    triangle and ring assembly; ms[3] edge counts and processing order. */
@@ -259,14 +266,14 @@ int rich_batch_add(rich_batch *b, const rich_config *cfg, int64_t n, const doubl
                    const double *rho, const double *vx, const double *vy, const double *p, double t_end,
                    int64_t max_steps, int32_t *id);
 
-/* One step of every pending or running simulation.  With the staged
-   launch, the moved points are read back once the point motion is done and
-   the simulations that go on are tessellated for the next step while the
-   device finishes the sweep (the next call then tessellates only newly
-   admitted ones); results equal those without this overlap, bit for bit.
+/* One step of every pending or running simulation.  The meshes of the moved
+   points are updated on the device after the sweep; a step with the same
+   simulations as the last then starts with the sweep, and one with others
+   reads those meshes back and packs them with the host-built ones of the
+   newly admitted simulations.
    info (nullable): steps_done = simulations stepped, sweep_ms = device time
-   of the sweep, tess_ms = host tessellation wall time (both tessellations),
-   copy_ms = other host time outside the sweep. */
+   of the sweep, tess_ms = time of the host tessellations and of the mesh
+   updates, copy_ms = other host time outside the sweep. */
 int rich_batch_step(rich_batch *b, rich_step_info *info);
 
 /* State (RICH_SIM_*), error code of a failed simulation, its time and steps
@@ -414,12 +421,11 @@ void rich_server_destroy(rich_server *s);
    FP32).  Cells whose time step is +inf are skipped, as the sweep skips
    them; a cell whose time step is NaN, negative or -0.0 (a negative or NaN
    pressure or density) makes *dt_out a NaN instead of being skipped.
-   It allocates nothing: its scratch (one partial minimum per block of 256
-   cells and a completion counter, 512 KiB) is a fixed array in the
-   library's device image, which every GPU that loads the library holds until
-   the process exits.  The first call on each device looks up that array's
+   It allocates nothing: its scratch (one partial minimum per block and a
+   completion counter, 10 KB) is a fixed array in the library's device image,
+   which every GPU that loads the library holds until the process exits.  The first call on each device looks up that array's
    address (cudaGetSymbolAddress), so make it before any stream capture.
-   Every call shares the array and clears its counter: calls that overlap on
+   Every call shares the array: calls that overlap on
    the GPU (other streams, other host threads) race and must not be issued.
    Returns RICH_EINVAL for a configuration that rich_init_mesh rejects, a
    NULL array, or n outside [1, RICH_NOALLOC_MAX_CELLS], RICH_ECUDA if the
@@ -485,6 +491,24 @@ int rich_edge_list_check(const rich_config *cfg, int64_t n, const double *x, con
 int rich_mesh_update_check(const rich_config *cfg, int64_t n, int32_t steps, const double *xs, const double *ys,
                            int32_t threads, int32_t *mismatched, int64_t *updated, int64_t *rebuilt,
                            int64_t *reinserted);
+
+/* The device's mesh update against the host builder (host only; no GPU
+   needed): from the mesh of each of `steps` successive point sets (xs, ys:
+   steps x n, row-major, the same cells in each) the next set's mesh is made
+   by the update's per-cell code, run serially, and compared with a fresh
+   host build.  *mismatched counts entries that differ (rings, offsets,
+   processing order, ghosts), *updated the meshes made by the update (the
+   others it leaves to the host builder), *recomputed the stars built again.
+   Errors: RICH_EINVAL, tessellation errors. */
+int rich_device_update_check(const rich_config *cfg, int64_t n, int32_t steps, const double *xs, const double *ys,
+                             int64_t *mismatched, int64_t *updated, int64_t *recomputed);
+
+/* The handle's current mesh on the device against a fresh host build of its
+   points: *mismatched counts the entries that differ; *updates (nullable)
+   receives how many of the handle's meshes the device updated so far.
+   Errors: RICH_EINVAL, RICH_ESTATE (no current tessellation), RICH_ECUDA,
+   tessellation errors. */
+int rich_mesh_check(rich_sim *s, int64_t *mismatched, int64_t *updates);
 
 #ifdef __cplusplus
 }

@@ -14,8 +14,8 @@ CSRC = os.path.join(PKG, "csrc")
 OBJ = os.path.join(ROOT, "_build")
 LIB = os.path.join(PKG, "librich.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-CUDA_SOURCES = ["sweep.cu", "courant_noalloc.cu", "probe.cu", "layout.cu"]
-HOST_SOURCES = ["predicates.cpp", "mesh.cpp", "rich_api.cpp", "batch.cpp", "server.cpp"]
+CUDA_SOURCES = ["sweep.cu", "meshupdate.cu", "courant_noalloc.cu", "probe.cu", "layout.cu"]
+HOST_SOURCES = ["predicates.cpp", "mesh.cpp", "meshupdate_host.cpp", "rich_api.cpp", "batch.cpp", "server.cpp"]
 
 
 def _nvcc():
@@ -33,7 +33,9 @@ def _compile(src):
     path = os.path.join(CSRC, src)
     obj = os.path.join(OBJ, src + ".o")
     if src.endswith(".cu"):
-        cmd = [_nvcc(), *ARCH, "-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC,-ffp-contract=off",
+        # (the exact predicates' error bounds assume no contraction)
+        fmad = ["-fmad=false"] if src == "meshupdate.cu" else []
+        cmd = [_nvcc(), *ARCH, *fmad, "-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC,-ffp-contract=off",
                "-Xptxas", "-v", "-c", path, "-o", obj]
     else:
         cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-pthread", "-ffp-contract=off", "-fno-fast-math",

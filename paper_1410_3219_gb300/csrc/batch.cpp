@@ -32,6 +32,8 @@
 
 #include "api_internal.h"
 #include "mesh.h"
+#include "meshupdate.h"
+#include "meshupdate_dev.h"
 #include "sweep.cuh"
 #include "threadpool.h"
 
@@ -56,8 +58,7 @@ struct BatchSim {
     rich::MeshWork mw;           // (edge lists built on the device, packed)
     rich::HostMesh hm;
     int mesh_rc = 0;
-    // the mesh of its current points was built during the last step's sweep
-    // (mesh_rc is that build's result)
+    // hm is the mesh of its current points (read back from the device)
     bool prebuilt = false;
     double t = 0.0, t_end = 0.0, last_dt = 0.0;
     int64_t steps = 0, max_steps = 0;
@@ -103,18 +104,26 @@ struct rich_batch {
     rich::ThreadPool *pool = nullptr;
     cudaStream_t stream = nullptr;
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
-    // early read of a staged sweep's moved points and time steps (copied on
-    // their own stream once the point motion is done) into page-locked
-    // memory: x, y of the packed cells, then dt per simulation
-    cudaStream_t copy_stream = nullptr;
-    cudaEvent_t ev_moved = nullptr, ev_copied = nullptr;
-    rich::HBuf h_moved;
+    // The device's mesh update (meshupdate.h) for the packed cells: after a
+    // step dev_mesh says that the arrays of buffers mcur hold the meshes of
+    // the moved points of `packed` (those of simulations with a mesh flag
+    // excepted), dev_lists that the triangle and edge lists are built too
+    // and none is flagged.  A step whose simulations are the same then starts
+    // with the sweep; else the meshes are read back and packed again.
+    rich::MeshUpdater updater;
+    rich::MeshSizes msz;
+    int mcur = 0;
+    bool dev_mesh = false, dev_lists = false;
+    std::vector<int32_t> mesh_flag;
+    rich::HBuf h_back;  // dt, status per simulation, then the list builders' flags
+    cudaEvent_t ev2 = nullptr, ev3 = nullptr;
     bool diagnostics = false;
     int cur = 0;
     // device
-    DBuf x[2], y[2], U[2], A, o, W, cs, g, gl, alpha, w, tess, rounding, p64, cell_ptr, cell_inst, initW, src;
+    DBuf x[2], y[2], U[2], A, o, W, cs, g, gl, alpha, w, tess, rounding, p64, cell_inst, initW, src;
     DBuf corder, psrc;
-    DBuf gx, gy, gsrc, gxf, tri, ccx, ccy, slot_nb, slot_tri, slot_edge;
+    DBuf cell_ptr[2], slot_nb[2], gsrc[2], gimg[2];
+    DBuf gx, gy, gxf, tri, ccx, ccy, slot_tri, slot_edge;
     DBuf edge_l, edge_r, edge_ta, edge_tb, eL, emlx, emly, emrx, emry, enx, eny, eqx, eqy, F, ePM;
     DBuf instp, dtmin, dtout, status, dsizes, gsync, eoff, toff, gshift, edgebad;
     // launch shape: autotuned over the first steps unless fixed by the caller
@@ -141,13 +150,12 @@ struct rich_batch {
     int32_t inject_spin = 0;
     // host staging of the packed mesh
     std::vector<double> h_x, h_y, h_gx, h_gy, h_W0;
-    std::vector<double> h_dlx, h_dly;  // the points downloaded at the start of a step
+    std::vector<double> h_dlx, h_dly, h_dgx, h_dgy;  // the points (and a mesh's ghosts) downloaded at the start of a step
+    std::vector<int32_t> h_dptr, h_dnb, h_dgsrc, h_dgxf, h_dgshift, h_dgimg, h_dtoff, h_deoff, h_dorder;
     std::vector<int32_t> h_gsrc, h_gxf, h_cell_ptr, h_slot_nb, h_cell_inst;
     std::vector<int32_t> h_corder;
-    std::vector<int32_t> h_src, h_eoff, h_toff, h_gshift;
+    std::vector<int32_t> h_src, h_eoff, h_toff, h_gshift, h_gimg;
     std::vector<rich::InstParams> h_inst;
-    std::vector<double> h_dt;
-    std::vector<int32_t> h_status;
     int64_t nG = 0, nT = 0, nE = 0, nS = 0;
 
     explicit rich_batch(int threads) : own_pool(new rich::ThreadPool(threads)), pool(own_pool.get()) {}
@@ -159,14 +167,14 @@ struct rich_batch {
             if (gexec[k]) cudaGraphExecDestroy(gexec[k]);
             if (graph[k]) cudaGraphDestroy(graph[k]);
         }
-        if (copy_stream) cudaStreamSynchronize(copy_stream);
-        if (ev0) cudaEventDestroy(ev0);
-        if (ev1) cudaEventDestroy(ev1);
-        if (ev_moved) cudaEventDestroy(ev_moved);
-        if (ev_copied) cudaEventDestroy(ev_copied);
-        if (copy_stream) cudaStreamDestroy(copy_stream);
+        for (cudaEvent_t e : {ev0, ev1, ev2, ev3})
+            if (e) cudaEventDestroy(e);
         if (stream) cudaStreamDestroy(stream);
     }
+
+    double *dt_back() const { return h_back.as<double>(); }
+    int32_t *status_back() const { return reinterpret_cast<int32_t *>(h_back.as<double>() + packed.size()); }
+    int32_t *list_flags() const { return reinterpret_cast<int32_t *>(h_back.as<char>() + h_back.cap) - 2; }
 
     size_t rsize() const { return precision == RICH_FP32_SPLIT ? sizeof(float) : sizeof(double); }
 
@@ -186,11 +194,11 @@ struct rich_batch {
         p.x = x[cur].as<double>(); p.y = y[cur].as<double>();
         p.xn = x[1 - cur].as<double>(); p.yn = y[1 - cur].as<double>();
         p.gx = gx.as<double>(); p.gy = gy.as<double>();
-        p.tri = tri.as<int32_t>(); p.cell_ptr = cell_ptr.as<int32_t>(); p.cell_order = corder.as<int32_t>();
-        p.slot_nb = slot_nb.as<int32_t>(); p.slot_tri = slot_tri.as<int32_t>(); p.slot_edge = slot_edge.as<int32_t>();
+        p.tri = tri.as<int32_t>(); p.cell_ptr = cell_ptr[mcur].as<int32_t>(); p.cell_order = corder.as<int32_t>();
+        p.slot_nb = slot_nb[mcur].as<int32_t>(); p.slot_tri = slot_tri.as<int32_t>(); p.slot_edge = slot_edge.as<int32_t>();
         p.edge_l = edge_l.as<int32_t>(); p.edge_r = edge_r.as<int32_t>();
         p.edge_ta = edge_ta.as<int32_t>(); p.edge_tb = edge_tb.as<int32_t>();
-        p.ghost_src = gsrc.as<int32_t>(); p.ghost_xf = gxf.as<int32_t>();
+        p.ghost_src = gsrc[mcur].as<int32_t>(); p.ghost_xf = gxf.as<int32_t>();
         p.ccx = ccx.as<double>(); p.ccy = ccy.as<double>(); p.A = A.as<double>();
         p.eL = eL.as<R>(); p.emlx = emlx.as<R>(); p.emly = emly.as<R>();
         p.emrx = emrx.as<R>(); p.emry = emry.as<R>();
@@ -242,6 +250,7 @@ rich::InstParams inst_params(const BatchSim &s, bool init)
     ip.remaining = s.t_end - s.t;
     ip.boundary = c.boundary; ip.motion = c.motion; ip.limiter = c.limiter;
     ip.init = init ? 1 : 0;
+    rich::mesh_params(rich::BoxConfig{c.boundary, c.x0, c.x1, c.y0, c.y1}, s.n, ip);
     return ip;
 }
 
@@ -292,6 +301,7 @@ void pack_part(rich_batch *b, BatchSim &s, const PackTask &t)
             b->h_gsrc[go + q] = (int32_t)(co + m.ghost_src[q]);
             b->h_gxf[go + q] = m.ghost_xf[q];
             b->h_gshift[go + q] = m.ghost_shift[q];
+            b->h_gimg[go + q] = m.ghost_img[q];
         }
         break;
     }
@@ -337,6 +347,7 @@ int ensure_device(rich_batch *b)
     CUDA_TRY(b->ePM.ensure(4 * E * r + 32));
     CUDA_TRY(b->instp.ensure(K * sizeof(rich::InstParams) + 8));
     CUDA_TRY(b->dtmin.ensure(K * 8 + 8)); CUDA_TRY(b->dtout.ensure(K * 8 + 8)); CUDA_TRY(b->status.ensure(K * 4 + 8));
+    CUDA_TRY(b->h_back.ensure(K * 12 + 64));
     CUDA_TRY(b->dsizes.ensure(sizeof(rich::DeviceSizes))); CUDA_TRY(b->gsync.ensure(sizeof(rich::GridSync)));
     (void)G;
     return RICH_OK;
@@ -446,27 +457,175 @@ template <class R> int run_persistent(rich_batch *b, int block)
     return RICH_OK;
 }
 
-// The sweep stage by stage; with read_moved the moved points and each
-// simulation's dt are copied into h_moved as soon as the point motion is
-// done (ev_copied marks their arrival) while the other stages run.
-int run_staged(rich_batch *b, bool read_moved = false)
+// The sweep stage by stage.
+int run_staged(rich_batch *b)
 {
     CUDA_TRY(cudaMemsetAsync(b->status.p, 0, b->status.cap, b->stream));
-    for (int k = 0; k < rich::NUM_STAGES; k++) {
-        b->launch(k, nullptr);
-        if (read_moved && k == rich::K_ADVANCE) {
-            const size_t N = (size_t)b->n_packed, I = b->packed.size();
-            double *h = b->h_moved.as<double>();
-            CUDA_TRY(cudaEventRecord(b->ev_moved, b->stream));
-            CUDA_TRY(cudaStreamWaitEvent(b->copy_stream, b->ev_moved, 0));
-            CUDA_TRY(cudaMemcpyAsync(h, b->x[1 - b->cur].p, N * 8, cudaMemcpyDeviceToHost, b->copy_stream));
-            CUDA_TRY(cudaMemcpyAsync(h + N, b->y[1 - b->cur].p, N * 8, cudaMemcpyDeviceToHost, b->copy_stream));
-            CUDA_TRY(cudaMemcpyAsync(h + 2 * N, b->dtout.p, I * 8, cudaMemcpyDeviceToHost, b->copy_stream));
-            CUDA_TRY(cudaEventRecord(b->ev_copied, b->copy_stream));
-        }
-    }
+    for (int k = 0; k < rich::NUM_STAGES; k++) b->launch(k, nullptr);
     CUDA_TRY(cudaGetLastError());
     b->staged_launches++;
+    return RICH_OK;
+}
+
+// The packed triangle and edge lists, built on the device from the rings of
+// buffers `mesh` (each cell's box type from its simulation's parameters),
+// with the builders' flags copied into h_back; the caller checks them before
+// any kernel reads the lists.
+int build_lists(rich_batch *b, int mesh)
+{
+    const size_t T = (size_t)b->nT, E = (size_t)b->nE, S = (size_t)b->nS;
+    CUDA_TRY(b->tri.ensure(T * 12 + 12));
+    CUDA_TRY(b->slot_tri.ensure(S * 4 + 4));
+    CUDA_TRY(b->slot_edge.ensure(S * 4 + 4));
+    for (DBuf *e : {&b->edge_l, &b->edge_r, &b->edge_ta, &b->edge_tb}) CUDA_TRY(e->ensure(E * 4 + 4));
+    CUDA_TRY(b->edgebad.ensure(8));
+    int32_t *bad = b->edgebad.as<int32_t>();
+    const int32_t N = (int32_t)b->n_packed;
+    const int32_t *ptr = b->cell_ptr[mesh].as<int32_t>(), *nb = b->slot_nb[mesh].as<int32_t>();
+    CUDA_TRY(rich::launch_build_tris(N, (int32_t)S, ptr, nb, b->toff.as<int32_t>(), b->tri.as<int32_t>(),
+                                     b->slot_tri.as<int32_t>(), bad + 1, b->stream));
+    CUDA_TRY(rich::launch_build_edges(N, (int32_t)S, ptr, nb, b->slot_tri.as<int32_t>(), b->gsrc[mesh].as<int32_t>(),
+                                      b->gshift.as<int32_t>(), b->eoff.as<int32_t>(), 0,
+                                      b->instp.as<rich::InstParams>(), b->cell_inst.as<int32_t>(),
+                                      b->slot_edge.as<int32_t>(), b->edge_l.as<int32_t>(), b->edge_r.as<int32_t>(),
+                                      b->edge_ta.as<int32_t>(), b->edge_tb.as<int32_t>(), bad, b->stream));
+    CUDA_TRY(cudaMemcpyAsync(b->list_flags(), bad, 8, cudaMemcpyDeviceToHost, b->stream));
+    return RICH_OK;
+}
+
+int check_lists(rich_batch *b)
+{
+    const int32_t *bad = b->list_flags();
+    if (bad[1]) return fail(RICH_ETESS, "a triangle of a ring is missing from its owner's ring");
+    if (bad[0]) return fail(RICH_ETESS, "an edge of a ring has no partner in the other cell's ring");
+    return RICH_OK;
+}
+
+rich::MeshArrays mesh_arrays(rich_batch *b, int q)
+{
+    rich::MeshArrays a{};
+    a.n = (int32_t)b->n_packed;
+    a.n_inst = (int32_t)b->packed.size();
+    a.inst = b->instp.as<rich::InstParams>();
+    a.cell_inst = b->cell_inst.as<int32_t>();
+    a.x = b->x[q].as<double>();
+    a.y = b->y[q].as<double>();
+    a.cell_ptr = b->cell_ptr[b->mcur].as<int32_t>();
+    a.slot_nb = b->slot_nb[b->mcur].as<int32_t>();
+    a.ghost_src = b->gsrc[b->mcur].as<int32_t>();
+    a.ghost_img = b->gimg[b->mcur].as<int32_t>();
+    return a;
+}
+
+// The updated meshes of the points in buffers q written, after the update's
+// first part was waited for; with `lists` (the next step has the same
+// simulations, as far as is known) the triangle and edge lists too.
+int finish_update(rich_batch *b, int q, bool lists)
+{
+    b->dev_mesh = b->dev_lists = false;
+    rich::MeshSizes z;
+    bool ok = false;
+    const rich::MeshArrays a = mesh_arrays(b, q);
+    CUDA_TRY(b->updater.settle(a, ok, z, b->stream));
+    if (!ok) return RICH_OK;
+    b->mesh_flag.assign(b->updater.flags(), b->updater.flags() + a.n_inst);
+    for (int32_t f : b->mesh_flag) lists = lists && !f;
+    const int m = 1 - b->mcur;
+    const size_t N = (size_t)b->n_packed, G = (size_t)z.ghosts + 1;
+    CUDA_TRY(b->cell_ptr[m].ensure((N + 1) * 4));
+    CUDA_TRY(b->slot_nb[m].ensure(((size_t)z.slots + 1) * 4));
+    CUDA_TRY(b->gsrc[m].ensure(G * 4)); CUDA_TRY(b->gimg[m].ensure(G * 4));
+    CUDA_TRY(b->gx.ensure(G * 8)); CUDA_TRY(b->gy.ensure(G * 8));
+    CUDA_TRY(b->gxf.ensure(G * 4)); CUDA_TRY(b->gshift.ensure(G * 4));
+    rich::MeshOutput o{};
+    o.cell_ptr = b->cell_ptr[m].as<int32_t>();
+    o.slot_nb = b->slot_nb[m].as<int32_t>();
+    o.tri_off = b->toff.as<int32_t>();
+    o.edge_off = b->eoff.as<int32_t>();
+    o.cell_order = b->corder.as<int32_t>();
+    o.gx = b->gx.as<double>();
+    o.gy = b->gy.as<double>();
+    o.ghost_src = b->gsrc[m].as<int32_t>();
+    o.ghost_xf = b->gxf.as<int32_t>();
+    o.ghost_shift = b->gshift.as<int32_t>();
+    o.ghost_img = b->gimg[m].as<int32_t>();
+    CUDA_TRY(b->updater.finish(a, o, b->stream));
+    b->mcur = m;
+    b->msz = z;
+    b->nG = z.ghosts;
+    b->nT = z.tris;
+    b->nE = z.edges;
+    b->nS = z.slots;
+    if (lists) {
+        int rc = build_lists(b, m);
+        if (rc) return rc;
+    }
+    b->dev_mesh = true;
+    b->dev_lists = lists;
+    return RICH_OK;
+}
+
+// The meshes of the simulations that go on, read back from the device into
+// their hm (with their points), for a step that packs other simulations.
+int read_meshes(rich_batch *b)
+{
+    const size_t N = (size_t)b->n_packed, G = (size_t)b->nG, S = (size_t)b->nS;
+    auto down = [&](auto &v, const DBuf &d, size_t k) -> cudaError_t {
+        if (v.size() < k) v.resize(k);
+        if (k == 0) return cudaSuccess;
+        return cudaMemcpyAsync(v.data(), d.p, k * sizeof(v[0]), cudaMemcpyDeviceToHost, b->stream);
+    };
+    const int m = b->mcur;
+    CUDA_TRY(down(b->h_dlx, b->x[b->cur], N)); CUDA_TRY(down(b->h_dly, b->y[b->cur], N));
+    CUDA_TRY(down(b->h_dptr, b->cell_ptr[m], N + 1)); CUDA_TRY(down(b->h_dnb, b->slot_nb[m], S));
+    CUDA_TRY(down(b->h_dtoff, b->toff, N + 1)); CUDA_TRY(down(b->h_deoff, b->eoff, N + 1));
+    CUDA_TRY(down(b->h_dorder, b->corder, N));
+    CUDA_TRY(down(b->h_dgx, b->gx, G)); CUDA_TRY(down(b->h_dgy, b->gy, G));
+    CUDA_TRY(down(b->h_dgsrc, b->gsrc[m], G)); CUDA_TRY(down(b->h_dgxf, b->gxf, G));
+    CUDA_TRY(down(b->h_dgshift, b->gshift, G)); CUDA_TRY(down(b->h_dgimg, b->gimg[m], G));
+    CUDA_TRY(cudaStreamSynchronize(b->stream));
+    // (ghosts follow their cells' order, so a simulation's are consecutive)
+    std::vector<int64_t> g0(b->packed.size() + 1, (int64_t)G);
+    for (size_t k = 0; k < b->packed.size(); k++)
+        g0[k] = std::lower_bound(b->h_dgsrc.begin(), b->h_dgsrc.begin() + G, (int32_t)b->packed[k]->cell_off) -
+                b->h_dgsrc.begin();
+    // a window of the processing order is 1024 packed cells: it may hold
+    // cells of two simulations, so each simulation's order is made again
+    b->pool->parallel_for((int64_t)b->packed.size(), [&](int64_t k) {
+        BatchSim *s = b->packed[k];
+        if (s->state != RUNNING || b->mesh_flag[k]) return;
+        const int64_t co = s->cell_off, n = s->n, go = g0[k], ge = g0[k + 1];
+        rich::HostMesh &h = s->hm;
+        h.n = s->n;
+        h.g = (int32_t)(ge - go);
+        auto slice = [&](auto &dst, const auto &src, int64_t i0, int64_t i1, int32_t shift) {
+            dst.resize(i1 - i0);
+            for (int64_t i = i0; i < i1; i++) dst[i - i0] = src[i] - shift;
+        };
+        const int32_t so = b->h_dptr[co], se = b->h_dptr[co + n];
+        slice(h.cell_ptr, b->h_dptr, co, co + n + 1, so);
+        slice(h.tri_off, b->h_dtoff, co, co + n + 1, b->h_dtoff[co]);
+        slice(h.edge_off, b->h_deoff, co, co + n + 1, b->h_deoff[co]);
+        h.n_tris = h.tri_off[n];
+        h.n_edges = h.edge_off[n];
+        h.slot_nb.resize(se - so);
+        for (int32_t q = so; q < se; q++) {
+            const int32_t id = b->h_dnb[q];
+            h.slot_nb[q - so] = id < (int32_t)N ? id - (int32_t)co : (int32_t)(n + (id - (int64_t)N - go));
+        }
+        slice(h.gx, b->h_dgx, go, ge, 0);
+        slice(h.gy, b->h_dgy, go, ge, 0);
+        slice(h.ghost_src, b->h_dgsrc, go, ge, (int32_t)co);
+        slice(h.ghost_xf, b->h_dgxf, go, ge, 0);
+        slice(h.ghost_shift, b->h_dgshift, go, ge, 0);
+        slice(h.ghost_img, b->h_dgimg, go, ge, 0);
+        h.cell_order.resize(n);
+        rich::degree_order((int32_t)n, h.cell_ptr.data(), h.cell_order.data());
+        std::memcpy(s->hx.data(), &b->h_dlx[co], sizeof(double) * n);
+        std::memcpy(s->hy.data(), &b->h_dly[co], sizeof(double) * n);
+        s->mesh_rc = 0;
+        s->prebuilt = true;
+    });
     return RICH_OK;
 }
 
@@ -522,10 +681,8 @@ int batch_create(int32_t precision, int64_t max_cells, int32_t host_threads, Thr
     b->precision = precision;
     b->max_cells = max_cells;
     if (cudaStreamCreateWithFlags(&b->stream, cudaStreamNonBlocking) != cudaSuccess ||
-        cudaStreamCreateWithFlags(&b->copy_stream, cudaStreamNonBlocking) != cudaSuccess ||
         cudaEventCreate(&b->ev0) != cudaSuccess || cudaEventCreate(&b->ev1) != cudaSuccess ||
-        cudaEventCreateWithFlags(&b->ev_moved, cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventCreateWithFlags(&b->ev_copied, cudaEventDisableTiming) != cudaSuccess) {
+        cudaEventCreate(&b->ev2) != cudaSuccess || cudaEventCreate(&b->ev3) != cudaSuccess) {
         delete b;
         return fail(RICH_ECUDA, "stream or event creation failed");
     }
@@ -621,16 +778,16 @@ void tessellate_members(rich_batch *b, const std::vector<BatchSim *> &sims)
     });
 }
 
-}  // namespace
-
-int rich_batch_step(rich_batch *b, rich_step_info *info)
+// Steps 1 to 5 of a step whose meshes are not all on the device: the points
+// and meshes of `list` on the host, packed, uploaded, and new simulations
+// initialised.  t1, t2: when the host tessellations began and ended.
+int pack_step(rich_batch *b, const std::vector<BatchSim *> &list, double &t1, double &t2)
 {
-    rich::Range range("rich batch step");
-    if (!b) return fail(RICH_EINVAL, "NULL handle");
-    if (info) std::memset(info, 0, sizeof(*info));
-    const double t0 = now_ms();
-    // 1. points of the running simulations back to the host (those whose
-    //    mesh was built during the last sweep have them already)
+    // 1. the meshes the device updated, and the points of the other running
+    //    simulations, back to the host
+    int rc;
+    if (b->dev_mesh && (rc = read_meshes(b))) return rc;
+    b->dev_mesh = b->dev_lists = false;
     bool need_points = false;
     for (BatchSim *s : b->packed) need_points |= s->state == RUNNING && !s->prebuilt;
     if (b->n_packed > 0 && need_points) {
@@ -651,21 +808,10 @@ int rich_batch_step(rich_batch *b, rich_step_info *info)
             std::memcpy(s->hy.data(), &hy[s->cell_off], sizeof(double) * s->n);
         });
     }
-    // the simulations of this step: running ones in their previous order, then new ones
-    std::vector<BatchSim *> list;
-    for (BatchSim *s : b->packed)
-        if (s->state == RUNNING) list.push_back(s);
-    for (auto &s : b->sims)
-        if (s->state == PENDING) list.push_back(s.get());
     for (BatchSim *s : list) s->prev_cell_off = s->state == RUNNING ? s->cell_off : -1;
-    if (list.empty()) {
-        b->packed.clear();
-        b->n_packed = 0;
-        return RICH_OK;
-    }
-    // 2. tessellations in parallel (of the simulations without a mesh
-    //    built during the last sweep)
-    const double t1 = now_ms();
+    // 2. tessellations in parallel (of the simulations whose mesh the device
+    //    did not have)
+    t1 = now_ms();
     {
         std::vector<BatchSim *> todo;
         for (BatchSim *s : list)
@@ -673,7 +819,7 @@ int rich_batch_step(rich_batch *b, rich_step_info *info)
         tessellate_members(b, todo);
         for (BatchSim *s : list) s->prebuilt = false;
     }
-    const double t2 = now_ms();
+    t2 = now_ms();
     std::vector<BatchSim *> ok;
     for (BatchSim *s : list) {
         if (s->mesh_rc == 0) {
@@ -721,6 +867,7 @@ int rich_batch_step(rich_batch *b, rich_step_info *info)
     b->h_cell_ptr.resize(N + 1); b->h_corder.resize(N);
     b->h_slot_nb.resize(so);
     b->h_eoff.resize(N + 1); b->h_toff.resize(N + 1); b->h_gshift.resize(go);
+    b->h_gimg.resize(go);
     if (any_pending) b->h_W0.assign(4 * N, 0.0);
     pack_all(b, ok);
     b->h_cell_ptr[N] = (int32_t)so;
@@ -729,8 +876,7 @@ int rich_batch_step(rich_batch *b, rich_step_info *info)
     b->h_inst.resize(ok.size());
     for (size_t k = 0; k < ok.size(); k++) b->h_inst[k] = inst_params(*ok[k], ok[k]->state == PENDING);
     // 4. device buffers and uploads
-    int rc = ensure_device(b);
-    if (rc) return rc;
+    if ((rc = ensure_device(b))) return rc;
     const int nxt = 1 - b->cur;
     if (!same_layout && n_old > 0) {
         // regather the conserved state of continuing simulations into the other
@@ -752,40 +898,20 @@ int rich_batch_step(rich_batch *b, rich_step_info *info)
     CUDA_TRY(upload(b->cell_inst, b->h_cell_inst, b->stream));
     CUDA_TRY(upload(b->gx, b->h_gx, b->stream));
     CUDA_TRY(upload(b->gy, b->h_gy, b->stream));
-    CUDA_TRY(upload(b->gsrc, b->h_gsrc, b->stream));
+    CUDA_TRY(upload(b->gsrc[b->mcur], b->h_gsrc, b->stream));
+    CUDA_TRY(upload(b->gimg[b->mcur], b->h_gimg, b->stream));
     CUDA_TRY(upload(b->gxf, b->h_gxf, b->stream));
-    CUDA_TRY(upload(b->cell_ptr, b->h_cell_ptr, b->stream));
+    CUDA_TRY(upload(b->cell_ptr[b->mcur], b->h_cell_ptr, b->stream));
     CUDA_TRY(upload(b->corder, b->h_corder, b->stream));
-    CUDA_TRY(upload(b->slot_nb, b->h_slot_nb, b->stream));
+    CUDA_TRY(upload(b->slot_nb[b->mcur], b->h_slot_nb, b->stream));
     CUDA_TRY(upload(b->toff, b->h_toff, b->stream));
     CUDA_TRY(upload(b->eoff, b->h_eoff, b->stream));
     CUDA_TRY(upload(b->gshift, b->h_gshift, b->stream));
     CUDA_TRY(upload(b->instp, b->h_inst, b->stream));
-    // the packed triangle and edge lists, built on the device from the rings
-    // (each cell's box type from its simulation's parameters); checked before
-    // any kernel reads them
-    {
-        CUDA_TRY(b->tri.ensure((size_t)to * 12 + 12));
-        CUDA_TRY(b->slot_tri.ensure((size_t)so * 4 + 4));
-        CUDA_TRY(b->slot_edge.ensure((size_t)so * 4 + 4));
-        for (DBuf *e : {&b->edge_l, &b->edge_r, &b->edge_ta, &b->edge_tb}) CUDA_TRY(e->ensure((size_t)eo * 4 + 4));
-        CUDA_TRY(b->edgebad.ensure(8));
-        int32_t *bad = b->edgebad.as<int32_t>();
-        CUDA_TRY(rich::launch_build_tris((int32_t)N, (int32_t)so, b->cell_ptr.as<int32_t>(), b->slot_nb.as<int32_t>(),
-                                         b->toff.as<int32_t>(), b->tri.as<int32_t>(), b->slot_tri.as<int32_t>(),
-                                         bad + 1, b->stream));
-        CUDA_TRY(rich::launch_build_edges((int32_t)N, (int32_t)so, b->cell_ptr.as<int32_t>(), b->slot_nb.as<int32_t>(),
-                                          b->slot_tri.as<int32_t>(), b->gsrc.as<int32_t>(), b->gshift.as<int32_t>(),
-                                          b->eoff.as<int32_t>(), 0, b->instp.as<rich::InstParams>(),
-                                          b->cell_inst.as<int32_t>(), b->slot_edge.as<int32_t>(),
-                                          b->edge_l.as<int32_t>(), b->edge_r.as<int32_t>(), b->edge_ta.as<int32_t>(),
-                                          b->edge_tb.as<int32_t>(), bad, b->stream));
-        int32_t bad_h[2] = {0, 0};
-        CUDA_TRY(cudaMemcpyAsync(bad_h, bad, 8, cudaMemcpyDeviceToHost, b->stream));
-        CUDA_TRY(cudaStreamSynchronize(b->stream));
-        if (bad_h[1]) return fail(RICH_ETESS, "a triangle of a ring is missing from its owner's ring");
-        if (bad_h[0]) return fail(RICH_ETESS, "an edge of a ring has no partner in the other cell's ring");
-    }
+    // the packed triangle and edge lists, checked before any kernel reads them
+    if ((rc = build_lists(b, b->mcur))) return rc;
+    CUDA_TRY(cudaStreamSynchronize(b->stream));
+    if ((rc = check_lists(b))) return rc;
     CUDA_TRY(cudaMemsetAsync(b->status.p, 0, ok.size() * 4, b->stream));
     if (any_pending) CUDA_TRY(upload(b->initW, b->h_W0, b->stream));
     // 5. admission: conserved variables of new simulations from their first geometry
@@ -802,44 +928,57 @@ int rich_batch_step(rich_batch *b, rich_step_info *info)
         for (size_t k = 0; k < ok.size(); k++) b->h_inst[k].init = 0;
         CUDA_TRY(upload(b->instp, b->h_inst, b->stream));
     }
+    return RICH_OK;
+}
+
+}  // namespace
+
+int rich_batch_step(rich_batch *b, rich_step_info *info)
+{
+    rich::Range range("rich batch step");
+    if (!b) return fail(RICH_EINVAL, "NULL handle");
+    if (info) std::memset(info, 0, sizeof(*info));
+    const double t0 = now_ms();
+    // the simulations of this step: running ones in their previous order, then new ones
+    std::vector<BatchSim *> list;
+    for (BatchSim *s : b->packed)
+        if (s->state == RUNNING) list.push_back(s);
+    for (auto &s : b->sims)
+        if (s->state == PENDING) list.push_back(s.get());
+    if (list.empty()) {
+        b->packed.clear();
+        b->n_packed = 0;
+        b->dev_mesh = b->dev_lists = false;
+        return RICH_OK;
+    }
+    int rc;
+    double t1 = now_ms(), t2 = t1;
+    if (b->dev_lists && list == b->packed) {
+        // their meshes, lists and points are on the device already
+        for (size_t k = 0; k < list.size(); k++) b->h_inst[k] = inst_params(*list[k], false);
+        CUDA_TRY(cudaStreamSynchronize(b->stream));
+        if ((rc = check_lists(b))) return rc;
+        b->dev_mesh = b->dev_lists = false;
+        if ((rc = ensure_device(b))) return rc;
+        CUDA_TRY(upload(b->instp, b->h_inst, b->stream));
+    } else if ((rc = pack_step(b, list, t1, t2))) {
+        return rc;
+    }
+    if (b->packed.empty()) return RICH_OK;
     const double t3 = now_ms();
-    // 6. the sweep over every cell of every simulation; staged, its moved
-    //    points are read back once the point motion is done, and the host
-    //    tessellates them for the next step while the device finishes
+    // 6. the sweep over every cell of every simulation, then the first part
+    //    of the mesh update for the moved points (one wait for both)
+    const std::vector<BatchSim *> ok = b->packed;
+    const size_t N = (size_t)b->n_packed;
     const LaunchShape shape = pick_shape(b);
-    if (!shape.persistent) CUDA_TRY(b->h_moved.ensure((2 * N + ok.size() + 1) * sizeof(double)));
     CUDA_TRY(cudaEventRecord(b->ev0, b->stream));
     if (shape.persistent) {
         rc = b->precision == RICH_FP32_SPLIT ? run_persistent<float>(b, shape.block) : run_persistent<double>(b, shape.block);
     } else {
-        rc = run_staged(b, true);
+        rc = run_staged(b);
     }
     if (rc) return rc;
     CUDA_TRY(cudaEventRecord(b->ev1, b->stream));
-    double t_pre = 0.0;
-    if (!shape.persistent) {
-        CUDA_TRY(cudaEventSynchronize(b->ev_copied));
-        const double tp = now_ms();
-        const double *h = b->h_moved.as<double>();
-        // the simulations that go on after this step (the bookkeeping below
-        // takes the same decision), unless the step fails
-        std::vector<BatchSim *> next;
-        for (size_t k = 0; k < ok.size(); k++) {
-            BatchSim *s = ok[k];
-            const double dt = h[2 * N + k], rem = s->t_end - s->t;
-            const double tn = dt >= rem ? s->t_end : s->t + dt;
-            if (tn >= s->t_end || s->steps + 1 >= s->max_steps) continue;
-            next.push_back(s);
-        }
-        b->pool->parallel_for((int64_t)next.size(), [&](int64_t k) {
-            BatchSim *s = next[k];
-            std::memcpy(s->hx.data(), h + s->cell_off, sizeof(double) * s->n);
-            std::memcpy(s->hy.data(), h + N + s->cell_off, sizeof(double) * s->n);
-        });
-        tessellate_members(b, next);
-        for (BatchSim *s : next) s->prebuilt = true;
-        t_pre = now_ms() - tp;
-    }
     if (shape.persistent) {
         int32_t timeout = 0;
         CUDA_TRY(cudaMemcpyAsync(&timeout, (char *)b->gsync.p + offsetof(rich::GridSync, timeout), 4,
@@ -856,22 +995,27 @@ int rich_batch_step(rich_batch *b, rich_step_info *info)
             CUDA_TRY(cudaEventRecord(b->ev1, b->stream));
         }
     }
-    b->h_dt.resize(ok.size());
-    b->h_status.resize(ok.size());
-    CUDA_TRY(cudaMemcpyAsync(b->h_dt.data(), b->dtout.p, ok.size() * 8, cudaMemcpyDeviceToHost, b->stream));
-    CUDA_TRY(cudaMemcpyAsync(b->h_status.data(), b->status.p, ok.size() * 4, cudaMemcpyDeviceToHost, b->stream));
+    const bool update = (int64_t)N >= rich::kMeshUpdateMin && (int64_t)N <= rich::kMeshUpdateMax;
+    CUDA_TRY(cudaEventRecord(b->ev2, b->stream));
+    if (update) CUDA_TRY(b->updater.start(mesh_arrays(b, 1 - b->cur), b->stream));
+    CUDA_TRY(cudaEventRecord(b->ev3, b->stream));
+    CUDA_TRY(cudaMemcpyAsync(b->dt_back(), b->dtout.p, ok.size() * 8, cudaMemcpyDeviceToHost, b->stream));
+    CUDA_TRY(cudaMemcpyAsync(b->status_back(), b->status.p, ok.size() * 4, cudaMemcpyDeviceToHost, b->stream));
     CUDA_TRY(cudaStreamSynchronize(b->stream));
     float ms = 0.0f;
     cudaEventElapsedTime(&ms, b->ev0, b->ev1);
     record_timing(b, shape, ms);
+    float up_ms = 0.0f;
+    cudaEventElapsedTime(&up_ms, b->ev2, b->ev3);
     // 7. per-simulation bookkeeping; a failed step keeps that simulation's old state
     const int nxt2 = 1 - b->cur;
     const double tnow = now_ms();
+    const int32_t *status = b->status_back();
+    size_t going = 0;
     for (size_t k = 0; k < ok.size(); k++) {
         BatchSim *s = ok[k];
-        if (b->h_status[k]) {
-            s->prebuilt = false;
-            s->err = (b->h_status[k] & rich::ST_NAN) ? RICH_ENAN : RICH_ENEGATIVE;
+        if (status[k]) {
+            s->err = (status[k] & rich::ST_NAN) ? RICH_ENAN : RICH_ENEGATIVE;
             s->err_msg = "step rejected (non-finite, non-positive mass or thermal energy, or a point left the box)";
             finish_copy_out(b, *s, b->cur);
             s->state = FAILED;
@@ -880,7 +1024,7 @@ int rich_batch_step(rich_batch *b, rich_step_info *info)
             continue;
         }
         const double rem = s->t_end - s->t;
-        s->last_dt = b->h_dt[k];
+        s->last_dt = b->dt_back()[k];
         s->t = s->last_dt >= rem ? s->t_end : s->t + s->last_dt;
         s->steps++;
         if (s->t >= s->t_end || s->steps >= s->max_steps) {
@@ -888,15 +1032,21 @@ int rich_batch_step(rich_batch *b, rich_step_info *info)
             s->state = DONE;
             s->t_finish = tnow;
             b->cells_admitted -= s->n;
+        } else {
+            going++;
         }
     }
-    CUDA_TRY(cudaStreamSynchronize(b->stream));
+    if (going < ok.size()) CUDA_TRY(cudaStreamSynchronize(b->stream));
     b->cur = nxt2;
+    // 8. the updated meshes of the simulations that go on
+    const double tf = now_ms();
+    if (update && going > 0 && (rc = finish_update(b, nxt2, going == ok.size()))) return rc;
+    const double t_fin = now_ms() - tf;
     if (info) {
         info->steps_done = (int64_t)ok.size();
         info->sweep_ms = ms;
-        info->tess_ms = (t2 - t1) + t_pre;
-        info->copy_ms = (t1 - t0) + (t3 - t2) + (now_ms() - tnow);
+        info->tess_ms = (t2 - t1) + up_ms + t_fin;
+        info->copy_ms = (t1 - t0) + (t3 - t2) + (now_ms() - tnow) - t_fin;
         info->n_ghost = b->nG;
         info->n_tri = b->nT;
         info->n_edges = b->nE;

@@ -1,0 +1,774 @@
+// Update of a tessellation for moved points (a0), per-cell bodies shared by
+// the device kernels (meshupdate.cu) and a serial host run that checks them
+// (meshupdate_host.cpp).
+//
+// The mesh is the set of stars: every real cell's ring of Delaunay
+// neighbours in counter-clockwise order.  Between steps the points move a
+// fraction of a cell, and 0.01-2.6 % of the triangles change, so
+//   verify    every cell checks its own star at the new positions: triangles
+//             counter-clockwise, one turn, every edge locally Delaunay, the
+//             circumdisks inside the ghost band; the cells of a failed check
+//             are listed;
+//   recompute a listed cell builds its star again by gift wrapping over the
+//             sources of its ring and of its neighbours' rings (and their
+//             images, near a wall);
+//   check     a new star's triangles must be in the rings of their other two
+//             vertices, and a dropped neighbour must have dropped the cell;
+//             where not, the cells involved are listed for another round and
+//             told of the vertices they lack.
+// This is star splaying (Shewchuk, "Star splaying: an algorithm for
+// repairing Delaunay triangulations and convex hulls", 2005): stars that
+// are all locally Delaunay and agree with each other form the Delaunay
+// triangulation, which the symbolic tie-break makes unique, so the result is
+// the host builder's mesh, ring for ring.  What the bodies do not handle (a
+// circumdisk beyond the ghost band, more than kMaxDeg neighbours, rounds that
+// do not converge, coordinates the exact predicates cannot hold) sets a flag,
+// and the caller builds that mesh on the host.
+//
+// Neighbours are references src * 16 + img: the image img = (a + 1) +
+// 3 (b + 1), a, b in {-1, 0, 1}, of real cell src (4: the cell itself).  In a
+// periodic box every neighbour is the source's image nearest to the cell,
+// which holds while circumdisks are smaller than a quarter of the box
+// (checked); across walls the image is part of the reference.
+//
+// Predicates: the sign of a determinant is taken from FP32 when it exceeds
+// its error bound (FP64 runs at 1/64 of the FP32 rate on GB300; fewer than
+// one edge in 10^4 goes on), else from FP64 with the host's bounds, else from
+// exact integers.  This file must be compiled without floating-point
+// contraction.
+#pragma once
+
+#include <cmath>
+#include <cstdint>
+
+#include "exactint.h"
+#include "mesh.h"
+#include "predicates.h"
+#include "sweep.cuh"
+
+namespace rich {
+
+constexpr int kMaxDeg = 32;     // neighbours of a recomputed cell
+constexpr int kMaxCand = 96;    // candidates of a recomputed cell
+constexpr int kMaxExtra = 8;    // vertices another cell can tell it of per round
+constexpr int kMaxRounds = 12;  // rounds before the host takes over
+
+enum : int32_t {
+    MU_FAR = 1,       // a circumdisk near or beyond the ghost band
+    MU_SIZE = 2,      // too many candidates, neighbours or recomputed cells
+    MU_STAR = 4,      // a star did not close (coincident points)
+    MU_EXACT = 8,     // coordinates beyond the exact predicates' grid
+    MU_IMAGE = 16,    // a neighbour image outside the ghost band
+};
+
+// Counters of one update (device memory, cleared at its start).
+struct MeshUpdateCount {
+    int32_t listed[kMaxRounds + 1];  // cells listed for each round
+    int32_t overrides;               // cells recomputed so far
+    int32_t slots, edges, tris, ghosts;
+};
+
+struct MeshUpdate {
+    int32_t n, n_inst;
+    const InstParams *inst;
+    const int32_t *cell_inst;  // nullptr: one simulation
+    const double *x, *y;       // new positions of the real cells
+    // the mesh being updated
+    const int32_t *cell_ptr, *slot_nb, *ghost_src, *ghost_img;
+    // cells listed: stamp of the round a cell was last listed for, and the
+    // rounds' lists (alternating).  Stamps grow from update to update, so
+    // nothing is cleared between them.
+    int32_t stamp;
+    int32_t *mark, *list[2];
+    // recomputed stars: per cell (stamp << 2 | first << 1 | version) of its
+    // last recomputation and its place, per place two versions of the ring
+    int32_t *ring_info, *ring_at;
+    int32_t max_rings;
+    int32_t *ring_deg, *ring_ref;
+    // vertices other cells found missing from a listed cell's star
+    int32_t *extra_n, *extra;
+    MeshUpdateCount *count;
+    // MU_* of each simulation: a flagged one lists no more cells, and its
+    // mesh is left to the host builder
+    int32_t *flags;
+    // per cell: owned edges, triangles, ghost images, degree (8 bits each)
+    // and the mask of its images inside the ghost band
+    uint32_t *sizes;
+    uint16_t *images;
+    // the updated mesh
+    int32_t *out_ptr, *out_nb, *tri_off, *edge_off, *ghost_off;
+    double *gx, *gy;
+    int32_t *gsrc, *gxf, *gshift, *gimg;
+};
+
+namespace mu {
+
+#ifdef __CUDA_ARCH__
+__device__ __forceinline__ int32_t a_exch(int32_t *p, int32_t v) { return atomicExch(p, v); }
+__device__ __forceinline__ int32_t a_add(int32_t *p, int32_t v) { return atomicAdd(p, v); }
+__device__ __forceinline__ void a_or(int32_t *p, int32_t v) { atomicOr(p, v); }
+__device__ __forceinline__ int32_t vol(const int32_t *p) { return *(const volatile int32_t *)p; }
+#else
+inline int32_t a_exch(int32_t *p, int32_t v) { const int32_t o = *p; *p = v; return o; }
+inline int32_t a_add(int32_t *p, int32_t v) { const int32_t o = *p; *p += v; return o; }
+inline void a_or(int32_t *p, int32_t v) { *p |= v; }
+inline int32_t vol(const int32_t *p) { return *p; }
+#endif
+
+// a < b by an order-preserving integer key (FP64 compares issue on the FP64 pipe)
+RICH_HD inline bool less(double a, double b)
+{
+#ifdef __CUDA_ARCH__
+    long long p = __double_as_longlong(a), q = __double_as_longlong(b);
+    p ^= (p >> 63) & 0x7fffffffffffffffll;
+    q ^= (q >> 63) & 0x7fffffffffffffffll;
+    p = p == -1 ? 0 : p;
+    q = q == -1 ? 0 : q;
+    return p < q;
+#else
+    return a < b;
+#endif
+}
+
+RICH_HD inline double image_coord(double v, double lo, double hi, int a, bool periodic)
+{
+    if (a == 0) return v;
+    if (!periodic) return a < 0 ? (lo + lo) - v : (hi + hi) - v;
+    return a > 0 ? v + (hi - lo) : v - (hi - lo);
+}
+
+// One cell's frame: its position, its simulation's box, and a length scale
+// that keeps FP32 products of neighbour offsets in range.
+struct Frame {
+    const MeshUpdate *m;
+    int32_t i;
+    int32_t *flags;
+    double xi, yi;
+    double x0, x1, y0, y1, hx, hy;  // box and half its sides
+    float scale, rlim2, rper2, reach;
+    bool periodic;
+};
+
+RICH_HD inline int32_t inst_at(const MeshUpdate &m, int32_t i) { return m.cell_inst ? m.cell_inst[i] : 0; }
+
+RICH_HD inline Frame frame_of(const MeshUpdate &m, int32_t i)
+{
+    const int32_t k = inst_at(m, i);
+    const InstParams &ip = m.inst[k];
+    Frame f;
+    f.flags = m.flags + k;
+    f.m = &m;
+    f.i = i;
+    f.xi = m.x[i];
+    f.yi = m.y[i];
+    f.x0 = ip.x0; f.x1 = ip.x1; f.y0 = ip.y0; f.y1 = ip.y1;
+    f.hx = ip.half_x; f.hy = ip.half_y;
+    f.scale = ip.mesh_scale;
+    f.rlim2 = ip.mesh_rlim2;
+    f.rper2 = ip.mesh_rper2;
+    f.reach = ip.mesh_reach;
+    f.periodic = ip.boundary == 1;
+    return f;
+}
+
+struct Point {
+    double x, y;     // absolute position (as the host's ghost list has it)
+    float fx, fy, l;  // scaled offset from the cell and its square
+    int32_t ref;
+};
+
+RICH_HD inline float to_float(double v)
+{
+#ifdef __CUDA_ARCH__
+    return __double2float_rn(v);
+#else
+    return (float)v;
+#endif
+}
+
+// the point of a reference; in a periodic box the source's nearest image
+// (whatever image the reference names)
+RICH_HD inline Point point_of(const Frame &f, int32_t ref)
+{
+    const int32_t src = ref >> 4;
+    Point p;
+    p.x = f.m->x[src];
+    p.y = f.m->y[src];
+    double dx, dy;
+    if (f.periodic) {
+        dx = p.x - f.xi;
+        dy = p.y - f.yi;
+        int a = 0, b = 0;
+        if (less(f.hx, dx)) a = -1;
+        else if (less(dx, -f.hx)) a = 1;
+        if (less(f.hy, dy)) b = -1;
+        else if (less(dy, -f.hy)) b = 1;
+        if (a) {
+            p.x = image_coord(p.x, f.x0, f.x1, a, true);
+            dx = p.x - f.xi;
+        }
+        if (b) {
+            p.y = image_coord(p.y, f.y0, f.y1, b, true);
+            dy = p.y - f.yi;
+        }
+        p.ref = src * 16 + (a + 1) + 3 * (b + 1);
+    } else {
+        const int32_t img = ref & 15;
+        if (img != 4) {
+            p.x = image_coord(p.x, f.x0, f.x1, img % 3 - 1, false);
+            p.y = image_coord(p.y, f.y0, f.y1, img / 3 - 1, false);
+        }
+        dx = p.x - f.xi;
+        dy = p.y - f.yi;
+        p.ref = ref;
+    }
+    p.fx = to_float(dx) * f.scale;
+    p.fy = to_float(dy) * f.scale;
+    p.l = p.fx * p.fx + p.fy * p.fy;
+    return p;
+}
+
+// FP32 determinants of offsets: relative error of a product of k rounded
+// factors below (2 k + 2) 2^-24 of the permanent; the bounds are a few times
+// that.
+constexpr float kCrossBound = 1e-6f;
+constexpr float kCircleBound = 3e-6f;
+
+#ifdef __CUDA_ARCH__
+#define RICH_MU_SLOW __device__ __noinline__
+#else
+#define RICH_MU_SLOW inline
+#endif
+
+// orientation of a, b, c from FP64 with the host's bound, else exact
+// (0 with MU_EXACT set when the integers cannot hold it)
+RICH_MU_SLOW int orient_slow(int32_t *flags, double ax, double ay, double bx, double by, double cx, double cy)
+{
+    const double l = (bx - ax) * (cy - ay), r = (by - ay) * (cx - ax);
+    const double det = l - r, bound = kOrientBound * (fabs(l) + fabs(r));
+    if (det > bound) return 1;
+    if (-det > bound) return -1;
+    const int s = exactint::orient_sign(ax, ay, bx, by, cx, cy);
+    if (s == exactint::kUnknown) a_or(flags, MU_EXACT);
+    return s == exactint::kUnknown ? 0 : s;
+}
+
+RICH_HD inline bool lex_less(double px, double py, double qx, double qy)
+{
+    return px < qx || (px == qx && py < qy);
+}
+
+// in-circle of counter-clockwise a, b, c and d, likewise, with the symbolic
+// tie-break of predicates.h: > 0 when d is inside
+RICH_MU_SLOW int circle_slow(int32_t *flags, double ax, double ay, double bx, double by, double cx, double cy,
+                             double dx, double dy)
+{
+    {
+        const double adx = ax - dx, ady = ay - dy, bdx = bx - dx, bdy = by - dy, cdx = cx - dx, cdy = cy - dy;
+        const double p1 = bdx * cdy, p2 = cdx * bdy, p3 = cdx * ady, p4 = adx * cdy, p5 = adx * bdy, p6 = bdx * ady;
+        const double la = adx * adx + ady * ady, lb = bdx * bdx + bdy * bdy, lc = cdx * cdx + cdy * cdy;
+        const double det = la * (p1 - p2) + lb * (p3 - p4) + lc * (p5 - p6);
+        const double bound = kIncircleBound * (la * (fabs(p1) + fabs(p2)) + lb * (fabs(p3) + fabs(p4)) +
+                                               lc * (fabs(p5) + fabs(p6)));
+        // (infinities and NaNs fail the comparisons)
+        if (det > bound && det < 1e300) return 1;
+        if (-det > bound && -det < 1e300) return -1;
+    }
+    const int s = exactint::incircle_sign(ax, ay, bx, by, cx, cy, dx, dy);
+    if (s == exactint::kUnknown) {
+        a_or(flags, MU_EXACT);
+        return 0;
+    }
+    if (s) return s;
+    int k = 0;
+    double mx = ax, my = ay;
+    if (lex_less(bx, by, mx, my)) { k = 1; mx = bx; my = by; }
+    if (lex_less(cx, cy, mx, my)) { k = 2; mx = cx; my = cy; }
+    if (lex_less(dx, dy, mx, my)) { k = 3; }
+    switch (k) {
+    case 0: return orient_slow(flags, bx, by, cx, cy, dx, dy);
+    case 1: return -orient_slow(flags, ax, ay, cx, cy, dx, dy);
+    case 2: return orient_slow(flags, ax, ay, bx, by, dx, dy);
+    default: return -orient_slow(flags, ax, ay, bx, by, cx, cy);
+    }
+}
+
+RICH_HD inline int orient_slow(const Frame &f, const Point &a, const Point &b)
+{
+    return orient_slow(f.flags, f.xi, f.yi, a.x, a.y, b.x, b.y);
+}
+
+// d against the circle of the counter-clockwise (cell, a, b)
+RICH_HD inline int circle_slow(const Frame &f, const Point &a, const Point &b, const Point &d)
+{
+    return circle_slow(f.flags, f.xi, f.yi, a.x, a.y, b.x, b.y, d.x, d.y);
+}
+
+// Whether the circumdisk of (cell, a, b) is certainly inside the ghost band
+// (and, in a periodic box, smaller than a quarter of it).  A disk through
+// the cell reaches past a wall by less than its diameter, so a radius below
+// 0.48 bands is enough; larger disks are placed.  In FP32, with margins of
+// 2 %.
+RICH_HD inline bool disk_ok(const Frame &f, const Point &a, const Point &b)
+{
+    const float cr = a.fx * b.fy - a.fy * b.fx;
+    const float ex = a.fx - b.fx, ey = a.fy - b.fy;
+    const float q = a.l * b.l * (ex * ex + ey * ey), c4 = 4.0f * cr * cr;
+    if (q <= c4 * f.rlim2) return true;
+    if (!(q <= c4 * f.rper2)) return false;
+    const float i2 = 0.5f / cr;
+    const float ux = (b.fy * a.l - a.fy * b.l) * i2, uy = (a.fx * b.l - b.fx * a.l) * i2;
+    const float R = sqrtf(ux * ux + uy * uy) * 1.001f;
+    const float lx = to_float(f.xi - f.x0) * f.scale, rx = to_float(f.x1 - f.xi) * f.scale;
+    const float ly = to_float(f.yi - f.y0) * f.scale, ry = to_float(f.y1 - f.yi) * f.scale;
+    return R - ux - lx <= f.reach && R + ux - rx <= f.reach && R - uy - ly <= f.reach && R + uy - ry <= f.reach;
+}
+
+// List a cell for the round of `stamp` (once).
+RICH_HD inline void list_cell(const MeshUpdate &m, int32_t v, int32_t round)
+{
+    if (vol(m.flags + inst_at(m, v)) || vol(m.mark + v) == m.stamp + round || a_exch(m.mark + v, m.stamp + round) == m.stamp + round) return;
+    m.list[round & 1][a_add(&m.count->listed[round], 1)] = v;
+}
+
+RICH_HD inline int32_t base_ref(const MeshUpdate &m, int32_t q)
+{
+    return q < m.n ? q * 16 + 4 : m.ghost_src[q - m.n] * 16 + m.ghost_img[q - m.n];
+}
+
+// A cell's ring as another cell sees it.  While round `computing` is being
+// recomputed its cells still show their previous star (-1: their latest).
+struct Ring {
+    const MeshUpdate *m;
+    const int32_t *p;
+    int32_t deg;
+    bool base;
+    RICH_HD int32_t operator[](int32_t k) const { return base ? base_ref(*m, p[k]) : p[k]; }
+};
+
+RICH_HD inline Ring ring_of(const MeshUpdate &m, int32_t v, int32_t computing)
+{
+    const int32_t info = vol(m.ring_info + v);
+    bool base = (info >> 2) < m.stamp;
+    int ver = info & 1;
+    if (!base && computing >= 0 && (info >> 2) == m.stamp + computing) {
+        if (info & 2) base = true;
+        else ver ^= 1;
+    }
+    Ring r;
+    r.m = &m;
+    r.base = base;
+    if (base) {
+        r.p = m.slot_nb + m.cell_ptr[v];
+        r.deg = m.cell_ptr[v + 1] - m.cell_ptr[v];
+    } else {
+        const int32_t at = 2 * m.ring_at[v] + ver;
+        r.p = m.ring_ref + (int64_t)at * kMaxDeg;
+        r.deg = m.ring_deg[at];
+    }
+    return r;
+}
+
+// ---- the bodies --------------------------------------------------------------
+
+// Cell i's star at the new positions.
+RICH_HD inline void verify(const MeshUpdate &m, int32_t i)
+{
+    const Frame f = frame_of(m, i);
+    const int32_t lo = m.cell_ptr[i], deg = m.cell_ptr[i + 1] - lo;
+    const int32_t *nb = m.slot_nb + lo;
+    if (!f.periodic) {
+        // a cell with mirror images: their coordinates are rounded, so its
+        // star is always built again
+        bool wall = false;
+        for (int32_t k = 0; k < deg; k++) wall |= nb[k] >= m.n;
+        if (wall) {
+            list_cell(m, i, 0);
+            return;
+        }
+    }
+    Point a = point_of(f, base_ref(m, nb[deg - 2])), b = point_of(f, base_ref(m, nb[deg - 1]));
+    float cab;
+    {
+        // (a x b: the orientation of the triangle before the first)
+        cab = a.fx * b.fy - a.fy * b.fx;
+    }
+    int turns = 0;
+    bool self = false;
+    for (int32_t k = 0; k < deg; k++) {
+        const int32_t ref = base_ref(m, nb[k]);
+        const Point d = point_of(f, ref);
+        const float p = b.fx * d.fy, q = b.fy * d.fx, cbd = p - q;
+        bool bad = false;
+        if (!(cbd > kCrossBound * (fabsf(p) + fabsf(q)))) bad = orient_slow(f, b, d) <= 0;
+        if (!bad) {
+            const float p3 = a.fx * d.fy, p4 = a.fy * d.fx, p5 = a.fx * b.fy, p6 = a.fy * b.fx;
+            const float det = a.l * cbd - b.l * (p3 - p4) + d.l * cab;
+            const float bound = kCircleBound * (a.l * (fabsf(p) + fabsf(q)) + b.l * (fabsf(p3) + fabsf(p4)) +
+                                                d.l * (fabsf(p5) + fabsf(p6)));
+            if (!(det > bound)) bad = -det > bound || circle_slow(f, a, b, d) >= 0;
+        }
+        if (bad) {
+            list_cell(m, a.ref >> 4, 0);
+            list_cell(m, b.ref >> 4, 0);
+            list_cell(m, d.ref >> 4, 0);
+            self = true;
+        }
+        // another image than the mesh had, or a disk near the band's edge:
+        // this cell alone
+        if (d.ref != ref || !disk_ok(f, b, d)) self = true;
+        turns += (b.fy < 0.0f && d.fy >= 0.0f) ? 1 : 0;
+        a = b;
+        b = d;
+        cab = cbd;
+    }
+    if (self || turns != 1) list_cell(m, i, 0);
+}
+
+// Cell i's star built again from the candidates around it.
+RICH_HD inline void recompute(const MeshUpdate &m, int32_t i, int32_t round)
+{
+    const Frame f = frame_of(m, i);
+    int32_t src[kMaxCand];
+    int ns = 0;
+    uint32_t imgs = 1u << 4;
+    bool full = false;
+    auto add = [&](int32_t s) {
+        for (int k = 0; k < ns; k++)
+            if (src[k] == s) return;
+        if (ns == kMaxCand) full = true;
+        else src[ns++] = s;
+    };
+    // sources of the ring and of what others reported, then of their rings
+    const Ring own = ring_of(m, i, round);
+    for (int32_t k = 0; k < own.deg; k++) {
+        const int32_t r = own[k];
+        imgs |= 1u << (r & 15);
+        if ((r >> 4) != i) add(r >> 4);
+    }
+    const int32_t told = m.extra_n[i], ne = told < kMaxExtra ? told : kMaxExtra;
+    m.extra_n[i] = 0;
+    for (int32_t k = 0; k < ne; k++) {
+        const int32_t r = m.extra[(int64_t)i * kMaxExtra + k];
+        imgs |= 1u << (r & 15);
+        if ((r >> 4) != i) add(r >> 4);
+    }
+    const int first = ns;
+    for (int k = 0; k < first; k++) {
+        const Ring r = ring_of(m, src[k], round);
+        for (int32_t j = 0; j < r.deg; j++) {
+            const int32_t q = r[j];
+            imgs |= 1u << (q & 15);
+            if ((q >> 4) != i) add(q >> 4);
+        }
+    }
+    // the candidates: nearest images, or every source's images across the
+    // walls that any of these rings meets (the cell's own images too)
+    int32_t ref[kMaxCand];
+    float fx[kMaxCand], fy[kMaxCand], fl[kMaxCand];
+    int nc = 0;
+    int near = -1;
+    double dmin = 0.0;
+    auto put = [&](int32_t r) {
+        if (nc == kMaxCand) {
+            full = true;
+            return;
+        }
+        const Point p = point_of(f, r);
+        ref[nc] = p.ref;
+        fx[nc] = p.fx;
+        fy[nc] = p.fy;
+        fl[nc] = p.l;
+        const double dx = p.x - f.xi, dy = p.y - f.yi, d2 = dx * dx + dy * dy;
+        if (near < 0 || d2 < dmin) {
+            near = nc;
+            dmin = d2;
+        }
+        nc++;
+    };
+    for (int k = 0; k < ns; k++) put(src[k] * 16 + 4);
+    if (!f.periodic && imgs != 1u << 4)
+        for (int img = 0; img < 9; img++) {
+            if (img == 4 || !(imgs >> img & 1)) continue;
+            put(i * 16 + img);
+            for (int k = 0; k < ns; k++) put(src[k] * 16 + img);
+        }
+    if (full || nc < 3) {
+        a_or(f.flags, MU_SIZE);
+        return;
+    }
+    auto point = [&](int k) {
+        Point p;
+        p.fx = fx[k];
+        p.fy = fy[k];
+        p.l = fl[k];
+        p.ref = ref[k];
+        return p;
+    };
+    // (FP32 in-circle: with offsets from the cell, d is inside the circle of
+    // the counter-clockwise (cell, a, b) when |a|^2 (b x d) - |b|^2 (a x d) +
+    // |d|^2 (a x b) < 0)
+    // the absolute coordinates, wanted only by the slow predicates
+    auto whole = [&](int k) { return point_of(f, ref[k]); };
+    // gift wrapping from the nearest candidate (always a neighbour): the next
+    // one is the point to the left of the last whose circle with the cell and
+    // the last is empty
+    int32_t out[kMaxDeg];
+    int deg = 0, last = near, turns = 0;
+    bool bad = false;
+    do {
+        if (deg == kMaxDeg) {
+            bad = true;
+            break;
+        }
+        out[deg++] = ref[last];
+        const Point a = point(last);
+        int best = -1;
+        for (int k = 0; k < nc; k++) {
+            if (k == last) continue;
+            const float p = a.fx * fy[k], q = a.fy * fx[k], c = p - q;
+            const float cb = kCrossBound * (fabsf(p) + fabsf(q));
+            bool left = c > cb;
+            if (!left && !(-c > cb)) left = orient_slow(f, whole(last), whole(k)) > 0;
+            if (!left) continue;
+            if (best < 0) {
+                best = k;
+                continue;
+            }
+            const Point b = point(best);
+            const float p1 = b.fx * fy[k], p2 = b.fy * fx[k], p5 = a.fx * b.fy, p6 = a.fy * b.fx;
+            const float det = a.l * (p1 - p2) - b.l * c + fl[k] * (p5 - p6);
+            const float bound = kCircleBound * (a.l * (fabsf(p1) + fabsf(p2)) + b.l * (fabsf(p) + fabsf(q)) +
+                                                fl[k] * (fabsf(p5) + fabsf(p6)));
+            if (det > bound) continue;
+            if (-det > bound || circle_slow(f, whole(last), whole(best), whole(k)) > 0) best = k;
+        }
+        if (best < 0) {
+            bad = true;
+            break;
+        }
+        if (!disk_ok(f, a, point(best))) a_or(f.flags, MU_FAR);
+        turns += (a.fy < 0.0f && fy[best] >= 0.0f) ? 1 : 0;
+        last = best;
+    } while (last != near);
+    if (bad || deg < 3 || turns != 1) {
+        a_or(f.flags, MU_STAR);
+        return;
+    }
+    // into the version that no other cell reads in this round
+    const int32_t info = m.ring_info[i];
+    const bool fresh = (info >> 2) < m.stamp;
+    int32_t at, ver;
+    if (fresh) {
+        at = a_add(&m.count->overrides, 1);
+        if (at >= m.max_rings) {
+            a_or(f.flags, MU_SIZE);
+            return;
+        }
+        m.ring_at[i] = at;
+        ver = 0;
+    } else {
+        at = m.ring_at[i];
+        ver = (info & 1) ^ 1;
+    }
+    int32_t *dst = m.ring_ref + (int64_t)(2 * at + ver) * kMaxDeg;
+    for (int k = 0; k < deg; k++) dst[k] = out[k];
+    m.ring_deg[2 * at + ver] = deg;
+    m.ring_info[i] = (m.stamp + round) << 2 | (fresh ? 2 : 0) | ver;
+}
+
+// Cell v lacks the references r and q (in its own frame): list it for the
+// next round and tell it.
+RICH_HD inline void tell(const MeshUpdate &m, int32_t v, int32_t round, int32_t r, int32_t q)
+{
+    list_cell(m, v, round + 1);
+    const int32_t e[2] = {r, q};
+    for (int k = 0; k < 2; k++) {
+        if (e[k] < 0) continue;
+        const int32_t at = a_add(m.extra_n + v, 1);
+        if (at < kMaxExtra) m.extra[(int64_t)v * kMaxExtra + at] = e[k];
+    }
+}
+
+// whether the ring of v has r followed by q (by source in a periodic box)
+RICH_HD inline bool has_pair(const MeshUpdate &m, bool periodic, int32_t v, int32_t r, int32_t q)
+{
+    const Ring g = ring_of(m, v, -1);
+    int32_t prev = g[g.deg - 1];
+    for (int32_t k = 0; k < g.deg; k++) {
+        const int32_t cur = g[k];
+        if (periodic ? ((prev >> 4) == (r >> 4) && (cur >> 4) == (q >> 4)) : (prev == r && cur == q)) return true;
+        prev = cur;
+    }
+    return false;
+}
+
+// The new star of cell i against its neighbours' rings.
+RICH_HD inline void check(const MeshUpdate &m, int32_t i, int32_t round)
+{
+    const int32_t info = m.ring_info[i];
+    if ((info >> 2) != m.stamp + round) return;  // not recomputed: a flag is set
+    const bool periodic = m.inst[inst_at(m, i)].boundary == 1;
+    const Ring g = ring_of(m, i, -1);
+    const int32_t me = i * 16 + 4;
+    int32_t a = g[g.deg - 1];
+    for (int32_t k = 0; k < g.deg; k++) {
+        const int32_t b = g[k];
+        // the triangle (i, a, b) in the rings of a and b (the cells
+        // themselves, not their images across a wall)
+        if ((periodic || (a & 15) == 4) && !has_pair(m, periodic, a >> 4, b, me)) {
+            tell(m, a >> 4, round, b, me);
+            list_cell(m, i, round + 1);
+        }
+        if ((periodic || (b & 15) == 4) && !has_pair(m, periodic, b >> 4, me, a)) {
+            tell(m, b >> 4, round, me, a);
+            list_cell(m, i, round + 1);
+        }
+        a = b;
+    }
+    // neighbours of the previous star that the new one dropped must have
+    // dropped the cell
+    const Ring old = ring_of(m, i, round);
+    for (int32_t k = 0; k < old.deg; k++) {
+        const int32_t r = old[k];
+        if ((r >> 4) == i || (!periodic && (r & 15) != 4)) continue;
+        bool kept = false;
+        for (int32_t j = 0; j < g.deg; j++) kept |= periodic ? (g[j] >> 4) == (r >> 4) : g[j] == r;
+        if (kept) continue;
+        const Ring o = ring_of(m, r >> 4, -1);
+        for (int32_t j = 0; j < o.deg; j++)
+            if (periodic ? (o[j] >> 4) == i : o[j] == me) {
+                list_cell(m, r >> 4, round + 1);
+                break;
+            }
+    }
+}
+
+// The images of point (x, y) inside the ghost band, in the host builder's
+// order (bit img of the mask; make_ghosts).
+RICH_HD inline uint32_t image_mask(const InstParams &ip, double x, double y)
+{
+    if (less(ip.in_x0, x) && less(x, ip.in_x1) && less(ip.in_y0, y) && less(y, ip.in_y1)) return 0;
+    const bool per = ip.boundary == 1;
+    const double lox = ip.x0 - ip.band, hix = ip.x1 + ip.band, loy = ip.y0 - ip.band, hiy = ip.y1 + ip.band;
+    uint32_t ox = 0, oy = 0;
+    for (int a = -1; a <= 1; a++) {
+        const double X = image_coord(x, ip.x0, ip.x1, a, per), Y = image_coord(y, ip.y0, ip.y1, a, per);
+        if (!(X < lox || X > hix)) ox |= 1u << (a + 1);
+        if (!(Y < loy || Y > hiy)) oy |= 1u << (a + 1);
+    }
+    if (!((ox | oy) & 5u)) return 0;
+    uint32_t mask = 0;
+    for (int b = 0; b < 3; b++)
+        if (oy >> b & 1) mask |= ox << (3 * b);
+    return mask & ~(1u << 4);
+}
+
+RICH_HD inline int popcount(uint32_t v)
+{
+#ifdef __CUDA_ARCH__
+    return __popc(v);
+#else
+    return __builtin_popcount(v);
+#endif
+}
+
+// position of image img among the images of `mask` in the host's order:
+// a (x) outer, b (y) inner
+RICH_HD inline int image_rank(uint32_t mask, int img)
+{
+    const int a = img % 3, b = img / 3;
+    int r = 0;
+    for (int q = 0; q < 9; q++) {
+        if (!(mask >> q & 1)) continue;
+        const int qa = q % 3, qb = q / 3;
+        r += (qa < a || (qa == a && qb < b)) ? 1 : 0;
+    }
+    return r;
+}
+
+// The cell's degree, owned edges and triangles, and ghost images.
+RICH_HD inline uint32_t measure(const MeshUpdate &m, int32_t i)
+{
+    const InstParams &ip = m.inst[inst_at(m, i)];
+    const bool periodic = ip.boundary == 1;
+    const Ring g = ring_of(m, i, -1);
+    uint32_t ne = 0, nt = 0;
+    int32_t prev = g[g.deg - 1];
+    bool prev_up = (prev & 15) != 4 || (prev >> 4) > i;
+    for (int32_t k = 0; k < g.deg; k++) {
+        const int32_t r = g[k];
+        const bool real = (r & 15) == 4, up = !real || (r >> 4) > i;
+        ne += real || periodic ? (r >> 4) > i : 1;
+        nt += (prev_up && up) ? 1 : 0;
+        prev_up = up;
+    }
+    const uint32_t mask = image_mask(ip, m.x[i], m.y[i]);
+    m.images[i] = (uint16_t)mask;
+    if (g.deg > 255) a_or(m.flags + inst_at(m, i), MU_SIZE);
+    const uint32_t s = (uint32_t)g.deg | ne << 8 | nt << 16 | (uint32_t)popcount(mask) << 24;
+    m.sizes[i] = s;
+    return s;
+}
+
+// The ghosts of cell i, from ghost_off[i] on.
+RICH_HD inline void place_ghosts(const MeshUpdate &m, int32_t i)
+{
+    const uint32_t mask = m.images[i];
+    if (!mask) return;
+    const InstParams &ip = m.inst[inst_at(m, i)];
+    const bool per = ip.boundary == 1;
+    int32_t k = m.ghost_off[i];
+    for (int a = -1; a <= 1; a++)
+        for (int b = -1; b <= 1; b++) {
+            const int img = (a + 1) + 3 * (b + 1);
+            if (!(mask >> img & 1)) continue;
+            m.gx[k] = image_coord(m.x[i], ip.x0, ip.x1, a, per);
+            m.gy[k] = image_coord(m.y[i], ip.y0, ip.y1, b, per);
+            m.gsrc[k] = i;
+            m.gxf[k] = per ? 0 : ((a ? XF_MIRROR_X : 0) | (b ? XF_MIRROR_Y : 0));
+            m.gshift[k] = per ? img : 4;
+            m.gimg[k] = img;
+            k++;
+        }
+}
+
+// Cell i's ring with this mesh's point ids, from its smallest neighbour on.
+RICH_HD inline void place_ring(const MeshUpdate &m, int32_t i)
+{
+    const Ring g = ring_of(m, i, -1);
+    int32_t *dst = m.out_nb + m.out_ptr[i];
+    auto id_of = [&](int32_t r) {
+        const int32_t src = r >> 4, img = r & 15;
+        if (img == 4) return src;
+        const uint32_t mask = m.images[src];
+        if (!(mask >> img & 1)) {
+            a_or(m.flags + inst_at(m, i), MU_IMAGE);
+            return src;
+        }
+        return m.n + m.ghost_off[src] + image_rank(mask, img);
+    };
+    int32_t best = INT32_MAX, at = 0;
+    for (int32_t k = 0; k < g.deg; k++) {
+        const int32_t id = id_of(g[k]);
+        if (id < best) {
+            best = id;
+            at = k;
+        }
+    }
+    for (int32_t k = 0; k < g.deg; k++) dst[k] = id_of(g[at + k < g.deg ? at + k : at + k - g.deg]);
+}
+
+}  // namespace mu
+
+// The update's constants in a simulation's parameters (host): its ghost band
+// as build_host_mesh takes it first, and the FP32 limits on circumdisks.
+void mesh_params(const BoxConfig &box, int32_t n, InstParams &ip);
+
+// The update of `mesh` (a build_host_mesh result, or this function's) for
+// new points by the device bodies, run serially on the host.  Returns 1, or
+// 0 with `flags` set when the host builder has to take the mesh.
+int mesh_update_serial(const BoxConfig &box, int32_t n, const double *x, const double *y, HostMesh &mesh,
+                       int32_t &flags, int32_t &rounds, int32_t &recomputed);
+
+}  // namespace rich

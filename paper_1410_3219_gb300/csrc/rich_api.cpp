@@ -19,6 +19,8 @@
 #include "../../include/rich.h"
 #include "api_internal.h"
 #include "mesh.h"
+#include "meshupdate.h"
+#include "meshupdate_dev.h"
 #include "sweep.cuh"
 #include "threadpool.h"
 
@@ -85,7 +87,19 @@ struct rich_sim {
     double *hx() const { return hpts.as<double>(); }
     double *hy() const { return hpts.as<double>() + n; }
     rich::MeshWork mw;  // (edge list built on the device: see tessellate)
-    rich::HostMesh hm;
+    rich::HostMesh hm;  // the last mesh the host built
+    // The mesh on the device (buffers mcur of the arrays that an update reads
+    // while it writes the new ones): its sizes, and whether the update may
+    // start from it.  After an update the check of its lists (bad_host) is
+    // read at the next wait.
+    int mcur = 0;
+    rich::MeshSizes msz;
+    bool mesh_on_device = false, lists_unchecked = false;
+    rich::MeshUpdater updater;
+    int64_t updates = 0;   // meshes made by it
+    rich::HBuf bad_host;   // two flags of the list builders, then the step's dt and status
+    DBuf mesh_inst;        // the box and mesh_params
+    cudaEvent_t ev_up0 = nullptr, ev_up1 = nullptr;
     std::unique_ptr<rich::ThreadPool> pool;  // host threads of the tile-parallel tessellation
     rich_sim() { mw.host_edges = false; }
     double t = 0.0;
@@ -100,22 +114,19 @@ struct rich_sim {
     cudaStream_t stream = nullptr;
     cudaStream_t own_stream = nullptr;
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
-    // early read of a sweep's new points (rich_step): copied on their own
-    // stream once the point motion is done, while the sweep goes on
-    cudaStream_t copy_stream = nullptr;
-    cudaEvent_t ev_moved = nullptr, ev_copied = nullptr;
     bool profiling = false;
     cudaEvent_t kev[rich::NUM_STAGES + 1] = {};
     double kms[rich::NUM_STAGES] = {};
     double last_dt = 0.0;
     // device buffers
     DBuf x[3], y[3], U[3];
-    DBuf A, o, W, cs, g, gl, alpha, w, tess, cell_ptr, corder, initW, rounding, p64, psrc;
+    DBuf A, o, W, cs, g, gl, alpha, w, tess, corder, initW, rounding, p64, psrc;
     bool diagnostics = true;
-    DBuf gx, gy, gsrc, gxf, gshift, eoff, toff;
+    DBuf gx, gy, gxf, gshift, eoff, toff;
+    DBuf cell_ptr[2], slot_nb[2], gsrc[2], gimg[2];
     DBuf perm_dev, unperm;  // caller index of each internal cell; reordered state for reads
     DBuf tri, ccx, ccy;
-    DBuf slot_nb, slot_tri, slot_edge;
+    DBuf slot_tri, slot_edge;
     DBuf edge_l, edge_r, edge_ta, edge_tb, eL, emlx, emly, emrx, emry, enx, eny, eqx, eqy, F, ePM;
     DBuf scal;   // dtmin bits, dt, status
     DBuf instp;  // one InstParams
@@ -125,9 +136,8 @@ struct rich_sim {
     {
         if (ev0) cudaEventDestroy(ev0);
         if (ev1) cudaEventDestroy(ev1);
-        if (ev_moved) cudaEventDestroy(ev_moved);
-        if (ev_copied) cudaEventDestroy(ev_copied);
-        if (copy_stream) cudaStreamDestroy(copy_stream);
+        if (ev_up0) cudaEventDestroy(ev_up0);
+        if (ev_up1) cudaEventDestroy(ev_up1);
         for (cudaEvent_t e : kev)
             if (e) cudaEventDestroy(e);
         if (own_stream) cudaStreamDestroy(own_stream);
@@ -142,10 +152,10 @@ struct rich_sim {
         p.diagnostics = diagnostics ? 1 : 0;
         p.motion = 1;
         p.n = n;
-        p.ng = hm.g;
-        p.T = hm.n_tris;
-        p.E = hm.n_edges;
-        p.S = (int32_t)hm.slot_nb.size();
+        p.ng = msz.ghosts;
+        p.T = msz.tris;
+        p.E = msz.edges;
+        p.S = msz.slots;
         // extrapolated fluxes: [cur] -> [1 - cur].  Time-centred: [cur] -> [2]
         // by half a step, then primitives and mesh of [2], update of [cur]
         // into [1 - cur]
@@ -154,11 +164,11 @@ struct rich_sim {
         p.xn = x[dst].as<double>(); p.yn = y[dst].as<double>();
         p.x0 = x[cur].as<double>(); p.y0 = y[cur].as<double>();
         p.gx = gx.as<double>(); p.gy = gy.as<double>();
-        p.tri = tri.as<int32_t>(); p.cell_ptr = cell_ptr.as<int32_t>(); p.cell_order = corder.as<int32_t>();
-        p.slot_nb = slot_nb.as<int32_t>(); p.slot_tri = slot_tri.as<int32_t>(); p.slot_edge = slot_edge.as<int32_t>();
+        p.tri = tri.as<int32_t>(); p.cell_ptr = cell_ptr[mcur].as<int32_t>(); p.cell_order = corder.as<int32_t>();
+        p.slot_nb = slot_nb[mcur].as<int32_t>(); p.slot_tri = slot_tri.as<int32_t>(); p.slot_edge = slot_edge.as<int32_t>();
         p.edge_l = edge_l.as<int32_t>(); p.edge_r = edge_r.as<int32_t>();
         p.edge_ta = edge_ta.as<int32_t>(); p.edge_tb = edge_tb.as<int32_t>();
-        p.ghost_src = gsrc.as<int32_t>(); p.ghost_xf = gxf.as<int32_t>();
+        p.ghost_src = gsrc[mcur].as<int32_t>(); p.ghost_xf = gxf.as<int32_t>();
         p.ccx = ccx.as<double>(); p.ccy = ccy.as<double>(); p.A = A.as<double>();
         p.eL = eL.as<R>(); p.emlx = emlx.as<R>(); p.emly = emly.as<R>();
         p.emrx = emrx.as<R>(); p.emry = emry.as<R>();
@@ -215,9 +225,21 @@ struct rich_sim {
         }
     }
 
-    // the mesh sizes of the current tessellation
-    int32_t nT() const { return hm.n_tris; }
-    int32_t nE() const { return hm.n_edges; }
+    // the mesh update's input: the mesh on the device and new positions
+    rich::MeshArrays mesh_arrays(int q) const
+    {
+        rich::MeshArrays a{};
+        a.n = n;
+        a.n_inst = 1;
+        a.inst = mesh_inst.as<rich::InstParams>();
+        a.x = x[q].as<double>();
+        a.y = y[q].as<double>();
+        a.cell_ptr = cell_ptr[mcur].as<int32_t>();
+        a.slot_nb = slot_nb[mcur].as<int32_t>();
+        a.ghost_src = gsrc[mcur].as<int32_t>();
+        a.ghost_img = gimg[mcur].as<int32_t>();
+        return a;
+    }
 };
 
 namespace {
@@ -238,6 +260,12 @@ int alloc_cells(rich_sim *s)
     CUDA_TRY(s->scal.ensure(64));
     CUDA_TRY(cudaMemsetAsync(s->scal.p, 0, 64, s->stream));
     CUDA_TRY(s->instp.ensure(sizeof(rich::InstParams)));
+    CUDA_TRY(s->bad_host.ensure(64));
+    CUDA_TRY(s->mesh_inst.ensure(sizeof(rich::InstParams)));
+    rich::InstParams ip = s->inst_params(0.0);
+    rich::mesh_params(rich::BoxConfig{s->cfg.boundary, s->cfg.x0, s->cfg.x1, s->cfg.y0, s->cfg.y1}, s->n, ip);
+    CUDA_TRY(cudaMemcpyAsync(s->mesh_inst.p, &ip, sizeof(ip), cudaMemcpyHostToDevice, s->stream));
+    CUDA_TRY(cudaStreamSynchronize(s->stream));
     return RICH_OK;
 }
 
@@ -253,66 +281,160 @@ int build_mesh(rich_sim *s, rich_step_info *info)
     return rc ? mesh_rc(rc) : RICH_OK;
 }
 
-// upload of the host mesh; the triangle and edge lists are built on the
-// device from the rings (the host sends each cell's first owned triangle
-// and edge, and the ghosts' periodic shifts).  Nothing on the stream may
-// still read the old mesh: buffers that grow are reallocated.
-int upload_mesh(rich_sim *s, rich_step_info *info)
+// Room for a mesh of these sizes in the arrays beside its rings, and the
+// triangle and edge lists built from the rings of buffers `mesh` (enqueued
+// with the copy of the builders' flags to bad_host).  Nothing on the stream
+// may still read the old lists: buffers that grow are reallocated.
+int build_lists(rich_sim *s, int mesh)
 {
-    const double t2 = now_ms();
-    const rich::HostMesh &m = s->hm;
-    const size_t T = (size_t)m.n_tris, E = (size_t)m.n_edges, d = sizeof(double);
-    CUDA_TRY(upload(s->gx, m.gx, s->stream));
-    CUDA_TRY(upload(s->gy, m.gy, s->stream));
-    CUDA_TRY(upload(s->gsrc, m.ghost_src, s->stream));
-    CUDA_TRY(upload(s->gxf, m.ghost_xf, s->stream));
-    CUDA_TRY(upload(s->cell_ptr, m.cell_ptr, s->stream));
-    CUDA_TRY(upload(s->corder, m.cell_order, s->stream));
-    CUDA_TRY(upload(s->slot_nb, m.slot_nb, s->stream));
-    CUDA_TRY(upload(s->toff, m.tri_off, s->stream));
-    CUDA_TRY(upload(s->eoff, m.edge_off, s->stream));
-    CUDA_TRY(upload(s->gshift, m.ghost_shift, s->stream));
-    const size_t S = m.slot_nb.size();
+    const size_t T = (size_t)s->msz.tris, E = (size_t)s->msz.edges, S = (size_t)s->msz.slots, d = sizeof(double);
+    const size_t r = s->rsize();
     CUDA_TRY(s->tri.ensure((3 * T + 3) * sizeof(int32_t)));
     CUDA_TRY(s->slot_tri.ensure((S + 1) * sizeof(int32_t)));
     CUDA_TRY(s->slot_edge.ensure((S + 1) * sizeof(int32_t)));
     for (DBuf *b : {&s->edge_l, &s->edge_r, &s->edge_ta, &s->edge_tb}) CUDA_TRY(b->ensure((E + 1) * sizeof(int32_t)));
     int32_t *bad = reinterpret_cast<int32_t *>(s->scal.as<char>() + 24);
     int32_t *bad_tri = reinterpret_cast<int32_t *>(s->scal.as<char>() + 28);
-    CUDA_TRY(rich::launch_build_tris(s->n, (int32_t)S, s->cell_ptr.as<int32_t>(), s->slot_nb.as<int32_t>(),
-                                     s->toff.as<int32_t>(), s->tri.as<int32_t>(), s->slot_tri.as<int32_t>(), bad_tri,
-                                     s->stream));
-    CUDA_TRY(rich::launch_build_edges(s->n, (int32_t)S, s->cell_ptr.as<int32_t>(), s->slot_nb.as<int32_t>(),
-                                      s->slot_tri.as<int32_t>(), s->gsrc.as<int32_t>(), s->gshift.as<int32_t>(),
-                                      s->eoff.as<int32_t>(), s->cfg.boundary == RICH_BC_PERIODIC ? 1 : 0,
-                                      nullptr, nullptr, s->slot_edge.as<int32_t>(), s->edge_l.as<int32_t>(), s->edge_r.as<int32_t>(),
+    const int32_t *ptr = s->cell_ptr[mesh].as<int32_t>(), *nb = s->slot_nb[mesh].as<int32_t>();
+    CUDA_TRY(rich::launch_build_tris(s->n, (int32_t)S, ptr, nb, s->toff.as<int32_t>(), s->tri.as<int32_t>(),
+                                     s->slot_tri.as<int32_t>(), bad_tri, s->stream));
+    CUDA_TRY(rich::launch_build_edges(s->n, (int32_t)S, ptr, nb, s->slot_tri.as<int32_t>(), s->gsrc[mesh].as<int32_t>(),
+                                      s->gshift.as<int32_t>(), s->eoff.as<int32_t>(),
+                                      s->cfg.boundary == RICH_BC_PERIODIC ? 1 : 0, nullptr, nullptr,
+                                      s->slot_edge.as<int32_t>(), s->edge_l.as<int32_t>(), s->edge_r.as<int32_t>(),
                                       s->edge_ta.as<int32_t>(), s->edge_tb.as<int32_t>(), bad, s->stream));
-    int32_t bad_h[2] = {0, 0};
-    CUDA_TRY(cudaMemcpyAsync(bad_h, bad, 2 * sizeof(int32_t), cudaMemcpyDeviceToHost, s->stream));
-    const size_t r = s->rsize();
+    CUDA_TRY(cudaMemcpyAsync(s->bad_host.p, bad, 2 * sizeof(int32_t), cudaMemcpyDeviceToHost, s->stream));
+    s->lists_unchecked = true;
     CUDA_TRY(s->ccx.ensure((T + 1) * d)); CUDA_TRY(s->ccy.ensure((T + 1) * d));
     for (DBuf *b : {&s->eL, &s->emlx, &s->emly, &s->emrx, &s->emry, &s->enx, &s->eny, &s->eqx, &s->eqy})
         CUDA_TRY(b->ensure((E + 1) * r));
     CUDA_TRY(s->F.ensure((4 * E + 4) * sizeof(double)));
     CUDA_TRY(s->ePM.ensure((4 * E + 4) * r));
-    CUDA_TRY(cudaStreamSynchronize(s->stream));
-    const double t3 = now_ms();
-    if (bad_h[1]) return fail(RICH_ETESS, "a triangle of a ring is missing from its owner's ring");
-    if (bad_h[0]) return fail(RICH_ETESS, "an edge of a ring has no partner in the other cell's ring");
-    s->tess_current = true;
-    if (info) {
-        info->copy_ms += t3 - t2;
-        info->n_ghost = m.g;
-        info->n_tri = (int64_t)T;
-        info->n_edges = (int64_t)E;
-        info->n_slots = (int64_t)m.slot_nb.size();
-    }
     return RICH_OK;
 }
 
-// host tessellation of the current points + upload of the connectivity
+// After a wait: the list builders' flags of the mesh last built.
+int check_lists(rich_sim *s)
+{
+    if (!s->lists_unchecked) return RICH_OK;
+    s->lists_unchecked = false;
+    const int32_t *bad = s->bad_host.as<int32_t>();
+    if (!bad[0] && !bad[1]) return RICH_OK;
+    s->tess_current = s->mesh_on_device = false;
+    if (bad[1]) return fail(RICH_ETESS, "a triangle of a ring is missing from its owner's ring");
+    return fail(RICH_ETESS, "an edge of a ring has no partner in the other cell's ring");
+}
+
+void report_sizes(const rich_sim *s, rich_step_info *info)
+{
+    if (!info) return;
+    info->n_ghost = s->msz.ghosts;
+    info->n_tri = s->msz.tris;
+    info->n_edges = s->msz.edges;
+    info->n_slots = s->msz.slots;
+}
+
+// upload of the host mesh; the triangle and edge lists are built on the
+// device from the rings (the host sends each cell's first owned triangle
+// and edge, and the ghosts' images)
+int upload_mesh(rich_sim *s, rich_step_info *info)
+{
+    const double t2 = now_ms();
+    const rich::HostMesh &m = s->hm;
+    const int q = s->mcur;
+    s->mesh_on_device = false;
+    CUDA_TRY(upload(s->gx, m.gx, s->stream));
+    CUDA_TRY(upload(s->gy, m.gy, s->stream));
+    CUDA_TRY(upload(s->gsrc[q], m.ghost_src, s->stream));
+    CUDA_TRY(upload(s->gimg[q], m.ghost_img, s->stream));
+    CUDA_TRY(upload(s->gxf, m.ghost_xf, s->stream));
+    CUDA_TRY(upload(s->cell_ptr[q], m.cell_ptr, s->stream));
+    CUDA_TRY(upload(s->corder, m.cell_order, s->stream));
+    CUDA_TRY(upload(s->slot_nb[q], m.slot_nb, s->stream));
+    CUDA_TRY(upload(s->toff, m.tri_off, s->stream));
+    CUDA_TRY(upload(s->eoff, m.edge_off, s->stream));
+    CUDA_TRY(upload(s->gshift, m.ghost_shift, s->stream));
+    s->msz = rich::MeshSizes{m.g, m.n_tris, m.n_edges, (int32_t)m.slot_nb.size()};
+    int rc = build_lists(s, q);
+    if (rc != RICH_OK) return rc;
+    CUDA_TRY(cudaStreamSynchronize(s->stream));
+    if ((rc = check_lists(s)) != RICH_OK) return rc;
+    s->tess_current = s->mesh_on_device = true;
+    if (info) info->copy_ms += now_ms() - t2;
+    report_sizes(s, info);
+    return RICH_OK;
+}
+
+// Whether the mesh of new points can be an update of the one on the device.
+bool can_update(const rich_sim *s)
+{
+    return s->mesh_on_device && s->n >= rich::kMeshUpdateMin && s->n <= rich::kMeshUpdateMax;
+}
+
+// The updated mesh of the points in buffers q written and made the current
+// one, after the update's first part was waited for (enqueued, not waited
+// for; the caller of the next sweep checks the lists).  ok = false: the host
+// has to build this mesh; the mesh on the device is unchanged.
+int finish_update(rich_sim *s, int q, bool &ok, rich_step_info *info)
+{
+    rich::MeshSizes z;
+    const rich::MeshArrays a = s->mesh_arrays(q);
+    CUDA_TRY(s->updater.settle(a, ok, z, s->stream));
+    ok = ok && !s->updater.flags()[0];
+    if (!ok) return RICH_OK;
+    const int m = 1 - s->mcur;
+    const size_t i4 = sizeof(int32_t), N = (size_t)s->n, G = (size_t)z.ghosts + 1;
+    // (the old ghosts' positions are read by nothing any more)
+    CUDA_TRY(s->cell_ptr[m].ensure((N + 1) * i4));
+    CUDA_TRY(s->slot_nb[m].ensure(((size_t)z.slots + 1) * i4));
+    CUDA_TRY(s->gsrc[m].ensure(G * i4)); CUDA_TRY(s->gimg[m].ensure(G * i4));
+    CUDA_TRY(s->gx.ensure(G * 8)); CUDA_TRY(s->gy.ensure(G * 8));
+    CUDA_TRY(s->gxf.ensure(G * i4)); CUDA_TRY(s->gshift.ensure(G * i4));
+    rich::MeshOutput o{};
+    o.cell_ptr = s->cell_ptr[m].as<int32_t>();
+    o.slot_nb = s->slot_nb[m].as<int32_t>();
+    o.tri_off = s->toff.as<int32_t>();
+    o.edge_off = s->eoff.as<int32_t>();
+    o.cell_order = s->corder.as<int32_t>();
+    o.gx = s->gx.as<double>();
+    o.gy = s->gy.as<double>();
+    o.ghost_src = s->gsrc[m].as<int32_t>();
+    o.ghost_xf = s->gxf.as<int32_t>();
+    o.ghost_shift = s->gshift.as<int32_t>();
+    o.ghost_img = s->gimg[m].as<int32_t>();
+    // (from here on the old mesh's offsets are overwritten)
+    s->tess_current = s->mesh_on_device = false;
+    CUDA_TRY(s->updater.finish(a, o, s->stream));
+    s->mcur = m;
+    s->msz = z;
+    s->updates++;
+    const int rc = build_lists(s, m);
+    if (rc != RICH_OK) return rc;
+    s->tess_current = s->mesh_on_device = true;
+    report_sizes(s, info);
+    return RICH_OK;
+}
+
+// a0 for the current points: the mesh on the device updated, or else built on
+// the host and its connectivity uploaded.  fetch_points false: the host copy
+// of the points is current, and there is no mesh to update.
 int tessellate(rich_sim *s, rich_step_info *info, bool fetch_points)
 {
+    if (fetch_points && can_update(s)) {
+        const double t0 = now_ms();
+        const int q = s->pts();
+        CUDA_TRY(s->updater.start(s->mesh_arrays(q), s->stream));
+        CUDA_TRY(cudaStreamSynchronize(s->stream));
+        bool ok = false;
+        int rc = finish_update(s, q, ok, info);
+        if (rc != RICH_OK) return rc;
+        if (ok) {
+            CUDA_TRY(cudaStreamSynchronize(s->stream));
+            if ((rc = check_lists(s)) != RICH_OK) return rc;
+            if (info) info->tess_ms += now_ms() - t0;
+            return RICH_OK;
+        }
+    }
     if (fetch_points) {
         const double t0 = now_ms();
         const int q = s->pts();
@@ -433,11 +555,8 @@ static int create_sim(const rich_config *cfg, int64_t n, const double *x, const 
         return bail(fail(RICH_ECUDA, "stream creation failed"));
     s->stream = s->own_stream;
     if (cudaEventCreate(&s->ev0) != cudaSuccess || cudaEventCreate(&s->ev1) != cudaSuccess ||
-        cudaEventCreateWithFlags(&s->ev_moved, cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventCreateWithFlags(&s->ev_copied, cudaEventDisableTiming) != cudaSuccess)
+        cudaEventCreate(&s->ev_up0) != cudaSuccess || cudaEventCreate(&s->ev_up1) != cudaSuccess)
         return bail(fail(RICH_ECUDA, "event creation failed"));
-    if (cudaStreamCreateWithFlags(&s->copy_stream, cudaStreamNonBlocking) != cudaSuccess)
-        return bail(fail(RICH_ECUDA, "stream creation failed"));
     if ((rc = alloc_cells(s)) != RICH_OK) return bail(rc);
     if (s->x[0].ensure(n * 8) != cudaSuccess) return bail(fail(RICH_ENOMEM, "device points"));
     if (upload(s->perm_dev, s->perm, s->stream) != cudaSuccess) return bail(fail(RICH_ENOMEM, "device order"));
@@ -538,33 +657,24 @@ int rich_tessellate(rich_sim *s, rich_step_info *info)
     return tessellate(s, info, true);
 }
 
-// Launch the sweep; with read_points the moved points and the step's dt
-// are copied into hpts on the copy stream as soon as the point motion is
-// done (ev_copied marks their arrival) while the rest of the sweep runs.
-static int launch_sweep(rich_sim *s, double t_end, bool read_points)
+static int launch_sweep(rich_sim *s, double t_end)
 {
     rich::Range range("rich sweep launch (a1-a9)");
     if (!s) return fail(RICH_EINVAL, "NULL handle");
     if (!s->tess_current) return fail(RICH_ESTATE, "no current tessellation");
     if (s->pending) return fail(RICH_ESTATE, "a sweep is pending; call rich_sync first");
     if (!(t_end > s->t)) return fail(RICH_EINVAL, "t_end must exceed the current time");
-    CUDA_TRY(cudaStreamSynchronize(s->stream));  // the staging struct may be in flight
+    // the staging struct may be in flight, and the lists of an updated mesh
+    // are checked before any kernel reads them
+    CUDA_TRY(cudaStreamSynchronize(s->stream));
+    int rc = check_lists(s);
+    if (rc != RICH_OK) return rc;
     s->inst_host = s->inst_params(t_end - s->t);
     CUDA_TRY(cudaMemcpyAsync(s->instp.p, &s->inst_host, sizeof(rich::InstParams), cudaMemcpyHostToDevice, s->stream));
     CUDA_TRY(cudaEventRecord(s->ev0, s->stream));
     for (int k = 0; k < rich::NUM_STAGES; k++) {
         if (s->profiling) CUDA_TRY(cudaEventRecord(s->kev[k], s->stream));
         s->launch(k, nullptr);
-        if (read_points && k == rich::K_ADVANCE) {
-            const size_t N = (size_t)s->n;
-            const int q = s->next_pts();
-            CUDA_TRY(cudaEventRecord(s->ev_moved, s->stream));
-            CUDA_TRY(cudaStreamWaitEvent(s->copy_stream, s->ev_moved, 0));
-            CUDA_TRY(cudaMemcpyAsync(s->hx(), s->x[q].p, N * 8, cudaMemcpyDeviceToHost, s->copy_stream));
-            CUDA_TRY(cudaMemcpyAsync(s->hy(), s->y[q].p, N * 8, cudaMemcpyDeviceToHost, s->copy_stream));
-            CUDA_TRY(cudaMemcpyAsync(s->hy() + N, s->scal.as<char>() + 8, 8, cudaMemcpyDeviceToHost, s->copy_stream));
-            CUDA_TRY(cudaEventRecord(s->ev_copied, s->copy_stream));
-        }
     }
     if (s->profiling) CUDA_TRY(cudaEventRecord(s->kev[rich::NUM_STAGES], s->stream));
     CUDA_TRY(cudaGetLastError());
@@ -573,7 +683,7 @@ static int launch_sweep(rich_sim *s, double t_end, bool read_points)
     return RICH_OK;
 }
 
-int rich_sweep(rich_sim *s, double t_end) { return launch_sweep(s, t_end, false); }
+int rich_sweep(rich_sim *s, double t_end) { return launch_sweep(s, t_end); }
 
 int rich_sync(rich_sim *s, rich_step_info *info)
 {
@@ -581,12 +691,14 @@ int rich_sync(rich_sim *s, rich_step_info *info)
     if (!s) return fail(RICH_EINVAL, "NULL handle");
     if (!s->pending) return fail(RICH_ESTATE, "no sweep pending");
     double t0 = now_ms();
-    double dt = 0.0;
-    int32_t status = 0;
     char *sc = s->scal.as<char>();
-    CUDA_TRY(cudaMemcpyAsync(&dt, sc + 8, 8, cudaMemcpyDeviceToHost, s->stream));
-    CUDA_TRY(cudaMemcpyAsync(&status, sc + 16, 4, cudaMemcpyDeviceToHost, s->stream));
+    // (into page-locked memory: dt, then the status)
+    double *dt_host = s->bad_host.as<double>() + 1;
+    int32_t *status_host = reinterpret_cast<int32_t *>(dt_host + 1);
+    CUDA_TRY(cudaMemcpyAsync(dt_host, sc + 8, 12, cudaMemcpyDeviceToHost, s->stream));
     CUDA_TRY(cudaStreamSynchronize(s->stream));
+    const double dt = *dt_host;
+    const int32_t status = *status_host;
     s->pending = false;
     float ms = 0.0f;
     cudaEventElapsedTime(&ms, s->ev0, s->ev1);
@@ -632,33 +744,37 @@ int rich_sync(rich_sim *s, rich_step_info *info)
     return RICH_OK;
 }
 
-// One sweep of rich_step: while the device computes the gradients, fluxes
-// and update, the host builds the mesh of the moved points (which it reads
-// as soon as the point motion is done) unless the sweep ends the run at
-// t_end; after the sweep that mesh is uploaded.  A failed sweep leaves the
-// host mesh ahead of the device one: the next use tessellates again.
-static int pipelined_sweep(rich_sim *s, double t_end, rich_step_info *info)
+// One sweep of rich_step: the update of the mesh for the moved points follows
+// the sweep on the stream (its first part reads only the points and the old
+// mesh), so one wait serves both; unless the sweep failed or landed on t_end,
+// the updated mesh is then written (not waited for).  A mesh that the update
+// cannot make is left to the next tessellation.
+static int step_sweep(rich_sim *s, double t_end, rich_step_info *info)
 {
-    int rc = launch_sweep(s, t_end, true);
+    int rc = launch_sweep(s, t_end);
     if (rc != RICH_OK) return rc;
-    const double t0 = now_ms();
-    CUDA_TRY(cudaEventSynchronize(s->ev_copied));
-    if (info) info->copy_ms += now_ms() - t0;
-    const double dt = s->hy()[s->n];
-    // the half-step points always get a mesh; after a full step, the points
-    // get one unless the step lands on t_end
-    const bool build = (s->time_centred() && s->tc_phase == 0) || dt < t_end - s->t;
-    int brc = RICH_OK;
-    if (build) {
-        s->tess_current = false;
-        brc = build_mesh(s, info);
+    const int q = s->next_pts();
+    const bool update = can_update(s);
+    if (update) {
+        CUDA_TRY(cudaEventRecord(s->ev_up0, s->stream));
+        CUDA_TRY(s->updater.start(s->mesh_arrays(q), s->stream));
+        CUDA_TRY(cudaEventRecord(s->ev_up1, s->stream));
     }
-    rc = rich_sync(s, info);
-    if (rc != RICH_OK) return rc;
-    // (a mesh that could not be built is reported by the next step's
-    // tessellation of the same points, as without the early build)
-    if (!build || brc != RICH_OK) return RICH_OK;
-    return upload_mesh(s, info);
+    const bool half = s->time_centred() && s->tc_phase == 0;
+    const double before = s->t;
+    if ((rc = rich_sync(s, info)) != RICH_OK) return rc;
+    if (!update) return RICH_OK;
+    float ms = 0.0f;
+    cudaEventElapsedTime(&ms, s->ev_up0, s->ev_up1);
+    if (info) info->tess_ms += ms;
+    // the half-step points always get a mesh; after a full step, the points
+    // get one unless the step landed on t_end
+    if (!half && !(s->last_dt < t_end - before)) return RICH_OK;
+    const double t0 = now_ms();
+    bool ok = false;
+    rc = finish_update(s, q, ok, info);
+    if (info) info->tess_ms += now_ms() - t0;
+    return rc;
 }
 
 int rich_step(rich_sim *s, int32_t max_steps, double t_end, rich_step_info *info)
@@ -672,12 +788,12 @@ int rich_step(rich_sim *s, int32_t max_steps, double t_end, rich_step_info *info
         int rc;
         if (!s->tess_current && (rc = tessellate(s, info, true)) != RICH_OK) return rc;
         double before = s->t;
-        if ((rc = pipelined_sweep(s, t_end, info)) != RICH_OK) return rc;
+        if ((rc = step_sweep(s, t_end, info)) != RICH_OK) return rc;
         if (s->tc_phase == 1) {
             // time-centred: the full step on the mesh of the half-step points
             // (meshed again here, to report its error, if the early build failed)
             if (!s->tess_current && (rc = tessellate(s, info, true)) != RICH_OK) return rc;
-            if ((rc = pipelined_sweep(s, t_end, info)) != RICH_OK) return rc;
+            if ((rc = step_sweep(s, t_end, info)) != RICH_OK) return rc;
         }
         if (s->last_dt >= t_end - before) s->t = t_end;  // landed on t_end
         if (info) info->t = s->t;
@@ -694,6 +810,11 @@ static int ensure_geometry(rich_sim *s)
     if (s->pending) return fail(RICH_ESTATE, "a sweep is pending; call rich_sync first");
     if (!s->tess_current) {
         int rc = tessellate(s, nullptr, true);
+        if (rc) return rc;
+    }
+    if (s->lists_unchecked) {
+        CUDA_TRY(cudaStreamSynchronize(s->stream));
+        int rc = check_lists(s);
         if (rc) return rc;
     }
     for (int k = 0; k < rich::GEOMETRY_STAGES; k++) s->launch(k, nullptr, nullptr, false);
@@ -1010,6 +1131,95 @@ int rich_mesh_update_check(const rich_config *cfg, int64_t n, int32_t steps, con
     *updated = kept.kinetic_tiles;
     *rebuilt = kept.fresh_tiles;
     *reinserted = kept.reinserted;
+    return RICH_OK;
+}
+
+// entries of the device mesh update's output that differ from a fresh host build
+static int64_t mesh_differences(const rich::HostMesh &a, const rich::HostMesh &b)
+{
+    int64_t bad = 0;
+    auto cmp = [&](const auto &u, const auto &v) {
+        if (u.size() != v.size()) {
+            bad++;
+            return;
+        }
+        for (size_t k = 0; k < u.size(); k++) bad += u[k] != v[k];
+    };
+    cmp(a.cell_ptr, b.cell_ptr);
+    cmp(a.slot_nb, b.slot_nb);
+    cmp(a.tri_off, b.tri_off);
+    cmp(a.edge_off, b.edge_off);
+    cmp(a.cell_order, b.cell_order);
+    cmp(a.gx, b.gx);
+    cmp(a.gy, b.gy);
+    cmp(a.ghost_src, b.ghost_src);
+    cmp(a.ghost_xf, b.ghost_xf);
+    cmp(a.ghost_shift, b.ghost_shift);
+    cmp(a.ghost_img, b.ghost_img);
+    return bad;
+}
+
+int rich_device_update_check(const rich_config *cfg, int64_t n, int32_t steps, const double *xs, const double *ys,
+                             int64_t *mismatched, int64_t *updated, int64_t *recomputed)
+{
+    if (!valid_config(cfg) || n < 3 || n > rich::kMeshUpdateMax || steps < 1 || !xs || !ys || !mismatched || !updated ||
+        !recomputed)
+        return fail(RICH_EINVAL, "bad arguments");
+    for (int64_t i = 0; i < (int64_t)steps * n; i++)
+        if (!point_inside(cfg, xs[i], ys[i])) return fail(RICH_EINVAL, "point outside the box");
+    const rich::BoxConfig box{cfg->boundary, cfg->x0, cfg->x1, cfg->y0, cfg->y1};
+    rich::ThreadPool pool((int)std::max(1u, std::thread::hardware_concurrency()));
+    rich::HostMesh m;
+    *mismatched = *updated = *recomputed = 0;
+    for (int32_t k = 0; k < steps; k++) {
+        const double *x = xs + (size_t)k * n, *y = ys + (size_t)k * n;
+        rich::MeshWork work;
+        work.host_edges = false;
+        rich::HostMesh f;
+        const int rc = rich::build_host_mesh(box, (int32_t)n, x, y, work, f, &pool);
+        if (rc) return mesh_rc(rc);
+        int32_t flags = 0, rounds = 0, listed = 0;
+        if (k > 0 && rich::mesh_update_serial(box, (int32_t)n, x, y, m, flags, rounds, listed)) {
+            *mismatched += mesh_differences(m, f);
+            *updated += 1;
+            *recomputed += listed;
+        }
+        m = std::move(f);
+    }
+    return RICH_OK;
+}
+
+int rich_mesh_check(rich_sim *s, int64_t *mismatched, int64_t *updates)
+{
+    if (!s || !mismatched) return fail(RICH_EINVAL, "bad arguments");
+    if (s->pending) return fail(RICH_ESTATE, "a sweep is pending; call rich_sync first");
+    if (!s->tess_current) return fail(RICH_ESTATE, "no current tessellation");
+    CUDA_TRY(cudaStreamSynchronize(s->stream));
+    int rc = check_lists(s);
+    if (rc != RICH_OK) return rc;
+    rich::HostMesh d, f;
+    const size_t N = (size_t)s->n, G = (size_t)s->msz.ghosts, S = (size_t)s->msz.slots;
+    std::vector<double> x(N), y(N);
+    auto down = [&](auto &v, const DBuf &b, size_t k) -> cudaError_t {
+        v.resize(k);
+        if (k == 0) return cudaSuccess;
+        return cudaMemcpyAsync(v.data(), b.p, k * sizeof(v[0]), cudaMemcpyDeviceToHost, s->stream);
+    };
+    const int q = s->pts(), m = s->mcur;
+    CUDA_TRY(down(x, s->x[q], N)); CUDA_TRY(down(y, s->y[q], N));
+    CUDA_TRY(down(d.cell_ptr, s->cell_ptr[m], N + 1)); CUDA_TRY(down(d.slot_nb, s->slot_nb[m], S));
+    CUDA_TRY(down(d.tri_off, s->toff, N + 1)); CUDA_TRY(down(d.edge_off, s->eoff, N + 1));
+    CUDA_TRY(down(d.cell_order, s->corder, N));
+    CUDA_TRY(down(d.gx, s->gx, G)); CUDA_TRY(down(d.gy, s->gy, G));
+    CUDA_TRY(down(d.ghost_src, s->gsrc[m], G)); CUDA_TRY(down(d.ghost_xf, s->gxf, G));
+    CUDA_TRY(down(d.ghost_shift, s->gshift, G)); CUDA_TRY(down(d.ghost_img, s->gimg[m], G));
+    CUDA_TRY(cudaStreamSynchronize(s->stream));
+    rich::MeshWork work;
+    work.host_edges = false;
+    const rich::BoxConfig box{s->cfg.boundary, s->cfg.x0, s->cfg.x1, s->cfg.y0, s->cfg.y1};
+    if ((rc = rich::build_host_mesh(box, s->n, x.data(), y.data(), work, f, s->pool.get()))) return mesh_rc(rc);
+    *mismatched = mesh_differences(d, f);
+    if (updates) *updates = s->updates;
     return RICH_OK;
 }
 

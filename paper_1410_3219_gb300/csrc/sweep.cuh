@@ -70,6 +70,13 @@ struct InstParams {
     // host), for the split-precision stages
     float gamma_f, igm1_f, chi_f, theta_f, delta_v_f;
     int32_t pad;
+    // constants of the device mesh update (mesh_params in meshupdate.h):
+    // half the box's sides, the ghost band and the box inside which no point
+    // has an image in it, and in FP32, in mean point spacings (lengths times
+    // mesh_scale), the squared circumradii that need no placing and that a
+    // periodic box allows, and how far a disk may reach past a wall
+    double half_x, half_y, band, in_x0, in_x1, in_y0, in_y1;
+    float mesh_scale, mesh_rlim2, mesh_rper2, mesh_reach;
 };
 
 template <class R> struct SweepParams {

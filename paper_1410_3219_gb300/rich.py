@@ -36,7 +36,8 @@ EXPORTS = ["rich_default_config", "rich_init_mesh", "rich_step", "rich_get_state
            "rich_server_query", "rich_server_fetch", "rich_server_batch", "rich_server_destroy",
            "rich_init_conserved", "rich_get_order", "rich_time", "rich_mesh_update_check",
            "rich_probe_pipe_peaks", "rich_batch_inject_barrier_timeout", "rich_server_start",
-           "rich_server_stats", "rich_edge_list_check", "rich_tess_phases"]
+           "rich_server_stats", "rich_edge_list_check", "rich_tess_phases", "rich_device_update_check",
+           "rich_mesh_check"]
 
 REQ_STATES = {0: "queued", 1: "running", 2: "done", 3: "failed"}
 
@@ -148,6 +149,8 @@ def _lib():
         L.rich_server_start.argtypes = [P, I32, I64, I64]
         L.rich_tess_phases.argtypes = [P, _D]
         L.rich_edge_list_check.argtypes = [C.POINTER(rich_config), I64, _D, _D, C.POINTER(I64), C.POINTER(I64)]
+        L.rich_device_update_check.argtypes = [C.POINTER(rich_config), I64, I32, _D, _D] + [C.POINTER(I64)] * 3
+        L.rich_mesh_check.argtypes = [P, C.POINTER(I64), C.POINTER(I64)]
         L.rich_server_stats.argtypes = [P, C.POINTER(I64)] + [_D] * 4
         _handle = L
     return _handle
@@ -350,6 +353,26 @@ def rich_mesh_update_check(cfg, xs, ys, threads=4):
                                          C.byref(re), C.byref(ri)))
     return mis.value, up.value, re.value, ri.value
 
+
+def rich_device_update_check(cfg, xs, ys):
+    """Meshes of successive point sets made by the device update's per-cell
+    code (run on the host) against fresh host builds: (entries that differ,
+    meshes updated, stars built again)."""
+    c = cfg if isinstance(cfg, rich_config) else rich_config.from_dict(cfg)
+    xs, ys = np.atleast_2d(xs), np.atleast_2d(ys)
+    steps, n = xs.shape
+    xs, ys = _f64(xs.ravel()), _f64(ys.ravel())
+    v = [C.c_int64() for _ in range(3)]
+    _check(_lib().rich_device_update_check(C.byref(c), n, steps, _p(xs), _p(ys), *[C.byref(k) for k in v]))
+    return tuple(k.value for k in v)
+
+
+def rich_mesh_check(h):
+    """(entries of the device mesh that differ from a fresh host build,
+    meshes the device has updated so far)."""
+    a, b = C.c_int64(), C.c_int64()
+    _check(_lib().rich_mesh_check(h, C.byref(a), C.byref(b)))
+    return a.value, b.value
 
 
 def rich_batch_create(precision=0, max_cells=1 << 24, host_threads=0):

@@ -1,0 +1,98 @@
+"""The mesh a simulation holds on the device after steps, updated there from
+step to step, equals a fresh host build of its points entry by entry, and the
+steps are made by the update and not by the host builder."""
+import numpy as np
+import pytest
+
+from paper_1410_3219_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def R():
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_1410_3219_gb300 import rich
+    return rich
+
+
+def _drift():
+    wl = W.kelvin_helmholtz(n_side=64)
+    wl["vx"] = wl["vx"] + 40.0  # several cells a step through the boundary
+    return wl
+
+
+@pytest.mark.parametrize("name,make,steps,share", [
+    ("sod_64", lambda: W.sod(n_side=64), 60, 1.0),
+    ("sod_rough_53", lambda: W.sod(n_side=53, jitter=0.45), 40, 1.0),
+    ("kh_128", lambda: W.kelvin_helmholtz(n_side=128, amp=0.1), 40, 1.0),
+    ("kh_drift", _drift, 40, 1.0),
+    ("advection_lattice", lambda: W.advection(n_side=32), 20, 1.0),
+    ("static", lambda: W.uniform(n_side=40, motion=W.MESH_EULERIAN), 8, 1.0),
+    ("sedov_20000", lambda: W.sedov(n=20000, seed=2), 12, 0.5),
+    ("random_257", lambda: W.random_smooth(n=257), 20, 0.5),
+    ("small_8", lambda: W.gresho(n_side=8), 20, 0.5),
+    ("below_the_update", lambda: W.gresho(n_side=7), 4, 0.0),
+])
+@pytest.mark.parametrize("scheme", [W.SCHEME_EXTRAPOLATED, W.SCHEME_TIME_CENTRED])
+def test_device_mesh_equals_fresh_build(R, name, make, steps, share, scheme):
+    wl = make()
+    wl["cfg"]["scheme"] = scheme
+    sim = R.Sim(wl)
+    meshes = steps * (2 if scheme == W.SCHEME_TIME_CENTRED else 1)
+    for k in range(4):
+        sim.step(steps // 4)
+        mismatched, updates = R.rich_mesh_check(sim.h)
+        assert mismatched == 0, (k, updates)
+    assert updates >= share * meshes - 1, (updates, meshes)
+    if share == 0.0:
+        assert updates == 0
+    sim.close()
+
+
+def test_failed_and_repeated_steps_keep_the_mesh(R):
+    """A failed step leaves the mesh of the points it started from; the
+    pieces API updates the same mesh again."""
+    wl = W.random_mixed(n=400, seed=8)
+    wl["p"] = np.where(np.arange(400) == 7, 1e12, wl["p"])
+    sim = R.Sim(wl)
+    failed = False
+    for _ in range(30):
+        try:
+            sim.step(1)
+        except R.RichError:
+            failed = True
+            break
+    sim.tessellate()
+    assert R.rich_mesh_check(sim.h)[0] == 0
+    sim.tessellate()
+    assert R.rich_mesh_check(sim.h)[0] == 0
+    assert failed or sim.conserved()["m"].min() > 0
+    sim.close()
+
+
+def test_batch_membership_changes_repack_updated_meshes(R):
+    """Simulations that leave and join between steps: the others' meshes come
+    from the device, and every result equals its solo run bit for bit."""
+    wls = [W.sod(n_side=24, seed=1), W.gresho(n_side=30, seed=2), W.kelvin_helmholtz(n_side=20, seed=3),
+           W.sod(n_side=31, seed=4), W.gresho(n_side=6, seed=5)]
+    budget = [9, 4, 14, 6, 5]
+    b = R.Batch(max_cells=1 << 20)
+    ids = [b.add(w, max_steps=k) for w, k in zip(wls[:3], budget[:3])]
+    for k in range(14):
+        if k == 2:
+            ids.append(b.add(wls[3], max_steps=budget[3]))
+        if k == 7:
+            ids.append(b.add(wls[4], max_steps=budget[4]))
+        b.step()
+    for w, sid, k in zip(wls, ids, budget):
+        q = b.query(sid)
+        assert q["state"] == "done" and q["steps"] == k
+        solo = R.Sim(w)
+        solo.step(k)
+        got, want = b.conserved(sid), solo.conserved()
+        for f in want:
+            assert np.array_equal(got[f], want[f]), (sid, f)
+        solo.close()
+    b.close()

@@ -1,0 +1,106 @@
+"""The device's mesh update (star splaying over the cells whose neighbours
+changed) run serially on the host: its meshes equal fresh host builds entry
+by entry (rings, offsets, processing order, ghosts), over periodic and walled
+boxes, co-circular lattices (every edge decided by the exact predicates and
+the tie-break), points crossing walls and periodic boundaries, sheared rows
+(large reconnections), drifts of several cells a step, elongated and offset
+boxes, and the smallest sizes."""
+import numpy as np
+import pytest
+
+from paper_1410_3219_gb300 import rich as R
+from paper_1410_3219_gb300 import workloads as W
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    import __graft_entry__
+    __graft_entry__.build_library()
+
+
+def _walk(box, boundary, nx, ny, jitter, step, steps, drift=0.0, rows=0.0, seed=0):
+    """Successive point sets: a jittered lattice whose points move by up to
+    `step` spacings at random, drift together, and slide in alternate bands."""
+    x0, x1, y0, y1 = box
+    rng = np.random.default_rng(seed)
+    hx, hy = (x1 - x0) / nx, (y1 - y0) / ny
+    x, y = W.jittered_lattice(nx, ny, x0, x1, y0, y1, jitter, rng)
+    xs, ys = [x], [y]
+    for _ in range(steps - 1):
+        x = x + rng.uniform(-step, step, x.size) * hx + drift * hx * rng.uniform(-1, 1)
+        y = y + rng.uniform(-step, step, y.size) * hy + drift * hy * rng.uniform(-1, 1)
+        if rows:
+            u = (x - x0) / (x1 - x0)
+            x = x + np.where(np.floor((y - y0) / (y1 - y0) * 8) % 2 == 0, rows, -rows) * hx * (
+                1.0 if boundary else 4.0 * u * (1.0 - u))
+        if boundary == W.BC_PERIODIC:
+            x, y = x0 + np.mod(x - x0, x1 - x0), y0 + np.mod(y - y0, y1 - y0)
+            x, y = np.where(x >= x1, x0, x), np.where(y >= y1, y0, y)
+        else:
+            x = np.where(x <= x0, 2 * x0 - x, np.where(x >= x1, 2 * x1 - x, x))
+            y = np.where(y <= y0, 2 * y0 - y, np.where(y >= y1, 2 * y1 - y, y))
+        xs.append(x)
+        ys.append(y)
+    return np.array(xs), np.array(ys)
+
+
+UNIT = (0.0, 1.0, 0.0, 1.0)
+
+
+@pytest.mark.parametrize("boundary", [W.BC_PERIODIC, W.BC_REFLECTIVE])
+@pytest.mark.parametrize("name,kw,least", [
+    ("jittered", dict(box=UNIT, nx=40, ny=40, jitter=0.1, step=0.02, steps=12), 11),
+    ("rough", dict(box=UNIT, nx=33, ny=37, jitter=0.45, step=0.1, steps=12), 11),
+    ("lattice_at_rest", dict(box=UNIT, nx=32, ny=32, jitter=0.0, step=0.0, steps=3), 2),
+    ("lattice_inexact", dict(box=(-0.3, 0.7, 0.1, 1.1), nx=29, ny=29, jitter=0.0, step=0.0, steps=3), 2),
+    ("lattice_sheared", dict(box=UNIT, nx=32, ny=32, jitter=0.0, step=0.0, rows=0.25, steps=9), 8),
+    ("large_moves", dict(box=UNIT, nx=32, ny=32, jitter=0.1, step=0.25, steps=10), 9),
+    ("sliding_rows", dict(box=UNIT, nx=48, ny=48, jitter=0.1, step=0.02, rows=0.4, steps=12), 11),
+    ("elongated_box", dict(box=(-4.0, 12.0, 3.0, 5.0), nx=96, ny=12, jitter=0.2, step=0.05, steps=10), 9),
+    ("tiny_box_far_away", dict(box=(7.0, 7.0 + 1e-6, -3.0, -3.0 + 1e-6), nx=24, ny=24, jitter=0.2, step=0.05, steps=6),
+     5),
+    ("eight_by_eight", dict(box=UNIT, nx=8, ny=8, jitter=0.1, step=0.03, steps=12), 6),
+])
+def test_update_equals_fresh_build(name, kw, least, boundary):
+    xs, ys = _walk(boundary=boundary, **kw)
+    box = kw["box"]
+    cfg = W.default_cfg(boundary=boundary, x0=box[0], x1=box[1], y0=box[2], y1=box[3])
+    mismatched, updated, _ = R.rich_device_update_check(cfg, xs, ys)
+    assert mismatched == 0
+    assert updated >= least
+
+
+def test_update_follows_a_drift_through_the_periodic_boundary():
+    xs, ys = _walk(UNIT, W.BC_PERIODIC, 32, 32, 0.1, 0.02, 20, drift=3.0)
+    mismatched, updated, _ = R.rich_device_update_check(W.default_cfg(), xs, ys)
+    assert (mismatched, updated) == (0, 19)
+
+
+@pytest.mark.parametrize("n", [3, 5, 16, 64, 257, 1023, 1025])
+@pytest.mark.parametrize("boundary", [W.BC_PERIODIC, W.BC_REFLECTIVE])
+def test_random_points_of_ragged_sizes(n, boundary):
+    """What the update cannot make (small boxes) it leaves to the host; what
+    it makes equals the fresh build."""
+    rng = np.random.default_rng(n)
+    x, y = rng.uniform(0.02, 0.98, n), rng.uniform(0.02, 0.98, n)
+    d = 0.05 / np.sqrt(n)
+    sets = []
+    for _ in range(6):
+        sets.append((x, y))
+        x = np.clip(x + rng.uniform(-d, d, n), 0.001, 0.999)
+        y = np.clip(y + rng.uniform(-d, d, n), 0.001, 0.999)
+    cfg = W.default_cfg(boundary=boundary)
+    mismatched, updated, _ = R.rich_device_update_check(cfg, np.array([s[0] for s in sets]),
+                                                        np.array([s[1] for s in sets]))
+    assert mismatched == 0
+    if n >= 257:
+        assert updated == 5
+
+
+def test_coincident_points_are_left_to_the_host_builder():
+    rng = np.random.default_rng(3)
+    x, y = W.jittered_lattice(16, 16, 0.0, 1.0, 0.0, 1.0, 0.1, rng)
+    x2, y2 = x.copy(), y.copy()
+    x2[17], y2[17] = x[18], y[18]
+    with pytest.raises(R.RichError, match="EDUPLICATE"):
+        R.rich_device_update_check(W.default_cfg(), np.array([x, x2]), np.array([y, y2]))
