@@ -130,9 +130,10 @@ int rich_init_mesh(const rich_config *cfg, int64_t n, const double *x, const dou
    device for the current points and mesh, then a0 for the moved points
    (twice, with a0 for the half-step points in between, in the time-centred
    scheme).  A step that does not land on t_end thus leaves the mesh of its
-   points built, and the next step or call starts with the sweep; the device
+   points updated, and the next step or call starts with the sweep; the device
    may still be writing that mesh when the call returns, and later calls wait
-   for it.  Results equal those of rich_tessellate / rich_sweep / rich_sync in
+   for it.  A mesh left to the host (see rich_tessellate) is built by the next
+   step or call.  Results equal those of rich_tessellate / rich_sweep / rich_sync in
    turn, bit for bit.  info may be NULL.
    Errors: RICH_ENEGATIVE / RICH_ENAN (state left at the last good step),
    RICH_ETESS, RICH_EDUPLICATE, RICH_ECUDA. */

@@ -107,15 +107,18 @@ struct rich_batch {
     // The device's mesh update (meshupdate.h) for the packed cells: after a
     // step dev_mesh says that the arrays of buffers mcur hold the meshes of
     // the moved points of `packed` (those of simulations with a mesh flag
-    // excepted), dev_lists that the triangle and edge lists are built too
-    // and none is flagged.  A step whose simulations are the same then starts
+    // excepted), dev_lists that none is flagged and the triangle and edge
+    // lists are good.  A step whose simulations are the same then starts
     // with the sweep; else the meshes are read back and packed again.
     rich::MeshUpdater updater;
-    rich::MeshSizes msz;
     int mcur = 0;
     bool dev_mesh = false, dev_lists = false;
     std::vector<int32_t> mesh_flag;
-    rich::HBuf h_back;  // dt, status per simulation, then the list builders' flags
+    // reads: the caller's index of each packed cell (within its simulation),
+    // and a simulation's state in that order on the device and page-locked
+    DBuf perm_dev, read_dev;
+    rich::HBuf read_host;
+    rich::HBuf h_back;  // dt, status per simulation, then the list builder's flag
     cudaEvent_t ev2 = nullptr, ev3 = nullptr;
     bool diagnostics = false;
     int cur = 0;
@@ -125,7 +128,7 @@ struct rich_batch {
     DBuf cell_ptr[2], slot_nb[2], gsrc[2], gimg[2];
     DBuf gx, gy, gxf, tri, ccx, ccy, slot_tri, slot_edge;
     DBuf edge_l, edge_r, edge_ta, edge_tb, eL, emlx, emly, emrx, emry, enx, eny, eqx, eqy, F, ePM;
-    DBuf instp, dtmin, dtout, status, dsizes, gsync, eoff, toff, gshift, edgebad;
+    DBuf instp, dtmin, dtout, status, dsizes, gsync, eoff, toff, gshift, listbad;
     // launch shape: autotuned over the first steps unless fixed by the caller
     int launch_mode = 0;  // 0 autotune, 1 staged, 2 persistent
     int fixed_block = 256;
@@ -154,7 +157,7 @@ struct rich_batch {
     std::vector<int32_t> h_dptr, h_dnb, h_dgsrc, h_dgxf, h_dgshift, h_dgimg, h_dtoff, h_deoff, h_dorder;
     std::vector<int32_t> h_gsrc, h_gxf, h_cell_ptr, h_slot_nb, h_cell_inst;
     std::vector<int32_t> h_corder;
-    std::vector<int32_t> h_src, h_eoff, h_toff, h_gshift, h_gimg;
+    std::vector<int32_t> h_src, h_eoff, h_toff, h_gshift, h_gimg, h_perm;
     std::vector<rich::InstParams> h_inst;
     int64_t nG = 0, nT = 0, nE = 0, nS = 0;
 
@@ -174,7 +177,7 @@ struct rich_batch {
 
     double *dt_back() const { return h_back.as<double>(); }
     int32_t *status_back() const { return reinterpret_cast<int32_t *>(h_back.as<double>() + packed.size()); }
-    int32_t *list_flags() const { return reinterpret_cast<int32_t *>(h_back.as<char>() + h_back.cap) - 2; }
+    int32_t *list_flag() const { return reinterpret_cast<int32_t *>(h_back.as<char>() + h_back.cap) - 2; }
 
     size_t rsize() const { return precision == RICH_FP32_SPLIT ? sizeof(float) : sizeof(double); }
 
@@ -280,6 +283,7 @@ void pack_part(rich_batch *b, BatchSim &s, const PackTask &t)
         std::memcpy(&b->h_y[co + i0], s.hy.data() + i0, sizeof(double) * (i1 - i0));
         for (int64_t i = i0; i < i1; i++) {
             b->h_cell_inst[co + i] = t.k;
+            b->h_perm[co + i] = s.perm[i];
             b->h_cell_ptr[co + i] = (int32_t)(so + m.cell_ptr[i]);
             b->h_corder[co + i] = (int32_t)(co + m.cell_order[i]);
             b->h_eoff[co + i] = (int32_t)(eo + m.edge_off[i]);
@@ -327,8 +331,7 @@ void pack_all(rich_batch *b, const std::vector<BatchSim *> &ok)
 
 int ensure_device(rich_batch *b)
 {
-    const size_t N = (size_t)b->n_packed, d = sizeof(double), r = b->rsize();
-    const size_t G = (size_t)b->nG, T = (size_t)b->nT, E = (size_t)b->nE, K = b->packed.size();
+    const size_t N = (size_t)b->n_packed, d = sizeof(double), r = b->rsize(), K = b->packed.size();
     for (int k = 0; k < 2; k++) {
         CUDA_TRY(b->x[k].ensure(N * d + 8));
         CUDA_TRY(b->y[k].ensure(N * d + 8));
@@ -340,16 +343,10 @@ int ensure_device(rich_batch *b)
     CUDA_TRY(b->alpha.ensure(4 * N * r + 32)); CUDA_TRY(b->w.ensure(2 * N * r + 16));
     CUDA_TRY(b->tess.ensure(N * 4 + 4)); CUDA_TRY(b->rounding.ensure(N + 8)); CUDA_TRY(b->p64.ensure(N * d + 8));
     CUDA_TRY(b->psrc.ensure(4 * N * r + 32));
-    CUDA_TRY(b->ccx.ensure(T * d + 8)); CUDA_TRY(b->ccy.ensure(T * d + 8));
-    for (DBuf *e : {&b->eL, &b->emlx, &b->emly, &b->emrx, &b->emry, &b->enx, &b->eny, &b->eqx, &b->eqy})
-        CUDA_TRY(e->ensure(E * r + 8));
-    CUDA_TRY(b->F.ensure(4 * E * sizeof(double) + 32));
-    CUDA_TRY(b->ePM.ensure(4 * E * r + 32));
     CUDA_TRY(b->instp.ensure(K * sizeof(rich::InstParams) + 8));
     CUDA_TRY(b->dtmin.ensure(K * 8 + 8)); CUDA_TRY(b->dtout.ensure(K * 8 + 8)); CUDA_TRY(b->status.ensure(K * 4 + 8));
     CUDA_TRY(b->h_back.ensure(K * 12 + 64));
     CUDA_TRY(b->dsizes.ensure(sizeof(rich::DeviceSizes))); CUDA_TRY(b->gsync.ensure(sizeof(rich::GridSync)));
-    (void)G;
     return RICH_OK;
 }
 
@@ -467,38 +464,75 @@ int run_staged(rich_batch *b)
     return RICH_OK;
 }
 
-// The packed triangle and edge lists, built on the device from the rings of
-// buffers `mesh` (each cell's box type from its simulation's parameters),
-// with the builders' flags copied into h_back; the caller checks them before
-// any kernel reads the lists.
-int build_lists(rich_batch *b, int mesh)
+rich::MeshLists mesh_lists(const rich_batch *b)
 {
-    const size_t T = (size_t)b->nT, E = (size_t)b->nE, S = (size_t)b->nS;
-    CUDA_TRY(b->tri.ensure(T * 12 + 12));
-    CUDA_TRY(b->slot_tri.ensure(S * 4 + 4));
-    CUDA_TRY(b->slot_edge.ensure(S * 4 + 4));
-    for (DBuf *e : {&b->edge_l, &b->edge_r, &b->edge_ta, &b->edge_tb}) CUDA_TRY(e->ensure(E * 4 + 4));
-    CUDA_TRY(b->edgebad.ensure(8));
-    int32_t *bad = b->edgebad.as<int32_t>();
-    const int32_t N = (int32_t)b->n_packed;
-    const int32_t *ptr = b->cell_ptr[mesh].as<int32_t>(), *nb = b->slot_nb[mesh].as<int32_t>();
-    CUDA_TRY(rich::launch_build_tris(N, (int32_t)S, ptr, nb, b->toff.as<int32_t>(), b->tri.as<int32_t>(),
-                                     b->slot_tri.as<int32_t>(), bad + 1, b->stream));
-    CUDA_TRY(rich::launch_build_edges(N, (int32_t)S, ptr, nb, b->slot_tri.as<int32_t>(), b->gsrc[mesh].as<int32_t>(),
-                                      b->gshift.as<int32_t>(), b->eoff.as<int32_t>(), 0,
-                                      b->instp.as<rich::InstParams>(), b->cell_inst.as<int32_t>(),
-                                      b->slot_edge.as<int32_t>(), b->edge_l.as<int32_t>(), b->edge_r.as<int32_t>(),
-                                      b->edge_ta.as<int32_t>(), b->edge_tb.as<int32_t>(), bad, b->stream));
-    CUDA_TRY(cudaMemcpyAsync(b->list_flags(), bad, 8, cudaMemcpyDeviceToHost, b->stream));
+    rich::MeshLists l{};
+    l.tri = b->tri.as<int32_t>();
+    l.slot_tri = b->slot_tri.as<int32_t>();
+    l.slot_edge = b->slot_edge.as<int32_t>();
+    l.edge_l = b->edge_l.as<int32_t>(); l.edge_r = b->edge_r.as<int32_t>();
+    l.edge_ta = b->edge_ta.as<int32_t>(); l.edge_tb = b->edge_tb.as<int32_t>();
+    return l;
+}
+
+// Room for the rings of packed meshes of these sizes in buffers m, and for
+// the rest of them (nothing on the stream may still use the arrays).
+int reserve_rings(rich_batch *b, int m, const rich::MeshSizes &z)
+{
+    const size_t G = (size_t)z.ghosts + 1;
+    CUDA_TRY(b->cell_ptr[m].ensure(((size_t)b->n_packed + 1) * 4));
+    CUDA_TRY(b->slot_nb[m].ensure(((size_t)z.slots + 1) * 4));
+    CUDA_TRY(b->gsrc[m].ensure(G * 4)); CUDA_TRY(b->gimg[m].ensure(G * 4));
     return RICH_OK;
 }
 
-int check_lists(rich_batch *b)
+int reserve_mesh(rich_batch *b, const rich::MeshSizes &z)
 {
-    const int32_t *bad = b->list_flags();
-    if (bad[1]) return fail(RICH_ETESS, "a triangle of a ring is missing from its owner's ring");
-    if (bad[0]) return fail(RICH_ETESS, "an edge of a ring has no partner in the other cell's ring");
+    const size_t N = (size_t)b->n_packed, G = (size_t)z.ghosts + 1, T = (size_t)z.tris + 1, E = (size_t)z.edges + 1;
+    const size_t S = (size_t)z.slots + 1, r = b->rsize(), d = sizeof(double);
+    CUDA_TRY(b->gx.ensure(G * 8)); CUDA_TRY(b->gy.ensure(G * 8));
+    CUDA_TRY(b->gxf.ensure(G * 4)); CUDA_TRY(b->gshift.ensure(G * 4));
+    CUDA_TRY(b->toff.ensure((N + 1) * 4)); CUDA_TRY(b->eoff.ensure((N + 1) * 4)); CUDA_TRY(b->corder.ensure(N * 4));
+    CUDA_TRY(b->tri.ensure(T * 12));
+    CUDA_TRY(b->slot_tri.ensure(S * 4));
+    CUDA_TRY(b->slot_edge.ensure(S * 4));
+    for (DBuf *e : {&b->edge_l, &b->edge_r, &b->edge_ta, &b->edge_tb}) CUDA_TRY(e->ensure(E * 4));
+    CUDA_TRY(b->ccx.ensure(T * d)); CUDA_TRY(b->ccy.ensure(T * d));
+    for (DBuf *e : {&b->eL, &b->emlx, &b->emly, &b->emrx, &b->emry, &b->enx, &b->eny, &b->eqx, &b->eqy})
+        CUDA_TRY(e->ensure(E * r));
+    CUDA_TRY(b->F.ensure(4 * E * sizeof(double)));
+    CUDA_TRY(b->ePM.ensure(4 * E * r));
     return RICH_OK;
+}
+
+// where an update writes (its rings to buffers m), as far as the arrays reach
+rich::MeshOutput mesh_output(const rich_batch *b, int m)
+{
+    rich::MeshOutput o{};
+    o.cell_ptr = b->cell_ptr[m].as<int32_t>();
+    o.slot_nb = b->slot_nb[m].as<int32_t>();
+    o.tri_off = b->toff.as<int32_t>();
+    o.edge_off = b->eoff.as<int32_t>();
+    o.cell_order = b->corder.as<int32_t>();
+    o.gx = b->gx.as<double>();
+    o.gy = b->gy.as<double>();
+    o.ghost_src = b->gsrc[m].as<int32_t>();
+    o.ghost_xf = b->gxf.as<int32_t>();
+    o.ghost_shift = b->gshift.as<int32_t>();
+    o.ghost_img = b->gimg[m].as<int32_t>();
+    const size_t r = b->rsize();
+    size_t e = std::min(b->F.cap / 32, b->ePM.cap / (4 * r));
+    for (const DBuf *k : {&b->edge_l, &b->edge_r, &b->edge_ta, &b->edge_tb}) e = std::min(e, k->cap / 4);
+    for (const DBuf *k : {&b->eL, &b->emlx, &b->emly, &b->emrx, &b->emry, &b->enx, &b->eny, &b->eqx, &b->eqy})
+        e = std::min(e, k->cap / r);
+    const size_t g = std::min({b->gx.cap / 8, b->gy.cap / 8, b->gsrc[m].cap / 4, b->gimg[m].cap / 4, b->gxf.cap / 4,
+                               b->gshift.cap / 4});
+    const size_t t = std::min({b->tri.cap / 12, b->ccx.cap / 8, b->ccy.cap / 8});
+    const size_t q = std::min({b->slot_nb[m].cap / 4, b->slot_tri.cap / 4, b->slot_edge.cap / 4});
+    auto i32 = [](size_t v) { return (int32_t)std::min<size_t>(v, INT32_MAX / 4); };
+    o.max = rich::MeshSizes{i32(g), i32(t), i32(e), i32(q)};
+    o.lists = mesh_lists(b);
+    return o;
 }
 
 rich::MeshArrays mesh_arrays(rich_batch *b, int q)
@@ -517,52 +551,34 @@ rich::MeshArrays mesh_arrays(rich_batch *b, int q)
     return a;
 }
 
-// The updated meshes of the points in buffers q written, after the update's
-// first part was waited for; with `lists` (the next step has the same
-// simulations, as far as is known) the triangle and edge lists too.
-int finish_update(rich_batch *b, int q, bool lists)
+// After the update for the points in buffers q was waited for: the meshes of
+// the packed simulations on the device, as far as it made them.
+int finish_update(rich_batch *b, int q)
 {
     b->dev_mesh = b->dev_lists = false;
-    rich::MeshSizes z;
-    bool ok = false;
     const rich::MeshArrays a = mesh_arrays(b, q);
-    CUDA_TRY(b->updater.settle(a, ok, z, b->stream));
-    if (!ok) return RICH_OK;
-    b->mesh_flag.assign(b->updater.flags(), b->updater.flags() + a.n_inst);
-    for (int32_t f : b->mesh_flag) lists = lists && !f;
     const int m = 1 - b->mcur;
-    const size_t N = (size_t)b->n_packed, G = (size_t)z.ghosts + 1;
-    CUDA_TRY(b->cell_ptr[m].ensure((N + 1) * 4));
-    CUDA_TRY(b->slot_nb[m].ensure(((size_t)z.slots + 1) * 4));
-    CUDA_TRY(b->gsrc[m].ensure(G * 4)); CUDA_TRY(b->gimg[m].ensure(G * 4));
-    CUDA_TRY(b->gx.ensure(G * 8)); CUDA_TRY(b->gy.ensure(G * 8));
-    CUDA_TRY(b->gxf.ensure(G * 4)); CUDA_TRY(b->gshift.ensure(G * 4));
-    rich::MeshOutput o{};
-    o.cell_ptr = b->cell_ptr[m].as<int32_t>();
-    o.slot_nb = b->slot_nb[m].as<int32_t>();
-    o.tri_off = b->toff.as<int32_t>();
-    o.edge_off = b->eoff.as<int32_t>();
-    o.cell_order = b->corder.as<int32_t>();
-    o.gx = b->gx.as<double>();
-    o.gy = b->gy.as<double>();
-    o.ghost_src = b->gsrc[m].as<int32_t>();
-    o.ghost_xf = b->gxf.as<int32_t>();
-    o.ghost_shift = b->gshift.as<int32_t>();
-    o.ghost_img = b->gimg[m].as<int32_t>();
-    CUDA_TRY(b->updater.finish(a, o, b->stream));
-    b->mcur = m;
-    b->msz = z;
-    b->nG = z.ghosts;
-    b->nT = z.tris;
-    b->nE = z.edges;
-    b->nS = z.slots;
-    if (lists) {
-        int rc = build_lists(b, m);
+    rich::MeshResult r;
+    CUDA_TRY(b->updater.settle(a, mesh_output(b, m), r, b->stream));
+    if (r.state == rich::MeshResult::kGrow) {
+        int rc = reserve_mesh(b, r.sizes);
+        if (!rc) rc = reserve_rings(b, m, r.sizes);
         if (rc) return rc;
+        CUDA_TRY(b->updater.again(a, mesh_output(b, m), r, b->stream));
     }
+    if (r.state != rich::MeshResult::kDone || (r.bad && !r.flagged)) {
+        b->updater.forget();
+        return RICH_OK;
+    }
+    b->mesh_flag.assign(b->updater.flags(), b->updater.flags() + a.n_inst);
+    b->mcur = m;
+    b->nG = r.sizes.ghosts;
+    b->nT = r.sizes.tris;
+    b->nE = r.sizes.edges;
+    b->nS = r.sizes.slots;
     b->dev_mesh = true;
-    b->dev_lists = lists;
-    return RICH_OK;
+    b->dev_lists = !r.flagged;
+    return reserve_rings(b, 1 - m, r.sizes);
 }
 
 // The meshes of the simulations that go on, read back from the device into
@@ -863,6 +879,7 @@ int pack_step(rich_batch *b, const std::vector<BatchSim *> &list, double &t1, do
     bool any_pending = false;
     for (BatchSim *s : ok) any_pending |= s->state == PENDING;
     b->h_x.resize(N); b->h_y.resize(N); b->h_cell_inst.resize(N); b->h_src.resize(N);
+    b->h_perm.resize(N);
     b->h_gx.resize(go); b->h_gy.resize(go); b->h_gsrc.resize(go); b->h_gxf.resize(go);
     b->h_cell_ptr.resize(N + 1); b->h_corder.resize(N);
     b->h_slot_nb.resize(so);
@@ -877,6 +894,9 @@ int pack_step(rich_batch *b, const std::vector<BatchSim *> &list, double &t1, do
     for (size_t k = 0; k < ok.size(); k++) b->h_inst[k] = inst_params(*ok[k], ok[k]->state == PENDING);
     // 4. device buffers and uploads
     if ((rc = ensure_device(b))) return rc;
+    const rich::MeshSizes z{(int32_t)go, (int32_t)to, (int32_t)eo, (int32_t)so};
+    b->updater.forget();
+    if ((rc = reserve_mesh(b, z)) || (rc = reserve_rings(b, 0, z)) || (rc = reserve_rings(b, 1, z))) return rc;
     const int nxt = 1 - b->cur;
     if (!same_layout && n_old > 0) {
         // regather the conserved state of continuing simulations into the other
@@ -896,6 +916,7 @@ int pack_step(rich_batch *b, const std::vector<BatchSim *> &list, double &t1, do
     CUDA_TRY(upload(b->x[b->cur], b->h_x, b->stream));
     CUDA_TRY(upload(b->y[b->cur], b->h_y, b->stream));
     CUDA_TRY(upload(b->cell_inst, b->h_cell_inst, b->stream));
+    CUDA_TRY(upload(b->perm_dev, b->h_perm, b->stream));
     CUDA_TRY(upload(b->gx, b->h_gx, b->stream));
     CUDA_TRY(upload(b->gy, b->h_gy, b->stream));
     CUDA_TRY(upload(b->gsrc[b->mcur], b->h_gsrc, b->stream));
@@ -909,9 +930,25 @@ int pack_step(rich_batch *b, const std::vector<BatchSim *> &list, double &t1, do
     CUDA_TRY(upload(b->gshift, b->h_gshift, b->stream));
     CUDA_TRY(upload(b->instp, b->h_inst, b->stream));
     // the packed triangle and edge lists, checked before any kernel reads them
-    if ((rc = build_lists(b, b->mcur))) return rc;
-    CUDA_TRY(cudaStreamSynchronize(b->stream));
-    if ((rc = check_lists(b))) return rc;
+    {
+        CUDA_TRY(b->listbad.ensure(8));
+        rich::MeshLists l = mesh_lists(b);
+        l.n = (int32_t)N;
+        l.cell_inst = b->cell_inst.as<int32_t>();
+        l.inst = b->instp.as<rich::InstParams>();
+        l.cell_ptr = b->cell_ptr[b->mcur].as<int32_t>();
+        l.slot_nb = b->slot_nb[b->mcur].as<int32_t>();
+        l.tri_off = b->toff.as<int32_t>();
+        l.edge_off = b->eoff.as<int32_t>();
+        l.ghost_src = b->gsrc[b->mcur].as<int32_t>();
+        l.ghost_shift = b->gshift.as<int32_t>();
+        l.bad = b->listbad.as<int32_t>();
+        CUDA_TRY(cudaMemsetAsync(l.bad, 0, 4, b->stream));
+        CUDA_TRY(rich::launch_lists(l, b->stream));
+        CUDA_TRY(cudaMemcpyAsync(b->list_flag(), l.bad, 4, cudaMemcpyDeviceToHost, b->stream));
+        CUDA_TRY(cudaStreamSynchronize(b->stream));
+        if (*b->list_flag()) return fail(RICH_ETESS, "the rings of a mesh do not close");
+    }
     CUDA_TRY(cudaMemsetAsync(b->status.p, 0, ok.size() * 4, b->stream));
     if (any_pending) CUDA_TRY(upload(b->initW, b->h_W0, b->stream));
     // 5. admission: conserved variables of new simulations from their first geometry
@@ -956,18 +993,15 @@ int rich_batch_step(rich_batch *b, rich_step_info *info)
     if (b->dev_lists && list == b->packed) {
         // their meshes, lists and points are on the device already
         for (size_t k = 0; k < list.size(); k++) b->h_inst[k] = inst_params(*list[k], false);
-        CUDA_TRY(cudaStreamSynchronize(b->stream));
-        if ((rc = check_lists(b))) return rc;
         b->dev_mesh = b->dev_lists = false;
-        if ((rc = ensure_device(b))) return rc;
         CUDA_TRY(upload(b->instp, b->h_inst, b->stream));
     } else if ((rc = pack_step(b, list, t1, t2))) {
         return rc;
     }
     if (b->packed.empty()) return RICH_OK;
     const double t3 = now_ms();
-    // 6. the sweep over every cell of every simulation, then the first part
-    //    of the mesh update for the moved points (one wait for both)
+    // 6. the sweep over every cell of every simulation, then the mesh update
+    //    for the moved points (one wait for both)
     const std::vector<BatchSim *> ok = b->packed;
     const size_t N = (size_t)b->n_packed;
     const LaunchShape shape = pick_shape(b);
@@ -997,7 +1031,8 @@ int rich_batch_step(rich_batch *b, rich_step_info *info)
     }
     const bool update = (int64_t)N >= rich::kMeshUpdateMin && (int64_t)N <= rich::kMeshUpdateMax;
     CUDA_TRY(cudaEventRecord(b->ev2, b->stream));
-    if (update) CUDA_TRY(b->updater.start(mesh_arrays(b, 1 - b->cur), b->stream));
+    if (update)
+        CUDA_TRY(b->updater.start(mesh_arrays(b, 1 - b->cur), mesh_output(b, 1 - b->mcur), b->stream));
     CUDA_TRY(cudaEventRecord(b->ev3, b->stream));
     CUDA_TRY(cudaMemcpyAsync(b->dt_back(), b->dtout.p, ok.size() * 8, cudaMemcpyDeviceToHost, b->stream));
     CUDA_TRY(cudaMemcpyAsync(b->status_back(), b->status.p, ok.size() * 4, cudaMemcpyDeviceToHost, b->stream));
@@ -1040,7 +1075,8 @@ int rich_batch_step(rich_batch *b, rich_step_info *info)
     b->cur = nxt2;
     // 8. the updated meshes of the simulations that go on
     const double tf = now_ms();
-    if (update && going > 0 && (rc = finish_update(b, nxt2, going == ok.size()))) return rc;
+    if (update && going > 0 && (rc = finish_update(b, nxt2))) return rc;
+    if (update && going == 0) b->updater.forget();
     const double t_fin = now_ms() - tf;
     if (info) {
         info->steps_done = (int64_t)ok.size();
@@ -1078,30 +1114,29 @@ int rich_batch_get_conserved(rich_batch *b, int32_t id, int64_t n, double *x, do
     if (!b) return fail(RICH_EINVAL, "NULL handle");
     BatchSim *s = b->find(id);
     if (!s || n != s->n) return fail(RICH_EINVAL, "unknown simulation id or wrong size");
-    std::vector<double> buf;
-    const double *src = nullptr;
+    double *outs[6] = {x, y, m, px, py, E};
     if (s->state == DONE || s->state == FAILED) {
         if (s->fin.empty()) return fail(RICH_ESTATE, "no state recorded");
-        src = s->fin.data();
+        const double *src = s->fin.data();
+        for (int f = 0; f < 6; f++) {
+            if (!outs[f]) continue;
+            for (int32_t k = 0; k < s->n; k++) outs[f][s->perm[k]] = src[(size_t)f * s->n + k];
+        }
     } else if (s->state == RUNNING) {
-        const size_t nn = (size_t)s->n, N = (size_t)b->n_packed;
-        buf.resize(6 * nn);
-        CUDA_TRY(cudaMemcpyAsync(&buf[0], b->x[b->cur].as<double>() + s->cell_off, nn * 8, cudaMemcpyDeviceToHost,
-                                 b->stream));
-        CUDA_TRY(cudaMemcpyAsync(&buf[nn], b->y[b->cur].as<double>() + s->cell_off, nn * 8, cudaMemcpyDeviceToHost,
-                                 b->stream));
-        for (int c = 0; c < 4; c++)
-            CUDA_TRY(cudaMemcpyAsync(&buf[(2 + c) * nn], b->U[b->cur].as<double>() + c * N + s->cell_off, nn * 8,
-                                     cudaMemcpyDeviceToHost, b->stream));
+        // put in the caller's order on the device, one copy down
+        const size_t nn = (size_t)s->n, N = (size_t)b->n_packed, co = (size_t)s->cell_off;
+        const double *U = b->U[b->cur].as<double>() + co;
+        const double *src[6] = {b->x[b->cur].as<double>() + co, b->y[b->cur].as<double>() + co, U, U + N, U + 2 * N,
+                                U + 3 * N};
+        CUDA_TRY(b->read_dev.ensure(6 * nn * 8));
+        CUDA_TRY(b->read_host.ensure(6 * nn * 8));
+        CUDA_TRY(rich::launch_unpermute(s->n, b->perm_dev.as<int32_t>() + co, src, b->read_dev.as<double>(), b->stream));
+        CUDA_TRY(cudaMemcpyAsync(b->read_host.p, b->read_dev.p, 6 * nn * 8, cudaMemcpyDeviceToHost, b->stream));
         CUDA_TRY(cudaStreamSynchronize(b->stream));
-        src = buf.data();
+        for (int f = 0; f < 6; f++)
+            if (outs[f]) std::memcpy(outs[f], b->read_host.as<double>() + (size_t)f * nn, nn * 8);
     } else {
         return fail(RICH_ESTATE, "simulation not admitted yet");
-    }
-    double *outs[6] = {x, y, m, px, py, E};
-    for (int f = 0; f < 6; f++) {
-        if (!outs[f]) continue;
-        for (int32_t k = 0; k < s->n; k++) outs[f][s->perm[k]] = src[(size_t)f * s->n + k];
     }
     return RICH_OK;
 }

@@ -5,6 +5,8 @@
 
 #include <cuda_runtime.h>
 
+#include "sweep.cuh"
+
 namespace rich {
 namespace {
 
@@ -22,7 +24,39 @@ __global__ void k_unpermute(int32_t n, const int32_t *__restrict__ perm, const d
         if (src[f]) dst[(int64_t)f * n + u] = src[f][k];
 }
 
+// Eight fields of every cell for rich_get_state, in the caller's order: the
+// points, the primitives (rho, vx, vy, p side by side per cell, in the
+// simulation's precision) and the area
+template <class R>
+__global__ void k_unpermute_state(int32_t n, const int32_t *__restrict__ perm, const double *__restrict__ x,
+                                  const double *__restrict__ y, const Vec4<R> *__restrict__ W,
+                                  const double *__restrict__ area, double *__restrict__ dst)
+{
+    const int32_t k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= n) return;
+    const int64_t u = perm[k], N = n;
+    const Vec4<R> w = W[k];
+    dst[u] = x[k];
+    dst[N + u] = y[k];
+    dst[2 * N + u] = (double)w.x;
+    dst[3 * N + u] = (double)w.y;
+    dst[4 * N + u] = (double)w.z;
+    dst[5 * N + u] = (double)w.w;
+    dst[6 * N + u] = area[k];
+}
+
 }  // namespace
+
+cudaError_t launch_unpermute_state(int32_t n, const int32_t *perm, const double *x, const double *y, const void *W,
+                                   bool single, const double *area, double *dst, cudaStream_t st)
+{
+    const int b = (n + 255) / 256;
+    if (n > 0 && single)
+        k_unpermute_state<float><<<b, 256, 0, st>>>(n, perm, x, y, static_cast<const Vec4<float> *>(W), area, dst);
+    else if (n > 0)
+        k_unpermute_state<double><<<b, 256, 0, st>>>(n, perm, x, y, static_cast<const Vec4<double> *>(W), area, dst);
+    return cudaGetLastError();
+}
 
 cudaError_t launch_unpermute(int32_t n, const int32_t *perm, const double *const src[6], double *dst,
                              cudaStream_t st)

@@ -11,28 +11,476 @@ namespace rich {
 namespace {
 
 constexpr int kVerifyBlock = 128;
-constexpr int kListBlock = 64;
+constexpr int kListWarps = 4;  // listed cells per block, a warp each
+constexpr int kListBlock = 32 * kListWarps;
 constexpr int kWindow = kOrderWindow;  // cells per block of the size and ring passes
 static_assert(kWindow == 1024, "the scans and the order pass run one window per 1024-thread block");
+constexpr unsigned kAll = 0xffffffffu;
 
+// mu::verify<true> with eight lanes per cell, a ring slot each: a thread per
+// cell walked its ring through a chain of dependent loads, slot after slot
+// (327 us at 1M cells; 24 us at 4,096).  Cells of more than eight neighbours
+// (3 % of a random mesh) go to the undecided ones.
 __global__ void __launch_bounds__(kVerifyBlock) k_mesh_verify(MeshUpdate m)
 {
-    const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < m.n) mu::verify(m, i);
+    using namespace mu;
+    const int lane = threadIdx.x & 31, k = lane & 7, group = lane & 24;
+    const int32_t t = (blockIdx.x * blockDim.x + threadIdx.x) >> 3;
+    const bool live = t < m.n;
+    const int32_t i = live ? t : m.n - 1;
+    const Frame f = frame_of(m, i);
+    const int32_t lo = m.cell_ptr[i], deg = m.cell_ptr[i + 1] - lo;
+    const bool mine = live && k < deg && deg <= 8;
+    const int32_t ref = base_ref(m, m.slot_nb[lo + (k < deg ? k : 0)]);
+    const Point d = point_of(f, ref);
+    const int kb = k ? k - 1 : min(deg, 8) - 1, ka = kb ? kb - 1 : min(deg, 8) - 1;
+    Point a, b;
+    b.fx = __shfl_sync(kAll, d.fx, group | kb);
+    b.fy = __shfl_sync(kAll, d.fy, group | kb);
+    b.ref = __shfl_sync(kAll, d.ref, group | kb);
+    a.fx = __shfl_sync(kAll, d.fx, group | ka);
+    a.fy = __shfl_sync(kAll, d.fy, group | ka);
+    a.ref = __shfl_sync(kAll, d.ref, group | ka);
+    a.l = a.fx * a.fx + a.fy * a.fy;
+    b.l = b.fx * b.fx + b.fy * b.fy;
+    const float p = b.fx * d.fy, q = b.fy * d.fx, cbd = p - q;
+    const float p3 = a.fx * d.fy, p4 = a.fy * d.fx, p5 = a.fx * b.fy, p6 = a.fy * b.fx;
+    const float det = a.l * cbd - b.l * (p3 - p4) + d.l * (p5 - p6);
+    const float bound = kCircleBound * (a.l * (fabsf(p) + fabsf(q)) + b.l * (fabsf(p3) + fabsf(p4)) +
+                                        d.l * (fabsf(p5) + fabsf(p6)));
+    bool bad = -det > bound;
+    bool open = deg > 8 || !(cbd > kCrossBound * (fabsf(p) + fabsf(q))) || !(det > bound || bad);
+    if (!f.periodic) open = open || ((b.ref & 15) != 4 && (d.ref & 15) != 4);
+    open = live && open && (mine || deg > 8);
+    bad = bad && mine;
+    const bool self = mine && (bad || d.ref != ref || !disk_ok(f, b, d));
+    const bool turn = mine && b.fy < 0.0f && d.fy >= 0.0f;
+    const unsigned byte = 0xffu << group;
+    const unsigned opens = __ballot_sync(kAll, open) & byte, selves = __ballot_sync(kAll, self) & byte;
+    const unsigned turns = __ballot_sync(kAll, turn) & byte;
+    // the block's cells are listed together: one counter took an atomic for
+    // each of the 400,000 cells of a lively step (266 us for this kernel at
+    // 1M cells, 110 where few are listed)
+    constexpr int kMost = kVerifyBlock / 8 * 32;  // 8 slots x 3 cells + 1, per cell
+    __shared__ int32_t cells[kMost];
+    __shared__ int32_t listed, at;
+    if (threadIdx.x == 0) listed = 0;
+    if (!__syncthreads_or(live && (opens || selves || __popc(turns) != 1))) return;
+    auto put = [&](int32_t v) {
+        if (vol(m.flags + inst_at(m, v)) || vol(m.mark + v) == m.stamp || a_exch(m.mark + v, m.stamp) == m.stamp) return;
+        cells[atomicAdd(&listed, 1)] = v;
+    };
+    if (live && opens) {
+        if (k == 0) m.list[1][atomicAdd(&m.count->open, 1)] = i;
+    } else if (live) {
+        // (list_bad)
+        if (bad) {
+            put(b.ref >> 4);
+            put(a.ref >> 4);
+            put(d.ref >> 4);
+            if (f.periodic || (a.ref & 15) == 4) tell_only(m, a.ref >> 4, d.ref);
+            if (f.periodic || (d.ref & 15) == 4) tell_only(m, d.ref >> 4, a.ref);
+        }
+        if (k == 0 && (selves || __popc(turns) != 1)) put(i);
+    }
+    __syncthreads();
+    const int32_t most = listed;
+    if (threadIdx.x == 0 && most > 0) at = atomicAdd(&m.count->listed[0], most);
+    __syncthreads();
+    for (int32_t q = threadIdx.x; q < most; q += kVerifyBlock) m.list[0][at + q] = cells[q];
+}
+
+// The cells FP32 left open, a warp each: a lane per ring slot, and for the
+// triangles of two images a lane per image that might lie in their circle.
+// (A thread per cell spent 127 us on the walls of 4,096 cells.)
+__global__ void __launch_bounds__(kListBlock) k_mesh_verify_open(MeshUpdate m)
+{
+    using namespace mu;
+    const int lane = threadIdx.x & 31;
+    const int32_t count = m.count->open;
+    for (int32_t c = blockIdx.x * kListWarps + (threadIdx.x >> 5); c < count; c += gridDim.x * kListWarps) {
+        const int32_t i = m.list[1][c];
+        const Frame f = frame_of(m, i);
+        const int32_t lo = m.cell_ptr[i], deg = m.cell_ptr[i + 1] - lo;
+        const int32_t *nb = m.slot_nb + lo;
+        bool self = false;
+        int turns = 0;
+        uint32_t imgs = 0;
+        if (!f.periodic)
+            for (int32_t k = lane; k < deg; k += 32) imgs |= 1u << (base_ref(m, nb[k]) & 15);
+        imgs = __reduce_or_sync(kAll, imgs) & ~(1u << 4);
+        for (int32_t base = 0; base < deg; base += 32) {
+            const int32_t k = base + lane;
+            bool pair = false;
+            if (k < deg) {
+                const int32_t kb = k ? k - 1 : deg - 1, ka = kb ? kb - 1 : deg - 1, ref = base_ref(m, nb[k]);
+                const Point a = point_of(f, base_ref(m, nb[ka])), b = point_of(f, base_ref(m, nb[kb]));
+                const Point d = point_of(f, ref);
+                if (orient_slow(f, b, d) <= 0 || incircle(f, a, b, d) >= 0) {
+                    list_bad(m, f.periodic, a.ref, b.ref, d.ref);
+                    self = true;
+                }
+                if (d.ref != ref || !disk_ok(f, b, d)) self = true;
+                turns += (b.fy < 0.0f && d.fy >= 0.0f) ? 1 : 0;
+                pair = !f.periodic && (b.ref & 15) != 4 && (d.ref & 15) != 4;
+            }
+            for (unsigned pairs = __ballot_sync(kAll, pair); pairs; pairs &= pairs - 1) {
+                const int32_t kp = base + __ffs(pairs) - 1;
+                const Point b = point_of(f, base_ref(m, nb[kp ? kp - 1 : deg - 1])), d = point_of(f, base_ref(m, nb[kp]));
+                const int32_t tests = __popc(imgs) * (deg + 1);
+                for (int32_t t = lane; t < tests; t += 32) {
+                    const int img = (int)__fns(imgs, 0, t / (deg + 1) + 1);
+                    const int32_t s = t % (deg + 1);
+                    const int32_t r = (s == deg ? i : base_ref(m, nb[s]) >> 4) * 16 + img;
+                    if (r != b.ref && r != d.ref && incircle(f, b, d, point_of(f, r)) > 0) self = true;
+                }
+                __syncwarp();
+            }
+        }
+        turns = __reduce_add_sync(kAll, turns);
+        if ((__any_sync(kAll, self) || turns != 1) && lane == 0) list_cell(m, i, 0);
+    }
+}
+
+// A recomputed star of `deg` neighbours, held one per lane (of `width` lanes
+// from lane `first`), into the version that no other cell reads in this round,
+// with the cell's sizes.  False when the stars' storage is full.
+__device__ __forceinline__ bool commit_star(const MeshUpdate &m, const mu::Frame &f, int32_t round, int32_t ref,
+                                            int deg, int first, int width, bool live)
+{
+    const int lane = threadIdx.x & 31, k = lane - first;
+    const int32_t info = m.ring_info[f.i];
+    const bool fresh = (info >> 2) < m.stamp;
+    int32_t place = 0;
+    if (live && k == 0) place = fresh ? atomicAdd(&m.count->overrides, 1) : m.ring_at[f.i];
+    place = __shfl_sync(kAll, place, first);
+    const bool fits = place < m.max_rings;
+    const int32_t ver = fresh ? 0 : (info & 1) ^ 1;
+    // owned edges and triangles (mu::ring_sizes)
+    const int32_t prev = __shfl_sync(kAll, ref, first + (k ? k - 1 : deg - 1 < 0 ? 0 : deg - 1));
+    const bool in = live && k < deg;
+    const bool up = (ref & 15) != 4 || (ref >> 4) > f.i, prev_up = (prev & 15) != 4 || (prev >> 4) > f.i;
+    const bool edge = (ref & 15) == 4 || f.periodic ? (ref >> 4) > f.i : true;
+    const unsigned group = width == 32 ? kAll : ((1u << width) - 1) << first;
+    const unsigned ne = __ballot_sync(kAll, in && edge) & group, nt = __ballot_sync(kAll, in && up && prev_up) & group;
+    if (in && fits) m.ring_ref[(int64_t)(2 * place + ver) * kMaxDeg + k] = ref;
+    if (live && k == 0) {
+        if (!fits) {
+            mu::a_or(f.flags, MU_SIZE);
+        } else {
+            if (fresh) m.ring_at[f.i] = place;
+            m.ring_deg[2 * place + ver] = deg;
+            m.ring_info[f.i] = (m.stamp + round) << 2 | (fresh ? 2 : 0) | ver;
+            m.sizes[f.i] = (uint32_t)deg | __popc(ne) << 8 | __popc(nt) << 16;
+        }
+        m.extra_n[f.i] = 0;
+    }
+    return fits;
+}
+
+// mu::recompute_light for the first round's cells, a lane per candidate and
+// sixteen lanes per cell: the wrapping finds each next neighbour by a
+// tournament.  (A thread per cell took as long at 4,096 cells, 48 us, as at
+// 262,144: one cell's chain of steps.)
+__global__ void __launch_bounds__(kListBlock) k_mesh_recompute_light(MeshUpdate m)
+{
+    using namespace mu;
+    static_assert(kLight == 16, "a half warp per cell");
+    const int lane = threadIdx.x & 31, c = lane & 15, first = lane & 16;
+    const unsigned half = 0xffffu << first;
+    const int32_t count = m.count->listed[0];
+    for (int32_t k0 = (blockIdx.x * kListWarps + (threadIdx.x >> 5)) * 2; k0 < count; k0 += gridDim.x * kListWarps * 2) {
+        const int32_t kk = k0 + (first >> 4);
+        const bool live = kk < count;
+        const int32_t i = m.list[0][live ? kk : k0];
+        const Frame f = frame_of(m, i);
+        const Ring own = ring_of(m, i, 0);
+        const int32_t ne = m.extra_n[i], n = own.deg + ne;
+        bool ok = live && n <= kLight && ne <= kMaxExtra;
+        int32_t r = i * 16 + 4;
+        if (c < own.deg) r = own[c];
+        else if (c < n && ne <= kMaxExtra) r = m.extra[(int64_t)i * kMaxExtra + (c - own.deg)];
+        bool mine = c < n;
+        // a cell at a wall, or an image of itself, goes to the full recomputation
+        if (mine && ((!f.periodic && (r & 15) != 4) || (r >> 4) == i)) ok = false;
+        ok = (__ballot_sync(kAll, ok) & half) == half;
+        for (int t = 0; t < 15; t++) {
+            const int32_t s = __shfl_sync(kAll, r, first + t);
+            if (t < c && (s >> 4) == (r >> 4)) mine = false;
+        }
+        const Point d = point_of(f, r);
+        // (the nearest in FP32 is a neighbour unless another candidate lies
+        // within a thousandth of its distance of it; the wrapping then does
+        // not close)
+        float lmin = mine ? d.l : __int_as_float(0x7f800000);
+        int near = c;
+        for (int o = 8; o > 0; o >>= 1) {
+            const float l2 = __shfl_xor_sync(kAll, lmin, o);
+            const int n2 = __shfl_xor_sync(kAll, near, o);
+            if (l2 < lmin || (l2 == lmin && n2 < near)) {
+                lmin = l2;
+                near = n2;
+            }
+        }
+        int deg = 0, last = near, turns = 0, kept = 0;
+        bool open = ok;
+        while (__any_sync(kAll, open)) {
+            if (c == deg) kept = last;
+            Point a;
+            a.fx = __shfl_sync(kAll, d.fx, first + last);
+            a.fy = __shfl_sync(kAll, d.fy, first + last);
+            a.l = a.fx * a.fx + a.fy * a.fy;
+            const float p = a.fx * d.fy, q = a.fy * d.fx, cr = p - q, cb = kCrossBound * (fabsf(p) + fabsf(q));
+            const bool cand = mine && c != last;
+            bool unsure = cand && !(cr > cb) && !(-cr > cb);
+            int best = cand && cr > cb ? c : -1;
+            for (int o = 8; o > 0; o >>= 1) {
+                const int other = __shfl_xor_sync(kAll, best, o);
+                const int sb = first + (best < 0 ? 0 : best), so = first + (other < 0 ? 0 : other);
+                Point b, e;
+                b.fx = __shfl_sync(kAll, d.fx, sb);
+                b.fy = __shfl_sync(kAll, d.fy, sb);
+                e.fx = __shfl_sync(kAll, d.fx, so);
+                e.fy = __shfl_sync(kAll, d.fy, so);
+                if (other < 0 || other == best) continue;
+                if (best < 0) {
+                    best = other;
+                    continue;
+                }
+                b.l = b.fx * b.fx + b.fy * b.fy;
+                e.l = e.fx * e.fx + e.fy * e.fy;
+                const float p1 = b.fx * e.fy, p2 = b.fy * e.fx, p3 = a.fx * e.fy, p4 = a.fy * e.fx, p5 = a.fx * b.fy,
+                            p6 = a.fy * b.fx;
+                const float det = a.l * (p1 - p2) - b.l * (p3 - p4) + e.l * (p5 - p6);
+                const float bound = kCircleBound * (a.l * (fabsf(p1) + fabsf(p2)) + b.l * (fabsf(p3) + fabsf(p4)) +
+                                                    e.l * (fabsf(p5) + fabsf(p6)));
+                if (-det > bound) best = other;
+                else if (!(det > bound)) unsure = true;
+            }
+            const int nb = first + (best < 0 ? 0 : best);
+            Point b;
+            b.fx = __shfl_sync(kAll, d.fx, nb);
+            b.fy = __shfl_sync(kAll, d.fy, nb);
+            b.l = b.fx * b.fx + b.fy * b.fy;
+            const bool fail = unsure || best < 0 || !disk_ok(f, a, b);
+            const bool failed = (__ballot_sync(kAll, fail) & half) != 0;
+            if (open) {
+                deg++;
+                turns += (a.fy < 0.0f && b.fy >= 0.0f) ? 1 : 0;
+                last = best;
+                if (failed || (deg == kLight && last != near)) ok = open = false;
+                else if (last == near) open = false;
+            }
+        }
+        ok = ok && deg >= 3 && turns == 1;
+        const int32_t ref = __shfl_sync(kAll, d.ref, first + kept);
+        commit_star(m, f, 0, ref, deg, first, 16, ok);
+        if (live && !ok && c == 0) m.heavy[atomicAdd(&m.count->heavy, 1)] = i;
+    }
+}
+
+// One warp's working set for one cell.
+struct StarWork {
+    int32_t src[kMaxSources];
+    int32_t ref[kMaxCand];
+    float fx[kMaxCand], fy[kMaxCand];
+    int32_t out[kMaxDeg];
+};
+
+// mu::recompute with a warp per cell: the lanes read the neighbours' rings,
+// drop repeated sources, take a candidate or two each, and find the next
+// neighbour of the gift wrapping by a tournament of in-circle tests.  A step
+// lists a few hundred to a few per cent of the cells, so the pass is bound by
+// one cell's chain of dependent loads and tests: a thread per cell took 545 us
+// at 1M cells and 540 us for the wall cells of 4,096.
+__device__ void warp_recompute(const MeshUpdate &m, int32_t i, int32_t round, StarWork &w)
+{
+    using namespace mu;
+    const int lane = threadIdx.x & 31;
+    const Frame f = frame_of(m, i);
+    const Ring own = ring_of(m, i, round);
+    const int32_t told = m.extra_n[i], ne = told < kMaxExtra ? told : kMaxExtra;
+    __syncwarp();
+    if (lane == 0) m.extra_n[i] = 0;
+    if (own.deg + ne > 32) {
+        if (lane == 0) a_or(f.flags, MU_SIZE);
+        return;
+    }
+    // this lane's neighbour (or vertex told of), and its ring
+    const int first = own.deg + ne;
+    int32_t r = i * 16 + 4;
+    if (lane < own.deg) r = own[lane];
+    else if (lane < first) r = m.extra[(int64_t)i * kMaxExtra + (lane - own.deg)];
+    uint32_t imgs = 1u << (r & 15);
+    const bool far_own = (r >> 4) == i;  // an image of the cell itself (or no neighbour)
+    const Ring g = ring_of(m, r >> 4, round);
+    const int mine = far_own ? 0 : g.deg;
+    int at = mine;
+    for (int o = 1; o < 32; o <<= 1) {
+        const int u = __shfl_up_sync(kAll, at, o);
+        if (lane >= o) at += u;
+    }
+    const int total = first + __shfl_sync(kAll, at, 31);
+    at += first - mine;
+    if (total > kMaxSources) {
+        if (lane == 0) a_or(f.flags, MU_SIZE);
+        return;
+    }
+    if (lane < first) w.src[lane] = r >> 4;
+    for (int j = 0; j < mine; j++) {
+        const int32_t q = g[j];
+        imgs |= 1u << (q & 15);
+        w.src[at + j] = q >> 4;
+    }
+    imgs = __reduce_or_sync(kAll, imgs);
+    __syncwarp();
+    // distinct sources, the cell left out, to the front
+    int ns = 0;
+    for (int base = 0; base < total; base += 32) {
+        const int k = base + lane;
+        const int32_t s = k < total ? w.src[k] : i;
+        bool keep = s != i;
+        // (entries before this batch are the ones kept so far)
+        for (int q = 0; q < ns; q++) keep = keep && w.src[q] != s;
+        const unsigned same = __match_any_sync(kAll, s);
+        keep = keep && (same & ((1u << lane) - 1)) == 0;
+        const unsigned kept = __ballot_sync(kAll, keep);
+        __syncwarp();
+        // (place ns + rank is at most k: an entry already read)
+        if (keep) w.src[ns + __popc(kept & ((1u << lane) - 1))] = s;
+        __syncwarp();
+        ns += __popc(kept);
+    }
+    // the candidates: every source, and across walls every image that these
+    // rings meet, of the cell too
+    const bool walls = !f.periodic && (imgs & ~(1u << 4)) != 0;
+    const int per = walls ? ns + 1 : ns, sets = walls ? __popc(imgs | 1u << 4) : 1;
+    const int nc = per * sets;
+    if (nc > kMaxCand || nc < 3) {
+        if (lane == 0) a_or(f.flags, MU_SIZE);
+        return;
+    }
+    // (the cell itself, image 4 of the walls' sets, is no candidate)
+    unsigned long long dmin = ~0ull;
+    int near = -1;
+    for (int c = lane; c < nc; c += 32) {
+        int img = 4, k = c;
+        if (walls) {
+            const int set = c / per;
+            k = c % per;
+            img = (int)__fns(imgs | 1u << 4, 0, set + 1);
+        }
+        const int32_t src = k < ns ? w.src[k] : i;
+        if (src == i && img == 4) {
+            w.ref[c] = -1;
+            continue;
+        }
+        const Point p = point_of(f, src * 16 + img);
+        w.ref[c] = p.ref;
+        w.fx[c] = p.fx;
+        w.fy[c] = p.fy;
+        const double dx = p.x - f.xi, dy = p.y - f.yi;
+        const unsigned long long d2 = (unsigned long long)__double_as_longlong(dx * dx + dy * dy);
+        if (d2 < dmin) {
+            dmin = d2;
+            near = c;
+        }
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long d = __shfl_xor_sync(kAll, dmin, o);
+        const int n2 = __shfl_xor_sync(kAll, near, o);
+        if (d < dmin || (d == dmin && n2 > near)) {
+            dmin = d;
+            near = n2;
+        }
+    }
+    __syncwarp();
+    auto at_of = [&](int c) {
+        Point p;
+        p.ref = w.ref[c];
+        p.fx = w.fx[c];
+        p.fy = w.fy[c];
+        p.l = p.fx * p.fx + p.fy * p.fy;
+        return p;
+    };
+    // whether candidate d is inside the circle of (cell, a, b)
+    auto inside = [&](const Point &a, int b, int d) {
+        const Point pb = at_of(b), pd = at_of(d);
+        const float p1 = pb.fx * pd.fy, p2 = pb.fy * pd.fx, p3 = a.fx * pd.fy, p4 = a.fy * pd.fx, p5 = a.fx * pb.fy,
+                    p6 = a.fy * pb.fx;
+        const float det = a.l * (p1 - p2) - pb.l * (p3 - p4) + pd.l * (p5 - p6);
+        const float bound = kCircleBound * (a.l * (fabsf(p1) + fabsf(p2)) + pb.l * (fabsf(p3) + fabsf(p4)) +
+                                            pd.l * (fabsf(p5) + fabsf(p6)));
+        if (det > bound) return false;
+        if (-det > bound) return true;
+        return circle_slow(f, point_of(f, a.ref), point_of(f, pb.ref), point_of(f, pd.ref)) > 0;
+    };
+    int deg = 0, last = near, turns = 0;
+    bool bad = false;
+    do {
+        if (deg == kMaxDeg) {
+            bad = true;
+            break;
+        }
+        const Point a = at_of(last);
+        if (lane == 0) w.out[deg] = a.ref;
+        deg++;
+        int best = -1;
+        for (int c = lane; c < nc; c += 32) {
+            if (c == last || w.ref[c] < 0) continue;
+            const float p = a.fx * w.fy[c], q = a.fy * w.fx[c], cr = p - q;
+            const float cb = kCrossBound * (fabsf(p) + fabsf(q));
+            bool left = cr > cb;
+            if (!left && !(-cr > cb)) left = orient_slow(f, point_of(f, a.ref), point_of(f, w.ref[c])) > 0;
+            if (left && (best < 0 || inside(a, best, c))) best = c;
+        }
+        __syncwarp();
+        for (int o = 16; o > 0; o >>= 1) {
+            const int other = __shfl_xor_sync(kAll, best, o);
+            if (other >= 0 && other != best && (best < 0 || inside(a, best, other))) best = other;
+            __syncwarp();
+        }
+        if (best < 0) {
+            bad = true;
+            break;
+        }
+        const Point b = at_of(best);
+        if (lane == 0 && !disk_ok(f, a, b)) a_or(f.flags, MU_FAR);
+        turns += (a.fy < 0.0f && b.fy >= 0.0f) ? 1 : 0;
+        last = best;
+    } while (last != near);
+    __syncwarp();
+    if (bad || deg < 3 || turns != 1) {
+        if (lane == 0) a_or(f.flags, MU_STAR);
+        return;
+    }
+    commit_star(m, f, round, lane < deg ? w.out[lane] : 0, deg, 0, 32, true);
 }
 
 __global__ void __launch_bounds__(kListBlock) k_mesh_recompute(MeshUpdate m, int32_t round)
 {
-    const int32_t count = m.count->listed[round];
-    for (int32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < count; k += gridDim.x * blockDim.x)
-        mu::recompute(m, m.list[round & 1][k], round);
+    __shared__ StarWork work[kListWarps];
+    const int32_t count = round ? m.count->listed[round] : m.count->heavy;
+    const int32_t *list = round ? m.list[round & 1] : m.heavy;
+    for (int32_t k = blockIdx.x * kListWarps + (threadIdx.x >> 5); k < count; k += gridDim.x * kListWarps) {
+        warp_recompute(m, list[k], round, work[threadIdx.x >> 5]);
+        __syncwarp();
+    }
 }
 
+// eight lanes per cell, one per triangle and per dropped neighbour
 __global__ void __launch_bounds__(kListBlock) k_mesh_check(MeshUpdate m, int32_t round)
 {
-    const int32_t count = m.count->listed[round];
-    for (int32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < count; k += gridDim.x * blockDim.x)
-        mu::check(m, m.list[round & 1][k], round);
+    const int t = threadIdx.x & 7;
+    const int32_t count = m.count->listed[round], cells = kListBlock / 8;
+    for (int32_t k = blockIdx.x * cells + (threadIdx.x >> 3); k < count; k += gridDim.x * cells) {
+        const int32_t i = m.list[round & 1][k];
+        if (!mu::recomputed(m, i, round)) continue;
+        const bool periodic = m.inst[mu::inst_at(m, i)].boundary == 1;
+        const mu::Ring g = mu::ring_of(m, i, -1), old = mu::ring_of(m, i, round);
+        for (int32_t q = t; q < g.deg; q += 8) mu::check_triangle(m, periodic, g, i, round, q);
+        for (int32_t q = t; q < old.deg; q += 8) mu::check_dropped(m, periodic, g, old, i, round, q);
+    }
 }
 
 __device__ __forceinline__ int4 plus(int4 a, int4 b) { return make_int4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w); }
@@ -72,17 +520,23 @@ __device__ __forceinline__ int4 sizes_of(uint32_t s)
     return make_int4((int)(s & 255), (int)(s >> 8 & 255), (int)(s >> 16 & 255), (int)(s >> 24));
 }
 
-// sizes per cell and their sums per window
-__global__ void __launch_bounds__(kWindow) k_mesh_measure(MeshUpdate m, int4 *window_sums)
+// Sizes per cell and their sums per window.  A mesh's sizes are kept: the
+// recomputations set those of the rings they change, so that only the images
+// inside the ghost band are counted again (whole: every ring is measured, for
+// a mesh that the host built).
+__global__ void __launch_bounds__(kWindow) k_mesh_measure(MeshUpdate m, int4 *window_sums, int32_t whole)
 {
     __shared__ int4 ws[32];
     const int32_t i = blockIdx.x * kWindow + threadIdx.x;
-    const int4 v = block_sum(i < m.n ? sizes_of(mu::measure(m, i)) : make_int4(0, 0, 0, 0), ws);
+    int4 v = make_int4(0, 0, 0, 0);
+    if (i < m.n) v = sizes_of(whole ? mu::measure(m, i) : m.sizes[i] = mu::count_images(m, i, m.sizes[i]));
+    v = block_sum(v, ws);
     if (threadIdx.x == kWindow - 1) window_sums[blockIdx.x] = v;
 }
 
-// window sums -> the sums before each window, and the totals
-__global__ void __launch_bounds__(kWindow) k_mesh_totals(MeshUpdate m, int4 *window_sums, int32_t windows)
+// window sums -> the sums before each window, and the totals; the mesh can be
+// written when no cell is listed for round `last` and it fits its arrays
+__global__ void __launch_bounds__(kWindow) k_mesh_totals(MeshUpdate m, int4 *window_sums, int32_t windows, int32_t last)
 {
     __shared__ int4 ws[32];
     __shared__ int4 carry;
@@ -104,13 +558,17 @@ __global__ void __launch_bounds__(kWindow) k_mesh_totals(MeshUpdate m, int4 *win
         m.count->edges = carry.y;
         m.count->tris = carry.z;
         m.count->ghosts = carry.w;
+        const bool fits = carry.x >= 0 && carry.x <= m.max_slots && carry.y <= m.max_edges && carry.z <= m.max_tris &&
+                          carry.w <= m.max_ghosts;
+        m.count->ready = fits && m.count->listed[last] == 0 && !(m.n_inst == 1 && m.flags[0]) ? 1 : 0;
     }
 }
 
 // offsets per cell, the ghosts, and the processing order: within each window
 // cells by decreasing ring degree, stable (degree_order in mesh.cpp)
-__global__ void __launch_bounds__(kWindow) k_mesh_offsets(MeshUpdate m, const int4 *window_sums, int32_t *order)
+__global__ void __launch_bounds__(kWindow) k_mesh_offsets(MeshUpdate m, const int4 *window_sums)
 {
+    if (!m.count->ready) return;
     __shared__ int4 ws[32];
     __shared__ int32_t hist[32][65];  // cells of each degree in each warp, then their first places
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -152,19 +610,249 @@ __global__ void __launch_bounds__(kWindow) k_mesh_offsets(MeshUpdate m, const in
     if (deg >= 0) {
         int place = hist[wid][deg] + before;
         for (int d = deg + 1; d <= 64; d++) place += ((int *)ws)[d];
-        order[blockIdx.x * kWindow + place] = i;
+        m.cell_order[blockIdx.x * kWindow + place] = i;
     }
 }
 
+// mu::place_ring with eight lanes per cell, and the masks of each ring's
+// owned edges and triangles (cells of up to 32 neighbours), from which
+// k_mesh_lists takes every edge's and triangle's number.  A ring that no round
+// changed and that meets no image keeps its ids and their order.
 __global__ void __launch_bounds__(256) k_mesh_rings(MeshUpdate m)
 {
-    const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < m.n) mu::place_ring(m, i);
+    if (!m.count->ready) return;
+    using namespace mu;
+    const int32_t t = (blockIdx.x * blockDim.x + threadIdx.x) >> 3;
+    const int lane = threadIdx.x & 31, k = lane & 7, first = lane & 24;
+    const bool live = t < m.n;
+    const int32_t i = live ? t : m.n - 1;
+    const Ring g = ring_of(m, i, -1);
+    const bool periodic = m.inst[inst_at(m, i)].boundary == 1;
+    int32_t *dst = m.out_nb + m.out_ptr[i];
+    if (__all_sync(kAll, g.deg <= 8)) {
+        const bool in = live && k < g.deg;
+        const int32_t q = k < g.deg ? k : 0;
+        const bool plain = g.base && g.p[q] < m.n;
+        int32_t id = plain ? g.p[q] : 0;
+        int at = 0;
+        if (!__all_sync(kAll, plain)) {
+            if (!plain) id = point_id(m, i, g[q]);
+            int32_t best = id;
+            at = q;
+            for (int o = 4; o > 0; o >>= 1) {
+                const int32_t b2 = __shfl_xor_sync(kAll, best, o), a2 = __shfl_xor_sync(kAll, at, o);
+                if (b2 < best || (b2 == best && a2 < at)) {
+                    best = b2;
+                    at = a2;
+                }
+            }
+        }
+        const int pos = q >= at ? q - at : q - at + g.deg;
+        const int32_t next = __shfl_sync(kAll, id, first + (q + 1 < g.deg ? q + 1 : 0));
+        // (an image owns nothing; whether the cell owns a periodic edge to
+        // one follows from the source: images of the cell itself have no
+        // place in an updated mesh)
+        const bool edge = id < m.n || !periodic ? id > i : (g[q] >> 4) > i;
+        uint32_t own = in ? (edge ? 1u << pos : 0u) | (id > i && next > i ? 256u << pos : 0u) : 0u;
+        for (int o = 4; o > 0; o >>= 1) own |= __shfl_xor_sync(kAll, own, o);
+        if (in) dst[pos] = id;
+        if (live && k == 0) {
+            m.edge_mask[i] = own & 255u;
+            m.tri_mask[i] = own >> 8;
+        }
+        return;
+    }
+    // some ring of the warp has more than eight members
+    int32_t best = INT32_MAX, at = 0;
+    for (int32_t q = k; q < g.deg; q += 8) {
+        const int32_t id = point_id(m, i, g[q]);
+        if (id < best) {
+            best = id;
+            at = q;
+        }
+    }
+    for (int o = 4; o > 0; o >>= 1) {
+        const int32_t b2 = __shfl_xor_sync(kAll, best, o), a2 = __shfl_xor_sync(kAll, at, o);
+        if (b2 < best || (b2 == best && a2 < at)) {
+            best = b2;
+            at = a2;
+        }
+    }
+    uint32_t edges = 0, tris = 0;
+    for (int32_t q = k; q < g.deg; q += 8) {
+        const int32_t pos = q >= at ? q - at : q - at + g.deg, r = g[q];
+        const int32_t id = point_id(m, i, r), next = point_id(m, i, g[q + 1 < g.deg ? q + 1 : 0]);
+        if (live) dst[pos] = id;
+        if (pos < 32) {
+            if (id < m.n || !periodic ? id > i : (r >> 4) > i) edges |= 1u << pos;
+            if (id > i && next > i) tris |= 1u << pos;
+        }
+    }
+    for (int o = 4; o > 0; o >>= 1) {
+        edges |= __shfl_xor_sync(kAll, edges, o);
+        tris |= __shfl_xor_sync(kAll, tris, o);
+    }
+    if (live && k == 0) {
+        m.edge_mask[i] = edges;
+        m.tri_mask[i] = tris;
+    }
+}
+
+// owner of the edge between real cell i and point j (1: i, 0: the other
+// side, -1: inconsistent), the host builder's rule
+__device__ __forceinline__ int edge_owner(const MeshLists &l, bool periodic, int32_t i, int32_t j)
+{
+    if (j < l.n) return j > i ? 1 : (j < i ? 0 : -1);
+    if (!periodic) return 1;
+    const int32_t src = l.ghost_src[j - l.n];
+    if (src != i) return src > i ? 1 : 0;
+    const int32_t sh = l.ghost_shift[j - l.n];
+    const int32_t sx = sh % 3 - 1, sy = sh / 3 - 1;
+    return (sy < 0 || (sy == 0 && sx < 0)) ? 0 : 1;
+}
+
+// The triangle and edge lists from the rings, eight lanes per cell, a ring
+// slot each.  A slot whose neighbour is a smaller real cell finds this cell in
+// that one's ring: the edges and triangles that the neighbour owns before it
+// (from the masks of k_mesh_rings, or counted on the way in a mesh that the
+// host built) number the edge and both triangles beside it, so every slot is
+// written once, by its own cell, and needs no clearing and no later check.
+// (Three kernels before: triangles and edges with a walk per triangle and
+// per edge, and a check of both, 153 us at 1M cells.)
+__global__ void __launch_bounds__(128) k_mesh_lists(MeshLists l)
+{
+    if (l.ready && !*l.ready) return;
+    const int lane = threadIdx.x & 31, k = lane & 7, first = lane & 24;
+    const unsigned byte = 0xffu << first, below = ((1u << k) - 1) << first;
+    const int32_t cell = (blockIdx.x * blockDim.x + threadIdx.x) >> 3;
+    const bool live = cell < l.n;
+    const int32_t i = live ? cell : l.n - 1;
+    const bool periodic = l.cell_inst ? l.inst[l.cell_inst[i]].boundary == 1 : l.periodic != 0;
+    const int32_t lo = l.cell_ptr[i], deg = l.cell_ptr[i + 1] - lo;
+    const int32_t *nb = l.slot_nb + lo;
+    int32_t t = l.tri_off[i], e = l.edge_off[i];
+    const int32_t t_end = l.tri_off[i + 1], e_end = l.edge_off[i + 1];
+    bool bad = false;
+    int owner = -1;
+    // the loops run as long as any cell of the warp has slots
+    const int32_t steps = __reduce_max_sync(kAll, (deg + 7) >> 3);
+    for (int32_t s = 0; s < steps; s++) {
+        const int32_t q = 8 * s + k;
+        const bool in = live && q < deg;
+        const int32_t a = nb[in ? q : 0], b = nb[in && q + 1 < deg ? q + 1 : 0];
+        const bool own_tri = in && i < a && i < b;
+        const unsigned tris = __ballot_sync(kAll, own_tri) & byte;
+        if (own_tri) {
+            const int32_t num = t + __popc(tris & below);
+            if (num < t_end) {
+                l.tri[3 * num] = i;
+                l.tri[3 * num + 1] = a;
+                l.tri[3 * num + 2] = b;
+                l.slot_tri[lo + q] = num;
+            } else {
+                bad = true;
+            }
+        }
+        t += __popc(tris);
+        if (in) {
+            owner = edge_owner(l, periodic, i, a);
+            if (owner < 0) bad = true;
+        }
+        if (in && a < i) {
+            // this cell in the ring of a: edges and triangles of a before it
+            const int32_t prev = nb[q ? q - 1 : deg - 1];
+            const int32_t alo = l.cell_ptr[a], adeg = l.cell_ptr[a + 1] - alo;
+            const int32_t *an = l.slot_nb + alo;
+            int32_t ne = l.edge_off[a], nt = l.tri_off[a];
+            bool found = false;
+            int32_t j0 = 0;
+            if (l.edge_mask && adeg <= 32) {
+                while (j0 < adeg && an[j0] != i) j0++;
+                if (j0 < adeg) {
+                    const uint32_t passed = (1u << j0) - 1;
+                    ne += __popc(l.edge_mask[a] & passed);
+                    nt += __popc(l.tri_mask[a] & passed);
+                }
+            }
+            int32_t x = j0 < adeg ? an[j0] : -1, before = an[j0 ? j0 - 1 : adeg - 1];
+            for (int32_t j = j0; j < adeg; j++) {
+                const int32_t y = an[j + 1 < adeg ? j + 1 : 0];
+                if (x == i) {
+                    // (a; before, i) is this slot's triangle, (a; i, y) the last slot's
+                    l.slot_edge[lo + q] = 2 * ne + 1;
+                    if (a < b) {
+                        if (before != b) bad = true;
+                        l.slot_tri[lo + q] = j ? nt - 1 : l.tri_off[a + 1] - 1;
+                    }
+                    if (a < prev) {
+                        if (y != prev) bad = true;
+                        l.slot_tri[lo + (q ? q - 1 : deg - 1)] = nt;
+                    }
+                    found = true;
+                    break;
+                }
+                ne += edge_owner(l, periodic, a, x) > 0 ? 1 : 0;
+                nt += a < x && a < y ? 1 : 0;
+                before = x;
+                x = y;
+            }
+            if (!found) bad = true;
+        } else if (in && a >= l.n && owner == 0) {
+            // a periodic edge that the source of a owns: from its ring this
+            // cell is seen at the opposite shift
+            const int32_t src = l.ghost_src[a - l.n], sh = l.ghost_shift[a - l.n];
+            const int32_t want = (1 - (sh % 3 - 1)) + 3 * (1 - (sh / 3 - 1));
+            const int32_t alo = l.cell_ptr[src], adeg = l.cell_ptr[src + 1] - alo;
+            int32_t ne = l.edge_off[src];
+            bool found = false;
+            for (int32_t j = 0; j < adeg; j++) {
+                const int32_t x = l.slot_nb[alo + j];
+                if (x >= l.n && l.ghost_src[x - l.n] == i && l.ghost_shift[x - l.n] == want && alo + j != lo + q) {
+                    l.slot_edge[lo + q] = 2 * ne + 1;
+                    found = true;
+                    break;
+                }
+                ne += edge_owner(l, periodic, src, x) > 0 ? 1 : 0;
+            }
+            if (!found) bad = true;
+        }
+    }
+    if (live && t != t_end) bad = true;
+    // the owned edges, whose triangles are now all numbered
+    __syncwarp();
+    for (int32_t s = 0; s < steps; s++) {
+        const int32_t q = 8 * s + k;
+        const bool in = live && q < deg;
+        const int32_t a = nb[in ? q : 0];
+        const bool own = in && edge_owner(l, periodic, i, a) > 0;
+        const unsigned edges = __ballot_sync(kAll, own) & byte;
+        if (own) {
+            const int32_t num = e + __popc(edges & below);
+            if (num < e_end) {
+                l.edge_l[num] = i;
+                l.edge_r[num] = a;
+                l.edge_ta[num] = *(volatile const int32_t *)(l.slot_tri + lo + (q ? q - 1 : deg - 1));
+                l.edge_tb[num] = *(volatile const int32_t *)(l.slot_tri + lo + q);
+                l.slot_edge[lo + q] = 2 * num;
+            } else {
+                bad = true;
+            }
+        }
+        e += __popc(edges);
+    }
+    if (live && e != e_end) bad = true;
+    if (bad) *l.bad = 1;
 }
 
 inline int blocks(int64_t n, int b) { return (int)((n + b - 1) / b); }
 
 }  // namespace
+
+cudaError_t launch_lists(const MeshLists &l, cudaStream_t st)
+{
+    if (l.n > 0) k_mesh_lists<<<blocks(8 * (int64_t)l.n, 128), 128, 0, st>>>(l);
+    return cudaGetLastError();
+}
 
 #define MU_TRY(e)                               \
     do {                                        \
@@ -180,14 +868,18 @@ cudaError_t MeshUpdater::reserve(int32_t n, int32_t n_inst, cudaStream_t st)
     // stamps and counts that only ever grow must start at zero
     const bool fresh = !(mark_.p && mark_.cap >= N * i4);
     MU_TRY(mark_.ensure(N * i4)); MU_TRY(info_.ensure(N * i4)); MU_TRY(extra_n_.ensure(N * i4));
-    MU_TRY(list_[0].ensure(N * i4)); MU_TRY(list_[1].ensure(N * i4)); MU_TRY(at_.ensure(N * i4));
+    MU_TRY(list_[0].ensure(N * i4)); MU_TRY(list_[1].ensure(N * i4)); MU_TRY(heavy_.ensure(N * i4));
+    MU_TRY(at_.ensure(N * i4));
     MU_TRY(ring_deg_.ensure(2 * R * i4)); MU_TRY(ring_ref_.ensure(2 * R * kMaxDeg * i4));
     MU_TRY(extra_.ensure(N * kMaxExtra * i4));
+    if (sizes_.cap < N * 4) whole_ = true;
+    MU_TRY(edge_mask_.ensure(N * 4)); MU_TRY(tri_mask_.ensure(N * 4));
     MU_TRY(sizes_.ensure(N * 4)); MU_TRY(images_.ensure(N * 2)); MU_TRY(ghost_off_.ensure((N + 1) * i4));
     MU_TRY(sums_.ensure((size_t)blocks(n, kWindow) * sizeof(int4)));
-    MU_TRY(count_.ensure(sizeof(MeshUpdateCount)));
-    MU_TRY(flags_.ensure((size_t)n_inst * i4));
-    MU_TRY(host_.ensure(sizeof(MeshUpdateCount) + (size_t)n_inst * i4));
+    // the counters, then the simulations' flags
+    const size_t cb = sizeof(MeshUpdateCount) + (size_t)n_inst * i4;
+    MU_TRY(count_.ensure(cb));
+    MU_TRY(host_.ensure(cb));
     if (fresh || stamp_ > (1 << 28)) {
         MU_TRY(cudaMemsetAsync(mark_.p, 0, mark_.cap, st));
         MU_TRY(cudaMemsetAsync(info_.p, 0, info_.cap, st));
@@ -197,7 +889,7 @@ cudaError_t MeshUpdater::reserve(int32_t n, int32_t n_inst, cudaStream_t st)
     return cudaSuccess;
 }
 
-MeshUpdate MeshUpdater::params(const MeshArrays &a) const
+MeshUpdate MeshUpdater::params(const MeshArrays &a, const MeshOutput &o) const
 {
     MeshUpdate m{};
     m.n = a.n;
@@ -214,6 +906,7 @@ MeshUpdate MeshUpdater::params(const MeshArrays &a) const
     m.mark = mark_.as<int32_t>();
     m.list[0] = list_[0].as<int32_t>();
     m.list[1] = list_[1].as<int32_t>();
+    m.heavy = heavy_.as<int32_t>();
     m.ring_info = info_.as<int32_t>();
     m.ring_at = at_.as<int32_t>();
     m.max_rings = max_rings_;
@@ -222,88 +915,113 @@ MeshUpdate MeshUpdater::params(const MeshArrays &a) const
     m.extra_n = extra_n_.as<int32_t>();
     m.extra = extra_.as<int32_t>();
     m.count = count_.as<MeshUpdateCount>();
-    m.flags = flags_.as<int32_t>();
+    m.flags = reinterpret_cast<int32_t *>(m.count + 1);
     m.sizes = sizes_.as<uint32_t>();
     m.images = images_.as<uint16_t>();
     m.ghost_off = ghost_off_.as<int32_t>();
-    return m;
-}
-
-void MeshUpdater::launch_rounds(const MeshUpdate &m, int first, int last, cudaStream_t st) const
-{
-    // grids for the cells a step lists (a few per cent), looping beyond
-    const int g = std::max(1, std::min(blocks(m.n, 4 * kListBlock), 2048));
-    for (int r = first; r < last; r++) {
-        k_mesh_recompute<<<g, kListBlock, 0, st>>>(m, r);
-        k_mesh_check<<<g, kListBlock, 0, st>>>(m, r);
-    }
-    const int w = blocks(m.n, kWindow);
-    k_mesh_measure<<<w, kWindow, 0, st>>>(m, sums_.as<int4>());
-    k_mesh_totals<<<1, kWindow, 0, st>>>(m, sums_.as<int4>(), w);
-}
-
-// The rounds launched before the host looks: what nearly every step needs.
-constexpr int kFirstRounds = 2;
-
-cudaError_t MeshUpdater::start(const MeshArrays &a, cudaStream_t st)
-{
-    MU_TRY(reserve(a.n, a.n_inst, st));
-    stamp_ += 16;
-    static_assert(kMaxRounds + 1 < 16, "one update's stamps");
-    const MeshUpdate m = params(a);
-    MU_TRY(cudaMemsetAsync(count_.p, 0, sizeof(MeshUpdateCount), st));
-    MU_TRY(cudaMemsetAsync(flags_.p, 0, (size_t)a.n_inst * sizeof(int32_t), st));
-    k_mesh_verify<<<blocks(a.n, kVerifyBlock), kVerifyBlock, 0, st>>>(m);
-    launch_rounds(m, 0, kFirstRounds, st);
-    return read_counts(a, st);
-}
-
-cudaError_t MeshUpdater::read_counts(const MeshArrays &a, cudaStream_t st)
-{
-    MU_TRY(cudaMemcpyAsync(host_.p, count_.p, sizeof(MeshUpdateCount), cudaMemcpyDeviceToHost, st));
-    MU_TRY(cudaMemcpyAsync(host_.as<MeshUpdateCount>() + 1, flags_.p, (size_t)a.n_inst * sizeof(int32_t),
-                           cudaMemcpyDeviceToHost, st));
-    return cudaGetLastError();
-}
-
-cudaError_t MeshUpdater::settle(const MeshArrays &a, bool &ok, MeshSizes &sizes, cudaStream_t st)
-{
-    const MeshUpdateCount &c = *host_.as<MeshUpdateCount>();
-    int r = kFirstRounds;
-    static_assert((kMaxRounds - kFirstRounds) % 2 == 0, "further rounds come in pairs");
-    for (; c.listed[r] > 0 && r < kMaxRounds; r += 2) {
-        launch_rounds(params(a), r, r + 2, st);
-        MU_TRY(read_counts(a, st));
-        MU_TRY(cudaStreamSynchronize(st));
-    }
-    ok = c.listed[r] == 0 && c.slots >= 0 && c.slots <= INT32_MAX / 2;
-    const int32_t *f = flags();
-    bool flagged = false;
-    for (int32_t k = 0; k < a.n_inst; k++) flagged |= f[k] != 0;
-    // (what was reported to cells that no round recomputed is dropped)
-    if (!ok || flagged) MU_TRY(cudaMemsetAsync(extra_n_.p, 0, extra_n_.cap, st));
-    sizes = MeshSizes{c.ghosts, c.tris, c.edges, c.slots};
-    return cudaSuccess;
-}
-
-const int32_t *MeshUpdater::flags() const { return reinterpret_cast<const int32_t *>(host_.as<MeshUpdateCount>() + 1); }
-
-cudaError_t MeshUpdater::finish(const MeshArrays &a, const MeshOutput &o, cudaStream_t st)
-{
-    MeshUpdate m = params(a);
+    m.edge_mask = edge_mask_.as<uint32_t>();
+    m.tri_mask = tri_mask_.as<uint32_t>();
     m.out_ptr = o.cell_ptr;
     m.out_nb = o.slot_nb;
     m.tri_off = o.tri_off;
     m.edge_off = o.edge_off;
+    m.cell_order = o.cell_order;
     m.gx = o.gx;
     m.gy = o.gy;
     m.gsrc = o.ghost_src;
     m.gxf = o.ghost_xf;
     m.gshift = o.ghost_shift;
     m.gimg = o.ghost_img;
-    k_mesh_offsets<<<blocks(a.n, kWindow), kWindow, 0, st>>>(m, sums_.as<int4>(), o.cell_order);
-    k_mesh_rings<<<blocks(a.n, 256), 256, 0, st>>>(m);
-    return cudaGetLastError();
+    m.max_slots = o.max.slots;
+    m.max_edges = o.max.edges;
+    m.max_tris = o.max.tris;
+    m.max_ghosts = o.max.ghosts;
+    return m;
 }
+
+// rounds [first, last), then the new mesh if they settle it
+cudaError_t MeshUpdater::launch_rounds(const MeshArrays &a, const MeshOutput &o, int first, int last, cudaStream_t st)
+{
+    const MeshUpdate m = params(a, o);
+    // grids for the cells a step lists (a few per cent), looping beyond
+    const int g = std::max(1, std::min(blocks(m.n, 16 * kListWarps), 152 * 8));
+    for (int r = first; r < last; r++) {
+        if (r == 0) k_mesh_recompute_light<<<g, kListBlock, 0, st>>>(m);
+        k_mesh_recompute<<<g, kListBlock, 0, st>>>(m, r);
+        k_mesh_check<<<g, kListBlock, 0, st>>>(m, r);
+    }
+    const int w = blocks(m.n, kWindow);
+    k_mesh_measure<<<w, kWindow, 0, st>>>(m, sums_.as<int4>(), whole_ ? 1 : 0);
+    k_mesh_totals<<<1, kWindow, 0, st>>>(m, sums_.as<int4>(), w, last);
+    k_mesh_offsets<<<w, kWindow, 0, st>>>(m, sums_.as<int4>());
+    k_mesh_rings<<<blocks(8 * (int64_t)m.n, 256), 256, 0, st>>>(m);
+    MeshLists l = o.lists;
+    l.n = a.n;
+    l.cell_inst = a.cell_inst;
+    l.inst = a.inst;
+    l.cell_ptr = o.cell_ptr;
+    l.slot_nb = o.slot_nb;
+    l.tri_off = o.tri_off;
+    l.edge_off = o.edge_off;
+    l.ghost_src = o.ghost_src;
+    l.ghost_shift = o.ghost_shift;
+    l.edge_mask = m.edge_mask;
+    l.tri_mask = m.tri_mask;
+    l.ready = &m.count->ready;
+    l.bad = &m.count->bad;
+    MU_TRY(launch_lists(l, st));
+    return cudaMemcpyAsync(host_.p, count_.p, sizeof(MeshUpdateCount) + (size_t)a.n_inst * sizeof(int32_t),
+                           cudaMemcpyDeviceToHost, st);
+}
+
+// The rounds launched before the host looks: what nearly every step needs.
+constexpr int kFirstRounds = 2;
+
+cudaError_t MeshUpdater::start(const MeshArrays &a, const MeshOutput &o, cudaStream_t st)
+{
+    MU_TRY(reserve(a.n, a.n_inst, st));
+    stamp_ += 16;
+    static_assert(kMaxRounds + 1 < 16, "one update's stamps");
+    const MeshUpdate m = params(a, o);
+    MU_TRY(cudaMemsetAsync(count_.p, 0, sizeof(MeshUpdateCount) + (size_t)a.n_inst * sizeof(int32_t), st));
+    k_mesh_verify<<<blocks(8 * (int64_t)a.n, kVerifyBlock), kVerifyBlock, 0, st>>>(m);
+    k_mesh_verify_open<<<std::max(1, std::min(blocks(a.n, 16 * kListWarps), 152 * 8)), kListBlock, 0, st>>>(m);
+    last_round_ = kFirstRounds;
+    return launch_rounds(a, o, 0, kFirstRounds, st);
+}
+
+cudaError_t MeshUpdater::settle(const MeshArrays &a, const MeshOutput &o, MeshResult &result, cudaStream_t st)
+{
+    const MeshUpdateCount &c = *host_.as<MeshUpdateCount>();
+    int r = last_round_;
+    static_assert((kMaxRounds - kFirstRounds) % 2 == 0, "further rounds come in pairs");
+    for (; c.listed[r] > 0 && r < kMaxRounds; r += 2) {
+        MU_TRY(launch_rounds(a, o, r, r + 2, st));
+        MU_TRY(cudaStreamSynchronize(st));
+    }
+    result.sizes = MeshSizes{c.ghosts, c.tris, c.edges, c.slots};
+    result.flagged = false;
+    const int32_t *f = flags();
+    for (int32_t k = 0; k < a.n_inst; k++) result.flagged |= f[k] != 0;
+    const bool settled = c.listed[r] == 0 && c.slots >= 0 && c.slots <= INT32_MAX / 2;
+    result.state = !settled ? MeshResult::kHost : c.ready ? MeshResult::kDone : MeshResult::kGrow;
+    if (result.state == MeshResult::kGrow && a.n_inst == 1 && result.flagged) result.state = MeshResult::kHost;
+    result.bad = c.bad != 0;
+    // (what was reported to cells that no round recomputed is dropped, and
+    // sizes of rings that were not kept are measured again)
+    whole_ = result.state == MeshResult::kHost || result.flagged;
+    if (whole_) MU_TRY(cudaMemsetAsync(extra_n_.p, 0, extra_n_.cap, st));
+    last_round_ = r;
+    return cudaSuccess;
+}
+
+cudaError_t MeshUpdater::again(const MeshArrays &a, const MeshOutput &o, MeshResult &result, cudaStream_t st)
+{
+    MU_TRY(launch_rounds(a, o, last_round_, last_round_, st));
+    MU_TRY(cudaStreamSynchronize(st));
+    return settle(a, o, result, st);
+}
+
+const int32_t *MeshUpdater::flags() const { return reinterpret_cast<const int32_t *>(host_.as<MeshUpdateCount>() + 1); }
 
 }  // namespace rich

@@ -9,9 +9,10 @@
 //             counter-clockwise, one turn, every edge locally Delaunay, the
 //             circumdisks inside the ghost band; the cells of a failed check
 //             are listed;
-//   recompute a listed cell builds its star again by gift wrapping over the
-//             sources of its ring and of its neighbours' rings (and their
-//             images, near a wall);
+//   recompute a listed cell builds its star again by gift wrapping, at first
+//             over its ring and the vertices the failed checks name (an edge
+//             flip), else over the sources of its ring and of its neighbours'
+//             rings (and their images, near a wall);
 //   check     a new star's triangles must be in the rings of their other two
 //             vertices, and a dropped neighbour must have dropped the cell;
 //             where not, the cells involved are listed for another round and
@@ -49,7 +50,9 @@
 namespace rich {
 
 constexpr int kMaxDeg = 32;     // neighbours of a recomputed cell
+constexpr int kLight = 16;      // candidates of recompute_light
 constexpr int kMaxCand = 96;    // candidates of a recomputed cell
+constexpr int kMaxSources = 256;  // cells of its neighbours' rings, repeats included (device)
 constexpr int kMaxExtra = 8;    // vertices another cell can tell it of per round
 constexpr int kMaxRounds = 12;  // rounds before the host takes over
 
@@ -64,8 +67,12 @@ enum : int32_t {
 // Counters of one update (device memory, cleared at its start).
 struct MeshUpdateCount {
     int32_t listed[kMaxRounds + 1];  // cells listed for each round
+    int32_t open;                    // cells that FP32 could not verify
+    int32_t heavy;                   // listed cells that recompute_light left
     int32_t overrides;               // cells recomputed so far
     int32_t slots, edges, tris, ghosts;
+    int32_t ready;                   // the rounds are done and the new mesh fits its arrays
+    int32_t bad;                     // the lists of the new mesh do not close
 };
 
 struct MeshUpdate {
@@ -79,7 +86,8 @@ struct MeshUpdate {
     // rounds' lists (alternating).  Stamps grow from update to update, so
     // nothing is cleared between them.
     int32_t stamp;
-    int32_t *mark, *list[2];
+    int32_t *mark, *list[2];  // (verify's undecided cells wait in list[1])
+    int32_t *heavy;           // those of the first round that recompute_light left
     // recomputed stars: per cell (stamp << 2 | first << 1 | version) of its
     // last recomputation and its place, per place two versions of the ring
     int32_t *ring_info, *ring_at;
@@ -96,9 +104,13 @@ struct MeshUpdate {
     uint32_t *sizes;
     uint16_t *images;
     // the updated mesh
+    // (and for k_mesh_lists which of a ring's edges and triangles its cell owns)
+    uint32_t *edge_mask, *tri_mask;
     int32_t *out_ptr, *out_nb, *tri_off, *edge_off, *ghost_off;
     double *gx, *gy;
     int32_t *gsrc, *gxf, *gshift, *gimg;
+    int32_t *cell_order;
+    int32_t max_slots, max_edges, max_tris, max_ghosts;
 };
 
 namespace mu {
@@ -144,7 +156,8 @@ struct Frame {
     int32_t i;
     int32_t *flags;
     double xi, yi;
-    double x0, x1, y0, y1, hx, hy;  // box and half its sides
+    double x0, x1, y0, y1;  // box
+    float half_x, half_y;   // half its sides (scaled)
     float scale, rlim2, rper2, reach;
     bool periodic;
 };
@@ -162,7 +175,7 @@ RICH_HD inline Frame frame_of(const MeshUpdate &m, int32_t i)
     f.xi = m.x[i];
     f.yi = m.y[i];
     f.x0 = ip.x0; f.x1 = ip.x1; f.y0 = ip.y0; f.y1 = ip.y1;
-    f.hx = ip.half_x; f.hy = ip.half_y;
+    f.half_x = ip.half_x; f.half_y = ip.half_y;
     f.scale = ip.mesh_scale;
     f.rlim2 = ip.mesh_rlim2;
     f.rper2 = ip.mesh_rper2;
@@ -177,60 +190,70 @@ struct Point {
     int32_t ref;
 };
 
+// v in FP32 with its mantissa cut to 24 bits, on the integer pipe (FP64 to
+// FP32 conversions issue on the FP64 pipe); below FP32's normal range zero,
+// above it infinite
 RICH_HD inline float to_float(double v)
 {
 #ifdef __CUDA_ARCH__
-    return __double2float_rn(v);
+    const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
+    const unsigned e = (hi >> 20) & 0x7ffu;
+    unsigned u = __funnelshift_l(lo, hi, 3) - 0xc0000000u;
+    u = e < 897u ? 0u : (e > 1150u ? 0x7f800000u : u);
+    return __uint_as_float((u & 0x7fffffffu) | (hi & 0x80000000u));
 #else
-    return (float)v;
+    const uint64_t b = exactint::bits_of(v);
+    const unsigned hi = (unsigned)(b >> 32), lo = (unsigned)b, e = (hi >> 20) & 0x7ffu;
+    unsigned u = ((hi << 3) | (lo >> 29)) - 0xc0000000u;
+    u = e < 897u ? 0u : (e > 1150u ? 0x7f800000u : u);
+    u = (u & 0x7fffffffu) | (hi & 0x80000000u);
+    float f;
+    std::memcpy(&f, &u, 4);
+    return f;
 #endif
 }
 
 // the point of a reference; in a periodic box the source's nearest image
-// (whatever image the reference names)
+// (whatever image the reference names).  Neighbours are nearer than half the
+// box by far (disk_ok), so FP32 decides which image that is.
 RICH_HD inline Point point_of(const Frame &f, int32_t ref)
 {
     const int32_t src = ref >> 4;
     Point p;
     p.x = f.m->x[src];
     p.y = f.m->y[src];
-    double dx, dy;
-    if (f.periodic) {
-        dx = p.x - f.xi;
-        dy = p.y - f.yi;
-        int a = 0, b = 0;
-        if (less(f.hx, dx)) a = -1;
-        else if (less(dx, -f.hx)) a = 1;
-        if (less(f.hy, dy)) b = -1;
-        else if (less(dy, -f.hy)) b = 1;
-        if (a) {
-            p.x = image_coord(p.x, f.x0, f.x1, a, true);
-            dx = p.x - f.xi;
-        }
-        if (b) {
-            p.y = image_coord(p.y, f.y0, f.y1, b, true);
-            dy = p.y - f.yi;
-        }
-        p.ref = src * 16 + (a + 1) + 3 * (b + 1);
-    } else {
+    p.ref = ref;
+    if (!f.periodic) {
         const int32_t img = ref & 15;
         if (img != 4) {
             p.x = image_coord(p.x, f.x0, f.x1, img % 3 - 1, false);
             p.y = image_coord(p.y, f.y0, f.y1, img / 3 - 1, false);
         }
-        dx = p.x - f.xi;
-        dy = p.y - f.yi;
-        p.ref = ref;
     }
-    p.fx = to_float(dx) * f.scale;
-    p.fy = to_float(dy) * f.scale;
+    p.fx = to_float(p.x - f.xi) * f.scale;
+    p.fy = to_float(p.y - f.yi) * f.scale;
+    if (f.periodic) {
+        int a = 0, b = 0;
+        if (fabsf(p.fx) > f.half_x) {
+            a = p.fx > 0.0f ? -1 : 1;
+            p.x = image_coord(p.x, f.x0, f.x1, a, true);
+            p.fx = to_float(p.x - f.xi) * f.scale;
+        }
+        if (fabsf(p.fy) > f.half_y) {
+            b = p.fy > 0.0f ? -1 : 1;
+            p.y = image_coord(p.y, f.y0, f.y1, b, true);
+            p.fy = to_float(p.y - f.yi) * f.scale;
+        }
+        p.ref = src * 16 + (a + 1) + 3 * (b + 1);
+    }
     p.l = p.fx * p.fx + p.fy * p.fy;
     return p;
 }
 
-// FP32 determinants of offsets: relative error of a product of k rounded
-// factors below (2 k + 2) 2^-24 of the permanent; the bounds are a few times
-// that.
+// FP32 determinants of offsets, each offset within 3 2^-24 of its value (cut,
+// then scaled): a product of two is within 7 2^-24 and the cross product's
+// error below 9 2^-24 = 5.4e-7 of its permanent; |a|^2 is within 9 2^-24, and
+// the in-circle sum within 22 2^-24 = 1.3e-6 of its permanent.
 constexpr float kCrossBound = 1e-6f;
 constexpr float kCircleBound = 3e-6f;
 
@@ -248,6 +271,7 @@ RICH_MU_SLOW int orient_slow(int32_t *flags, double ax, double ay, double bx, do
     const double det = l - r, bound = kOrientBound * (fabs(l) + fabs(r));
     if (det > bound) return 1;
     if (-det > bound) return -1;
+    if ((ax == bx && bx == cx) || (ay == by && by == cy)) return 0;
     const int s = exactint::orient_sign(ax, ay, bx, by, cx, cy);
     if (s == exactint::kUnknown) a_or(flags, MU_EXACT);
     return s == exactint::kUnknown ? 0 : s;
@@ -256,6 +280,40 @@ RICH_MU_SLOW int orient_slow(int32_t *flags, double ax, double ay, double bx, do
 RICH_HD inline bool lex_less(double px, double py, double qx, double qy)
 {
     return px < qx || (px == qx && py < qy);
+}
+
+// a <=> b for the exact sums p + q and r + s
+RICH_HD inline int compare_sums(double p, double q, double r, double s, bool &known)
+{
+    const double s1 = p + q, v1 = s1 - p, e1 = (p - (s1 - v1)) + (q - v1);
+    const double s2 = r + s, v2 = s2 - r, e2 = (r - (s2 - v2)) + (s - v2);
+    const double d = (s1 - s2) + (e1 - e2);
+    known = s1 == s2 || d != 0.0;
+    return d > 0.0 ? 1 : (d < 0.0 ? -1 : 0);
+}
+
+// In-circle of four points that form two pairs of equal y (or x): the mirror
+// images of two cells, and every square of a lattice.  The circle's centre is
+// halfway between the other pair (r, s), so the power of d against that of
+// its own partner m is (d - m)(d + m - r - s) along x: two exact sums instead
+// of a 517-bit determinant.  1 inside, -1 outside, 0 on it, 2 when the points
+// are no such pairs.
+RICH_HD inline int circle_pairs(const double x[4], const double y[4])
+{
+    for (int k = 0; k < 3; k++) {  // the partner of d = point 3
+        const int r = k == 0 ? 1 : 0, q = 3 - k - r;
+        bool known = true;
+        int s = 2;
+        if (y[k] == y[3] && y[r] == y[q] && x[k] != x[3]) {
+            s = compare_sums(x[3], x[k], x[r], x[q], known);
+            s = x[3] > x[k] ? -s : s;
+        } else if (x[k] == x[3] && x[r] == x[q] && y[k] != y[3]) {
+            s = compare_sums(y[3], y[k], y[r], y[q], known);
+            s = y[3] > y[k] ? -s : s;
+        }
+        if (s != 2 && known) return s;
+    }
+    return 2;
 }
 
 // in-circle of counter-clockwise a, b, c and d, likewise, with the symbolic
@@ -274,7 +332,9 @@ RICH_MU_SLOW int circle_slow(int32_t *flags, double ax, double ay, double bx, do
         if (det > bound && det < 1e300) return 1;
         if (-det > bound && -det < 1e300) return -1;
     }
-    const int s = exactint::incircle_sign(ax, ay, bx, by, cx, cy, dx, dy);
+    const double px[4] = {ax, bx, cx, dx}, py[4] = {ay, by, cy, dy};
+    int s = circle_pairs(px, py);
+    if (s == 2) s = exactint::incircle_sign(ax, ay, bx, by, cx, cy, dx, dy);
     if (s == exactint::kUnknown) {
         a_or(flags, MU_EXACT);
         return 0;
@@ -304,6 +364,21 @@ RICH_HD inline int circle_slow(const Frame &f, const Point &a, const Point &b, c
     return circle_slow(f.flags, f.xi, f.yi, a.x, a.y, b.x, b.y, d.x, d.y);
 }
 
+// > 0 when d is inside the circumcircle of the counter-clockwise (cell, a, b).
+// With offsets from the cell the determinant is
+// -(|a|^2 (b x d) - |b|^2 (a x d) + |d|^2 (a x b)).
+RICH_HD inline int incircle(const Frame &f, const Point &a, const Point &b, const Point &d)
+{
+    const float p1 = b.fx * d.fy, p2 = b.fy * d.fx, p3 = a.fx * d.fy, p4 = a.fy * d.fx, p5 = a.fx * b.fy,
+                p6 = a.fy * b.fx;
+    const float det = a.l * (p1 - p2) - b.l * (p3 - p4) + d.l * (p5 - p6);
+    const float bound = kCircleBound * (a.l * (fabsf(p1) + fabsf(p2)) + b.l * (fabsf(p3) + fabsf(p4)) +
+                                        d.l * (fabsf(p5) + fabsf(p6)));
+    if (det > bound) return -1;
+    if (-det > bound) return 1;
+    return circle_slow(f, a, b, d);
+}
+
 // Whether the circumdisk of (cell, a, b) is certainly inside the ghost band
 // (and, in a periodic box, smaller than a quarter of it).  A disk through
 // the cell reaches past a wall by less than its diameter, so a radius below
@@ -329,6 +404,18 @@ RICH_HD inline void list_cell(const MeshUpdate &m, int32_t v, int32_t round)
 {
     if (vol(m.flags + inst_at(m, v)) || vol(m.mark + v) == m.stamp + round || a_exch(m.mark + v, m.stamp + round) == m.stamp + round) return;
     m.list[round & 1][a_add(&m.count->listed[round], 1)] = v;
+}
+
+// Tell a listed cell v of reference r (in its own frame).
+RICH_HD inline void tell_only(const MeshUpdate &m, int32_t v, int32_t r)
+{
+    const int32_t at = a_add(m.extra_n + v, 1);
+    if (at < kMaxExtra) m.extra[(int64_t)v * kMaxExtra + at] = r;
+}
+RICH_HD inline void tell(const MeshUpdate &m, int32_t v, int32_t round, int32_t r)
+{
+    list_cell(m, v, round);
+    tell_only(m, v, r);
 }
 
 RICH_HD inline int32_t base_ref(const MeshUpdate &m, int32_t q)
@@ -369,49 +456,78 @@ RICH_HD inline Ring ring_of(const MeshUpdate &m, int32_t v, int32_t computing)
     return r;
 }
 
+// Whether an image of a ring member (or of the cell) across the walls that
+// the ring meets lies in the circle of (cell, b, d).
+RICH_HD inline bool image_inside(const Frame &f, const int32_t *nb, int32_t deg, const Point &b, const Point &d)
+{
+    uint32_t imgs = 0;
+    for (int32_t k = 0; k < deg; k++) imgs |= 1u << (base_ref(*f.m, nb[k]) & 15);
+    for (int img = 0; img < 9; img++) {
+        if (img == 4 || !(imgs >> img & 1)) continue;
+        for (int32_t k = -1; k < deg; k++) {
+            const int32_t r = (k < 0 ? f.i : base_ref(*f.m, nb[k]) >> 4) * 16 + img;
+            if (r == b.ref || r == d.ref) continue;
+            if (incircle(f, b, d, point_of(f, r)) > 0) return true;
+        }
+    }
+    return false;
+}
+
 // ---- the bodies --------------------------------------------------------------
 
-// Cell i's star at the new positions.
-RICH_HD inline void verify(const MeshUpdate &m, int32_t i)
+// The edge from a cell to b between its neighbours a and d is not locally
+// Delaunay: its end loses it, and a and d may gain each other.
+RICH_HD inline void list_bad(const MeshUpdate &m, bool periodic, int32_t a, int32_t b, int32_t d)
+{
+    list_cell(m, b >> 4, 0);
+    // (across a wall a reference holds in the frame of a cell itself only)
+    if (periodic || (a & 15) == 4) tell(m, a >> 4, 0, d);
+    else list_cell(m, a >> 4, 0);
+    if (periodic || (d & 15) == 4) tell(m, d >> 4, 0, a);
+    else list_cell(m, d >> 4, 0);
+}
+
+// Cell i's star at the new positions.  With kFast the predicates stop at
+// FP32 and a star that they cannot decide is reported (true) instead, for a
+// second call without: the pass over every cell then holds no FP64 or exact
+// code, and its registers leave room for twice the warps.
+template <bool kFast> RICH_HD inline bool verify(const MeshUpdate &m, int32_t i)
 {
     const Frame f = frame_of(m, i);
     const int32_t lo = m.cell_ptr[i], deg = m.cell_ptr[i + 1] - lo;
     const int32_t *nb = m.slot_nb + lo;
-    if (!f.periodic) {
-        // a cell with mirror images: their coordinates are rounded, so its
-        // star is always built again
-        bool wall = false;
-        for (int32_t k = 0; k < deg; k++) wall |= nb[k] >= m.n;
-        if (wall) {
-            list_cell(m, i, 0);
-            return;
-        }
-    }
     Point a = point_of(f, base_ref(m, nb[deg - 2])), b = point_of(f, base_ref(m, nb[deg - 1]));
-    float cab;
-    {
-        // (a x b: the orientation of the triangle before the first)
-        cab = a.fx * b.fy - a.fy * b.fx;
-    }
+    // (a x b: the orientation of the triangle before the first)
+    float cab = a.fx * b.fy - a.fy * b.fx;
     int turns = 0;
-    bool self = false;
+    bool self = false, open = false;
     for (int32_t k = 0; k < deg; k++) {
         const int32_t ref = base_ref(m, nb[k]);
         const Point d = point_of(f, ref);
         const float p = b.fx * d.fy, q = b.fy * d.fx, cbd = p - q;
         bool bad = false;
-        if (!(cbd > kCrossBound * (fabsf(p) + fabsf(q)))) bad = orient_slow(f, b, d) <= 0;
-        if (!bad) {
-            const float p3 = a.fx * d.fy, p4 = a.fy * d.fx, p5 = a.fx * b.fy, p6 = a.fy * b.fx;
-            const float det = a.l * cbd - b.l * (p3 - p4) + d.l * cab;
-            const float bound = kCircleBound * (a.l * (fabsf(p) + fabsf(q)) + b.l * (fabsf(p3) + fabsf(p4)) +
-                                                d.l * (fabsf(p5) + fabsf(p6)));
-            if (!(det > bound)) bad = -det > bound || circle_slow(f, a, b, d) >= 0;
+        if (!(cbd > kCrossBound * (fabsf(p) + fabsf(q)))) {
+            if (kFast) open = true;
+            else bad = orient_slow(f, b, d) <= 0;
         }
-        if (bad) {
-            list_cell(m, a.ref >> 4, 0);
-            list_cell(m, b.ref >> 4, 0);
-            list_cell(m, d.ref >> 4, 0);
+        const float p3 = a.fx * d.fy, p4 = a.fy * d.fx, p5 = a.fx * b.fy, p6 = a.fy * b.fx;
+        const float det = a.l * cbd - b.l * (p3 - p4) + d.l * cab;
+        const float bound = kCircleBound * (a.l * (fabsf(p) + fabsf(q)) + b.l * (fabsf(p3) + fabsf(p4)) +
+                                            d.l * (fabsf(p5) + fabsf(p6)));
+        if (!(det > bound)) {
+            if (-det > bound) bad = true;
+            else if (kFast) open = true;
+            else if (!bad) bad = circle_slow(f, a, b, d) >= 0;
+        }
+        // both other vertices images across a wall: what lies beyond their
+        // edge is the image of a cell around this one, and no star of a cell
+        // tests it
+        if (!f.periodic && (b.ref & 15) != 4 && (d.ref & 15) != 4) {
+            if (kFast) open = true;
+            else if (!bad) bad = image_inside(f, nb, deg, b, d);
+        }
+        if (bad && !(kFast && open)) {
+            list_bad(m, f.periodic, a.ref, b.ref, d.ref);
             self = true;
         }
         // another image than the mesh had, or a disk near the band's edge:
@@ -422,10 +538,108 @@ RICH_HD inline void verify(const MeshUpdate &m, int32_t i)
         b = d;
         cab = cbd;
     }
+    if (kFast && open) return true;
     if (self || turns != 1) list_cell(m, i, 0);
+    return false;
 }
 
-// Cell i's star built again from the candidates around it.
+// Cell i's star from its ring and the vertices it was told of, in FP32: what
+// an edge flip asks for, and with it nearly every listed cell.  Returns
+// false, with nothing written, where that does not settle it (a cell at a wall, a
+// predicate beyond FP32, a large star or disk): recompute then.  (Serial; the
+// device's k_mesh_recompute_light takes a lane per candidate.)
+inline bool recompute_light(const MeshUpdate &m, int32_t i, int32_t round)
+{
+    int32_t ref[kLight];
+    float fx[kLight], fy[kLight];
+
+    const Frame f = frame_of(m, i);
+    const Ring own = ring_of(m, i, round);
+    const int32_t ne = m.extra_n[i];
+    if (own.deg + ne > kLight || ne > kMaxExtra) return false;
+    int nc = 0, near = 0;
+    float lmin = 0.0f;
+    for (int32_t k = 0; k < own.deg + ne; k++) {
+        const int32_t r = k < own.deg ? own[k] : m.extra[(int64_t)i * kMaxExtra + (k - own.deg)];
+        if (!f.periodic && (r & 15) != 4) return false;
+        if ((r >> 4) == i) return false;
+        bool have = false;
+        for (int c = 0; c < nc; c++) have |= (ref[c] >> 4) == (r >> 4);
+        if (have) continue;
+        const Point p = point_of(f, r);
+        ref[nc] = p.ref;
+        fx[nc] = p.fx;
+        fy[nc] = p.fy;
+        if (nc == 0 || p.l < lmin) {
+            lmin = p.l;
+            near = nc;
+        }
+        nc++;
+    }
+    // (the nearest candidate in FP32 is a neighbour unless another lies
+    // within a thousandth of its distance of it; the wrapping then does not
+    // close)
+    uint64_t out = 0;  // candidates in ring order, 4 bits each
+    int deg = 0, last = near, turns = 0;
+    do {
+        if (deg == 16) return false;
+        out |= (uint64_t)last << (4 * deg);
+        deg++;
+        Point a;
+        a.fx = fx[last];
+        a.fy = fy[last];
+        a.l = a.fx * a.fx + a.fy * a.fy;
+        int best = -1;
+        Point b;
+        for (int k = 0; k < nc; k++) {
+            if (k == last) continue;
+            Point d;
+            d.fx = fx[k];
+            d.fy = fy[k];
+            const float p3 = a.fx * d.fy, p4 = a.fy * d.fx, c = p3 - p4, cb = kCrossBound * (fabsf(p3) + fabsf(p4));
+            if (-c > cb) continue;
+            if (!(c > cb)) return false;
+            d.l = d.fx * d.fx + d.fy * d.fy;
+            if (best >= 0) {
+                const float p1 = b.fx * d.fy, p2 = b.fy * d.fx, p5 = a.fx * b.fy, p6 = a.fy * b.fx;
+                const float det = a.l * (p1 - p2) - b.l * c + d.l * (p5 - p6);
+                const float bound = kCircleBound * (a.l * (fabsf(p1) + fabsf(p2)) + b.l * (fabsf(p3) + fabsf(p4)) +
+                                                    d.l * (fabsf(p5) + fabsf(p6)));
+                if (det > bound) continue;
+                if (!(-det > bound)) return false;
+            }
+            best = k;
+            b = d;
+        }
+        if (best < 0 || !disk_ok(f, a, b)) return false;
+        turns += (a.fy < 0.0f && b.fy >= 0.0f) ? 1 : 0;
+        last = best;
+    } while (last != near);
+    if (deg < 3 || turns != 1) return false;
+    const int32_t info = m.ring_info[i];
+    const bool fresh = (info >> 2) < m.stamp;
+    int32_t at, ver = 0;
+    if (fresh) {
+        at = a_add(&m.count->overrides, 1);
+        if (at >= m.max_rings) {
+            a_or(f.flags, MU_SIZE);
+            return true;
+        }
+        m.ring_at[i] = at;
+    } else {
+        at = m.ring_at[i];
+        ver = (info & 1) ^ 1;
+    }
+    int32_t *dst = m.ring_ref + (int64_t)(2 * at + ver) * kMaxDeg;
+    for (int k = 0; k < deg; k++) dst[k] = ref[(int)(out >> (4 * k) & 15)];
+    m.ring_deg[2 * at + ver] = deg;
+    m.ring_info[i] = (m.stamp + round) << 2 | (fresh ? 2 : 0) | ver;
+    m.extra_n[i] = 0;
+    return true;
+}
+
+// Cell i's star built again from the candidates around it (serial; the device
+// runs the same steps with a warp per cell, see k_mesh_recompute).
 RICH_HD inline void recompute(const MeshUpdate &m, int32_t i, int32_t round)
 {
     const Frame f = frame_of(m, i);
@@ -577,19 +791,6 @@ RICH_HD inline void recompute(const MeshUpdate &m, int32_t i, int32_t round)
     m.ring_info[i] = (m.stamp + round) << 2 | (fresh ? 2 : 0) | ver;
 }
 
-// Cell v lacks the references r and q (in its own frame): list it for the
-// next round and tell it.
-RICH_HD inline void tell(const MeshUpdate &m, int32_t v, int32_t round, int32_t r, int32_t q)
-{
-    list_cell(m, v, round + 1);
-    const int32_t e[2] = {r, q};
-    for (int k = 0; k < 2; k++) {
-        if (e[k] < 0) continue;
-        const int32_t at = a_add(m.extra_n + v, 1);
-        if (at < kMaxExtra) m.extra[(int64_t)v * kMaxExtra + at] = e[k];
-    }
-}
-
 // whether the ring of v has r followed by q (by source in a periodic box)
 RICH_HD inline bool has_pair(const MeshUpdate &m, bool periodic, int32_t v, int32_t r, int32_t q)
 {
@@ -603,45 +804,46 @@ RICH_HD inline bool has_pair(const MeshUpdate &m, bool periodic, int32_t v, int3
     return false;
 }
 
-// The new star of cell i against its neighbours' rings.
-RICH_HD inline void check(const MeshUpdate &m, int32_t i, int32_t round)
+// The new star of cell i against its neighbours' rings: slot k's triangle,
+// and slot k of the star it replaced (the device's lanes take one k each).
+RICH_HD inline bool recomputed(const MeshUpdate &m, int32_t i, int32_t round)
 {
-    const int32_t info = m.ring_info[i];
-    if ((info >> 2) != m.stamp + round) return;  // not recomputed: a flag is set
-    const bool periodic = m.inst[inst_at(m, i)].boundary == 1;
-    const Ring g = ring_of(m, i, -1);
-    const int32_t me = i * 16 + 4;
-    int32_t a = g[g.deg - 1];
-    for (int32_t k = 0; k < g.deg; k++) {
-        const int32_t b = g[k];
-        // the triangle (i, a, b) in the rings of a and b (the cells
-        // themselves, not their images across a wall)
-        if ((periodic || (a & 15) == 4) && !has_pair(m, periodic, a >> 4, b, me)) {
-            tell(m, a >> 4, round, b, me);
-            list_cell(m, i, round + 1);
-        }
-        if ((periodic || (b & 15) == 4) && !has_pair(m, periodic, b >> 4, me, a)) {
-            tell(m, b >> 4, round, me, a);
-            list_cell(m, i, round + 1);
-        }
-        a = b;
+    return (m.ring_info[i] >> 2) == m.stamp + round;  // else a flag is set
+}
+
+RICH_HD inline void check_triangle(const MeshUpdate &m, bool periodic, const Ring &g, int32_t i, int32_t round,
+                                   int32_t k)
+{
+    const int32_t me = i * 16 + 4, a = g[k ? k - 1 : g.deg - 1], b = g[k];
+    // the triangle (i, a, b) in the rings of a and b (the cells themselves,
+    // not their images across a wall)
+    if ((periodic || (a & 15) == 4) && !has_pair(m, periodic, a >> 4, b, me)) {
+        tell(m, a >> 4, round + 1, b);
+        tell(m, a >> 4, round + 1, me);
+        list_cell(m, i, round + 1);
     }
-    // neighbours of the previous star that the new one dropped must have
-    // dropped the cell
-    const Ring old = ring_of(m, i, round);
-    for (int32_t k = 0; k < old.deg; k++) {
-        const int32_t r = old[k];
-        if ((r >> 4) == i || (!periodic && (r & 15) != 4)) continue;
-        bool kept = false;
-        for (int32_t j = 0; j < g.deg; j++) kept |= periodic ? (g[j] >> 4) == (r >> 4) : g[j] == r;
-        if (kept) continue;
-        const Ring o = ring_of(m, r >> 4, -1);
-        for (int32_t j = 0; j < o.deg; j++)
-            if (periodic ? (o[j] >> 4) == i : o[j] == me) {
-                list_cell(m, r >> 4, round + 1);
-                break;
-            }
+    if ((periodic || (b & 15) == 4) && !has_pair(m, periodic, b >> 4, me, a)) {
+        tell(m, b >> 4, round + 1, me);
+        tell(m, b >> 4, round + 1, a);
+        list_cell(m, i, round + 1);
     }
+}
+
+// a neighbour of the previous star that the new one dropped must have dropped
+// the cell
+RICH_HD inline void check_dropped(const MeshUpdate &m, bool periodic, const Ring &g, const Ring &old, int32_t i,
+                                  int32_t round, int32_t k)
+{
+    const int32_t me = i * 16 + 4, r = old[k];
+    if ((r >> 4) == i || (!periodic && (r & 15) != 4)) return;
+    for (int32_t j = 0; j < g.deg; j++)
+        if (periodic ? (g[j] >> 4) == (r >> 4) : g[j] == r) return;
+    const Ring o = ring_of(m, r >> 4, -1);
+    for (int32_t j = 0; j < o.deg; j++)
+        if (periodic ? (o[j] >> 4) == i : o[j] == me) {
+            list_cell(m, r >> 4, round + 1);
+            return;
+        }
 }
 
 // The images of point (x, y) inside the ghost band, in the host builder's
@@ -687,14 +889,11 @@ RICH_HD inline int image_rank(uint32_t mask, int img)
     return r;
 }
 
-// The cell's degree, owned edges and triangles, and ghost images.
-RICH_HD inline uint32_t measure(const MeshUpdate &m, int32_t i)
+// A ring's degree, owned edges and owned triangles (8 bits each).
+RICH_HD inline uint32_t ring_sizes(const MeshUpdate &m, bool periodic, int32_t i, const Ring &g)
 {
-    const InstParams &ip = m.inst[inst_at(m, i)];
-    const bool periodic = ip.boundary == 1;
-    const Ring g = ring_of(m, i, -1);
     uint32_t ne = 0, nt = 0;
-    int32_t prev = g[g.deg - 1];
+    const int32_t prev = g[g.deg - 1];
     bool prev_up = (prev & 15) != 4 || (prev >> 4) > i;
     for (int32_t k = 0; k < g.deg; k++) {
         const int32_t r = g[k];
@@ -703,12 +902,23 @@ RICH_HD inline uint32_t measure(const MeshUpdate &m, int32_t i)
         nt += (prev_up && up) ? 1 : 0;
         prev_up = up;
     }
-    const uint32_t mask = image_mask(ip, m.x[i], m.y[i]);
-    m.images[i] = (uint16_t)mask;
     if (g.deg > 255) a_or(m.flags + inst_at(m, i), MU_SIZE);
-    const uint32_t s = (uint32_t)g.deg | ne << 8 | nt << 16 | (uint32_t)popcount(mask) << 24;
-    m.sizes[i] = s;
-    return s;
+    return (uint32_t)(g.deg & 255) | ne << 8 | nt << 16;
+}
+
+// The cell's images inside the ghost band, counted into its sizes.
+RICH_HD inline uint32_t count_images(const MeshUpdate &m, int32_t i, uint32_t ring_part)
+{
+    const uint32_t mask = image_mask(m.inst[inst_at(m, i)], m.x[i], m.y[i]);
+    m.images[i] = (uint16_t)mask;
+    return (ring_part & 0xffffffu) | (uint32_t)popcount(mask) << 24;
+}
+
+// The cell's degree, owned edges and triangles, and ghost images.
+RICH_HD inline uint32_t measure(const MeshUpdate &m, int32_t i)
+{
+    const bool periodic = m.inst[inst_at(m, i)].boundary == 1;
+    return m.sizes[i] = count_images(m, i, ring_sizes(m, periodic, i, ring_of(m, i, -1)));
 }
 
 // The ghosts of cell i, from ghost_off[i] on.
@@ -733,30 +943,35 @@ RICH_HD inline void place_ghosts(const MeshUpdate &m, int32_t i)
         }
 }
 
-// Cell i's ring with this mesh's point ids, from its smallest neighbour on.
+// the updated mesh's point of a reference in cell i's ring
+RICH_HD inline int32_t point_id(const MeshUpdate &m, int32_t i, int32_t r)
+{
+    const int32_t src = r >> 4, img = r & 15;
+    if (img == 4) return src;
+    const uint32_t mask = m.images[src];
+    if (!(mask >> img & 1)) {
+        a_or(m.flags + inst_at(m, i), MU_IMAGE);
+        a_or(&m.count->bad, 1);
+        return src;
+    }
+    return m.n + m.ghost_off[src] + image_rank(mask, img);
+}
+
+// Cell i's ring with this mesh's point ids, from its smallest neighbour on
+// (serial; the device's k_mesh_rings takes eight lanes per cell).
 RICH_HD inline void place_ring(const MeshUpdate &m, int32_t i)
 {
     const Ring g = ring_of(m, i, -1);
     int32_t *dst = m.out_nb + m.out_ptr[i];
-    auto id_of = [&](int32_t r) {
-        const int32_t src = r >> 4, img = r & 15;
-        if (img == 4) return src;
-        const uint32_t mask = m.images[src];
-        if (!(mask >> img & 1)) {
-            a_or(m.flags + inst_at(m, i), MU_IMAGE);
-            return src;
-        }
-        return m.n + m.ghost_off[src] + image_rank(mask, img);
-    };
     int32_t best = INT32_MAX, at = 0;
     for (int32_t k = 0; k < g.deg; k++) {
-        const int32_t id = id_of(g[k]);
+        const int32_t id = point_id(m, i, g[k]);
         if (id < best) {
             best = id;
             at = k;
         }
     }
-    for (int32_t k = 0; k < g.deg; k++) dst[k] = id_of(g[at + k < g.deg ? at + k : at + k - g.deg]);
+    for (int32_t k = 0; k < g.deg; k++) dst[k] = point_id(m, i, g[at + k < g.deg ? at + k : at + k - g.deg]);
 }
 
 }  // namespace mu

@@ -26,37 +26,74 @@ struct MeshSizes {
     int32_t ghosts = 0, tris = 0, edges = 0, slots = 0;
 };
 
+// The triangle and edge lists of a mesh, built on the device from its rings.
+// The triangle of ring slot k of real cell i is (i, nb[k], nb[k+1]); it is
+// owned by its smallest vertex id (a real cell: ghost ids follow the real
+// ones), numbered in its owner's ring order from tri_off[owner] (tri_off[n] =
+// T) and written rotated to start at the owner.  Real cell i owns its edges to
+// larger real cells, to mirror images and (periodic box) to images of larger
+// cells or of itself shifted to the +x / +y side; its owned edges are numbered
+// in ring order from edge_off[i] (edge_off[n] = E).  Writes slot_edge (2 e, or
+// 2 e + 1 on the partner's slot) and edge_l / edge_r / edge_ta / edge_tb
+// (Voronoi edge from circumcentre ta to tb, counter-clockwise about the left
+// cell), and sets *bad where the rings do not agree with each other or with
+// the offsets.
+struct MeshLists {
+    int32_t n, periodic;        // box type where cell_inst is null
+    const int32_t *cell_inst;   // else each cell's box type from its simulation
+    const InstParams *inst;
+    const int32_t *cell_ptr, *slot_nb, *tri_off, *edge_off, *ghost_src, *ghost_shift;
+    int32_t *tri, *slot_tri, *slot_edge, *edge_l, *edge_r, *edge_ta, *edge_tb;
+    const uint32_t *edge_mask, *tri_mask;  // slots whose edge / triangle the cell owns (rings of up to 32), or nullptr
+    const int32_t *ready;       // nullptr, or 0 there: nothing is built
+    int32_t *bad;
+};
+cudaError_t launch_lists(const MeshLists &l, cudaStream_t st);
+
 // The updated mesh (cell_ptr, slot_nb, ghost_src and ghost_img apart from
-// the mesh being updated): what the host builder's upload holds.
+// the mesh being updated), the room its arrays have, and its lists' arrays.
 struct MeshOutput {
     int32_t *cell_ptr, *slot_nb, *tri_off, *edge_off, *cell_order;
     double *gx, *gy;
     int32_t *ghost_src, *ghost_xf, *ghost_shift, *ghost_img;
+    MeshSizes max;
+    MeshLists lists;  // (tri .. edge_tb and periodic; the rest is filled in)
+};
+
+struct MeshResult {
+    // kDone: the mesh and its lists are written (but for the meshes of
+    // simulations with flags()); kGrow: an array is too small for `sizes`;
+    // kHost: the rounds did not converge or the only simulation is flagged
+    enum { kDone, kGrow, kHost } state;
+    MeshSizes sizes;
+    bool flagged;  // some simulation's mesh is left to the host
+    bool bad;      // the lists do not close
 };
 
 class MeshUpdater {
 public:
-    // Enqueue the checks, the first rounds and the sizes of the updated
-    // mesh, with the counters' copy to the host.
-    cudaError_t start(const MeshArrays &a, cudaStream_t st);
-    // After the stream was waited for: the sizes, after more rounds if
-    // needed (ok = false: the rounds did not converge and the host builder
-    // has to take these meshes; those of simulations with flags() too).
-    cudaError_t settle(const MeshArrays &a, bool &ok, MeshSizes &sizes, cudaStream_t st);
+    // Enqueue the whole update, with the counters' copy to the host.
+    cudaError_t start(const MeshArrays &a, const MeshOutput &o, cudaStream_t st);
+    // After the stream was waited for: what came of it (after more rounds, if
+    // the cells did not agree yet).
+    cudaError_t settle(const MeshArrays &a, const MeshOutput &o, MeshResult &result, cudaStream_t st);
+    // After kGrow: the mesh written to larger arrays (waits).
+    cudaError_t again(const MeshArrays &a, const MeshOutput &o, MeshResult &result, cudaStream_t st);
     // Per simulation, after settle: non-zero when its mesh is left to the host.
     const int32_t *flags() const;
-    // Enqueue the writing of the updated mesh.
-    cudaError_t finish(const MeshArrays &a, const MeshOutput &o, cudaStream_t st);
+    // The next mesh to update is not the last update's (the host built it, or
+    // the update's was not kept).
+    void forget() { whole_ = true; }
 
 private:
     cudaError_t reserve(int32_t n, int32_t n_inst, cudaStream_t st);
-    cudaError_t read_counts(const MeshArrays &a, cudaStream_t st);
-    MeshUpdate params(const MeshArrays &a) const;
-    void launch_rounds(const MeshUpdate &m, int first, int last, cudaStream_t st) const;
+    MeshUpdate params(const MeshArrays &a, const MeshOutput &o) const;
+    cudaError_t launch_rounds(const MeshArrays &a, const MeshOutput &o, int first, int last, cudaStream_t st);
 
-    int32_t stamp_ = 0, max_rings_ = 0;
-    DBuf mark_, list_[2], info_, at_, ring_deg_, ring_ref_, extra_n_, extra_, count_, sizes_, images_, ghost_off_,
-        sums_, flags_;
+    int32_t stamp_ = 0, max_rings_ = 0, last_round_ = 0;
+    bool whole_ = true;  // sizes_ does not describe the mesh to update
+    DBuf mark_, list_[2], heavy_, info_, at_, ring_deg_, ring_ref_, extra_n_, extra_, count_, sizes_, images_,
+        ghost_off_, sums_, edge_mask_, tri_mask_;
     HBuf host_;
 };
 

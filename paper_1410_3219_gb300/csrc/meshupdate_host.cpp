@@ -15,8 +15,8 @@ void mesh_params(const BoxConfig &box, int32_t n, InstParams &ip)
     const double h = std::sqrt(Lx * Ly / std::max(n, 1));
     const double w = std::min(5.0 * h, lmin);
     const double margin = 1e-9 * (std::fabs(box.x0) + std::fabs(box.x1) + std::fabs(box.y0) + std::fabs(box.y1) + w);
-    ip.half_x = 0.5 * Lx;
-    ip.half_y = 0.5 * Ly;
+    ip.half_x = (float)(0.5 * Lx / h);
+    ip.half_y = (float)(0.5 * Ly / h);
     ip.band = w;
     ip.in_x0 = box.x0 + w + margin;
     ip.in_x1 = box.x1 - w - margin;
@@ -67,12 +67,24 @@ int mesh_update_serial(const BoxConfig &box, int32_t n, const double *x, const d
     m.flags = &flags;
     m.sizes = sizes.data();
     m.images = images.data();
-    for (int32_t i = 0; i < n; i++) mu::verify(m, i);
+    for (int32_t i = 0; i < n; i++)
+        if (mu::verify<true>(m, i)) m.list[1][cnt.open++] = i;
+    for (int32_t k = 0; k < cnt.open; k++) mu::verify<false>(m, m.list[1][k]);
     rounds = 0;
     recomputed = 0;
     for (; rounds < kMaxRounds && cnt.listed[rounds] > 0; rounds++) {
-        for (int32_t k = 0; k < cnt.listed[rounds]; k++) mu::recompute(m, m.list[rounds & 1][k], rounds);
-        for (int32_t k = 0; k < cnt.listed[rounds]; k++) mu::check(m, m.list[rounds & 1][k], rounds);
+        for (int32_t k = 0; k < cnt.listed[rounds]; k++) {
+            const int32_t i = m.list[rounds & 1][k];
+            if (rounds == 0 && mu::recompute_light(m, i, rounds)) continue;
+            mu::recompute(m, i, rounds);
+        }
+        for (int32_t k = 0; k < cnt.listed[rounds]; k++) {
+            const int32_t i = m.list[rounds & 1][k];
+            if (!mu::recomputed(m, i, rounds)) continue;
+            const mu::Ring g = mu::ring_of(m, i, -1), old = mu::ring_of(m, i, rounds);
+            for (int32_t t = 0; t < g.deg; t++) mu::check_triangle(m, box.boundary == 1, g, i, rounds, t);
+            for (int32_t t = 0; t < old.deg; t++) mu::check_dropped(m, box.boundary == 1, g, old, i, rounds, t);
+        }
         recomputed += cnt.listed[rounds];
     }
     if (flags || cnt.listed[rounds] > 0) return 0;

@@ -89,17 +89,16 @@ struct rich_sim {
     rich::MeshWork mw;  // (edge list built on the device: see tessellate)
     rich::HostMesh hm;  // the last mesh the host built
     // The mesh on the device (buffers mcur of the arrays that an update reads
-    // while it writes the new ones): its sizes, and whether the update may
-    // start from it.  After an update the check of its lists (bad_host) is
-    // read at the next wait.
+    // while it writes the new ones): its sizes, and whether an update may
+    // start from its rings
     int mcur = 0;
     rich::MeshSizes msz;
-    bool mesh_on_device = false, lists_unchecked = false;
+    bool mesh_on_device = false;
     rich::MeshUpdater updater;
     int64_t updates = 0;   // meshes made by it
-    rich::HBuf bad_host;   // two flags of the list builders, then the step's dt and status
+    rich::HBuf back;       // the step's dt and status, and the list builder's flag
     DBuf mesh_inst;        // the box and mesh_params
-    cudaEvent_t ev_up0 = nullptr, ev_up1 = nullptr;
+    cudaEvent_t ev_up = nullptr;
     std::unique_ptr<rich::ThreadPool> pool;  // host threads of the tile-parallel tessellation
     rich_sim() { mw.host_edges = false; }
     double t = 0.0;
@@ -136,8 +135,7 @@ struct rich_sim {
     {
         if (ev0) cudaEventDestroy(ev0);
         if (ev1) cudaEventDestroy(ev1);
-        if (ev_up0) cudaEventDestroy(ev_up0);
-        if (ev_up1) cudaEventDestroy(ev_up1);
+        if (ev_up) cudaEventDestroy(ev_up);
         for (cudaEvent_t e : kev)
             if (e) cudaEventDestroy(e);
         if (own_stream) cudaStreamDestroy(own_stream);
@@ -260,7 +258,7 @@ int alloc_cells(rich_sim *s)
     CUDA_TRY(s->scal.ensure(64));
     CUDA_TRY(cudaMemsetAsync(s->scal.p, 0, 64, s->stream));
     CUDA_TRY(s->instp.ensure(sizeof(rich::InstParams)));
-    CUDA_TRY(s->bad_host.ensure(64));
+    CUDA_TRY(s->back.ensure(64));
     CUDA_TRY(s->mesh_inst.ensure(sizeof(rich::InstParams)));
     rich::InstParams ip = s->inst_params(0.0);
     rich::mesh_params(rich::BoxConfig{s->cfg.boundary, s->cfg.x0, s->cfg.x1, s->cfg.y0, s->cfg.y1}, s->n, ip);
@@ -281,48 +279,78 @@ int build_mesh(rich_sim *s, rich_step_info *info)
     return rc ? mesh_rc(rc) : RICH_OK;
 }
 
-// Room for a mesh of these sizes in the arrays beside its rings, and the
-// triangle and edge lists built from the rings of buffers `mesh` (enqueued
-// with the copy of the builders' flags to bad_host).  Nothing on the stream
-// may still read the old lists: buffers that grow are reallocated.
-int build_lists(rich_sim *s, int mesh)
+// Room for the rings of a mesh of these sizes in buffers m, and for the rest
+// of it.  Nothing on the stream may still use the arrays: those that grow are
+// reallocated.
+int reserve_rings(rich_sim *s, int m, const rich::MeshSizes &z)
 {
-    const size_t T = (size_t)s->msz.tris, E = (size_t)s->msz.edges, S = (size_t)s->msz.slots, d = sizeof(double);
-    const size_t r = s->rsize();
-    CUDA_TRY(s->tri.ensure((3 * T + 3) * sizeof(int32_t)));
-    CUDA_TRY(s->slot_tri.ensure((S + 1) * sizeof(int32_t)));
-    CUDA_TRY(s->slot_edge.ensure((S + 1) * sizeof(int32_t)));
-    for (DBuf *b : {&s->edge_l, &s->edge_r, &s->edge_ta, &s->edge_tb}) CUDA_TRY(b->ensure((E + 1) * sizeof(int32_t)));
-    int32_t *bad = reinterpret_cast<int32_t *>(s->scal.as<char>() + 24);
-    int32_t *bad_tri = reinterpret_cast<int32_t *>(s->scal.as<char>() + 28);
-    const int32_t *ptr = s->cell_ptr[mesh].as<int32_t>(), *nb = s->slot_nb[mesh].as<int32_t>();
-    CUDA_TRY(rich::launch_build_tris(s->n, (int32_t)S, ptr, nb, s->toff.as<int32_t>(), s->tri.as<int32_t>(),
-                                     s->slot_tri.as<int32_t>(), bad_tri, s->stream));
-    CUDA_TRY(rich::launch_build_edges(s->n, (int32_t)S, ptr, nb, s->slot_tri.as<int32_t>(), s->gsrc[mesh].as<int32_t>(),
-                                      s->gshift.as<int32_t>(), s->eoff.as<int32_t>(),
-                                      s->cfg.boundary == RICH_BC_PERIODIC ? 1 : 0, nullptr, nullptr,
-                                      s->slot_edge.as<int32_t>(), s->edge_l.as<int32_t>(), s->edge_r.as<int32_t>(),
-                                      s->edge_ta.as<int32_t>(), s->edge_tb.as<int32_t>(), bad, s->stream));
-    CUDA_TRY(cudaMemcpyAsync(s->bad_host.p, bad, 2 * sizeof(int32_t), cudaMemcpyDeviceToHost, s->stream));
-    s->lists_unchecked = true;
-    CUDA_TRY(s->ccx.ensure((T + 1) * d)); CUDA_TRY(s->ccy.ensure((T + 1) * d));
-    for (DBuf *b : {&s->eL, &s->emlx, &s->emly, &s->emrx, &s->emry, &s->enx, &s->eny, &s->eqx, &s->eqy})
-        CUDA_TRY(b->ensure((E + 1) * r));
-    CUDA_TRY(s->F.ensure((4 * E + 4) * sizeof(double)));
-    CUDA_TRY(s->ePM.ensure((4 * E + 4) * r));
+    const size_t i4 = sizeof(int32_t), G = (size_t)z.ghosts + 1;
+    CUDA_TRY(s->cell_ptr[m].ensure(((size_t)s->n + 1) * i4));
+    CUDA_TRY(s->slot_nb[m].ensure(((size_t)z.slots + 1) * i4));
+    CUDA_TRY(s->gsrc[m].ensure(G * i4)); CUDA_TRY(s->gimg[m].ensure(G * i4));
     return RICH_OK;
 }
 
-// After a wait: the list builders' flags of the mesh last built.
-int check_lists(rich_sim *s)
+int reserve_mesh(rich_sim *s, const rich::MeshSizes &z)
 {
-    if (!s->lists_unchecked) return RICH_OK;
-    s->lists_unchecked = false;
-    const int32_t *bad = s->bad_host.as<int32_t>();
-    if (!bad[0] && !bad[1]) return RICH_OK;
-    s->tess_current = s->mesh_on_device = false;
-    if (bad[1]) return fail(RICH_ETESS, "a triangle of a ring is missing from its owner's ring");
-    return fail(RICH_ETESS, "an edge of a ring has no partner in the other cell's ring");
+    const size_t i4 = sizeof(int32_t), d = sizeof(double), r = s->rsize();
+    const size_t N = (size_t)s->n, G = (size_t)z.ghosts + 1, T = (size_t)z.tris + 1, E = (size_t)z.edges + 1;
+    const size_t S = (size_t)z.slots + 1;
+    CUDA_TRY(s->gx.ensure(G * d)); CUDA_TRY(s->gy.ensure(G * d));
+    CUDA_TRY(s->gxf.ensure(G * i4)); CUDA_TRY(s->gshift.ensure(G * i4));
+    CUDA_TRY(s->toff.ensure((N + 1) * i4)); CUDA_TRY(s->eoff.ensure((N + 1) * i4)); CUDA_TRY(s->corder.ensure(N * i4));
+    CUDA_TRY(s->tri.ensure(3 * T * i4));
+    CUDA_TRY(s->slot_tri.ensure(S * i4));
+    CUDA_TRY(s->slot_edge.ensure(S * i4));
+    for (DBuf *b : {&s->edge_l, &s->edge_r, &s->edge_ta, &s->edge_tb}) CUDA_TRY(b->ensure(E * i4));
+    CUDA_TRY(s->ccx.ensure(T * d)); CUDA_TRY(s->ccy.ensure(T * d));
+    for (DBuf *b : {&s->eL, &s->emlx, &s->emly, &s->emrx, &s->emry, &s->enx, &s->eny, &s->eqx, &s->eqy})
+        CUDA_TRY(b->ensure(E * r));
+    CUDA_TRY(s->F.ensure(4 * E * d));
+    CUDA_TRY(s->ePM.ensure(4 * E * r));
+    return RICH_OK;
+}
+
+rich::MeshLists mesh_lists(const rich_sim *s)
+{
+    rich::MeshLists l{};
+    l.periodic = s->cfg.boundary == RICH_BC_PERIODIC ? 1 : 0;
+    l.tri = s->tri.as<int32_t>();
+    l.slot_tri = s->slot_tri.as<int32_t>();
+    l.slot_edge = s->slot_edge.as<int32_t>();
+    l.edge_l = s->edge_l.as<int32_t>(); l.edge_r = s->edge_r.as<int32_t>();
+    l.edge_ta = s->edge_ta.as<int32_t>(); l.edge_tb = s->edge_tb.as<int32_t>();
+    return l;
+}
+
+// where an update writes (its rings to buffers m), as far as the arrays reach
+rich::MeshOutput mesh_output(const rich_sim *s, int m)
+{
+    rich::MeshOutput o{};
+    o.cell_ptr = s->cell_ptr[m].as<int32_t>();
+    o.slot_nb = s->slot_nb[m].as<int32_t>();
+    o.tri_off = s->toff.as<int32_t>();
+    o.edge_off = s->eoff.as<int32_t>();
+    o.cell_order = s->corder.as<int32_t>();
+    o.gx = s->gx.as<double>();
+    o.gy = s->gy.as<double>();
+    o.ghost_src = s->gsrc[m].as<int32_t>();
+    o.ghost_xf = s->gxf.as<int32_t>();
+    o.ghost_shift = s->gshift.as<int32_t>();
+    o.ghost_img = s->gimg[m].as<int32_t>();
+    const size_t r = s->rsize();
+    size_t e = std::min(s->F.cap / 32, s->ePM.cap / (4 * r));
+    for (const DBuf *b : {&s->edge_l, &s->edge_r, &s->edge_ta, &s->edge_tb}) e = std::min(e, b->cap / 4);
+    for (const DBuf *b : {&s->eL, &s->emlx, &s->emly, &s->emrx, &s->emry, &s->enx, &s->eny, &s->eqx, &s->eqy})
+        e = std::min(e, b->cap / r);
+    size_t g = std::min({s->gx.cap / 8, s->gy.cap / 8, s->gsrc[m].cap / 4, s->gimg[m].cap / 4, s->gxf.cap / 4,
+                         s->gshift.cap / 4});
+    const size_t t = std::min({s->tri.cap / 12, s->ccx.cap / 8, s->ccy.cap / 8});
+    const size_t q = std::min({s->slot_nb[m].cap / 4, s->slot_tri.cap / 4, s->slot_edge.cap / 4});
+    auto i32 = [](size_t v) { return (int32_t)std::min<size_t>(v, INT32_MAX / 4); };
+    o.max = rich::MeshSizes{i32(g), i32(t), i32(e), i32(q)};
+    o.lists = mesh_lists(s);
+    return o;
 }
 
 void report_sizes(const rich_sim *s, rich_step_info *info)
@@ -343,6 +371,11 @@ int upload_mesh(rich_sim *s, rich_step_info *info)
     const rich::HostMesh &m = s->hm;
     const int q = s->mcur;
     s->mesh_on_device = false;
+    s->updater.forget();
+    s->msz = rich::MeshSizes{m.g, m.n_tris, m.n_edges, (int32_t)m.slot_nb.size()};
+    int rc = reserve_mesh(s, s->msz);
+    for (int k = 0; k < 2 && rc == RICH_OK; k++) rc = reserve_rings(s, k, s->msz);
+    if (rc != RICH_OK) return rc;
     CUDA_TRY(upload(s->gx, m.gx, s->stream));
     CUDA_TRY(upload(s->gy, m.gy, s->stream));
     CUDA_TRY(upload(s->gsrc[q], m.ghost_src, s->stream));
@@ -354,11 +387,20 @@ int upload_mesh(rich_sim *s, rich_step_info *info)
     CUDA_TRY(upload(s->toff, m.tri_off, s->stream));
     CUDA_TRY(upload(s->eoff, m.edge_off, s->stream));
     CUDA_TRY(upload(s->gshift, m.ghost_shift, s->stream));
-    s->msz = rich::MeshSizes{m.g, m.n_tris, m.n_edges, (int32_t)m.slot_nb.size()};
-    int rc = build_lists(s, q);
-    if (rc != RICH_OK) return rc;
+    rich::MeshLists l = mesh_lists(s);
+    l.n = s->n;
+    l.cell_ptr = s->cell_ptr[q].as<int32_t>();
+    l.slot_nb = s->slot_nb[q].as<int32_t>();
+    l.tri_off = s->toff.as<int32_t>();
+    l.edge_off = s->eoff.as<int32_t>();
+    l.ghost_src = s->gsrc[q].as<int32_t>();
+    l.ghost_shift = s->gshift.as<int32_t>();
+    l.bad = reinterpret_cast<int32_t *>(s->scal.as<char>() + 24);
+    CUDA_TRY(cudaMemsetAsync(l.bad, 0, sizeof(int32_t), s->stream));
+    CUDA_TRY(rich::launch_lists(l, s->stream));
+    CUDA_TRY(cudaMemcpyAsync(s->back.p, l.bad, sizeof(int32_t), cudaMemcpyDeviceToHost, s->stream));
     CUDA_TRY(cudaStreamSynchronize(s->stream));
-    if ((rc = check_lists(s)) != RICH_OK) return rc;
+    if (*s->back.as<int32_t>()) return fail(RICH_ETESS, "the rings of the mesh do not close");
     s->tess_current = s->mesh_on_device = true;
     if (info) info->copy_ms += now_ms() - t2;
     report_sizes(s, info);
@@ -371,48 +413,45 @@ bool can_update(const rich_sim *s)
     return s->mesh_on_device && s->n >= rich::kMeshUpdateMin && s->n <= rich::kMeshUpdateMax;
 }
 
-// The updated mesh of the points in buffers q written and made the current
-// one, after the update's first part was waited for (enqueued, not waited
-// for; the caller of the next sweep checks the lists).  ok = false: the host
-// has to build this mesh; the mesh on the device is unchanged.
-int finish_update(rich_sim *s, int q, bool &ok, rich_step_info *info)
+// Enqueue the update of the mesh for the points in buffers q.  It reads the
+// rings of the present mesh and overwrites its lists.
+int start_update(rich_sim *s, int q)
 {
-    rich::MeshSizes z;
-    const rich::MeshArrays a = s->mesh_arrays(q);
-    CUDA_TRY(s->updater.settle(a, ok, z, s->stream));
-    ok = ok && !s->updater.flags()[0];
-    if (!ok) return RICH_OK;
-    const int m = 1 - s->mcur;
-    const size_t i4 = sizeof(int32_t), N = (size_t)s->n, G = (size_t)z.ghosts + 1;
-    // (the old ghosts' positions are read by nothing any more)
-    CUDA_TRY(s->cell_ptr[m].ensure((N + 1) * i4));
-    CUDA_TRY(s->slot_nb[m].ensure(((size_t)z.slots + 1) * i4));
-    CUDA_TRY(s->gsrc[m].ensure(G * i4)); CUDA_TRY(s->gimg[m].ensure(G * i4));
-    CUDA_TRY(s->gx.ensure(G * 8)); CUDA_TRY(s->gy.ensure(G * 8));
-    CUDA_TRY(s->gxf.ensure(G * i4)); CUDA_TRY(s->gshift.ensure(G * i4));
-    rich::MeshOutput o{};
-    o.cell_ptr = s->cell_ptr[m].as<int32_t>();
-    o.slot_nb = s->slot_nb[m].as<int32_t>();
-    o.tri_off = s->toff.as<int32_t>();
-    o.edge_off = s->eoff.as<int32_t>();
-    o.cell_order = s->corder.as<int32_t>();
-    o.gx = s->gx.as<double>();
-    o.gy = s->gy.as<double>();
-    o.ghost_src = s->gsrc[m].as<int32_t>();
-    o.ghost_xf = s->gxf.as<int32_t>();
-    o.ghost_shift = s->gshift.as<int32_t>();
-    o.ghost_img = s->gimg[m].as<int32_t>();
-    // (from here on the old mesh's offsets are overwritten)
-    s->tess_current = s->mesh_on_device = false;
-    CUDA_TRY(s->updater.finish(a, o, s->stream));
-    s->mcur = m;
-    s->msz = z;
-    s->updates++;
-    const int rc = build_lists(s, m);
-    if (rc != RICH_OK) return rc;
-    s->tess_current = s->mesh_on_device = true;
-    report_sizes(s, info);
+    s->tess_current = false;
+    CUDA_TRY(s->updater.start(s->mesh_arrays(q), mesh_output(s, 1 - s->mcur), s->stream));
     return RICH_OK;
+}
+
+// After the update was waited for: its mesh made the current one (keep), or
+// dropped; where it could not be made nothing is current, and the host has to
+// build it (the next update may still start from the present rings).
+int finish_update(rich_sim *s, int q, bool keep, rich_step_info *info)
+{
+    if (!keep) {
+        s->updater.forget();
+        return RICH_OK;
+    }
+    const rich::MeshArrays a = s->mesh_arrays(q);
+    const int m = 1 - s->mcur;
+    rich::MeshResult r;
+    CUDA_TRY(s->updater.settle(a, mesh_output(s, m), r, s->stream));
+    if (r.state == rich::MeshResult::kGrow) {
+        int rc = reserve_mesh(s, r.sizes);
+        if (rc == RICH_OK) rc = reserve_rings(s, m, r.sizes);
+        if (rc != RICH_OK) return rc;
+        CUDA_TRY(s->updater.again(a, mesh_output(s, m), r, s->stream));
+    }
+    if (r.state != rich::MeshResult::kDone || r.flagged || r.bad) {
+        s->updater.forget();
+        return RICH_OK;
+    }
+    s->mcur = m;
+    s->msz = r.sizes;
+    s->updates++;
+    s->tess_current = true;
+    report_sizes(s, info);
+    // (the next update's rings have as much room as these)
+    return reserve_rings(s, 1 - m, r.sizes);
 }
 
 // a0 for the current points: the mesh on the device updated, or else built on
@@ -423,17 +462,12 @@ int tessellate(rich_sim *s, rich_step_info *info, bool fetch_points)
     if (fetch_points && can_update(s)) {
         const double t0 = now_ms();
         const int q = s->pts();
-        CUDA_TRY(s->updater.start(s->mesh_arrays(q), s->stream));
-        CUDA_TRY(cudaStreamSynchronize(s->stream));
-        bool ok = false;
-        int rc = finish_update(s, q, ok, info);
+        int rc = start_update(s, q);
         if (rc != RICH_OK) return rc;
-        if (ok) {
-            CUDA_TRY(cudaStreamSynchronize(s->stream));
-            if ((rc = check_lists(s)) != RICH_OK) return rc;
-            if (info) info->tess_ms += now_ms() - t0;
-            return RICH_OK;
-        }
+        CUDA_TRY(cudaStreamSynchronize(s->stream));
+        if ((rc = finish_update(s, q, true, info)) != RICH_OK) return rc;
+        if (info) info->tess_ms += now_ms() - t0;
+        if (s->tess_current) return RICH_OK;
     }
     if (fetch_points) {
         const double t0 = now_ms();
@@ -555,7 +589,7 @@ static int create_sim(const rich_config *cfg, int64_t n, const double *x, const 
         return bail(fail(RICH_ECUDA, "stream creation failed"));
     s->stream = s->own_stream;
     if (cudaEventCreate(&s->ev0) != cudaSuccess || cudaEventCreate(&s->ev1) != cudaSuccess ||
-        cudaEventCreate(&s->ev_up0) != cudaSuccess || cudaEventCreate(&s->ev_up1) != cudaSuccess)
+        cudaEventCreate(&s->ev_up) != cudaSuccess)
         return bail(fail(RICH_ECUDA, "event creation failed"));
     if ((rc = alloc_cells(s)) != RICH_OK) return bail(rc);
     if (s->x[0].ensure(n * 8) != cudaSuccess) return bail(fail(RICH_ENOMEM, "device points"));
@@ -664,11 +698,6 @@ static int launch_sweep(rich_sim *s, double t_end)
     if (!s->tess_current) return fail(RICH_ESTATE, "no current tessellation");
     if (s->pending) return fail(RICH_ESTATE, "a sweep is pending; call rich_sync first");
     if (!(t_end > s->t)) return fail(RICH_EINVAL, "t_end must exceed the current time");
-    // the staging struct may be in flight, and the lists of an updated mesh
-    // are checked before any kernel reads them
-    CUDA_TRY(cudaStreamSynchronize(s->stream));
-    int rc = check_lists(s);
-    if (rc != RICH_OK) return rc;
     s->inst_host = s->inst_params(t_end - s->t);
     CUDA_TRY(cudaMemcpyAsync(s->instp.p, &s->inst_host, sizeof(rich::InstParams), cudaMemcpyHostToDevice, s->stream));
     CUDA_TRY(cudaEventRecord(s->ev0, s->stream));
@@ -693,7 +722,7 @@ int rich_sync(rich_sim *s, rich_step_info *info)
     double t0 = now_ms();
     char *sc = s->scal.as<char>();
     // (into page-locked memory: dt, then the status)
-    double *dt_host = s->bad_host.as<double>() + 1;
+    double *dt_host = s->back.as<double>() + 1;
     int32_t *status_host = reinterpret_cast<int32_t *>(dt_host + 1);
     CUDA_TRY(cudaMemcpyAsync(dt_host, sc + 8, 12, cudaMemcpyDeviceToHost, s->stream));
     CUDA_TRY(cudaStreamSynchronize(s->stream));
@@ -745,10 +774,9 @@ int rich_sync(rich_sim *s, rich_step_info *info)
 }
 
 // One sweep of rich_step: the update of the mesh for the moved points follows
-// the sweep on the stream (its first part reads only the points and the old
-// mesh), so one wait serves both; unless the sweep failed or landed on t_end,
-// the updated mesh is then written (not waited for).  A mesh that the update
-// cannot make is left to the next tessellation.
+// the sweep on the stream, so one wait serves both.  A failed sweep drops the
+// updated mesh (and the lists it overwrote); a mesh that the update cannot
+// make is left to the next tessellation.
 static int step_sweep(rich_sim *s, double t_end, rich_step_info *info)
 {
     int rc = launch_sweep(s, t_end);
@@ -756,25 +784,19 @@ static int step_sweep(rich_sim *s, double t_end, rich_step_info *info)
     const int q = s->next_pts();
     const bool update = can_update(s);
     if (update) {
-        CUDA_TRY(cudaEventRecord(s->ev_up0, s->stream));
-        CUDA_TRY(s->updater.start(s->mesh_arrays(q), s->stream));
-        CUDA_TRY(cudaEventRecord(s->ev_up1, s->stream));
+        if ((rc = start_update(s, q)) != RICH_OK) return rc;
+        CUDA_TRY(cudaEventRecord(s->ev_up, s->stream));
     }
-    const bool half = s->time_centred() && s->tc_phase == 0;
-    const double before = s->t;
-    if ((rc = rich_sync(s, info)) != RICH_OK) return rc;
-    if (!update) return RICH_OK;
+    rc = rich_sync(s, info);
+    if (!update) return rc;
+    if (rc != RICH_OK) {
+        finish_update(s, q, false, nullptr);
+        return rc;
+    }
     float ms = 0.0f;
-    cudaEventElapsedTime(&ms, s->ev_up0, s->ev_up1);
+    cudaEventElapsedTime(&ms, s->ev1, s->ev_up);
     if (info) info->tess_ms += ms;
-    // the half-step points always get a mesh; after a full step, the points
-    // get one unless the step landed on t_end
-    if (!half && !(s->last_dt < t_end - before)) return RICH_OK;
-    const double t0 = now_ms();
-    bool ok = false;
-    rc = finish_update(s, q, ok, info);
-    if (info) info->tess_ms += now_ms() - t0;
-    return rc;
+    return finish_update(s, q, true, info);
 }
 
 int rich_step(rich_sim *s, int32_t max_steps, double t_end, rich_step_info *info)
@@ -812,15 +834,10 @@ static int ensure_geometry(rich_sim *s)
         int rc = tessellate(s, nullptr, true);
         if (rc) return rc;
     }
-    if (s->lists_unchecked) {
-        CUDA_TRY(cudaStreamSynchronize(s->stream));
-        int rc = check_lists(s);
-        if (rc) return rc;
-    }
     for (int k = 0; k < rich::GEOMETRY_STAGES; k++) s->launch(k, nullptr, nullptr, false);
     CUDA_TRY(cudaGetLastError());
-    CUDA_TRY(cudaStreamSynchronize(s->stream));
-    // the cell geometry and primitives now describe the current points
+    // the cell geometry and primitives now describe the current points (once
+    // the stream gets there)
     s->geometry_current = true;
     s->diag_pts = s->pts();
     return RICH_OK;
@@ -856,22 +873,19 @@ int rich_get_state(rich_sim *s, int64_t n, double *x, double *y, double *rho, do
     if (!s || n != s->n) return fail(RICH_EINVAL, "bad handle or size");
     int rc = ensure_geometry(s);
     if (rc) return rc;
-    std::vector<double> h;
+    // put in the caller's order on the device, then copied straight into the
+    // caller's arrays with one wait (on the host the reordering took 2.4 ms of
+    // a 3.0 ms step and read at 262,144 cells)
     const size_t N = (size_t)s->n;
     const int q = s->pts();
-    if (x) { if ((rc = fetch(s, s->x[q].p, h, N))) return rc; unpermute(s, h.data(), x); }
-    if (y) { if ((rc = fetch(s, s->y[q].p, h, N))) return rc; unpermute(s, h.data(), y); }
-    double *outs[4] = {rho, vx, vy, p};
-    if (rho || vx || vy || p) {
-        if ((rc = fetch_r(s, s->W.p, h, 4 * N))) return rc;
-        std::vector<double> comp(N);
-        for (int v = 0; v < 4; v++) {
-            if (!outs[v]) continue;
-            for (size_t k = 0; k < N; k++) comp[k] = h[4 * k + v];
-            unpermute(s, comp.data(), outs[v]);
-        }
-    }
-    if (area) { if ((rc = fetch(s, s->A.p, h, N))) return rc; unpermute(s, h.data(), area); }
+    double *outs[7] = {x, y, rho, vx, vy, p, area};
+    CUDA_TRY(s->unperm.ensure(7 * N * sizeof(double)));
+    double *st = s->unperm.as<double>();
+    CUDA_TRY(rich::launch_unpermute_state(s->n, s->perm_dev.as<int32_t>(), s->x[q].as<double>(), s->y[q].as<double>(),
+                                          s->W.p, s->rsize() == sizeof(float), s->A.as<double>(), st, s->stream));
+    for (int f = 0; f < 7; f++)
+        if (outs[f]) CUDA_TRY(cudaMemcpyAsync(outs[f], st + (size_t)f * N, N * 8, cudaMemcpyDeviceToHost, s->stream));
+    CUDA_TRY(cudaStreamSynchronize(s->stream));
     return RICH_OK;
 }
 
@@ -1012,7 +1026,7 @@ int rich_edge_list_check(const rich_config *cfg, int64_t n, const double *x, con
     const size_t S = m.slot_nb.size(), E = (size_t)m.n_edges, T2 = (size_t)m2.n_tris;
     cudaStream_t st = nullptr;
     CUDA_TRY(cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking));
-    DBuf cell_ptr, slot_nb, slot_tri, gsrc, gshift, eoff, slot_edge, el, er, eta, etb, bad, toff, dtri, dslot_tri, bad2;
+    DBuf cell_ptr, slot_nb, gsrc, gshift, eoff, slot_edge, el, er, eta, etb, bad, toff, dtri, dslot_tri;
     auto up = [&](DBuf &d, const std::vector<int32_t> &h) -> cudaError_t {
         cudaError_t e = d.ensure((h.size() + 1) * sizeof(int32_t));
         if (e == cudaSuccess && !h.empty())
@@ -1020,30 +1034,35 @@ int rich_edge_list_check(const rich_config *cfg, int64_t n, const double *x, con
         return e;
     };
     std::vector<int32_t> dse(S), del(E), der(E), deta(E), detb(E), dt(3 * T2), dst(S);
-    int32_t bad_h = 0, bad2_h = 0;
+    int32_t bad_h = 0;
     cudaError_t e = up(cell_ptr, m.cell_ptr);
     if (e == cudaSuccess) e = up(slot_nb, m.slot_nb);
-    if (e == cudaSuccess) e = up(slot_tri, m.slot_tri);
     if (e == cudaSuccess) e = up(gsrc, m.ghost_src);
     if (e == cudaSuccess) e = up(gshift, m.ghost_shift);
     if (e == cudaSuccess) e = up(eoff, m.edge_off);
-    for (DBuf *b : {&slot_edge}) if (e == cudaSuccess) e = b->ensure((S + 1) * sizeof(int32_t));
+    if (e == cudaSuccess) e = up(toff, m2.tri_off);
+    // (every slot has to be written: an entry the builder leaves shows)
+    for (DBuf *b : {&slot_edge, &dslot_tri}) {
+        if (e == cudaSuccess) e = b->ensure((S + 1) * sizeof(int32_t));
+        if (e == cudaSuccess) e = cudaMemsetAsync(b->p, 0xff, b->cap, st);
+    }
     for (DBuf *b : {&el, &er, &eta, &etb}) if (e == cudaSuccess) e = b->ensure((E + 1) * sizeof(int32_t));
     if (e == cudaSuccess) e = bad.ensure(sizeof(int32_t));
-    if (e == cudaSuccess) e = up(toff, m2.tri_off);
+    if (e == cudaSuccess) e = cudaMemsetAsync(bad.p, 0, sizeof(int32_t), st);
     if (e == cudaSuccess) e = dtri.ensure((3 * T2 + 3) * sizeof(int32_t));
-    if (e == cudaSuccess) e = dslot_tri.ensure((S + 1) * sizeof(int32_t));
-    if (e == cudaSuccess) e = bad2.ensure(sizeof(int32_t));
-    if (e == cudaSuccess)
-        e = rich::launch_build_tris((int32_t)n, (int32_t)S, cell_ptr.as<int32_t>(), slot_nb.as<int32_t>(),
-                                    toff.as<int32_t>(), dtri.as<int32_t>(), dslot_tri.as<int32_t>(),
-                                    bad2.as<int32_t>(), st);
-    if (e == cudaSuccess)
-        e = rich::launch_build_edges((int32_t)n, (int32_t)S, cell_ptr.as<int32_t>(), slot_nb.as<int32_t>(),
-                                     slot_tri.as<int32_t>(), gsrc.as<int32_t>(), gshift.as<int32_t>(),
-                                     eoff.as<int32_t>(), cfg->boundary == RICH_BC_PERIODIC ? 1 : 0, nullptr, nullptr,
-                                     slot_edge.as<int32_t>(), el.as<int32_t>(), er.as<int32_t>(), eta.as<int32_t>(),
-                                     etb.as<int32_t>(), bad.as<int32_t>(), st);
+    if (e == cudaSuccess) {
+        rich::MeshLists l{};
+        l.n = (int32_t)n;
+        l.periodic = cfg->boundary == RICH_BC_PERIODIC ? 1 : 0;
+        l.cell_ptr = cell_ptr.as<int32_t>(); l.slot_nb = slot_nb.as<int32_t>();
+        l.tri_off = toff.as<int32_t>(); l.edge_off = eoff.as<int32_t>();
+        l.ghost_src = gsrc.as<int32_t>(); l.ghost_shift = gshift.as<int32_t>();
+        l.tri = dtri.as<int32_t>(); l.slot_tri = dslot_tri.as<int32_t>(); l.slot_edge = slot_edge.as<int32_t>();
+        l.edge_l = el.as<int32_t>(); l.edge_r = er.as<int32_t>();
+        l.edge_ta = eta.as<int32_t>(); l.edge_tb = etb.as<int32_t>();
+        l.bad = bad.as<int32_t>();
+        e = rich::launch_lists(l, st);
+    }
     auto down = [&](std::vector<int32_t> &h, DBuf &d) {
         if (e == cudaSuccess && !h.empty())
             e = cudaMemcpyAsync(h.data(), d.p, h.size() * sizeof(int32_t), cudaMemcpyDeviceToHost, st);
@@ -1056,11 +1075,10 @@ int rich_edge_list_check(const rich_config *cfg, int64_t n, const double *x, con
     down(dt, dtri);
     down(dst, dslot_tri);
     if (e == cudaSuccess) e = cudaMemcpyAsync(&bad_h, bad.p, sizeof(int32_t), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&bad2_h, bad2.p, sizeof(int32_t), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     cudaStreamDestroy(st);
     if (e != cudaSuccess) return fail(RICH_ECUDA, cudaGetErrorString(e));
-    int64_t bad_count = (bad_h ? 1 : 0) + (bad2_h ? 1 : 0);
+    int64_t bad_count = bad_h ? 1 : 0;
     for (size_t k = 0; k < S; k++) bad_count += dse[k] != m.slot_edge[k];
     // the device's triangle of every slot: the host's, vertex for vertex
     // (the numbering differs: the host's is per tile)
@@ -1072,9 +1090,16 @@ int rich_edge_list_check(const rich_config *cfg, int64_t n, const double *x, con
         }
         for (int c = 0; c < 3; c++) bad_count += dt[3 * (size_t)a + c] != m.tri[3 * (size_t)h + c];
     }
+    // (the edges' Voronoi vertices: the device's triangles, vertex for vertex)
+    auto same_tri = [&](int32_t a, int32_t h) {
+        if (a < 0 || (size_t)a >= T2) return false;
+        for (int c = 0; c < 3; c++)
+            if (dt[3 * (size_t)a + c] != m.tri[3 * (size_t)h + c]) return false;
+        return true;
+    };
     for (size_t k = 0; k < E; k++)
-        bad_count += (del[k] != m.edge_l[k]) + (der[k] != m.edge_r[k]) + (deta[k] != m.edge_ta[k]) +
-                     (detb[k] != m.edge_tb[k]);
+        bad_count += (del[k] != m.edge_l[k]) + (der[k] != m.edge_r[k]) + !same_tri(deta[k], m.edge_ta[k]) +
+                     !same_tri(detb[k], m.edge_tb[k]);
     *edges = (int64_t)E;
     *mismatched = bad_count;
     return RICH_OK;
@@ -1195,8 +1220,7 @@ int rich_mesh_check(rich_sim *s, int64_t *mismatched, int64_t *updates)
     if (s->pending) return fail(RICH_ESTATE, "a sweep is pending; call rich_sync first");
     if (!s->tess_current) return fail(RICH_ESTATE, "no current tessellation");
     CUDA_TRY(cudaStreamSynchronize(s->stream));
-    int rc = check_lists(s);
-    if (rc != RICH_OK) return rc;
+    int rc;
     rich::HostMesh d, f;
     const size_t N = (size_t)s->n, G = (size_t)s->msz.ghosts, S = (size_t)s->msz.slots;
     std::vector<double> x(N), y(N);

@@ -71,12 +71,12 @@ struct InstParams {
     float gamma_f, igm1_f, chi_f, theta_f, delta_v_f;
     int32_t pad;
     // constants of the device mesh update (mesh_params in meshupdate.h):
-    // half the box's sides, the ghost band and the box inside which no point
-    // has an image in it, and in FP32, in mean point spacings (lengths times
-    // mesh_scale), the squared circumradii that need no placing and that a
+    // the ghost band and the box inside which no point has an image in it,
+    // and in FP32, in mean point spacings (lengths times mesh_scale), half the
+    // box's sides, the squared circumradii that need no placing and that a
     // periodic box allows, and how far a disk may reach past a wall
-    double half_x, half_y, band, in_x0, in_x1, in_y0, in_y1;
-    float mesh_scale, mesh_rlim2, mesh_rper2, mesh_reach;
+    double band, in_x0, in_x1, in_y0, in_y1;
+    float half_x, half_y, mesh_scale, mesh_rlim2, mesh_rper2, mesh_reach;
 };
 
 template <class R> struct SweepParams {
@@ -188,33 +188,5 @@ template <class R> int persistent_blocks_per_sm(int block);
 // arrays of n_old and n_new cells); cells with src[i] < 0 are left alone.
 void launch_repack(const int32_t *src, int32_t n_new, int32_t n_old, const double *U_old, double *U_new,
                    cudaStream_t st);
-
-// The triangle list from the rings, on the device.  The triangle of ring
-// slot k of real cell i is (i, nb[k], nb[k+1]); it is owned by its smallest
-// vertex id (a real cell: ghost ids follow the real ones), numbered in its
-// owner's ring order from tri_off[owner] (tri_off[n] = T, from the host) and
-// written rotated to start at the owner, as the host builder writes it.
-// Writes tri (3 T) and slot_tri (S), and sets *bad to 1 if a cell owns more
-// or fewer triangles than tri_off gives, if a slot's triangle is missing
-// from its owner's ring, or if a slot ends without a triangle.
-cudaError_t launch_build_tris(int32_t n, int32_t S, const int32_t *cell_ptr, const int32_t *slot_nb,
-                              const int32_t *tri_off, int32_t *tri, int32_t *slot_tri, int32_t *bad, cudaStream_t st);
-
-// The edge list from the rings, on the device (the host then ships rings
-// only).  Real cell i owns its edges to larger real cells, to mirror images
-// and (periodic box) to images of larger cells or of itself shifted to the
-// +x / +y side; its owned edges are numbered in ring order from
-// edge_off[i] (edge_off[n] = E, from the host).  Writes slot_edge (2 e, or
-// 2 e + 1 on the partner's slot), edge_l / edge_r / edge_ta / edge_tb
-// (Voronoi edge from circumcentre ta to tb, counter-clockwise about the
-// left cell), and sets *bad to 1 if a slot ends without an edge.  S slots
-// in all; the ghost arrays are read only for a periodic box.  In a packed
-// batch (cell_inst non-null) each cell's box type comes from its
-// simulation's parameters instead of `periodic`.
-cudaError_t launch_build_edges(int32_t n, int32_t S, const int32_t *cell_ptr, const int32_t *slot_nb,
-                               const int32_t *slot_tri, const int32_t *ghost_src, const int32_t *ghost_shift,
-                               const int32_t *edge_off, int32_t periodic, const InstParams *inst,
-                               const int32_t *cell_inst, int32_t *slot_edge, int32_t *edge_l, int32_t *edge_r,
-                               int32_t *edge_ta, int32_t *edge_tb, int32_t *bad, cudaStream_t st);
 
 }  // namespace rich
