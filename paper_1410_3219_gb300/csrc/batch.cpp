@@ -105,12 +105,14 @@ struct rich_batch {
     cudaStream_t stream = nullptr;
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
     // The device's mesh update (meshupdate.h) for the packed cells: after a
-    // step dev_mesh says that the arrays of buffers mcur hold the meshes of
+    // step dev_mesh says that mesh[mcur] holds the meshes of
     // the moved points of `packed` (those of simulations with a mesh flag
     // excepted), dev_lists that none is flagged and the triangle and edge
     // lists are good.  A step whose simulations are the same then starts
     // with the sweep; else the meshes are read back and packed again.
     rich::MeshUpdater updater;
+    rich::MeshStore mesh[2];
+    rich::MeshStream mesh_stream;
     int mcur = 0;
     bool dev_mesh = false, dev_lists = false;
     std::vector<int32_t> mesh_flag;
@@ -119,16 +121,13 @@ struct rich_batch {
     DBuf perm_dev, read_dev;
     rich::HBuf read_host;
     rich::HBuf h_back;  // dt, status per simulation, then the list builder's flag
-    cudaEvent_t ev2 = nullptr, ev3 = nullptr;
+    cudaEvent_t ev2 = nullptr;
     bool diagnostics = false;
     int cur = 0;
     // device
     DBuf x[2], y[2], U[2], A, o, W, cs, g, gl, alpha, w, tess, rounding, p64, cell_inst, initW, src;
-    DBuf corder, psrc;
-    DBuf cell_ptr[2], slot_nb[2], gsrc[2], gimg[2];
-    DBuf gx, gy, gxf, tri, ccx, ccy, slot_tri, slot_edge;
-    DBuf edge_l, edge_r, edge_ta, edge_tb, eL, emlx, emly, emrx, emry, enx, eny, eqx, eqy, F, ePM;
-    DBuf instp, dtmin, dtout, status, dsizes, gsync, eoff, toff, gshift, listbad;
+    DBuf psrc, ccx, ccy, eL, emlx, emly, emrx, emry, enx, eny, eqx, eqy, F, ePM;
+    DBuf instp, dtmin, dtout, status, dsizes, gsync, listbad;
     // launch shape: autotuned over the first steps unless fixed by the caller
     int launch_mode = 0;  // 0 autotune, 1 staged, 2 persistent
     int fixed_block = 256;
@@ -154,7 +153,7 @@ struct rich_batch {
     // host staging of the packed mesh
     std::vector<double> h_x, h_y, h_gx, h_gy, h_W0;
     std::vector<double> h_dlx, h_dly, h_dgx, h_dgy;  // the points (and a mesh's ghosts) downloaded at the start of a step
-    std::vector<int32_t> h_dptr, h_dnb, h_dgsrc, h_dgxf, h_dgshift, h_dgimg, h_dtoff, h_deoff, h_dorder;
+    std::vector<int32_t> h_dptr, h_dnb, h_dgsrc, h_dgxf, h_dgshift, h_dgimg, h_dtoff, h_deoff;
     std::vector<int32_t> h_gsrc, h_gxf, h_cell_ptr, h_slot_nb, h_cell_inst;
     std::vector<int32_t> h_corder;
     std::vector<int32_t> h_src, h_eoff, h_toff, h_gshift, h_gimg, h_perm;
@@ -170,7 +169,7 @@ struct rich_batch {
             if (gexec[k]) cudaGraphExecDestroy(gexec[k]);
             if (graph[k]) cudaGraphDestroy(graph[k]);
         }
-        for (cudaEvent_t e : {ev0, ev1, ev2, ev3})
+        for (cudaEvent_t e : {ev0, ev1, ev2})
             if (e) cudaEventDestroy(e);
         if (stream) cudaStreamDestroy(stream);
     }
@@ -190,18 +189,9 @@ struct rich_batch {
         p.diagnostics = diagnostics ? 1 : 0;
         p.motion = 1;
         p.n = (int32_t)n_packed;
-        p.ng = (int32_t)nG;
-        p.T = (int32_t)nT;
-        p.E = (int32_t)nE;
-        p.S = (int32_t)nS;
+        mesh[mcur].describe(p, rich::MeshSizes{(int32_t)nG, (int32_t)nT, (int32_t)nE, (int32_t)nS});
         p.x = x[cur].as<double>(); p.y = y[cur].as<double>();
         p.xn = x[1 - cur].as<double>(); p.yn = y[1 - cur].as<double>();
-        p.gx = gx.as<double>(); p.gy = gy.as<double>();
-        p.tri = tri.as<int32_t>(); p.cell_ptr = cell_ptr[mcur].as<int32_t>(); p.cell_order = corder.as<int32_t>();
-        p.slot_nb = slot_nb[mcur].as<int32_t>(); p.slot_tri = slot_tri.as<int32_t>(); p.slot_edge = slot_edge.as<int32_t>();
-        p.edge_l = edge_l.as<int32_t>(); p.edge_r = edge_r.as<int32_t>();
-        p.edge_ta = edge_ta.as<int32_t>(); p.edge_tb = edge_tb.as<int32_t>();
-        p.ghost_src = gsrc[mcur].as<int32_t>(); p.ghost_xf = gxf.as<int32_t>();
         p.ccx = ccx.as<double>(); p.ccy = ccy.as<double>(); p.A = A.as<double>();
         p.eL = eL.as<R>(); p.emlx = emlx.as<R>(); p.emly = emly.as<R>();
         p.emrx = emrx.as<R>(); p.emry = emry.as<R>();
@@ -454,85 +444,17 @@ template <class R> int run_persistent(rich_batch *b, int block)
     return RICH_OK;
 }
 
-// The sweep stage by stage.
-int run_staged(rich_batch *b)
+// Room for the geometry of packed meshes of these sizes (which every sweep
+// computes afresh; nothing enqueued may still use the arrays).
+int reserve_geometry(rich_batch *b, const rich::MeshSizes &z)
 {
-    CUDA_TRY(cudaMemsetAsync(b->status.p, 0, b->status.cap, b->stream));
-    for (int k = 0; k < rich::NUM_STAGES; k++) b->launch(k, nullptr);
-    CUDA_TRY(cudaGetLastError());
-    b->staged_launches++;
-    return RICH_OK;
-}
-
-rich::MeshLists mesh_lists(const rich_batch *b)
-{
-    rich::MeshLists l{};
-    l.tri = b->tri.as<int32_t>();
-    l.slot_tri = b->slot_tri.as<int32_t>();
-    l.slot_edge = b->slot_edge.as<int32_t>();
-    l.edge_l = b->edge_l.as<int32_t>(); l.edge_r = b->edge_r.as<int32_t>();
-    l.edge_ta = b->edge_ta.as<int32_t>(); l.edge_tb = b->edge_tb.as<int32_t>();
-    return l;
-}
-
-// Room for the rings of packed meshes of these sizes in buffers m, and for
-// the rest of them (nothing on the stream may still use the arrays).
-int reserve_rings(rich_batch *b, int m, const rich::MeshSizes &z)
-{
-    const size_t G = (size_t)z.ghosts + 1;
-    CUDA_TRY(b->cell_ptr[m].ensure(((size_t)b->n_packed + 1) * 4));
-    CUDA_TRY(b->slot_nb[m].ensure(((size_t)z.slots + 1) * 4));
-    CUDA_TRY(b->gsrc[m].ensure(G * 4)); CUDA_TRY(b->gimg[m].ensure(G * 4));
-    return RICH_OK;
-}
-
-int reserve_mesh(rich_batch *b, const rich::MeshSizes &z)
-{
-    const size_t N = (size_t)b->n_packed, G = (size_t)z.ghosts + 1, T = (size_t)z.tris + 1, E = (size_t)z.edges + 1;
-    const size_t S = (size_t)z.slots + 1, r = b->rsize(), d = sizeof(double);
-    CUDA_TRY(b->gx.ensure(G * 8)); CUDA_TRY(b->gy.ensure(G * 8));
-    CUDA_TRY(b->gxf.ensure(G * 4)); CUDA_TRY(b->gshift.ensure(G * 4));
-    CUDA_TRY(b->toff.ensure((N + 1) * 4)); CUDA_TRY(b->eoff.ensure((N + 1) * 4)); CUDA_TRY(b->corder.ensure(N * 4));
-    CUDA_TRY(b->tri.ensure(T * 12));
-    CUDA_TRY(b->slot_tri.ensure(S * 4));
-    CUDA_TRY(b->slot_edge.ensure(S * 4));
-    for (DBuf *e : {&b->edge_l, &b->edge_r, &b->edge_ta, &b->edge_tb}) CUDA_TRY(e->ensure(E * 4));
+    const size_t T = (size_t)z.tris + 1, E = (size_t)z.edges + 1, r = b->rsize(), d = sizeof(double);
     CUDA_TRY(b->ccx.ensure(T * d)); CUDA_TRY(b->ccy.ensure(T * d));
     for (DBuf *e : {&b->eL, &b->emlx, &b->emly, &b->emrx, &b->emry, &b->enx, &b->eny, &b->eqx, &b->eqy})
         CUDA_TRY(e->ensure(E * r));
     CUDA_TRY(b->F.ensure(4 * E * sizeof(double)));
     CUDA_TRY(b->ePM.ensure(4 * E * r));
     return RICH_OK;
-}
-
-// where an update writes (its rings to buffers m), as far as the arrays reach
-rich::MeshOutput mesh_output(const rich_batch *b, int m)
-{
-    rich::MeshOutput o{};
-    o.cell_ptr = b->cell_ptr[m].as<int32_t>();
-    o.slot_nb = b->slot_nb[m].as<int32_t>();
-    o.tri_off = b->toff.as<int32_t>();
-    o.edge_off = b->eoff.as<int32_t>();
-    o.cell_order = b->corder.as<int32_t>();
-    o.gx = b->gx.as<double>();
-    o.gy = b->gy.as<double>();
-    o.ghost_src = b->gsrc[m].as<int32_t>();
-    o.ghost_xf = b->gxf.as<int32_t>();
-    o.ghost_shift = b->gshift.as<int32_t>();
-    o.ghost_img = b->gimg[m].as<int32_t>();
-    const size_t r = b->rsize();
-    size_t e = std::min(b->F.cap / 32, b->ePM.cap / (4 * r));
-    for (const DBuf *k : {&b->edge_l, &b->edge_r, &b->edge_ta, &b->edge_tb}) e = std::min(e, k->cap / 4);
-    for (const DBuf *k : {&b->eL, &b->emlx, &b->emly, &b->emrx, &b->emry, &b->enx, &b->eny, &b->eqx, &b->eqy})
-        e = std::min(e, k->cap / r);
-    const size_t g = std::min({b->gx.cap / 8, b->gy.cap / 8, b->gsrc[m].cap / 4, b->gimg[m].cap / 4, b->gxf.cap / 4,
-                               b->gshift.cap / 4});
-    const size_t t = std::min({b->tri.cap / 12, b->ccx.cap / 8, b->ccy.cap / 8});
-    const size_t q = std::min({b->slot_nb[m].cap / 4, b->slot_tri.cap / 4, b->slot_edge.cap / 4});
-    auto i32 = [](size_t v) { return (int32_t)std::min<size_t>(v, INT32_MAX / 4); };
-    o.max = rich::MeshSizes{i32(g), i32(t), i32(e), i32(q)};
-    o.lists = mesh_lists(b);
-    return o;
 }
 
 rich::MeshArrays mesh_arrays(rich_batch *b, int q)
@@ -544,41 +466,78 @@ rich::MeshArrays mesh_arrays(rich_batch *b, int q)
     a.cell_inst = b->cell_inst.as<int32_t>();
     a.x = b->x[q].as<double>();
     a.y = b->y[q].as<double>();
-    a.cell_ptr = b->cell_ptr[b->mcur].as<int32_t>();
-    a.slot_nb = b->slot_nb[b->mcur].as<int32_t>();
-    a.ghost_src = b->gsrc[b->mcur].as<int32_t>();
-    a.ghost_img = b->gimg[b->mcur].as<int32_t>();
+    const rich::MeshStore &m = b->mesh[b->mcur];
+    a.cell_ptr = m.cell_ptr.as<int32_t>();
+    a.slot_nb = m.slot_nb.as<int32_t>();
+    a.ghost_src = m.ghost_src.as<int32_t>();
+    a.ghost_img = m.ghost_img.as<int32_t>();
     return a;
 }
 
-// After the update for the points in buffers q was waited for: the meshes of
-// the packed simulations on the device, as far as it made them.
+// Enqueue the update of the packed meshes for the points in buffers q, on the
+// mesh stream from where the batch's stream is now; join_update makes the
+// batch's stream continue after it.
+int start_update(rich_batch *b, int q)
+{
+    rich::MeshStream &u = b->mesh_stream;
+    CUDA_TRY(cudaEventRecord(u.moved, b->stream));
+    CUDA_TRY(cudaStreamWaitEvent(u.stream, u.moved, 0));
+    CUDA_TRY(b->updater.start(mesh_arrays(b, q), b->mesh[1 - b->mcur].output(0), u.stream));
+    CUDA_TRY(cudaEventRecord(u.done, u.stream));
+    return RICH_OK;
+}
+
+int join_update(rich_batch *b)
+{
+    CUDA_TRY(cudaStreamWaitEvent(b->stream, b->mesh_stream.done, 0));
+    return RICH_OK;
+}
+
+// The sweep stage by stage; with `update` the mesh update for the moved points
+// runs on the mesh stream beside the stages after the point motion.
+int run_staged(rich_batch *b, bool update)
+{
+    CUDA_TRY(cudaMemsetAsync(b->status.p, 0, b->status.cap, b->stream));
+    for (int k = 0; k < rich::NUM_STAGES; k++) {
+        b->launch(k, nullptr);
+        if (update && k == rich::K_ADVANCE) {
+            const int rc = start_update(b, 1 - b->cur);
+            if (rc) return rc;
+        }
+    }
+    CUDA_TRY(cudaGetLastError());
+    b->staged_launches++;
+    return RICH_OK;
+}
+
+// After the batch's stream was waited for: the meshes of the packed
+// simulations on the device, as far as the update made them.
 int finish_update(rich_batch *b, int q)
 {
     b->dev_mesh = b->dev_lists = false;
     const rich::MeshArrays a = mesh_arrays(b, q);
-    const int m = 1 - b->mcur;
+    rich::MeshStore &to = b->mesh[1 - b->mcur];
+    cudaStream_t st = b->mesh_stream.stream;
     rich::MeshResult r;
-    CUDA_TRY(b->updater.settle(a, mesh_output(b, m), r, b->stream));
+    CUDA_TRY(b->updater.settle(a, to.output(0), r, st));
     if (r.state == rich::MeshResult::kGrow) {
-        int rc = reserve_mesh(b, r.sizes);
-        if (!rc) rc = reserve_rings(b, m, r.sizes);
-        if (rc) return rc;
-        CUDA_TRY(b->updater.again(a, mesh_output(b, m), r, b->stream));
+        CUDA_TRY(to.reserve(a.n, r.sizes));
+        CUDA_TRY(b->updater.again(a, to.output(0), r, st));
     }
     if (r.state != rich::MeshResult::kDone || (r.bad && !r.flagged)) {
         b->updater.forget();
         return RICH_OK;
     }
     b->mesh_flag.assign(b->updater.flags(), b->updater.flags() + a.n_inst);
-    b->mcur = m;
+    b->mcur = 1 - b->mcur;
     b->nG = r.sizes.ghosts;
     b->nT = r.sizes.tris;
     b->nE = r.sizes.edges;
     b->nS = r.sizes.slots;
     b->dev_mesh = true;
     b->dev_lists = !r.flagged;
-    return reserve_rings(b, 1 - m, r.sizes);
+    CUDA_TRY(b->mesh[1 - b->mcur].reserve(a.n, r.sizes));
+    return reserve_geometry(b, r.sizes);
 }
 
 // The meshes of the simulations that go on, read back from the device into
@@ -591,14 +550,13 @@ int read_meshes(rich_batch *b)
         if (k == 0) return cudaSuccess;
         return cudaMemcpyAsync(v.data(), d.p, k * sizeof(v[0]), cudaMemcpyDeviceToHost, b->stream);
     };
-    const int m = b->mcur;
+    const rich::MeshStore &m = b->mesh[b->mcur];
     CUDA_TRY(down(b->h_dlx, b->x[b->cur], N)); CUDA_TRY(down(b->h_dly, b->y[b->cur], N));
-    CUDA_TRY(down(b->h_dptr, b->cell_ptr[m], N + 1)); CUDA_TRY(down(b->h_dnb, b->slot_nb[m], S));
-    CUDA_TRY(down(b->h_dtoff, b->toff, N + 1)); CUDA_TRY(down(b->h_deoff, b->eoff, N + 1));
-    CUDA_TRY(down(b->h_dorder, b->corder, N));
-    CUDA_TRY(down(b->h_dgx, b->gx, G)); CUDA_TRY(down(b->h_dgy, b->gy, G));
-    CUDA_TRY(down(b->h_dgsrc, b->gsrc[m], G)); CUDA_TRY(down(b->h_dgxf, b->gxf, G));
-    CUDA_TRY(down(b->h_dgshift, b->gshift, G)); CUDA_TRY(down(b->h_dgimg, b->gimg[m], G));
+    CUDA_TRY(down(b->h_dptr, m.cell_ptr, N + 1)); CUDA_TRY(down(b->h_dnb, m.slot_nb, S));
+    CUDA_TRY(down(b->h_dtoff, m.tri_off, N + 1)); CUDA_TRY(down(b->h_deoff, m.edge_off, N + 1));
+    CUDA_TRY(down(b->h_dgx, m.gx, G)); CUDA_TRY(down(b->h_dgy, m.gy, G));
+    CUDA_TRY(down(b->h_dgsrc, m.ghost_src, G)); CUDA_TRY(down(b->h_dgxf, m.ghost_xf, G));
+    CUDA_TRY(down(b->h_dgshift, m.ghost_shift, G)); CUDA_TRY(down(b->h_dgimg, m.ghost_img, G));
     CUDA_TRY(cudaStreamSynchronize(b->stream));
     // (ghosts follow their cells' order, so a simulation's are consecutive)
     std::vector<int64_t> g0(b->packed.size() + 1, (int64_t)G);
@@ -698,7 +656,7 @@ int batch_create(int32_t precision, int64_t max_cells, int32_t host_threads, Thr
     b->max_cells = max_cells;
     if (cudaStreamCreateWithFlags(&b->stream, cudaStreamNonBlocking) != cudaSuccess ||
         cudaEventCreate(&b->ev0) != cudaSuccess || cudaEventCreate(&b->ev1) != cudaSuccess ||
-        cudaEventCreate(&b->ev2) != cudaSuccess || cudaEventCreate(&b->ev3) != cudaSuccess) {
+        cudaEventCreate(&b->ev2) != cudaSuccess || b->mesh_stream.create() != cudaSuccess) {
         delete b;
         return fail(RICH_ECUDA, "stream or event creation failed");
     }
@@ -896,7 +854,8 @@ int pack_step(rich_batch *b, const std::vector<BatchSim *> &list, double &t1, do
     if ((rc = ensure_device(b))) return rc;
     const rich::MeshSizes z{(int32_t)go, (int32_t)to, (int32_t)eo, (int32_t)so};
     b->updater.forget();
-    if ((rc = reserve_mesh(b, z)) || (rc = reserve_rings(b, 0, z)) || (rc = reserve_rings(b, 1, z))) return rc;
+    for (rich::MeshStore &m : b->mesh) CUDA_TRY(m.reserve((int32_t)N, z));
+    if ((rc = reserve_geometry(b, z))) return rc;
     const int nxt = 1 - b->cur;
     if (!same_layout && n_old > 0) {
         // regather the conserved state of continuing simulations into the other
@@ -917,31 +876,25 @@ int pack_step(rich_batch *b, const std::vector<BatchSim *> &list, double &t1, do
     CUDA_TRY(upload(b->y[b->cur], b->h_y, b->stream));
     CUDA_TRY(upload(b->cell_inst, b->h_cell_inst, b->stream));
     CUDA_TRY(upload(b->perm_dev, b->h_perm, b->stream));
-    CUDA_TRY(upload(b->gx, b->h_gx, b->stream));
-    CUDA_TRY(upload(b->gy, b->h_gy, b->stream));
-    CUDA_TRY(upload(b->gsrc[b->mcur], b->h_gsrc, b->stream));
-    CUDA_TRY(upload(b->gimg[b->mcur], b->h_gimg, b->stream));
-    CUDA_TRY(upload(b->gxf, b->h_gxf, b->stream));
-    CUDA_TRY(upload(b->cell_ptr[b->mcur], b->h_cell_ptr, b->stream));
-    CUDA_TRY(upload(b->corder, b->h_corder, b->stream));
-    CUDA_TRY(upload(b->slot_nb[b->mcur], b->h_slot_nb, b->stream));
-    CUDA_TRY(upload(b->toff, b->h_toff, b->stream));
-    CUDA_TRY(upload(b->eoff, b->h_eoff, b->stream));
-    CUDA_TRY(upload(b->gshift, b->h_gshift, b->stream));
+    rich::MeshStore &d = b->mesh[b->mcur];
+    CUDA_TRY(upload(d.gx, b->h_gx, b->stream));
+    CUDA_TRY(upload(d.gy, b->h_gy, b->stream));
+    CUDA_TRY(upload(d.ghost_src, b->h_gsrc, b->stream));
+    CUDA_TRY(upload(d.ghost_img, b->h_gimg, b->stream));
+    CUDA_TRY(upload(d.ghost_xf, b->h_gxf, b->stream));
+    CUDA_TRY(upload(d.ghost_shift, b->h_gshift, b->stream));
+    CUDA_TRY(upload(d.cell_ptr, b->h_cell_ptr, b->stream));
+    CUDA_TRY(upload(d.cell_order, b->h_corder, b->stream));
+    CUDA_TRY(upload(d.slot_nb, b->h_slot_nb, b->stream));
+    CUDA_TRY(upload(d.tri_off, b->h_toff, b->stream));
+    CUDA_TRY(upload(d.edge_off, b->h_eoff, b->stream));
     CUDA_TRY(upload(b->instp, b->h_inst, b->stream));
     // the packed triangle and edge lists, checked before any kernel reads them
     {
         CUDA_TRY(b->listbad.ensure(8));
-        rich::MeshLists l = mesh_lists(b);
-        l.n = (int32_t)N;
+        rich::MeshLists l = d.lists((int32_t)N, 0);
         l.cell_inst = b->cell_inst.as<int32_t>();
         l.inst = b->instp.as<rich::InstParams>();
-        l.cell_ptr = b->cell_ptr[b->mcur].as<int32_t>();
-        l.slot_nb = b->slot_nb[b->mcur].as<int32_t>();
-        l.tri_off = b->toff.as<int32_t>();
-        l.edge_off = b->eoff.as<int32_t>();
-        l.ghost_src = b->gsrc[b->mcur].as<int32_t>();
-        l.ghost_shift = b->gshift.as<int32_t>();
         l.bad = b->listbad.as<int32_t>();
         CUDA_TRY(cudaMemsetAsync(l.bad, 0, 4, b->stream));
         CUDA_TRY(rich::launch_lists(l, b->stream));
@@ -1000,16 +953,17 @@ int rich_batch_step(rich_batch *b, rich_step_info *info)
     }
     if (b->packed.empty()) return RICH_OK;
     const double t3 = now_ms();
-    // 6. the sweep over every cell of every simulation, then the mesh update
-    //    for the moved points (one wait for both)
+    // 6. the sweep over every cell of every simulation, and the mesh update for
+    //    the moved points (staged: beside the last stages; one wait for both)
     const std::vector<BatchSim *> ok = b->packed;
     const size_t N = (size_t)b->n_packed;
+    const bool update = (int64_t)N >= rich::kMeshUpdateMin && (int64_t)N <= rich::kMeshUpdateMax;
     const LaunchShape shape = pick_shape(b);
     CUDA_TRY(cudaEventRecord(b->ev0, b->stream));
     if (shape.persistent) {
         rc = b->precision == RICH_FP32_SPLIT ? run_persistent<float>(b, shape.block) : run_persistent<double>(b, shape.block);
     } else {
-        rc = run_staged(b);
+        rc = run_staged(b, update);
     }
     if (rc) return rc;
     CUDA_TRY(cudaEventRecord(b->ev1, b->stream));
@@ -1025,23 +979,23 @@ int rich_batch_step(rich_batch *b, rich_step_info *info)
             b->barrier_timeouts++;
             b->graph_note = "persistent sweep barrier timed out; staged launches used";
             CUDA_TRY(cudaEventRecord(b->ev0, b->stream));
-            if ((rc = run_staged(b))) return rc;
+            if ((rc = run_staged(b, false))) return rc;
             CUDA_TRY(cudaEventRecord(b->ev1, b->stream));
         }
     }
-    const bool update = (int64_t)N >= rich::kMeshUpdateMin && (int64_t)N <= rich::kMeshUpdateMax;
+    if (update && shape.persistent && (rc = start_update(b, 1 - b->cur))) return rc;
+    if (update && (rc = join_update(b))) return rc;
     CUDA_TRY(cudaEventRecord(b->ev2, b->stream));
-    if (update)
-        CUDA_TRY(b->updater.start(mesh_arrays(b, 1 - b->cur), mesh_output(b, 1 - b->mcur), b->stream));
-    CUDA_TRY(cudaEventRecord(b->ev3, b->stream));
     CUDA_TRY(cudaMemcpyAsync(b->dt_back(), b->dtout.p, ok.size() * 8, cudaMemcpyDeviceToHost, b->stream));
     CUDA_TRY(cudaMemcpyAsync(b->status_back(), b->status.p, ok.size() * 4, cudaMemcpyDeviceToHost, b->stream));
     CUDA_TRY(cudaStreamSynchronize(b->stream));
     float ms = 0.0f;
     cudaEventElapsedTime(&ms, b->ev0, b->ev1);
-    record_timing(b, shape, ms);
+    // (what the update takes beyond the end of the sweep; the launch shapes are
+    // compared by the whole)
     float up_ms = 0.0f;
-    cudaEventElapsedTime(&up_ms, b->ev2, b->ev3);
+    cudaEventElapsedTime(&up_ms, b->ev1, b->ev2);
+    record_timing(b, shape, ms + up_ms);
     // 7. per-simulation bookkeeping; a failed step keeps that simulation's old state
     const int nxt2 = 1 - b->cur;
     const double tnow = now_ms();

@@ -854,6 +854,92 @@ cudaError_t launch_lists(const MeshLists &l, cudaStream_t st)
     return cudaGetLastError();
 }
 
+cudaError_t MeshStore::reserve(int32_t n, const MeshSizes &z)
+{
+    const size_t i4 = sizeof(int32_t), N = (size_t)n, G = (size_t)z.ghosts + 1, T = (size_t)z.tris + 1;
+    const size_t E = (size_t)z.edges + 1, S = (size_t)z.slots + 1;
+    cudaError_t e = cudaSuccess;
+    auto need = [&](DBuf &b, size_t bytes) {
+        if (e == cudaSuccess) e = b.ensure(bytes);
+    };
+    need(cell_ptr, (N + 1) * i4);
+    need(tri_off, (N + 1) * i4);
+    need(edge_off, (N + 1) * i4);
+    need(cell_order, N * i4);
+    for (DBuf *b : {&slot_nb, &slot_tri, &slot_edge}) need(*b, S * i4);
+    need(tri, 3 * T * i4);
+    for (DBuf *b : {&edge_l, &edge_r, &edge_ta, &edge_tb}) need(*b, E * i4);
+    for (DBuf *b : {&gx, &gy}) need(*b, G * sizeof(double));
+    for (DBuf *b : {&ghost_src, &ghost_xf, &ghost_shift, &ghost_img}) need(*b, G * i4);
+    return e;
+}
+
+MeshLists MeshStore::lists(int32_t n, int32_t periodic) const
+{
+    MeshLists l{};
+    l.n = n;
+    l.periodic = periodic;
+    l.cell_ptr = cell_ptr.as<int32_t>();
+    l.slot_nb = slot_nb.as<int32_t>();
+    l.tri_off = tri_off.as<int32_t>();
+    l.edge_off = edge_off.as<int32_t>();
+    l.ghost_src = ghost_src.as<int32_t>();
+    l.ghost_shift = ghost_shift.as<int32_t>();
+    l.tri = tri.as<int32_t>();
+    l.slot_tri = slot_tri.as<int32_t>();
+    l.slot_edge = slot_edge.as<int32_t>();
+    l.edge_l = edge_l.as<int32_t>();
+    l.edge_r = edge_r.as<int32_t>();
+    l.edge_ta = edge_ta.as<int32_t>();
+    l.edge_tb = edge_tb.as<int32_t>();
+    return l;
+}
+
+MeshOutput MeshStore::output(int32_t periodic) const
+{
+    MeshOutput o{};
+    o.cell_ptr = cell_ptr.as<int32_t>();
+    o.slot_nb = slot_nb.as<int32_t>();
+    o.tri_off = tri_off.as<int32_t>();
+    o.edge_off = edge_off.as<int32_t>();
+    o.cell_order = cell_order.as<int32_t>();
+    o.gx = gx.as<double>();
+    o.gy = gy.as<double>();
+    o.ghost_src = ghost_src.as<int32_t>();
+    o.ghost_xf = ghost_xf.as<int32_t>();
+    o.ghost_shift = ghost_shift.as<int32_t>();
+    o.ghost_img = ghost_img.as<int32_t>();
+    const size_t i4 = sizeof(int32_t);
+    auto room = [](size_t entries) { return (int32_t)std::min<size_t>(entries, INT32_MAX / 4); };
+    o.max.slots = room(std::min({slot_nb.cap, slot_tri.cap, slot_edge.cap}) / i4);
+    o.max.edges = room(std::min({edge_l.cap, edge_r.cap, edge_ta.cap, edge_tb.cap}) / i4);
+    o.max.tris = room(tri.cap / (3 * i4));
+    o.max.ghosts = room(std::min({gx.cap / 8, gy.cap / 8, ghost_src.cap / i4, ghost_xf.cap / i4, ghost_shift.cap / i4,
+                                  ghost_img.cap / i4}));
+    o.lists = lists(0, periodic);
+    return o;
+}
+
+cudaError_t MeshStream::create()
+{
+    // of the highest priority: its small kernels take the slots that blocks of
+    // the sweep's large grids leave
+    int least = 0, greatest = 0;
+    cudaError_t e = cudaDeviceGetStreamPriorityRange(&least, &greatest);
+    if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&stream, cudaStreamNonBlocking, greatest);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&moved, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventCreate(&done);
+    return e;
+}
+
+MeshStream::~MeshStream()
+{
+    if (stream) cudaStreamSynchronize(stream);
+    if (moved) cudaEventDestroy(moved);
+    if (done) cudaEventDestroy(done);
+    if (stream) cudaStreamDestroy(stream);
+}
+
 #define MU_TRY(e)                               \
     do {                                        \
         const cudaError_t err_ = (e);           \

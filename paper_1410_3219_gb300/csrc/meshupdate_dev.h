@@ -60,6 +60,43 @@ struct MeshOutput {
     MeshLists lists;  // (tri .. edge_tb and periodic; the rest is filled in)
 };
 
+// The connectivity of one mesh in device memory, as host builds are uploaded
+// to it and updates write it.
+struct MeshStore {
+    DBuf cell_ptr, slot_nb, slot_tri, slot_edge, tri, tri_off, edge_off, cell_order;
+    DBuf edge_l, edge_r, edge_ta, edge_tb, gx, gy, ghost_src, ghost_xf, ghost_shift, ghost_img;
+    // Room for a mesh of these sizes.  Nothing enqueued may still use the
+    // arrays: those that grow are reallocated.
+    cudaError_t reserve(int32_t n, const MeshSizes &z);
+    // where an update writes, with the room there is
+    MeshOutput output(int32_t periodic) const;
+    // the list builder's arguments for the mesh held (its lists from its rings)
+    MeshLists lists(int32_t n, int32_t periodic) const;
+    // the sweep's view of it
+    template <class R> void describe(SweepParams<R> &p, const MeshSizes &z) const
+    {
+        p.ng = z.ghosts;
+        p.T = z.tris;
+        p.E = z.edges;
+        p.S = z.slots;
+        p.gx = gx.as<double>(); p.gy = gy.as<double>();
+        p.tri = tri.as<int32_t>(); p.cell_ptr = cell_ptr.as<int32_t>(); p.cell_order = cell_order.as<int32_t>();
+        p.slot_nb = slot_nb.as<int32_t>(); p.slot_tri = slot_tri.as<int32_t>(); p.slot_edge = slot_edge.as<int32_t>();
+        p.edge_l = edge_l.as<int32_t>(); p.edge_r = edge_r.as<int32_t>();
+        p.edge_ta = edge_ta.as<int32_t>(); p.edge_tb = edge_tb.as<int32_t>();
+        p.ghost_src = ghost_src.as<int32_t>(); p.ghost_xf = ghost_xf.as<int32_t>();
+    }
+};
+
+// The stream that updates run on beside the rest of a sweep, and the events
+// that order the two.
+struct MeshStream {
+    cudaStream_t stream = nullptr;
+    cudaEvent_t moved = nullptr, done = nullptr;
+    cudaError_t create();
+    ~MeshStream();
+};
+
 struct MeshResult {
     // kDone: the mesh and its lists are written (but for the meshes of
     // simulations with flags()); kGrow: an array is too small for `sizes`;

@@ -88,9 +88,10 @@ struct rich_sim {
     double *hy() const { return hpts.as<double>() + n; }
     rich::MeshWork mw;  // (edge list built on the device: see tessellate)
     rich::HostMesh hm;  // the last mesh the host built
-    // The mesh on the device (buffers mcur of the arrays that an update reads
-    // while it writes the new ones): its sizes, and whether an update may
-    // start from its rings
+    // The mesh on the device (mesh[mcur]; an update writes the other while the
+    // rest of the sweep reads this one): its sizes, and whether an update may
+    // start from it
+    rich::MeshStore mesh[2];
     int mcur = 0;
     rich::MeshSizes msz;
     bool mesh_on_device = false;
@@ -98,7 +99,7 @@ struct rich_sim {
     int64_t updates = 0;   // meshes made by it
     rich::HBuf back;       // the step's dt and status, and the list builder's flag
     DBuf mesh_inst;        // the box and mesh_params
-    cudaEvent_t ev_up = nullptr;
+    rich::MeshStream mesh_stream;
     std::unique_ptr<rich::ThreadPool> pool;  // host threads of the tile-parallel tessellation
     rich_sim() { mw.host_edges = false; }
     double t = 0.0;
@@ -119,14 +120,10 @@ struct rich_sim {
     double last_dt = 0.0;
     // device buffers
     DBuf x[3], y[3], U[3];
-    DBuf A, o, W, cs, g, gl, alpha, w, tess, corder, initW, rounding, p64, psrc;
+    DBuf A, o, W, cs, g, gl, alpha, w, tess, initW, rounding, p64, psrc;
     bool diagnostics = true;
-    DBuf gx, gy, gxf, gshift, eoff, toff;
-    DBuf cell_ptr[2], slot_nb[2], gsrc[2], gimg[2];
     DBuf perm_dev, unperm;  // caller index of each internal cell; reordered state for reads
-    DBuf tri, ccx, ccy;
-    DBuf slot_tri, slot_edge;
-    DBuf edge_l, edge_r, edge_ta, edge_tb, eL, emlx, emly, emrx, emry, enx, eny, eqx, eqy, F, ePM;
+    DBuf ccx, ccy, eL, emlx, emly, emrx, emry, enx, eny, eqx, eqy, F, ePM;
     DBuf scal;   // dtmin bits, dt, status
     DBuf instp;  // one InstParams
     rich::InstParams inst_host{};  // staging for the parameter upload
@@ -135,7 +132,6 @@ struct rich_sim {
     {
         if (ev0) cudaEventDestroy(ev0);
         if (ev1) cudaEventDestroy(ev1);
-        if (ev_up) cudaEventDestroy(ev_up);
         for (cudaEvent_t e : kev)
             if (e) cudaEventDestroy(e);
         if (own_stream) cudaStreamDestroy(own_stream);
@@ -150,10 +146,7 @@ struct rich_sim {
         p.diagnostics = diagnostics ? 1 : 0;
         p.motion = 1;
         p.n = n;
-        p.ng = msz.ghosts;
-        p.T = msz.tris;
-        p.E = msz.edges;
-        p.S = msz.slots;
+        mesh[mcur].describe(p, msz);
         // extrapolated fluxes: [cur] -> [1 - cur].  Time-centred: [cur] -> [2]
         // by half a step, then primitives and mesh of [2], update of [cur]
         // into [1 - cur]
@@ -161,12 +154,6 @@ struct rich_sim {
         p.x = x[src].as<double>(); p.y = y[src].as<double>();
         p.xn = x[dst].as<double>(); p.yn = y[dst].as<double>();
         p.x0 = x[cur].as<double>(); p.y0 = y[cur].as<double>();
-        p.gx = gx.as<double>(); p.gy = gy.as<double>();
-        p.tri = tri.as<int32_t>(); p.cell_ptr = cell_ptr[mcur].as<int32_t>(); p.cell_order = corder.as<int32_t>();
-        p.slot_nb = slot_nb[mcur].as<int32_t>(); p.slot_tri = slot_tri.as<int32_t>(); p.slot_edge = slot_edge.as<int32_t>();
-        p.edge_l = edge_l.as<int32_t>(); p.edge_r = edge_r.as<int32_t>();
-        p.edge_ta = edge_ta.as<int32_t>(); p.edge_tb = edge_tb.as<int32_t>();
-        p.ghost_src = gsrc[mcur].as<int32_t>(); p.ghost_xf = gxf.as<int32_t>();
         p.ccx = ccx.as<double>(); p.ccy = ccy.as<double>(); p.A = A.as<double>();
         p.eL = eL.as<R>(); p.emlx = emlx.as<R>(); p.emly = emly.as<R>();
         p.emrx = emrx.as<R>(); p.emry = emry.as<R>();
@@ -232,12 +219,13 @@ struct rich_sim {
         a.inst = mesh_inst.as<rich::InstParams>();
         a.x = x[q].as<double>();
         a.y = y[q].as<double>();
-        a.cell_ptr = cell_ptr[mcur].as<int32_t>();
-        a.slot_nb = slot_nb[mcur].as<int32_t>();
-        a.ghost_src = gsrc[mcur].as<int32_t>();
-        a.ghost_img = gimg[mcur].as<int32_t>();
+        a.cell_ptr = mesh[mcur].cell_ptr.as<int32_t>();
+        a.slot_nb = mesh[mcur].slot_nb.as<int32_t>();
+        a.ghost_src = mesh[mcur].ghost_src.as<int32_t>();
+        a.ghost_img = mesh[mcur].ghost_img.as<int32_t>();
         return a;
     }
+    int32_t periodic() const { return cfg.boundary == RICH_BC_PERIODIC ? 1 : 0; }
 };
 
 namespace {
@@ -279,78 +267,17 @@ int build_mesh(rich_sim *s, rich_step_info *info)
     return rc ? mesh_rc(rc) : RICH_OK;
 }
 
-// Room for the rings of a mesh of these sizes in buffers m, and for the rest
-// of it.  Nothing on the stream may still use the arrays: those that grow are
-// reallocated.
-int reserve_rings(rich_sim *s, int m, const rich::MeshSizes &z)
+// Room for the geometry of a mesh of these sizes (which every sweep computes
+// afresh; nothing enqueued may still use the arrays).
+int reserve_geometry(rich_sim *s, const rich::MeshSizes &z)
 {
-    const size_t i4 = sizeof(int32_t), G = (size_t)z.ghosts + 1;
-    CUDA_TRY(s->cell_ptr[m].ensure(((size_t)s->n + 1) * i4));
-    CUDA_TRY(s->slot_nb[m].ensure(((size_t)z.slots + 1) * i4));
-    CUDA_TRY(s->gsrc[m].ensure(G * i4)); CUDA_TRY(s->gimg[m].ensure(G * i4));
-    return RICH_OK;
-}
-
-int reserve_mesh(rich_sim *s, const rich::MeshSizes &z)
-{
-    const size_t i4 = sizeof(int32_t), d = sizeof(double), r = s->rsize();
-    const size_t N = (size_t)s->n, G = (size_t)z.ghosts + 1, T = (size_t)z.tris + 1, E = (size_t)z.edges + 1;
-    const size_t S = (size_t)z.slots + 1;
-    CUDA_TRY(s->gx.ensure(G * d)); CUDA_TRY(s->gy.ensure(G * d));
-    CUDA_TRY(s->gxf.ensure(G * i4)); CUDA_TRY(s->gshift.ensure(G * i4));
-    CUDA_TRY(s->toff.ensure((N + 1) * i4)); CUDA_TRY(s->eoff.ensure((N + 1) * i4)); CUDA_TRY(s->corder.ensure(N * i4));
-    CUDA_TRY(s->tri.ensure(3 * T * i4));
-    CUDA_TRY(s->slot_tri.ensure(S * i4));
-    CUDA_TRY(s->slot_edge.ensure(S * i4));
-    for (DBuf *b : {&s->edge_l, &s->edge_r, &s->edge_ta, &s->edge_tb}) CUDA_TRY(b->ensure(E * i4));
+    const size_t d = sizeof(double), r = s->rsize(), T = (size_t)z.tris + 1, E = (size_t)z.edges + 1;
     CUDA_TRY(s->ccx.ensure(T * d)); CUDA_TRY(s->ccy.ensure(T * d));
     for (DBuf *b : {&s->eL, &s->emlx, &s->emly, &s->emrx, &s->emry, &s->enx, &s->eny, &s->eqx, &s->eqy})
         CUDA_TRY(b->ensure(E * r));
     CUDA_TRY(s->F.ensure(4 * E * d));
     CUDA_TRY(s->ePM.ensure(4 * E * r));
     return RICH_OK;
-}
-
-rich::MeshLists mesh_lists(const rich_sim *s)
-{
-    rich::MeshLists l{};
-    l.periodic = s->cfg.boundary == RICH_BC_PERIODIC ? 1 : 0;
-    l.tri = s->tri.as<int32_t>();
-    l.slot_tri = s->slot_tri.as<int32_t>();
-    l.slot_edge = s->slot_edge.as<int32_t>();
-    l.edge_l = s->edge_l.as<int32_t>(); l.edge_r = s->edge_r.as<int32_t>();
-    l.edge_ta = s->edge_ta.as<int32_t>(); l.edge_tb = s->edge_tb.as<int32_t>();
-    return l;
-}
-
-// where an update writes (its rings to buffers m), as far as the arrays reach
-rich::MeshOutput mesh_output(const rich_sim *s, int m)
-{
-    rich::MeshOutput o{};
-    o.cell_ptr = s->cell_ptr[m].as<int32_t>();
-    o.slot_nb = s->slot_nb[m].as<int32_t>();
-    o.tri_off = s->toff.as<int32_t>();
-    o.edge_off = s->eoff.as<int32_t>();
-    o.cell_order = s->corder.as<int32_t>();
-    o.gx = s->gx.as<double>();
-    o.gy = s->gy.as<double>();
-    o.ghost_src = s->gsrc[m].as<int32_t>();
-    o.ghost_xf = s->gxf.as<int32_t>();
-    o.ghost_shift = s->gshift.as<int32_t>();
-    o.ghost_img = s->gimg[m].as<int32_t>();
-    const size_t r = s->rsize();
-    size_t e = std::min(s->F.cap / 32, s->ePM.cap / (4 * r));
-    for (const DBuf *b : {&s->edge_l, &s->edge_r, &s->edge_ta, &s->edge_tb}) e = std::min(e, b->cap / 4);
-    for (const DBuf *b : {&s->eL, &s->emlx, &s->emly, &s->emrx, &s->emry, &s->enx, &s->eny, &s->eqx, &s->eqy})
-        e = std::min(e, b->cap / r);
-    size_t g = std::min({s->gx.cap / 8, s->gy.cap / 8, s->gsrc[m].cap / 4, s->gimg[m].cap / 4, s->gxf.cap / 4,
-                         s->gshift.cap / 4});
-    const size_t t = std::min({s->tri.cap / 12, s->ccx.cap / 8, s->ccy.cap / 8});
-    const size_t q = std::min({s->slot_nb[m].cap / 4, s->slot_tri.cap / 4, s->slot_edge.cap / 4});
-    auto i32 = [](size_t v) { return (int32_t)std::min<size_t>(v, INT32_MAX / 4); };
-    o.max = rich::MeshSizes{i32(g), i32(t), i32(e), i32(q)};
-    o.lists = mesh_lists(s);
-    return o;
 }
 
 void report_sizes(const rich_sim *s, rich_step_info *info)
@@ -369,32 +296,26 @@ int upload_mesh(rich_sim *s, rich_step_info *info)
 {
     const double t2 = now_ms();
     const rich::HostMesh &m = s->hm;
-    const int q = s->mcur;
     s->mesh_on_device = false;
     s->updater.forget();
     s->msz = rich::MeshSizes{m.g, m.n_tris, m.n_edges, (int32_t)m.slot_nb.size()};
-    int rc = reserve_mesh(s, s->msz);
-    for (int k = 0; k < 2 && rc == RICH_OK; k++) rc = reserve_rings(s, k, s->msz);
+    // (the other buffers too: the first update then has room)
+    for (rich::MeshStore &k : s->mesh) CUDA_TRY(k.reserve(s->n, s->msz));
+    int rc = reserve_geometry(s, s->msz);
     if (rc != RICH_OK) return rc;
-    CUDA_TRY(upload(s->gx, m.gx, s->stream));
-    CUDA_TRY(upload(s->gy, m.gy, s->stream));
-    CUDA_TRY(upload(s->gsrc[q], m.ghost_src, s->stream));
-    CUDA_TRY(upload(s->gimg[q], m.ghost_img, s->stream));
-    CUDA_TRY(upload(s->gxf, m.ghost_xf, s->stream));
-    CUDA_TRY(upload(s->cell_ptr[q], m.cell_ptr, s->stream));
-    CUDA_TRY(upload(s->corder, m.cell_order, s->stream));
-    CUDA_TRY(upload(s->slot_nb[q], m.slot_nb, s->stream));
-    CUDA_TRY(upload(s->toff, m.tri_off, s->stream));
-    CUDA_TRY(upload(s->eoff, m.edge_off, s->stream));
-    CUDA_TRY(upload(s->gshift, m.ghost_shift, s->stream));
-    rich::MeshLists l = mesh_lists(s);
-    l.n = s->n;
-    l.cell_ptr = s->cell_ptr[q].as<int32_t>();
-    l.slot_nb = s->slot_nb[q].as<int32_t>();
-    l.tri_off = s->toff.as<int32_t>();
-    l.edge_off = s->eoff.as<int32_t>();
-    l.ghost_src = s->gsrc[q].as<int32_t>();
-    l.ghost_shift = s->gshift.as<int32_t>();
+    rich::MeshStore &d = s->mesh[s->mcur];
+    CUDA_TRY(upload(d.gx, m.gx, s->stream));
+    CUDA_TRY(upload(d.gy, m.gy, s->stream));
+    CUDA_TRY(upload(d.ghost_src, m.ghost_src, s->stream));
+    CUDA_TRY(upload(d.ghost_img, m.ghost_img, s->stream));
+    CUDA_TRY(upload(d.ghost_xf, m.ghost_xf, s->stream));
+    CUDA_TRY(upload(d.ghost_shift, m.ghost_shift, s->stream));
+    CUDA_TRY(upload(d.cell_ptr, m.cell_ptr, s->stream));
+    CUDA_TRY(upload(d.cell_order, m.cell_order, s->stream));
+    CUDA_TRY(upload(d.slot_nb, m.slot_nb, s->stream));
+    CUDA_TRY(upload(d.tri_off, m.tri_off, s->stream));
+    CUDA_TRY(upload(d.edge_off, m.edge_off, s->stream));
+    rich::MeshLists l = d.lists(s->n, s->periodic());
     l.bad = reinterpret_cast<int32_t *>(s->scal.as<char>() + 24);
     CUDA_TRY(cudaMemsetAsync(l.bad, 0, sizeof(int32_t), s->stream));
     CUDA_TRY(rich::launch_lists(l, s->stream));
@@ -413,18 +334,28 @@ bool can_update(const rich_sim *s)
     return s->mesh_on_device && s->n >= rich::kMeshUpdateMin && s->n <= rich::kMeshUpdateMax;
 }
 
-// Enqueue the update of the mesh for the points in buffers q.  It reads the
-// rings of the present mesh and overwrites its lists.
+// Enqueue the update of the mesh for the points in buffers q, on the mesh
+// stream after ev (recorded on the handle's stream once those points are
+// there); the handle's stream continues after it (join_update).
 int start_update(rich_sim *s, int q)
 {
-    s->tess_current = false;
-    CUDA_TRY(s->updater.start(s->mesh_arrays(q), mesh_output(s, 1 - s->mcur), s->stream));
+    rich::MeshStream &u = s->mesh_stream;
+    CUDA_TRY(cudaEventRecord(u.moved, s->stream));
+    CUDA_TRY(cudaStreamWaitEvent(u.stream, u.moved, 0));
+    CUDA_TRY(s->updater.start(s->mesh_arrays(q), s->mesh[1 - s->mcur].output(s->periodic()), u.stream));
+    CUDA_TRY(cudaEventRecord(u.done, u.stream));
     return RICH_OK;
 }
 
-// After the update was waited for: its mesh made the current one (keep), or
-// dropped; where it could not be made nothing is current, and the host has to
-// build it (the next update may still start from the present rings).
+int join_update(rich_sim *s)
+{
+    CUDA_TRY(cudaStreamWaitEvent(s->stream, s->mesh_stream.done, 0));
+    return RICH_OK;
+}
+
+// After the handle's stream was waited for: the updated mesh made the current
+// one (keep), or dropped.  Where it could not be made the present mesh stays
+// on the device, and the host has to build the points' own.
 int finish_update(rich_sim *s, int q, bool keep, rich_step_info *info)
 {
     if (!keep) {
@@ -432,26 +363,26 @@ int finish_update(rich_sim *s, int q, bool keep, rich_step_info *info)
         return RICH_OK;
     }
     const rich::MeshArrays a = s->mesh_arrays(q);
-    const int m = 1 - s->mcur;
+    rich::MeshStore &to = s->mesh[1 - s->mcur];
+    cudaStream_t st = s->mesh_stream.stream;
     rich::MeshResult r;
-    CUDA_TRY(s->updater.settle(a, mesh_output(s, m), r, s->stream));
+    CUDA_TRY(s->updater.settle(a, to.output(s->periodic()), r, st));
     if (r.state == rich::MeshResult::kGrow) {
-        int rc = reserve_mesh(s, r.sizes);
-        if (rc == RICH_OK) rc = reserve_rings(s, m, r.sizes);
-        if (rc != RICH_OK) return rc;
-        CUDA_TRY(s->updater.again(a, mesh_output(s, m), r, s->stream));
+        CUDA_TRY(to.reserve(s->n, r.sizes));
+        CUDA_TRY(s->updater.again(a, to.output(s->periodic()), r, st));
     }
     if (r.state != rich::MeshResult::kDone || r.flagged || r.bad) {
         s->updater.forget();
         return RICH_OK;
     }
-    s->mcur = m;
+    s->mcur = 1 - s->mcur;
     s->msz = r.sizes;
     s->updates++;
     s->tess_current = true;
     report_sizes(s, info);
-    // (the next update's rings have as much room as these)
-    return reserve_rings(s, 1 - m, r.sizes);
+    // (the next update's buffers have as much room as these)
+    CUDA_TRY(s->mesh[1 - s->mcur].reserve(s->n, r.sizes));
+    return reserve_geometry(s, r.sizes);
 }
 
 // a0 for the current points: the mesh on the device updated, or else built on
@@ -462,8 +393,9 @@ int tessellate(rich_sim *s, rich_step_info *info, bool fetch_points)
     if (fetch_points && can_update(s)) {
         const double t0 = now_ms();
         const int q = s->pts();
-        int rc = start_update(s, q);
-        if (rc != RICH_OK) return rc;
+        int rc;
+        if ((rc = start_update(s, q)) != RICH_OK || (rc = join_update(s)) != RICH_OK) return rc;
+        s->tess_current = false;
         CUDA_TRY(cudaStreamSynchronize(s->stream));
         if ((rc = finish_update(s, q, true, info)) != RICH_OK) return rc;
         if (info) info->tess_ms += now_ms() - t0;
@@ -589,7 +521,7 @@ static int create_sim(const rich_config *cfg, int64_t n, const double *x, const 
         return bail(fail(RICH_ECUDA, "stream creation failed"));
     s->stream = s->own_stream;
     if (cudaEventCreate(&s->ev0) != cudaSuccess || cudaEventCreate(&s->ev1) != cudaSuccess ||
-        cudaEventCreate(&s->ev_up) != cudaSuccess)
+        s->mesh_stream.create() != cudaSuccess)
         return bail(fail(RICH_ECUDA, "event creation failed"));
     if ((rc = alloc_cells(s)) != RICH_OK) return bail(rc);
     if (s->x[0].ensure(n * 8) != cudaSuccess) return bail(fail(RICH_ENOMEM, "device points"));
@@ -691,7 +623,7 @@ int rich_tessellate(rich_sim *s, rich_step_info *info)
     return tessellate(s, info, true);
 }
 
-static int launch_sweep(rich_sim *s, double t_end)
+static int launch_sweep(rich_sim *s, double t_end, bool update)
 {
     rich::Range range("rich sweep launch (a1-a9)");
     if (!s) return fail(RICH_EINVAL, "NULL handle");
@@ -704,6 +636,10 @@ static int launch_sweep(rich_sim *s, double t_end)
     for (int k = 0; k < rich::NUM_STAGES; k++) {
         if (s->profiling) CUDA_TRY(cudaEventRecord(s->kev[k], s->stream));
         s->launch(k, nullptr);
+        if (update && k == rich::K_ADVANCE) {
+            int rc = start_update(s, s->next_pts());
+            if (rc != RICH_OK) return rc;
+        }
     }
     if (s->profiling) CUDA_TRY(cudaEventRecord(s->kev[rich::NUM_STAGES], s->stream));
     CUDA_TRY(cudaGetLastError());
@@ -712,7 +648,7 @@ static int launch_sweep(rich_sim *s, double t_end)
     return RICH_OK;
 }
 
-int rich_sweep(rich_sim *s, double t_end) { return launch_sweep(s, t_end); }
+int rich_sweep(rich_sim *s, double t_end) { return launch_sweep(s, t_end, false); }
 
 int rich_sync(rich_sim *s, rich_step_info *info)
 {
@@ -773,30 +709,28 @@ int rich_sync(rich_sim *s, rich_step_info *info)
     return RICH_OK;
 }
 
-// One sweep of rich_step: the update of the mesh for the moved points follows
-// the sweep on the stream, so one wait serves both.  A failed sweep drops the
-// updated mesh (and the lists it overwrote); a mesh that the update cannot
-// make is left to the next tessellation.
+// One sweep of rich_step: the update of the mesh for the moved points runs on
+// the mesh stream beside the gradients, fluxes and update, from when the
+// points are there (those stages leave the memory pipes and the FP32 and
+// integer units idle, which the update lives on), and one wait serves both.
+// A failed sweep drops the updated mesh; one that the update cannot make is
+// left to the next tessellation.
 static int step_sweep(rich_sim *s, double t_end, rich_step_info *info)
 {
-    int rc = launch_sweep(s, t_end);
-    if (rc != RICH_OK) return rc;
     const int q = s->next_pts();
     const bool update = can_update(s);
-    if (update) {
-        if ((rc = start_update(s, q)) != RICH_OK) return rc;
-        CUDA_TRY(cudaEventRecord(s->ev_up, s->stream));
-    }
+    int rc = launch_sweep(s, t_end, update);
+    if (rc != RICH_OK) return rc;
+    if (update && (rc = join_update(s)) != RICH_OK) return rc;
     rc = rich_sync(s, info);
     if (!update) return rc;
-    if (rc != RICH_OK) {
-        finish_update(s, q, false, nullptr);
-        return rc;
-    }
+    const double t0 = now_ms();
+    const int urc = finish_update(s, q, rc == RICH_OK, info);
+    // (what the update takes beyond the end of the sweep)
     float ms = 0.0f;
-    cudaEventElapsedTime(&ms, s->ev1, s->ev_up);
-    if (info) info->tess_ms += ms;
-    return finish_update(s, q, true, info);
+    if (info && cudaEventElapsedTime(&ms, s->ev1, s->mesh_stream.done) == cudaSuccess && ms > 0.0f) info->tess_ms += ms;
+    if (info) info->tess_ms += now_ms() - t0;
+    return rc != RICH_OK ? rc : urc;
 }
 
 int rich_step(rich_sim *s, int32_t max_steps, double t_end, rich_step_info *info)
@@ -1229,14 +1163,15 @@ int rich_mesh_check(rich_sim *s, int64_t *mismatched, int64_t *updates)
         if (k == 0) return cudaSuccess;
         return cudaMemcpyAsync(v.data(), b.p, k * sizeof(v[0]), cudaMemcpyDeviceToHost, s->stream);
     };
-    const int q = s->pts(), m = s->mcur;
+    const int q = s->pts();
+    const rich::MeshStore &m = s->mesh[s->mcur];
     CUDA_TRY(down(x, s->x[q], N)); CUDA_TRY(down(y, s->y[q], N));
-    CUDA_TRY(down(d.cell_ptr, s->cell_ptr[m], N + 1)); CUDA_TRY(down(d.slot_nb, s->slot_nb[m], S));
-    CUDA_TRY(down(d.tri_off, s->toff, N + 1)); CUDA_TRY(down(d.edge_off, s->eoff, N + 1));
-    CUDA_TRY(down(d.cell_order, s->corder, N));
-    CUDA_TRY(down(d.gx, s->gx, G)); CUDA_TRY(down(d.gy, s->gy, G));
-    CUDA_TRY(down(d.ghost_src, s->gsrc[m], G)); CUDA_TRY(down(d.ghost_xf, s->gxf, G));
-    CUDA_TRY(down(d.ghost_shift, s->gshift, G)); CUDA_TRY(down(d.ghost_img, s->gimg[m], G));
+    CUDA_TRY(down(d.cell_ptr, m.cell_ptr, N + 1)); CUDA_TRY(down(d.slot_nb, m.slot_nb, S));
+    CUDA_TRY(down(d.tri_off, m.tri_off, N + 1)); CUDA_TRY(down(d.edge_off, m.edge_off, N + 1));
+    CUDA_TRY(down(d.cell_order, m.cell_order, N));
+    CUDA_TRY(down(d.gx, m.gx, G)); CUDA_TRY(down(d.gy, m.gy, G));
+    CUDA_TRY(down(d.ghost_src, m.ghost_src, G)); CUDA_TRY(down(d.ghost_xf, m.ghost_xf, G));
+    CUDA_TRY(down(d.ghost_shift, m.ghost_shift, G)); CUDA_TRY(down(d.ghost_img, m.ghost_img, G));
     CUDA_TRY(cudaStreamSynchronize(s->stream));
     rich::MeshWork work;
     work.host_edges = false;
