@@ -40,6 +40,49 @@ static __device__ __forceinline__ double sqrt_nonneg(double x)
 }
 static __device__ __forceinline__ float sqrt_nonneg(float x) { return sqrtf(x); }
 
+// num / den as num y (1 + e + e^2), the same reciprocal series without the
+// reciprocal's own rounding: four FP64 instructions.
+static __device__ __forceinline__ double quotient(double num, double den)
+{
+    const unsigned ex = ((unsigned)__double2hiint(den) >> 20) & 0x7ffu;
+    if (ex - 2u > 2040u) return num / den;
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(den));
+    const double e = fma(-den, y, 1.0), q = num * y;
+    return fma(q, fma(e, e, e), q);
+}
+
+// x / 2 on the integer pipe: one off the exponent field.  Zeros, infinities
+// and NaNs stay as they are, and so do magnitudes below 2^-1020.
+static __device__ __forceinline__ double halved(double x)
+{
+    const int hi = __double2hiint(x);
+    const bool scales = ((unsigned)hi & 0x7ff00000u) - 0x00300000u < 0x7fc00000u;
+    return __hiloint2double(scales ? hi - 0x00100000 : hi, __double2loint(x));
+}
+
+// FP32 estimates of FP64 values for decisions that FP64 repeats where FP32
+// cannot take them: |x| with its mantissa cut to 24 bits (relative error below
+// 2^-23), on the integer pipe, for an exponent field within 100 of 1023.
+static __device__ __forceinline__ bool estimable(double x)
+{
+    return (((unsigned)__double2hiint(x) >> 20) & 0x7ffu) - 923u <= 200u;
+}
+static __device__ __forceinline__ float magnitude(double x)
+{
+    return __uint_as_float((__funnelshift_l((unsigned)__double2loint(x), (unsigned)__double2hiint(x), 3) - 0xc0000000u) &
+                           0x7fffffffu);
+}
+// the same with the sign; magnitudes below 2^-126 become 0, those of 2^128
+// and above (and NaN) infinite
+static __device__ __forceinline__ float estimate(double x)
+{
+    const unsigned hi = (unsigned)__double2hiint(x), e = (hi >> 20) & 0x7ffu;
+    unsigned u = (__funnelshift_l((unsigned)__double2loint(x), hi, 3) - 0xc0000000u) & 0x7fffffffu;
+    u = e < 897u ? 0u : (e > 1150u ? 0x7f800000u : u);
+    return __uint_as_float(u | (hi & 0x80000000u));
+}
+
 // Conversions between FP64 and FP32 on the integer pipe (F2F conversions
 // issue on the FP64 pipe on this part).  Both give the hardware's results
 // bit for bit: d2f_rn rounds to nearest even, f2d widens exactly.  Normal

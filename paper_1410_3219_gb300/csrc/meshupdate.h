@@ -353,15 +353,49 @@ RICH_MU_SLOW int circle_slow(int32_t *flags, double ax, double ay, double bx, do
     }
 }
 
+// Positions for the slow predicates.  In a periodic box every cell of a
+// triangle or quadrilateral has to come to the same answer, but an image's
+// coordinates are rounded, differently from each cell's own frame: near-ties
+// (a drifting lattice is made of them) would then be decided differently on
+// the two sides of the boundary.  So the points are taken in the frame of the
+// smallest cell among them, one of the frames the host builder tests them in.
+RICH_HD inline double shifted(double v, double lo, double hi, int k)
+{
+    const double L = hi - lo;
+    return k == 0 ? v : (k > 0 ? v + (k > 1 ? L + L : L) : v - (k < -1 ? L + L : L));
+}
+
+RICH_HD inline void common_frame(const Frame &f, const int32_t *ref, int n, double *x, double *y)
+{
+    int32_t least = ref[0];
+    for (int k = 1; k < n; k++) least = (ref[k] >> 4) < (least >> 4) ? ref[k] : least;
+    const int a0 = (least & 15) % 3, b0 = (least & 15) / 3;
+    for (int k = 0; k < n; k++) {
+        x[k] = shifted(f.m->x[ref[k] >> 4], f.x0, f.x1, (ref[k] & 15) % 3 - a0);
+        y[k] = shifted(f.m->y[ref[k] >> 4], f.y0, f.y1, (ref[k] & 15) / 3 - b0);
+    }
+}
+
+// orientation of (cell, a, b)
 RICH_HD inline int orient_slow(const Frame &f, const Point &a, const Point &b)
 {
-    return orient_slow(f.flags, f.xi, f.yi, a.x, a.y, b.x, b.y);
+    double x[3] = {f.xi, a.x, b.x}, y[3] = {f.yi, a.y, b.y};
+    if (f.periodic) {
+        const int32_t ref[3] = {f.i * 16 + 4, a.ref, b.ref};
+        common_frame(f, ref, 3, x, y);
+    }
+    return orient_slow(f.flags, x[0], y[0], x[1], y[1], x[2], y[2]);
 }
 
 // d against the circle of the counter-clockwise (cell, a, b)
 RICH_HD inline int circle_slow(const Frame &f, const Point &a, const Point &b, const Point &d)
 {
-    return circle_slow(f.flags, f.xi, f.yi, a.x, a.y, b.x, b.y, d.x, d.y);
+    double x[4] = {f.xi, a.x, b.x, d.x}, y[4] = {f.yi, a.y, b.y, d.y};
+    if (f.periodic) {
+        const int32_t ref[4] = {f.i * 16 + 4, a.ref, b.ref, d.ref};
+        common_frame(f, ref, 4, x, y);
+    }
+    return circle_slow(f.flags, x[0], y[0], x[1], y[1], x[2], y[2], x[3], y[3]);
 }
 
 // > 0 when d is inside the circumcircle of the counter-clockwise (cell, a, b).

@@ -347,6 +347,33 @@ __device__ __forceinline__ double stage_cell_geometry(const SweepParams<R> &p, c
         }
     }
     p.w[i] = Vec2<R>{wx, wy};
+    if (sizeof(R) == sizeof(double)) {
+        // The Courant step costs 22 FP64 instructions; only a cell whose FP32
+        // estimate is within 4e-6 of its warp's smallest and of the smallest
+        // step found so far can hold the minimum, and only such warps take it
+        // (the estimate is within 1e-6; values beyond FP32's range always do).
+        // A moving cell's speed against its mesh point is zero, or chi c_s
+        // where the rounding velocity is on.
+        const double ma = (double)W.y, mb = (double)W.z;
+        bool known = estimable(A) && estimable((double)cs) && A > 0.0 && (double)cs > 0.0;
+        float speed = ip.motion == 0 ? (rounding ? ip.chi_f * magnitude((double)cs) : 0.0f) : 0.0f;
+        if (ip.motion != 0) {
+            const float fa = estimate(ma), fb = estimate(mb);
+            speed = sqrtf(fa * fa + fb * fb);
+        }
+        // (beyond 2^60 a square would overflow, and chi is the caller's)
+        known = known && speed < 1.15e18f;
+        const float est = sqrtf(magnitude(A) * 0.318309886f) / (magnitude((double)cs) + speed);
+        const unsigned act = __activemask();
+        unsigned least = known ? __float_as_uint(est) : 0x7f800000u;
+        // (lanes of one simulation share the warp's smallest; in a mixed warp
+        // each lane stands alone)
+        const int32_t lead = __shfl_sync(act, my_inst, __ffs(act) - 1);
+        if (__all_sync(act, my_inst == lead)) least = __reduce_min_sync(act, least);
+        const float far = estimate(__longlong_as_double((long long)__ldcg(p.dtmin_bits + my_inst)));
+        const float limit = fminf(__uint_as_float(least), far) * 1.000004f;
+        if (known && est > limit) return DBL_MAX;
+    }
     // Courant step R_i / (c_s + |v - w|), R_i = sqrt(A/pi) = (A/pi) rsqrt(A/pi)
     const R Api = to_R<R>(A) * (R(1) / R(M_PI));
     const R Rad = Api * rsqrt(Api);
@@ -410,6 +437,253 @@ template <class R> struct GlobalSlots {
         return p.p64[src_of(p, p.slot_nb[s], xf)];
     }
 };
+
+// TESS (Eq. 6): psi_ij = max(theta (phi_j - phi_i)/dphi, 0); the smallest
+// ratio is found by cross-multiplication, divided once
+template <class R, class Slots>
+__device__ __forceinline__ void tess_limit(const SweepParams<R> &p, int32_t lo, int32_t hi, const Slots &sl, const R Wi[4],
+                                           const R g[8], R ox, R oy, R Lmin, R theta, R an[4], R ad[4], bool lim[4])
+{
+    R bn[4] = {0, 0, 0, 0}, bd[4] = {0, 0, 0, 0};  // smallest |N|/|D| so far (bd == 0: none)
+    bool zero[4] = {false, false, false, false};
+    for (int32_t s = lo; s < hi; s++) {
+        if (!nonneg_less(Lmin, sl.L(s))) continue;
+        R mx, my;
+        sl.midpoint(s, mx, my);
+        const R offx = mx - ox, offy = my - oy;
+        const Vec4<R> Wv = sl.W(s);
+        const R Wj[4] = {Wv.x, Wv.y, Wv.z, Wv.w};
+#pragma unroll
+        for (int v = 0; v < 4; v++) {
+            R dphi = g[2 * v] * offx + g[2 * v + 1] * offy;
+            if (dphi == R(0)) continue;
+            R num = Wj[v] - Wi[v];
+            if (!(num * dphi > R(0))) { zero[v] = true; continue; }
+            R a_n = fabs(num), a_d = fabs(dphi);
+            if (bd[v] == R(0) || a_n * bd[v] < bn[v] * a_d) { bn[v] = a_n; bd[v] = a_d; }
+        }
+    }
+#pragma unroll
+    for (int v = 0; v < 4; v++) {
+        // alpha = 0, or min(1, theta bn / bd)
+        const R tn = theta * bn[v];
+        if (zero[v]) { an[v] = R(0); lim[v] = true; }
+        else if (bd[v] > R(0) && tn < bd[v]) { an[v] = tn; ad[v] = bd[v]; lim[v] = true; }
+    }
+}
+
+template <class R> __device__ __forceinline__ double step_dt(const SweepParams<R> &p, int32_t inst)
+{
+    const InstParams &ip = p.inst[inst];
+    // the second sweep of the time-centred scheme keeps the first one's dt
+    if (ip.phase == 2) return __ldcg(p.dt_out + inst);
+    // read through L2: in the persistent sweep the minimum was reset and then
+    // reduced with atomics earlier in the same launch, and a line of it may
+    // still sit stale in this SM's L1
+    double dt = ip.cfl * __longlong_as_double((long long)__ldcg(p.dtmin_bits + inst));
+    return nonneg_less(ip.remaining, dt) ? ip.remaining : dt;
+}
+
+// a3-a4 in FP64: as stage_cell_gradient below, with what an FP64 pipe of one
+// warp instruction per 16 clocks asks for (the FP32 and integer units idle
+// beside it): FP32 estimates take the two kinds of decisions that need no FP64
+// value, and FP64 takes over where they cannot.
+//  - The pressure-ratio test of the switch per neighbour.
+//  - The limiter (AREPO): which edge and sign bind each variable, so that FP64
+//    evaluates one extrapolated difference per limited variable (and none for
+//    an unlimited one) instead of four per edge; ties within the estimates'
+//    error go through every edge in FP64.
+// The prediction's cell terms come out folded: with the edge's midpoint m
+// (from the generator) and velocity w_f, Eq. 2 and the half-step prediction of
+// a side read C + g.(m + hdt w_f) with C = phi - g.(o + hdt v) - hdt S.  That
+// takes 12 FP64 instructions more per cell and 12 fewer per edge, and the flux
+// loads C in place of phi, o and S.
+// (Per cell of six slots: 204 FP64 instructions before, about 160 now.)
+template <class R, class Slots>
+__device__ __forceinline__ void stage_cell_gradient_fp64(const SweepParams<R> &p, int32_t i, int32_t lo, int32_t hi,
+                                                         const Slots &sl)
+{
+    const int32_t inst = inst_of(p, i);
+    const InstParams &ip = p.inst[inst];
+    const Vec4<R> W4 = p.W[i];
+    const double Wi[4] = {W4.x, W4.y, W4.z, W4.w};
+    double acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+    double Bx = 0, By = 0;
+    Extremes<double> ext[4];
+#pragma unroll
+    for (int v = 0; v < 4; v++) ext[v].init(Wi[v]);
+    bool shock = false;
+    const double A = p.A[i];
+    const double dp = ip.delta_p;
+    const float dpf = (float)dp;
+    // R_i = sqrt(A/pi) and 1/A from one reciprocal square root
+    const double Api = A * (1.0 / M_PI);
+    const double rR = rsqrt(Api);
+    const double Rad = Api * rR;
+    // point contacts: edges of at most 1e-9 sqrt(A)
+    const double Lmin = 1.7724538509055160273e-9 * Rad;
+    const float pif = magnitude(Wi[3]);
+    const bool pi_ok = estimable(Wi[3]);
+    float reach = 0.0f;  // the farthest midpoint (largest coordinate)
+    for (int32_t s = lo; s < hi; s++) {
+        const double L = sl.L(s);
+        double Ax, Ay, bx, by;
+        sl.weights(s, Ax, Ay, bx, by);
+        Bx += bx;
+        By += by;
+        const Vec4<R> Wv = sl.W(s);
+        const double Wj[4] = {Wv.x, Wv.y, Wv.z, Wv.w};
+#pragma unroll
+        for (int v = 0; v < 4; v++) {
+            acc[2 * v] = fma(Wj[v], Ax, acc[2 * v]);
+            acc[2 * v + 1] = fma(Wj[v], Ay, acc[2 * v + 1]);
+        }
+        if (nonneg_less(Lmin, L)) {
+#pragma unroll
+            for (int v = 0; v < 4; v++) ext[v].add(Wj[v]);
+            // min(p_i, p_j) < delta_p max(p_i, p_j)
+            const float pjf = magnitude(Wj[3]);
+            const float pmin = fminf(pif, pjf), pmax = fmaxf(pif, pjf) * dpf;
+            if (pi_ok && estimable(Wj[3]) && fabsf(pmin - pmax) > 1e-6f * pmax) {
+                if (pmin < pmax) shock = true;
+            } else {
+                const bool jl = nonneg_less(Wj[3], Wi[3]);
+                if (nonneg_less(jl ? Wj[3] : Wi[3], dp * (jl ? Wi[3] : Wj[3]))) shock = true;
+            }
+        }
+    }
+#pragma unroll
+    for (int v = 0; v < 4; v++) {
+        acc[2 * v] = fma(Wi[v], Bx, acc[2 * v]);
+        acc[2 * v + 1] = fma(Wi[v], By, acc[2 * v + 1]);
+    }
+    const double invA = rR * rR * (1.0 / M_PI);
+    double g[8];
+#pragma unroll
+    for (int c = 0; c < 8; c++) g[c] = acc[c] * invA;
+    // Eq. 7: -div v > delta_v c_s / R_i, as (delta_v c_s) < -(div v) R_i
+    if (key_less(ip.delta_v * p.cs[i], flip((g[2] + g[5]) * Rad, 0x8000000000000000ull))) shock = true;
+    const bool use_tess = ip.limiter == 2 || (ip.limiter == 0 && shock);
+    const Vec2<R> oi = p.o[i];
+    // alpha_v = an[v] / ad[v] (1 where the variable is not limited): the
+    // smallest of 1, (phi_max - phi_i)/dphi over the largest dphi of the
+    // edges, and (phi_i - phi_min)/-dphi over the smallest
+    double an[4] = {1, 1, 1, 1}, ad[4] = {1, 1, 1, 1};
+    bool lim[4] = {false, false, false, false};
+    if (!use_tess) {
+        const float oxf = estimate(oi.x), oyf = estimate(oi.y);
+        float gf[8], up[4] = {0, 0, 0, 0}, dn[4] = {0, 0, 0, 0};
+        int32_t su[4] = {lo, lo, lo, lo}, sd[4] = {lo, lo, lo, lo};
+#pragma unroll
+        for (int c = 0; c < 8; c++) gf[c] = estimate(g[c]);
+        // runners-up, to see ties
+        float up2[4] = {0, 0, 0, 0}, dn2[4] = {0, 0, 0, 0};
+        for (int32_t s = lo; s < hi; s++) {
+            if (!nonneg_less(Lmin, sl.L(s))) continue;
+            double mx, my;
+            sl.midpoint(s, mx, my);
+            const float fx = estimate(mx) - oxf, fy = estimate(my) - oyf;
+            reach = fmaxf(reach, fmaxf(fabsf(fx), fabsf(fy)));
+#pragma unroll
+            for (int v = 0; v < 4; v++) {
+                const float d = gf[2 * v] * fx + gf[2 * v + 1] * fy;
+                if (d > up[v]) { up2[v] = up[v]; up[v] = d; su[v] = s; }
+                else up2[v] = fmaxf(up2[v], d);
+                if (d < dn[v]) { dn2[v] = dn[v]; dn[v] = d; sd[v] = s; }
+                else dn2[v] = fminf(dn2[v], d);
+            }
+        }
+        reach += fmaxf(fabsf(oxf), fabsf(oyf));
+#pragma unroll
+        for (int v = 0; v < 4; v++) {
+            // an estimate's error: offsets within 3e-7 of reach, gradients
+            // within 2^-23, two products and a sum
+            const float gx = fabsf(gf[2 * v]), gy = fabsf(gf[2 * v + 1]), err = 1e-6f * (gx + gy) * reach;
+            const double n1 = ext[v].max() - Wi[v], n2 = Wi[v] - ext[v].min();
+            const float f1 = estimate(n1), f2 = estimate(n2);
+            // (products far from FP32's smallest numbers; a gradient of
+            // exactly zero is exact)
+            const bool known = reach > 1e-12f && (gx > 1e-22f || dkey0(g[2 * v]) == 0) &&
+                               (gy > 1e-22f || dkey0(g[2 * v + 1]) == 0);
+            // a side is free when its numerator clears its largest difference
+            const bool free1 = f1 >= (up[v] + err) * 1.000001f, free2 = f2 >= (err - dn[v]) * 1.000001f;
+            if (known && free1 && free2) continue;
+            if (known && ((up[v] > err && dkey0(n1) == 0) || (dn[v] < -err && dkey0(n2) == 0))) {
+                // an extremum: nothing may be added on that side
+                an[v] = 0.0;
+                lim[v] = true;
+                continue;
+            }
+            // which side binds: the smaller ratio, by cross-multiplication
+            const float c1 = f1 * (-dn[v]), c2 = f2 * up[v], ce = 1e-5f * (fabsf(c1) + fabsf(c2)) + err * (f1 + f2);
+            const bool one = known && up[v] > err && (free2 || (dn[v] < -err && c1 < c2 - ce));
+            const bool two = known && dn[v] < -err && (free1 || (up[v] > err && c2 < c1 - ce));
+            // (an infinite or NaN estimate fails these; a tie between edges or
+            // sides, or a difference of the size of its error, goes on)
+            if ((one && up2[v] < up[v] - 2.0f * err) || (two && dn2[v] > dn[v] + 2.0f * err)) {
+                double mx, my;
+                sl.midpoint(one ? su[v] : sd[v], mx, my);
+                const double k = fma(g[2 * v], oi.x, g[2 * v + 1] * oi.y);
+                const double d = flip(fma(g[2 * v], mx, fma(g[2 * v + 1], my, -k)), one ? 0ull : 0x8000000000000000ull);
+                const double n = one ? n1 : n2;
+                if (dkey0(d) > 0 && nonneg_less(n, d)) {
+                    an[v] = n;
+                    ad[v] = d;
+                    lim[v] = true;
+                }
+                continue;
+            }
+            // every edge in FP64
+            const double k = fma(g[2 * v], oi.x, g[2 * v + 1] * oi.y);
+            Extremes<double> dex;
+            dex.init(0.0);
+            for (int32_t s = lo; s < hi; s++) {
+                if (!nonneg_less(Lmin, sl.L(s))) continue;
+                double mx, my;
+                sl.midpoint(s, mx, my);
+                dex.add(fma(g[2 * v], mx, fma(g[2 * v + 1], my, -k)));
+            }
+            const double d1 = dex.max(), d2 = -dex.min();
+            const bool b1 = dex.max_positive() && nonneg_less(n1, d1);
+            const bool b2 = dex.min_negative() && nonneg_less(n2, d2);
+            if (b1 || b2) {
+                const bool use1 = b1 && (!b2 || nonneg_less(n1 * d2, n2 * d1));
+                an[v] = use1 ? n1 : n2;
+                ad[v] = use1 ? d1 : d2;
+                lim[v] = true;
+            }
+        }
+    } else {
+        tess_limit(p, lo, hi, sl, Wi, g, (double)oi.x, (double)oi.y, Lmin, ip.theta, an, ad, lim);
+    }
+    double alpha[4];
+#pragma unroll
+    for (int v = 0; v < 4; v++) alpha[v] = lim[v] ? an[v] * recip(ad[v]) : 1.0;
+    double lg[8];
+#pragma unroll
+    for (int c = 0; c < 8; c++) lg[c] = alpha[c >> 1] * g[c];
+    p.gl[2 * i] = Vec4<R>{lg[0], lg[1], lg[2], lg[3]};
+    p.gl[2 * i + 1] = Vec4<R>{lg[4], lg[5], lg[6], lg[7]};
+    {
+        // half the step's dt where edge states advance in time (the point
+        // motion, which records dt, runs beside this stage in the persistent
+        // sweep)
+        const double hdt = ip.phase == 0 ? halved(step_dt(p, inst)) : 0.0;
+        const double sx = fma(hdt, Wi[1], (double)oi.x), sy = fma(hdt, Wi[2], (double)oi.y);
+        const double hd = hdt * (lg[2] + lg[5]), hr = hdt * recip(Wi[0]), gp = ip.gamma * Wi[3];
+        const double C0 = fma(-Wi[0], hd, fma(-lg[1], sy, fma(-lg[0], sx, Wi[0])));
+        const double C1 = fma(-hr, lg[6], fma(-lg[3], sy, fma(-lg[2], sx, Wi[1])));
+        const double C2 = fma(-hr, lg[7], fma(-lg[5], sy, fma(-lg[4], sx, Wi[2])));
+        const double C3 = fma(-gp, hd, fma(-lg[7], sy, fma(-lg[6], sx, Wi[3])));
+        p.psrc[i] = Vec4<R>{C0, C1, C2, C3};
+    }
+    if (p.diagnostics) {
+        p.g[2 * i] = Vec4<R>{g[0], g[1], g[2], g[3]};
+        p.g[2 * i + 1] = Vec4<R>{g[4], g[5], g[6], g[7]};
+        p.alpha[i] = Vec4<R>{alpha[0], alpha[1], alpha[2], alpha[3]};
+        p.tess[i] = use_tess ? 1 : 0;
+    }
+}
 
 // a3-a4: Green-Gauss gradient (Eq. 1), limiter with the shock switch
 // (Eqs. 3-8), and the cell terms of the half-step prediction, for cell i
@@ -524,32 +798,7 @@ __device__ __forceinline__ void stage_cell_gradient(const SweepParams<R> &p, int
                 }
             }
         } else {
-            R bn[4] = {0, 0, 0, 0}, bd[4] = {0, 0, 0, 0};  // smallest |N|/|D| so far (bd == 0: none)
-            bool zero[4] = {false, false, false, false};
-            for (int32_t s = lo; s < hi; s++) {
-                if (!nonneg_less(Lmin, sl.L(s))) continue;
-                R mx, my;
-                sl.midpoint(s, mx, my);
-                const R offx = mx - ox, offy = my - oy;
-                const Vec4<R> Wv = sl.W(s);
-                const R Wj[4] = {Wv.x, Wv.y, Wv.z, Wv.w};
-#pragma unroll
-                for (int v = 0; v < 4; v++) {
-                    R dphi = g[2 * v] * offx + g[2 * v + 1] * offy;
-                    if (dphi == R(0)) continue;
-                    R num = Wj[v] - Wi[v];
-                    if (!(num * dphi > R(0))) { zero[v] = true; continue; }
-                    R a_n = fabs(num), a_d = fabs(dphi);
-                    if (bd[v] == R(0) || a_n * bd[v] < bn[v] * a_d) { bn[v] = a_n; bd[v] = a_d; }
-                }
-            }
-#pragma unroll
-            for (int v = 0; v < 4; v++) {
-                // alpha = 0, or min(1, theta bn / bd)
-                const R tn = inst_value<R>(ip.theta, ip.theta_f) * bn[v];
-                if (zero[v]) { an[v] = R(0); lim[v] = true; }
-                else if (bd[v] > R(0) && tn < bd[v]) { an[v] = tn; ad[v] = bd[v]; lim[v] = true; }
-            }
+            tess_limit(p, lo, hi, sl, Wi, g, ox, oy, Lmin, inst_value<R>(ip.theta, ip.theta_f), an, ad, lim);
         }
         // the cell's five quotients (alpha of each variable, 1/rho for the
         // prediction terms), each through one refined reciprocal
@@ -577,6 +826,16 @@ __device__ __forceinline__ void stage_cell_gradient(const SweepParams<R> &p, int
     }
 }
 
+// (each precision its own stage)
+__device__ __forceinline__ void cell_gradient(const SweepParams<double> &p, int32_t i)
+{
+    stage_cell_gradient_fp64(p, i, p.cell_ptr[i], p.cell_ptr[i + 1], GlobalSlots<double>{p});
+}
+__device__ __forceinline__ void cell_gradient(const SweepParams<float> &p, int32_t i)
+{
+    stage_cell_gradient(p, i, p.cell_ptr[i], p.cell_ptr[i + 1], GlobalSlots<float>{p});
+}
+
 // launched in blocks of 128 threads; six blocks per SM cap the FP64 build at
 // 80 registers (from 94, with a few spilled to L1), 24 warps instead of 20;
 // nine hold the FP32 build's 56 registers, 36 warps, which hide more of its
@@ -593,20 +852,8 @@ template <class R> __global__ void __launch_bounds__(128, sizeof(R) == 4 ? 9 : 6
     int32_t k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k < p.n) {
         const int32_t i = sizeof(R) == sizeof(double) ? cell_at(p, k) : k;
-        stage_cell_gradient(p, i, p.cell_ptr[i], p.cell_ptr[i + 1], GlobalSlots<R>{p});
+        cell_gradient(p, i);
     }
-}
-
-template <class R> __device__ __forceinline__ double step_dt(const SweepParams<R> &p, int32_t inst)
-{
-    const InstParams &ip = p.inst[inst];
-    // the second sweep of the time-centred scheme keeps the first one's dt
-    if (ip.phase == 2) return __ldcg(p.dt_out + inst);
-    // read through L2: in the persistent sweep the minimum was reset and then
-    // reduced with atomics earlier in the same launch, and a line of it may
-    // still sit stale in this SM's L1
-    double dt = ip.cfl * __longlong_as_double((long long)__ldcg(p.dtmin_bits + inst));
-    return nonneg_less(ip.remaining, dt) ? ip.remaining : dt;
 }
 
 // The step's dt in the stages after the point motion, which records it
@@ -683,6 +930,97 @@ template <class R> __device__ __forceinline__ void hllc(R gam, R igm1, const R L
     F[2] = F[0] * tK;
 }
 
+// a7 in FP64: as stage_edge_flux below, with 98 FP64 instructions per edge
+// instead of 132.  The sides' states come from the cells' folded terms
+// (stage_cell_gradient_fp64); only the normal velocity is taken relative to
+// the edge, and only side K's tangential velocity is formed, in the lab frame.
+// With the contact (or, beyond the outer waves, side K's own) speed S relative
+// to the edge, density f, pressure P and internal energy density ei, and
+// V = S + w_n in the lab frame, the flux through the moving edge is
+//   mass f S, normal momentum f S V + P, tangential momentum f S T,
+//   energy S ei + P V + f S (V^2 + T^2)/2,
+// the edge-frame HLLC flux boosted back (the star state of Toro,
+// rho* = m_K/(S_K - S), p* = p_K + m_K (S - u_K), with the kinetic parts of
+// its energy put together: ei* = p_K (igm1 (S_K - u_K) + S - u_K)/(S_K - S) +
+// rho* (S - u_K)^2/2).
+template <class R> __device__ __forceinline__ void stage_edge_flux_fp64(const SweepParams<R> &p, int32_t e)
+{
+    const int32_t l = p.edge_l[e];
+    const int32_t li = inst_of(p, l);
+    const InstParams &ip = p.inst[li];
+    const double hdt = ip.phase == 0 ? halved(recorded_dt(p, li)) : 0.0;
+    int32_t xf;
+    const int32_t k = src_of(p, p.edge_r[e], xf);
+    const unsigned long long mx = (xf & 1) ? 0x8000000000000000ull : 0ull;
+    const unsigned long long my = (xf & 2) ? 0x8000000000000000ull : 0ull;
+    const unsigned long long mxy = mx ^ my;
+    const Vec2<R> wl = p.w[l], wk = p.w[k];
+    const double nx = p.enx[e], ny = p.eny[e];
+    // velocity of the perpendicular bisector at the edge midpoint
+    const double wrx = flip(wk.x, mx), wry = flip(wk.y, my);
+    const double dwc = fma(wrx - wl.x, (double)p.eqx[e], (wry - wl.y) * p.eqy[e]);
+    const double wfx = fma(-dwc, nx, halved(wl.x + wrx)), wfy = fma(-dwc, ny, halved(wl.y + wry));
+    const double wn = fma(wfx, nx, wfy * ny);
+    double sL[4], sR[4];
+    {
+        const double ax = fma(hdt, wfx, (double)p.emlx[e]), ay = fma(hdt, wfy, (double)p.emly[e]);
+        const Vec4<R> C = p.psrc[l], g0 = p.gl[2 * l], g1 = p.gl[2 * l + 1];
+        sL[0] = fma(g0.x, ax, fma(g0.y, ay, C.x));
+        sL[1] = fma(g0.z, ax, fma(g0.w, ay, C.y));
+        sL[2] = fma(g1.x, ax, fma(g1.y, ay, C.z));
+        sL[3] = fma(g1.z, ax, fma(g1.w, ay, C.w));
+    }
+    {
+        // a mirrored source: each derivative takes the flip of its axis,
+        // velocity components also the flip of their own axis
+        const double ax = fma(hdt, wfx, (double)p.emrx[e]), ay = fma(hdt, wfy, (double)p.emry[e]);
+        const Vec4<R> C = p.psrc[k], g0 = p.gl[2 * k], g1 = p.gl[2 * k + 1];
+        sR[0] = fma(flip(g0.x, mx), ax, fma(flip(g0.y, my), ay, C.x));
+        sR[1] = fma(g0.z, ax, fma(flip(g0.w, mxy), ay, flip(C.y, mx)));
+        sR[2] = fma(flip(g1.x, mxy), ax, fma(g1.y, ay, flip(C.z, my)));
+        sR[3] = fma(flip(g1.z, mx), ax, fma(flip(g1.w, my), ay, C.w));
+    }
+    const double uL = fma(sL[1], nx, fma(sL[2], ny, -wn)), uR = fma(sR[1], nx, fma(sR[2], ny, -wn));
+    const double rL = sL[0], rR = sR[0], pL = sL[3], pR = sR[3];
+    // c = sqrt(gamma p / rho) = gamma p / sqrt(gamma p rho)
+    const double gam = ip.gamma, gpL = gam * pL, gpR = gam * pR;
+    const double cL = gpL * rsqrt(gpL * rL), cR = gpR * rsqrt(gpR * rR);
+    // Davis speeds, min / max chosen through integer keys
+    const double aL = uL - cL, aR = uR - cR, bL = uL + cL, bR = uR + cR;
+    const double SL = key_less(aR, aL) ? aR : aL, SR = key_less(bL, bR) ? bR : bL;
+    const bool supL = key_nonneg(SL), supR = !supL && key_nonpos(SR), sub = !(supL || supR);
+    // m_K = rho_K (S_K - u_K): m_L < 0 < m_R, so the contact speed
+    // S* = num / den has den = m_L - m_R < 0 and S* >= 0 exactly when num <= 0
+    const double dL = SL - uL, dR = SR - uR, mL = rL * dL, mR = rR * dR;
+    const double num = fma(-uR, mR, fma(uL, mL, pR - pL)), den = mL - mR;
+    const bool useL = supL || (sub && key_nonpos(num));
+    const double rK = useL ? rL : rR, uK = useL ? uL : uR, pK = useL ? pL : pR;
+    const double T = fma(useL ? sL[2] : sR[2], nx, -((useL ? sL[1] : sR[1]) * ny));
+    const double igm1 = ip.igm1;
+    double S = uK, f = rK, P = pK, ei;
+    if (sub) {
+        const double dK = useL ? dL : dR, mK = useL ? mL : mR;
+        S = quotient(num, den);
+        const double dS = S - uK, inv = recip(dK - dS);
+        f = mK * inv;
+        P = fma(mK, dS, pK);
+        ei = fma(pK * fma(igm1, dK, dS), inv, halved(f * dS) * dS);
+    } else {
+        ei = pK * igm1;
+    }
+    const double L = p.eL[e], V = S + wn, LP = L * P;
+    if (xf && k == l) {
+        // a wall: the cell faces its own mirror image; only the normal
+        // pressure flux remains (see stage_edge_flux)
+        const double Fn = fma(L * (f * S), S, LP);
+        p.F[e] = Vec4<R>{0.0, Fn * nx, Fn * ny, 0.0};
+        return;
+    }
+    const double F0 = L * (f * S), Fn = fma(F0, V, LP), Ft = F0 * T;
+    const double E1 = fma(LP, V, (L * S) * ei);
+    p.F[e] = Vec4<R>{F0, fma(Fn, nx, -(Ft * ny)), fma(Fn, ny, Ft * nx), fma(halved(F0), fma(V, V, T * T), E1)};
+}
+
 // a7: one flux per edge in the frame of the moving edge
 template <class R> __device__ __forceinline__ void stage_edge_flux(const SweepParams<R> &p, int32_t e)
 {
@@ -747,6 +1085,9 @@ template <class R> __device__ __forceinline__ void stage_edge_flux(const SweepPa
                      L * (Fe[3] + Fmx * wfx + Fmy * wfy + R(0.5) * (wfx * wfx + wfy * wfy) * Fe[0])};
 }
 
+__device__ __forceinline__ void edge_flux(const SweepParams<double> &p, int32_t e) { stage_edge_flux_fp64(p, e); }
+__device__ __forceinline__ void edge_flux(const SweepParams<float> &p, int32_t e) { stage_edge_flux(p, e); }
+
 // launched in blocks of 128 threads; ten blocks per SM cap the FP64 build
 // at 48 registers (a few spilled to L1): the FP64 flux times the same as
 // with 62 registers; sixteen cap the FP32 build at 32 (4 bytes spilled),
@@ -754,7 +1095,7 @@ template <class R> __device__ __forceinline__ void stage_edge_flux(const SweepPa
 template <class R> __global__ void __launch_bounds__(128, sizeof(R) == 4 ? 16 : 10) k_edge_flux(SweepParams<R> p)
 {
     int32_t e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e < p.E) stage_edge_flux(p, e);
+    if (e < p.E) edge_flux(p, e);
 }
 
 // a9: advance the generating points in FP64, x <- x0 + hdt w, wrapped
@@ -932,10 +1273,10 @@ __global__ void __launch_bounds__(512) k_sweep_persistent(SweepParams<R> p, cons
     for (int32_t i = tid; i < p.n; i += stride) stage_advance(p, i);
     for (int32_t k = tid; k < p.n; k += stride) {
         const int32_t i = cell_at(p, k);
-        stage_cell_gradient(p, i, p.cell_ptr[i], p.cell_ptr[i + 1], GlobalSlots<R>{p});
+        cell_gradient(p, i);
     }
     if (!grid_sync(gs, nb, lim)) return;
-    for (int32_t e = tid; e < p.E; e += stride) stage_edge_flux(p, e);
+    for (int32_t e = tid; e < p.E; e += stride) edge_flux(p, e);
     if (!grid_sync(gs, nb, lim)) return;
     for (int32_t k = tid; k < p.n; k += stride) stage_cell_update(p, cell_at(p, k));
 }
