@@ -10,7 +10,7 @@
 namespace rich {
 namespace {
 
-constexpr int kVerifyBlock = 128;
+constexpr int kVerifyBlock = 128;  // (as pass_blocks)
 constexpr int kListWarps = 4;  // listed cells per block, a warp each
 constexpr int kListBlock = 32 * kListWarps;
 constexpr int kWindow = kOrderWindow;  // cells per block of the size and ring passes
@@ -20,74 +20,92 @@ constexpr unsigned kAll = 0xffffffffu;
 // mu::verify<true> with eight lanes per cell, a ring slot each: a thread per
 // cell walked its ring through a chain of dependent loads, slot after slot
 // (327 us at 1M cells; 24 us at 4,096).  Cells of more than eight neighbours
-// (3 % of a random mesh) go to the undecided ones.
+// (3 % of a random mesh) go to the undecided ones.  The warps loop over the
+// cells, four at a time, and have the next four's ring slots in flight.
 __global__ void __launch_bounds__(kVerifyBlock) k_mesh_verify(MeshUpdate m)
 {
     using namespace mu;
     const int lane = threadIdx.x & 31, k = lane & 7, group = lane & 24;
-    const int32_t t = (blockIdx.x * blockDim.x + threadIdx.x) >> 3;
-    const bool live = t < m.n;
-    const int32_t i = live ? t : m.n - 1;
-    const Frame f = frame_of(m, i);
-    const int32_t lo = m.cell_ptr[i], deg = m.cell_ptr[i + 1] - lo;
-    const bool mine = live && k < deg && deg <= 8;
-    const int32_t ref = base_ref(m, m.slot_nb[lo + (k < deg ? k : 0)]);
-    const Point d = point_of(f, ref);
-    const int kb = k ? k - 1 : min(deg, 8) - 1, ka = kb ? kb - 1 : min(deg, 8) - 1;
-    Point a, b;
-    b.fx = __shfl_sync(kAll, d.fx, group | kb);
-    b.fy = __shfl_sync(kAll, d.fy, group | kb);
-    b.ref = __shfl_sync(kAll, d.ref, group | kb);
-    a.fx = __shfl_sync(kAll, d.fx, group | ka);
-    a.fy = __shfl_sync(kAll, d.fy, group | ka);
-    a.ref = __shfl_sync(kAll, d.ref, group | ka);
-    a.l = a.fx * a.fx + a.fy * a.fy;
-    b.l = b.fx * b.fx + b.fy * b.fy;
-    const float p = b.fx * d.fy, q = b.fy * d.fx, cbd = p - q;
-    const float p3 = a.fx * d.fy, p4 = a.fy * d.fx, p5 = a.fx * b.fy, p6 = a.fy * b.fx;
-    const float det = a.l * cbd - b.l * (p3 - p4) + d.l * (p5 - p6);
-    const float bound = kCircleBound * (a.l * (fabsf(p) + fabsf(q)) + b.l * (fabsf(p3) + fabsf(p4)) +
-                                        d.l * (fabsf(p5) + fabsf(p6)));
-    bool bad = -det > bound;
-    bool open = deg > 8 || !(cbd > kCrossBound * (fabsf(p) + fabsf(q))) || !(det > bound || bad);
-    if (!f.periodic) open = open || ((b.ref & 15) != 4 && (d.ref & 15) != 4);
-    open = live && open && (mine || deg > 8);
-    bad = bad && mine;
-    const bool self = mine && (bad || d.ref != ref || !disk_ok(f, b, d));
-    const bool turn = mine && b.fy < 0.0f && d.fy >= 0.0f;
     const unsigned byte = 0xffu << group;
-    const unsigned opens = __ballot_sync(kAll, open) & byte, selves = __ballot_sync(kAll, self) & byte;
-    const unsigned turns = __ballot_sync(kAll, turn) & byte;
-    // the block's cells are listed together: one counter took an atomic for
-    // each of the 400,000 cells of a lively step (266 us for this kernel at
-    // 1M cells, 110 where few are listed)
-    constexpr int kMost = kVerifyBlock / 8 * 32;  // 8 slots x 3 cells + 1, per cell
-    __shared__ int32_t cells[kMost];
-    __shared__ int32_t listed, at;
-    if (threadIdx.x == 0) listed = 0;
-    if (!__syncthreads_or(live && (opens || selves || __popc(turns) != 1))) return;
-    auto put = [&](int32_t v) {
-        if (vol(m.flags + inst_at(m, v)) || vol(m.mark + v) == m.stamp || a_exch(m.mark + v, m.stamp) == m.stamp) return;
-        cells[atomicAdd(&listed, 1)] = v;
+    // a warp lists its cells together: one counter took an atomic for each of
+    // the 400,000 cells of a lively step (266 us for this kernel at 1M cells)
+    constexpr int kMost = 4 * (8 * 3 + 1);
+    __shared__ int32_t listed[kVerifyBlock / 32][kMost];
+    __shared__ int32_t listed_n[kVerifyBlock / 32];
+    int32_t *cells = listed[threadIdx.x >> 5], *count = &listed_n[threadIdx.x >> 5];
+    if (lane == 0) *count = 0;
+    const int32_t quads = (m.n + 3) >> 2, stride = gridDim.x * (kVerifyBlock / 32);
+    int32_t quad = blockIdx.x * (kVerifyBlock / 32) + (threadIdx.x >> 5);
+    auto slots_of = [&](int32_t q, int32_t &i, int32_t &deg, int32_t &id) {
+        i = min(4 * q + (group >> 3), m.n - 1);
+        const int32_t lo = m.cell_ptr[i];
+        deg = m.cell_ptr[i + 1] - lo;
+        id = m.slot_nb[lo + (k < deg ? k : 0)];
     };
-    if (live && opens) {
-        if (k == 0) m.list[1][atomicAdd(&m.count->open, 1)] = i;
-    } else if (live) {
-        // (list_bad)
-        if (bad) {
-            put(b.ref >> 4);
-            put(a.ref >> 4);
-            put(d.ref >> 4);
-            if (f.periodic || (a.ref & 15) == 4) tell_only(m, a.ref >> 4, d.ref);
-            if (f.periodic || (d.ref & 15) == 4) tell_only(m, d.ref >> 4, a.ref);
+    int32_t i, deg, id;
+    if (quad < quads) slots_of(quad, i, deg, id);
+    for (; quad < quads; quad += stride) {
+        const bool live = 4 * quad + (group >> 3) < m.n;
+        const Frame f = frame_of(m, i);
+        const int32_t ref = base_ref(m, id);
+        const Point d = point_of(f, ref);
+        const bool small = deg <= 8, mine = live && k < deg && small;
+        const int last = min(deg, 8) - 1;
+        const int32_t cell = i;
+        if (quad + stride < quads) slots_of(quad + stride, i, deg, id);
+        const int kb = k ? k - 1 : last, ka = kb ? kb - 1 : last;
+        Point a, b;
+        b.fx = __shfl_sync(kAll, d.fx, group | kb);
+        b.fy = __shfl_sync(kAll, d.fy, group | kb);
+        b.ref = __shfl_sync(kAll, d.ref, group | kb);
+        a.fx = __shfl_sync(kAll, d.fx, group | ka);
+        a.fy = __shfl_sync(kAll, d.fy, group | ka);
+        a.ref = __shfl_sync(kAll, d.ref, group | ka);
+        a.l = a.fx * a.fx + a.fy * a.fy;
+        b.l = b.fx * b.fx + b.fy * b.fy;
+        const float p = b.fx * d.fy, q = b.fy * d.fx, cbd = p - q;
+        const float p3 = a.fx * d.fy, p4 = a.fy * d.fx, p5 = a.fx * b.fy, p6 = a.fy * b.fx;
+        const float det = a.l * cbd - b.l * (p3 - p4) + d.l * (p5 - p6);
+        const float bound = kCircleBound * (a.l * (fabsf(p) + fabsf(q)) + b.l * (fabsf(p3) + fabsf(p4)) +
+                                            d.l * (fabsf(p5) + fabsf(p6)));
+        bool bad = -det > bound;
+        bool open = !small || !(cbd > kCrossBound * (fabsf(p) + fabsf(q))) || !(det > bound || bad);
+        if (!f.periodic) open = open || ((b.ref & 15) != 4 && (d.ref & 15) != 4);
+        open = live && open && (mine || !small);
+        bad = bad && mine;
+        const bool self = mine && (bad || d.ref != ref || !disk_ok(f, b, d));
+        const bool turn = mine && b.fy < 0.0f && d.fy >= 0.0f;
+        const unsigned opens = __ballot_sync(kAll, open) & byte, selves = __ballot_sync(kAll, self) & byte;
+        const unsigned turns = __ballot_sync(kAll, turn) & byte;
+        if (!__any_sync(kAll, live && (opens || selves || __popc(turns) != 1))) continue;
+        auto put = [&](int32_t v) {
+            if (vol(m.flags + inst_at(m, v)) || vol(m.mark + v) == m.stamp || a_exch(m.mark + v, m.stamp) == m.stamp)
+                return;
+            cells[atomicAdd(count, 1)] = v;
+        };
+        if (live && opens) {
+            if (k == 0) m.list[1][atomicAdd(&m.count->open, 1)] = cell;
+        } else if (live) {
+            // (list_bad)
+            if (bad) {
+                put(b.ref >> 4);
+                put(a.ref >> 4);
+                put(d.ref >> 4);
+                if (f.periodic || (a.ref & 15) == 4) tell_only(m, a.ref >> 4, d.ref);
+                if (f.periodic || (d.ref & 15) == 4) tell_only(m, d.ref >> 4, a.ref);
+            }
+            if (k == 0 && (selves || __popc(turns) != 1)) put(cell);
         }
-        if (k == 0 && (selves || __popc(turns) != 1)) put(i);
+        __syncwarp();
+        const int32_t most = *count;
+        int32_t at = 0;
+        if (lane == 0 && most > 0) at = atomicAdd(&m.count->listed[0], most);
+        at = __shfl_sync(kAll, at, 0);
+        for (int32_t t = lane; t < most; t += 32) m.list[0][at + t] = cells[t];
+        __syncwarp();
+        if (lane == 0) *count = 0;
+        __syncwarp();
     }
-    __syncthreads();
-    const int32_t most = listed;
-    if (threadIdx.x == 0 && most > 0) at = atomicAdd(&m.count->listed[0], most);
-    __syncthreads();
-    for (int32_t q = threadIdx.x; q < most; q += kVerifyBlock) m.list[0][at + q] = cells[q];
 }
 
 // The cells FP32 left open, a warp each: a lane per ring slot, and for the
@@ -618,83 +636,86 @@ __global__ void __launch_bounds__(kWindow) k_mesh_offsets(MeshUpdate m, const in
 // owned edges and triangles (cells of up to 32 neighbours), from which
 // k_mesh_lists takes every edge's and triangle's number.  A ring that no round
 // changed and that meets no image keeps its ids and their order.
-__global__ void __launch_bounds__(256) k_mesh_rings(MeshUpdate m)
+__global__ void __launch_bounds__(128) k_mesh_rings(MeshUpdate m)
 {
     if (!m.count->ready) return;
     using namespace mu;
-    const int32_t t = (blockIdx.x * blockDim.x + threadIdx.x) >> 3;
     const int lane = threadIdx.x & 31, k = lane & 7, first = lane & 24;
-    const bool live = t < m.n;
-    const int32_t i = live ? t : m.n - 1;
-    const Ring g = ring_of(m, i, -1);
-    const bool periodic = m.inst[inst_at(m, i)].boundary == 1;
-    int32_t *dst = m.out_nb + m.out_ptr[i];
-    if (__all_sync(kAll, g.deg <= 8)) {
-        const bool in = live && k < g.deg;
-        const int32_t q = k < g.deg ? k : 0;
-        const bool plain = g.base && g.p[q] < m.n;
-        int32_t id = plain ? g.p[q] : 0;
-        int at = 0;
-        if (!__all_sync(kAll, plain)) {
-            if (!plain) id = point_id(m, i, g[q]);
-            int32_t best = id;
-            at = q;
-            for (int o = 4; o > 0; o >>= 1) {
-                const int32_t b2 = __shfl_xor_sync(kAll, best, o), a2 = __shfl_xor_sync(kAll, at, o);
-                if (b2 < best || (b2 == best && a2 < at)) {
-                    best = b2;
-                    at = a2;
+    const int32_t quads = (m.n + 3) >> 2, stride = gridDim.x * (blockDim.x >> 5);
+    for (int32_t quad = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); quad < quads; quad += stride) {
+        const int32_t t = 4 * quad + (first >> 3);
+        const bool live = t < m.n;
+        const int32_t i = live ? t : m.n - 1;
+        const Ring g = ring_of(m, i, -1);
+        const bool periodic = m.inst[inst_at(m, i)].boundary == 1;
+        int32_t *dst = m.out_nb + m.out_ptr[i];
+        if (__all_sync(kAll, g.deg <= 8)) {
+            const bool in = live && k < g.deg;
+            const int32_t q = k < g.deg ? k : 0;
+            const bool plain = g.base && g.p[q] < m.n;
+            int32_t id = plain ? g.p[q] : 0;
+            int at = 0;
+            if (!__all_sync(kAll, plain)) {
+                if (!plain) id = point_id(m, i, g[q]);
+                int32_t best = id;
+                at = q;
+                for (int o = 4; o > 0; o >>= 1) {
+                    const int32_t b2 = __shfl_xor_sync(kAll, best, o), a2 = __shfl_xor_sync(kAll, at, o);
+                    if (b2 < best || (b2 == best && a2 < at)) {
+                        best = b2;
+                        at = a2;
+                    }
                 }
             }
+            const int pos = q >= at ? q - at : q - at + g.deg;
+            const int32_t next = __shfl_sync(kAll, id, first + (q + 1 < g.deg ? q + 1 : 0));
+            // (an image owns nothing; whether the cell owns a periodic edge to
+            // one follows from the source: images of the cell itself have no
+            // place in an updated mesh)
+            const bool edge = id < m.n || !periodic ? id > i : (g[q] >> 4) > i;
+            uint32_t own = in ? (edge ? 1u << pos : 0u) | (id > i && next > i ? 256u << pos : 0u) : 0u;
+            for (int o = 4; o > 0; o >>= 1) own |= __shfl_xor_sync(kAll, own, o);
+            if (in) dst[pos] = id;
+            if (live && k == 0) {
+                m.edge_mask[i] = own & 255u;
+                m.tri_mask[i] = own >> 8;
+            }
+            continue;
         }
-        const int pos = q >= at ? q - at : q - at + g.deg;
-        const int32_t next = __shfl_sync(kAll, id, first + (q + 1 < g.deg ? q + 1 : 0));
-        // (an image owns nothing; whether the cell owns a periodic edge to
-        // one follows from the source: images of the cell itself have no
-        // place in an updated mesh)
-        const bool edge = id < m.n || !periodic ? id > i : (g[q] >> 4) > i;
-        uint32_t own = in ? (edge ? 1u << pos : 0u) | (id > i && next > i ? 256u << pos : 0u) : 0u;
-        for (int o = 4; o > 0; o >>= 1) own |= __shfl_xor_sync(kAll, own, o);
-        if (in) dst[pos] = id;
+        // some ring of the warp has more than eight members
+        int32_t best = INT32_MAX, at = 0;
+        for (int32_t q = k; q < g.deg; q += 8) {
+            const int32_t id = point_id(m, i, g[q]);
+            if (id < best) {
+                best = id;
+                at = q;
+            }
+        }
+        for (int o = 4; o > 0; o >>= 1) {
+            const int32_t b2 = __shfl_xor_sync(kAll, best, o), a2 = __shfl_xor_sync(kAll, at, o);
+            if (b2 < best || (b2 == best && a2 < at)) {
+                best = b2;
+                at = a2;
+            }
+        }
+        uint32_t edges = 0, tris = 0;
+        for (int32_t q = k; q < g.deg; q += 8) {
+            const int32_t pos = q >= at ? q - at : q - at + g.deg, r = g[q];
+            const int32_t id = point_id(m, i, r), next = point_id(m, i, g[q + 1 < g.deg ? q + 1 : 0]);
+            if (live) dst[pos] = id;
+            if (pos < 32) {
+                if (id < m.n || !periodic ? id > i : (r >> 4) > i) edges |= 1u << pos;
+                if (id > i && next > i) tris |= 1u << pos;
+            }
+        }
+        for (int o = 4; o > 0; o >>= 1) {
+            edges |= __shfl_xor_sync(kAll, edges, o);
+            tris |= __shfl_xor_sync(kAll, tris, o);
+        }
         if (live && k == 0) {
-            m.edge_mask[i] = own & 255u;
-            m.tri_mask[i] = own >> 8;
+            m.edge_mask[i] = edges;
+            m.tri_mask[i] = tris;
         }
-        return;
-    }
-    // some ring of the warp has more than eight members
-    int32_t best = INT32_MAX, at = 0;
-    for (int32_t q = k; q < g.deg; q += 8) {
-        const int32_t id = point_id(m, i, g[q]);
-        if (id < best) {
-            best = id;
-            at = q;
-        }
-    }
-    for (int o = 4; o > 0; o >>= 1) {
-        const int32_t b2 = __shfl_xor_sync(kAll, best, o), a2 = __shfl_xor_sync(kAll, at, o);
-        if (b2 < best || (b2 == best && a2 < at)) {
-            best = b2;
-            at = a2;
-        }
-    }
-    uint32_t edges = 0, tris = 0;
-    for (int32_t q = k; q < g.deg; q += 8) {
-        const int32_t pos = q >= at ? q - at : q - at + g.deg, r = g[q];
-        const int32_t id = point_id(m, i, r), next = point_id(m, i, g[q + 1 < g.deg ? q + 1 : 0]);
-        if (live) dst[pos] = id;
-        if (pos < 32) {
-            if (id < m.n || !periodic ? id > i : (r >> 4) > i) edges |= 1u << pos;
-            if (id > i && next > i) tris |= 1u << pos;
-        }
-    }
-    for (int o = 4; o > 0; o >>= 1) {
-        edges |= __shfl_xor_sync(kAll, edges, o);
-        tris |= __shfl_xor_sync(kAll, tris, o);
-    }
-    if (live && k == 0) {
-        m.edge_mask[i] = edges;
-        m.tri_mask[i] = tris;
     }
 }
 
@@ -711,23 +732,13 @@ __device__ __forceinline__ int edge_owner(const MeshLists &l, bool periodic, int
     return (sy < 0 || (sy == 0 && sx < 0)) ? 0 : 1;
 }
 
-// The triangle and edge lists from the rings, eight lanes per cell, a ring
-// slot each.  A slot whose neighbour is a smaller real cell finds this cell in
-// that one's ring: the edges and triangles that the neighbour owns before it
-// (from the masks of k_mesh_rings, or counted on the way in a mesh that the
-// host built) number the edge and both triangles beside it, so every slot is
-// written once, by its own cell, and needs no clearing and no later check.
-// (Three kernels before: triangles and edges with a walk per triangle and
-// per edge, and a check of both, 153 us at 1M cells.)
-__global__ void __launch_bounds__(128) k_mesh_lists(MeshLists l)
+// The lists of four cells (eight lanes each) of any degree, in a mesh of the
+// update or of the host: k_mesh_lists for the cells that its own code, for
+// rings of up to eight with masks, does not take.
+__device__ __noinline__ bool lists_of_any(const MeshLists &l, int32_t i, bool live, bool periodic)
 {
-    if (l.ready && !*l.ready) return;
     const int lane = threadIdx.x & 31, k = lane & 7, first = lane & 24;
     const unsigned byte = 0xffu << first, below = ((1u << k) - 1) << first;
-    const int32_t cell = (blockIdx.x * blockDim.x + threadIdx.x) >> 3;
-    const bool live = cell < l.n;
-    const int32_t i = live ? cell : l.n - 1;
-    const bool periodic = l.cell_inst ? l.inst[l.cell_inst[i]].boundary == 1 : l.periodic != 0;
     const int32_t lo = l.cell_ptr[i], deg = l.cell_ptr[i + 1] - lo;
     const int32_t *nb = l.slot_nb + lo;
     int32_t t = l.tri_off[i], e = l.edge_off[i];
@@ -841,16 +852,135 @@ __global__ void __launch_bounds__(128) k_mesh_lists(MeshLists l)
         e += __popc(edges);
     }
     if (live && e != e_end) bad = true;
+    return bad;
+}
+
+// The triangle and edge lists from the rings, eight lanes per cell, a ring
+// slot each.  A slot whose neighbour is a smaller real cell finds this cell in
+// that one's ring: the edges and triangles that the neighbour owns before it
+// (from the masks of k_mesh_rings, or counted on the way in a mesh that the
+// host built) number the edge and both triangles beside it, so every slot is
+// written once, by its own cell, and needs no clearing and no later check.
+// (Three kernels before: triangles and edges with a walk per triangle and
+// per edge, and a check of both, 153 us at 1M cells.)
+__global__ void __launch_bounds__(128) k_mesh_lists(MeshLists l)
+{
+    if (l.ready && !*l.ready) return;
+    const int lane = threadIdx.x & 31, k = lane & 7, first = lane & 24;
+    const int32_t quads = (l.n + 3) >> 2, stride = gridDim.x * (blockDim.x >> 5);
+    bool bad = false;
+    for (int32_t quad = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); quad < quads; quad += stride) {
+        const int32_t cell = 4 * quad + (first >> 3);
+        const bool live = cell < l.n;
+        const int32_t i = live ? cell : l.n - 1;
+        const bool periodic = l.cell_inst ? l.inst[l.cell_inst[i]].boundary == 1 : l.periodic != 0;
+        const int32_t lo = l.cell_ptr[i], deg = l.cell_ptr[i + 1] - lo;
+        if (!__all_sync(kAll, l.edge_mask && deg <= 8)) {
+            bad |= lists_of_any(l, i, live, periodic);
+            continue;
+        }
+        const int q = k < deg ? k : 0;
+        const int32_t t0 = l.tri_off[i], e0 = l.edge_off[i];
+        const int32_t own_edges = (int32_t)l.edge_mask[i], own_tris = (int32_t)l.tri_mask[i];
+        // (a mesh left to the host may not agree with its counts)
+        const bool counted = __popc(own_tris) == l.tri_off[i + 1] - t0 && __popc(own_edges) == l.edge_off[i + 1] - e0;
+        const bool in = live && counted && k < deg;
+        bad |= !counted;
+        const int32_t a = l.slot_nb[lo + q];
+        const int32_t b = __shfl_sync(kAll, a, first + (q + 1 < deg ? q + 1 : 0));
+        const int32_t prev = __shfl_sync(kAll, a, first + (q ? q - 1 : deg - 1));
+        const bool own_tri = in && (own_tris >> q & 1), own_edge = in && (own_edges >> q & 1);
+        // this slot's triangle and the one before it, where known here
+        int32_t tri = own_tri ? t0 + __popc(own_tris & ((1 << q) - 1)) : -1, tri_before = -1;
+        if (own_tri) {
+            l.tri[3 * tri] = i;
+            l.tri[3 * tri + 1] = a;
+            l.tri[3 * tri + 2] = b;
+        }
+        if (in && a < i) {
+            const int32_t alo = l.cell_ptr[a], adeg = l.cell_ptr[a + 1] - alo;
+            const uint32_t em = l.edge_mask[a], tm = l.tri_mask[a];
+            const int32_t te = l.tri_off[a + 1], ta = l.tri_off[a], ea = l.edge_off[a];
+            const int32_t *an = l.slot_nb + alo;
+            // (eight loads at once: a loop would wait for each)
+            int32_t ring[8];
+#pragma unroll
+            for (int c = 0; c < 8; c++) ring[c] = c < adeg ? an[c] : -1;
+            int32_t at = adeg;
+#pragma unroll
+            for (int c = 7; c >= 0; c--) at = ring[c] == i ? c : at;
+            if (at == adeg)
+                for (at = 8; at < adeg && an[at] != i; at++) {}
+            if (at >= adeg || adeg > 32) {
+                bad = true;
+            } else {
+                const uint32_t passed = (1u << at) - 1;
+                const int32_t ne = ea + __popc(em & passed), nt = ta + __popc(tm & passed);
+                l.slot_edge[lo + q] = 2 * ne + 1;
+                // (a; b, i) is this slot's triangle, (a; i, prev) the one before
+                if (a < b) {
+                    bad |= an[at ? at - 1 : adeg - 1] != b;
+                    tri = at ? nt - 1 : te - 1;
+                }
+                if (a < prev) {
+                    bad |= an[at + 1 < adeg ? at + 1 : 0] != prev;
+                    tri_before = nt;
+                }
+            }
+        } else if (in && !own_edge) {
+            // a periodic edge that the source of a owns: from its ring this
+            // cell is seen at the opposite shift
+            bool found = false;
+            if (a >= l.n) {
+                const int32_t src = l.ghost_src[a - l.n], sh = l.ghost_shift[a - l.n];
+                const int32_t want = (1 - (sh % 3 - 1)) + 3 * (1 - (sh / 3 - 1));
+                const int32_t alo = l.cell_ptr[src], adeg = l.cell_ptr[src + 1] - alo;
+                for (int32_t j = 0; j < adeg && j < 32 && !found; j++) {
+                    const int32_t x = l.slot_nb[alo + j];
+                    if (x < l.n || l.ghost_src[x - l.n] != i || l.ghost_shift[x - l.n] != want) continue;
+                    l.slot_edge[lo + q] = 2 * (l.edge_off[src] + __popc(l.edge_mask[src] & ((1u << j) - 1))) + 1;
+                    found = true;
+                }
+            }
+            bad |= !found;
+        }
+        const int32_t from_next = __shfl_sync(kAll, tri_before, first + (q + 1 < deg ? q + 1 : 0));
+        if (tri < 0) tri = from_next;
+        const int32_t before = __shfl_sync(kAll, tri, first + (q ? q - 1 : deg - 1));
+        if (in) {
+            bad |= tri < 0;
+            l.slot_tri[lo + q] = tri;
+        }
+        if (own_edge) {
+            const int32_t num = e0 + __popc(own_edges & ((1 << q) - 1));
+            l.edge_l[num] = i;
+            l.edge_r[num] = a;
+            l.edge_ta[num] = before;
+            l.edge_tb[num] = tri;
+            l.slot_edge[lo + q] = 2 * num;
+        }
+    }
     if (bad) *l.bad = 1;
 }
 
 inline int blocks(int64_t n, int b) { return (int)((n + b - 1) / b); }
 
+// Blocks of 128 threads for a pass over every cell, four cells per warp,
+// looping beyond `per SM` blocks on each of 152 SMs.  The update runs beside the
+// FP64 stages of a sweep, which keep their pace as long as they hold most of
+// the registers: at 1M cells a step and its read take 1.80 ms with 4 blocks
+// per SM, 1.87 with 8, 1.88 with 16 and 2.09 with 2; at 262,144 cells in split
+// precision, whose sweep is short, 1.10, 1.07, 1.08 and 1.19.
+inline int pass_blocks(int64_t n)
+{
+    return std::max(1, std::min(blocks(8 * n, 128), 152 * (n >= (1 << 19) ? 4 : 8)));
+}
+
 }  // namespace
 
 cudaError_t launch_lists(const MeshLists &l, cudaStream_t st)
 {
-    if (l.n > 0) k_mesh_lists<<<blocks(8 * (int64_t)l.n, 128), 128, 0, st>>>(l);
+    if (l.n > 0) k_mesh_lists<<<pass_blocks(l.n), 128, 0, st>>>(l);
     return cudaGetLastError();
 }
 
@@ -1040,7 +1170,7 @@ cudaError_t MeshUpdater::launch_rounds(const MeshArrays &a, const MeshOutput &o,
     k_mesh_measure<<<w, kWindow, 0, st>>>(m, sums_.as<int4>(), whole_ ? 1 : 0);
     k_mesh_totals<<<1, kWindow, 0, st>>>(m, sums_.as<int4>(), w, last);
     k_mesh_offsets<<<w, kWindow, 0, st>>>(m, sums_.as<int4>());
-    k_mesh_rings<<<blocks(8 * (int64_t)m.n, 256), 256, 0, st>>>(m);
+    k_mesh_rings<<<pass_blocks(m.n), 128, 0, st>>>(m);
     MeshLists l = o.lists;
     l.n = a.n;
     l.cell_inst = a.cell_inst;
@@ -1070,7 +1200,7 @@ cudaError_t MeshUpdater::start(const MeshArrays &a, const MeshOutput &o, cudaStr
     static_assert(kMaxRounds + 1 < 16, "one update's stamps");
     const MeshUpdate m = params(a, o);
     MU_TRY(cudaMemsetAsync(count_.p, 0, sizeof(MeshUpdateCount) + (size_t)a.n_inst * sizeof(int32_t), st));
-    k_mesh_verify<<<blocks(8 * (int64_t)a.n, kVerifyBlock), kVerifyBlock, 0, st>>>(m);
+    k_mesh_verify<<<pass_blocks(a.n), kVerifyBlock, 0, st>>>(m);
     k_mesh_verify_open<<<std::max(1, std::min(blocks(a.n, 16 * kListWarps), 152 * 8)), kListBlock, 0, st>>>(m);
     last_round_ = kFirstRounds;
     return launch_rounds(a, o, 0, kFirstRounds, st);
