@@ -1,0 +1,45 @@
+// Kernels of one stream that follow each other closely.  In a small simulation
+// a step is a chain of some twenty kernels of 4 to 20 us, and the gap between
+// one's end and the next one's first instruction is a good part of it.  A
+// kernel launched as a programmatic dependent is set up while the one before
+// it still runs, and waits for that one's end (and for its writes) where it
+// calls chained().  Every kernel of the chain calls it before it touches
+// memory, so the order is that of the plain launches.
+#pragma once
+
+#include <cstdint>
+
+#include <cuda_runtime.h>
+
+namespace rich {
+
+#ifdef __CUDACC__
+__device__ __forceinline__ void chained()
+{
+    // let the next kernel be set up, then wait for the one before (both do
+    // nothing in a plain launch)
+    asm volatile("griddepcontrol.launch_dependents;");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+#endif
+
+// From this many cells on kernels are launched plainly: the next one's
+// waiting blocks would take the room of the running one's.
+constexpr int64_t kChainedBelow = 1 << 17;
+
+template <class... P, class... A>
+cudaError_t launch_chained(void (*kernel)(P...), int grid, int block, cudaStream_t st, int64_t cells, A... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = cells < kChainedBelow ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
+}  // namespace rich

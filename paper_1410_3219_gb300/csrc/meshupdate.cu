@@ -17,6 +17,12 @@ constexpr int kWindow = kOrderWindow;  // cells per block of the size and ring p
 static_assert(kWindow == 1024, "the scans and the order pass run one window per 1024-thread block");
 constexpr unsigned kAll = 0xffffffffu;
 
+// the counters of the next update, cleared by this one's last pass
+__device__ __forceinline__ void clear_counters(int32_t *next, int32_t words)
+{
+    for (int32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < words; k += gridDim.x * blockDim.x) next[k] = 0;
+}
+
 // mu::verify<true> with eight lanes per cell, a ring slot each: a thread per
 // cell walked its ring through a chain of dependent loads, slot after slot
 // (327 us at 1M cells; 24 us at 4,096).  Cells of more than eight neighbours
@@ -24,6 +30,7 @@ constexpr unsigned kAll = 0xffffffffu;
 // cells, four at a time, and have the next four's ring slots in flight.
 __global__ void __launch_bounds__(kVerifyBlock) k_mesh_verify(MeshUpdate m)
 {
+    chained();
     using namespace mu;
     const int lane = threadIdx.x & 31, k = lane & 7, group = lane & 24;
     const unsigned byte = 0xffu << group;
@@ -113,6 +120,7 @@ __global__ void __launch_bounds__(kVerifyBlock) k_mesh_verify(MeshUpdate m)
 // (A thread per cell spent 127 us on the walls of 4,096 cells.)
 __global__ void __launch_bounds__(kListBlock) k_mesh_verify_open(MeshUpdate m)
 {
+    chained();
     using namespace mu;
     const int lane = threadIdx.x & 31;
     const int32_t count = m.count->open;
@@ -145,12 +153,12 @@ __global__ void __launch_bounds__(kListBlock) k_mesh_verify_open(MeshUpdate m)
             for (unsigned pairs = __ballot_sync(kAll, pair); pairs; pairs &= pairs - 1) {
                 const int32_t kp = base + __ffs(pairs) - 1;
                 const Point b = point_of(f, base_ref(m, nb[kp ? kp - 1 : deg - 1])), d = point_of(f, base_ref(m, nb[kp]));
-                const int32_t tests = __popc(imgs) * (deg + 1);
-                for (int32_t t = lane; t < tests; t += 32) {
-                    const int img = (int)__fns(imgs, 0, t / (deg + 1) + 1);
-                    const int32_t s = t % (deg + 1);
-                    const int32_t r = (s == deg ? i : base_ref(m, nb[s]) >> 4) * 16 + img;
-                    if (r != b.ref && r != d.ref && incircle(f, b, d, point_of(f, r)) > 0) self = true;
+                for (uint32_t rest = imgs; rest; rest &= rest - 1) {
+                    const int img = __ffs((int)rest) - 1;
+                    for (int32_t s = lane; s <= deg; s += 32) {
+                        const int32_t r = (s == deg ? i : base_ref(m, nb[s]) >> 4) * 16 + img;
+                        if (r != b.ref && r != d.ref && incircle(f, b, d, point_of(f, r)) > 0) self = true;
+                    }
                 }
                 __syncwarp();
             }
@@ -202,6 +210,7 @@ __device__ __forceinline__ bool commit_star(const MeshUpdate &m, const mu::Frame
 // 262,144: one cell's chain of steps.)
 __global__ void __launch_bounds__(kListBlock) k_mesh_recompute_light(MeshUpdate m)
 {
+    chained();
     using namespace mu;
     static_assert(kLight == 16, "a half warp per cell");
     const int lane = threadIdx.x & 31, c = lane & 15, first = lane & 16;
@@ -384,9 +393,9 @@ __device__ void warp_recompute(const MeshUpdate &m, int32_t i, int32_t round, St
     for (int c = lane; c < nc; c += 32) {
         int img = 4, k = c;
         if (walls) {
-            const int set = c / per;
-            k = c % per;
-            img = (int)__fns(imgs | 1u << 4, 0, set + 1);
+            uint32_t rest = imgs | 1u << 4;
+            for (; k >= per; k -= per) rest &= rest - 1;
+            img = __ffs((int)rest) - 1;
         }
         const int32_t src = k < ns ? w.src[k] : i;
         if (src == i && img == 4) {
@@ -477,6 +486,7 @@ __device__ void warp_recompute(const MeshUpdate &m, int32_t i, int32_t round, St
 
 __global__ void __launch_bounds__(kListBlock) k_mesh_recompute(MeshUpdate m, int32_t round)
 {
+    chained();
     __shared__ StarWork work[kListWarps];
     const int32_t count = round ? m.count->listed[round] : m.count->heavy;
     const int32_t *list = round ? m.list[round & 1] : m.heavy;
@@ -489,6 +499,7 @@ __global__ void __launch_bounds__(kListBlock) k_mesh_recompute(MeshUpdate m, int
 // eight lanes per cell, one per triangle and per dropped neighbour
 __global__ void __launch_bounds__(kListBlock) k_mesh_check(MeshUpdate m, int32_t round)
 {
+    chained();
     const int t = threadIdx.x & 7;
     const int32_t count = m.count->listed[round], cells = kListBlock / 8;
     for (int32_t k = blockIdx.x * cells + (threadIdx.x >> 3); k < count; k += gridDim.x * cells) {
@@ -502,6 +513,15 @@ __global__ void __launch_bounds__(kListBlock) k_mesh_check(MeshUpdate m, int32_t
 }
 
 __device__ __forceinline__ int4 plus(int4 a, int4 b) { return make_int4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w); }
+
+__device__ __forceinline__ int4 warp_total(int4 v)
+{
+    v.x = __reduce_add_sync(kAll, v.x);
+    v.y = __reduce_add_sync(kAll, v.y);
+    v.z = __reduce_add_sync(kAll, v.z);
+    v.w = __reduce_add_sync(kAll, v.w);
+    return v;
+}
 
 // inclusive sum over the block's 1024 threads
 __device__ __forceinline__ int4 block_sum(int4 v, int4 *warp_sums)
@@ -544,55 +564,69 @@ __device__ __forceinline__ int4 sizes_of(uint32_t s)
 // a mesh that the host built).
 __global__ void __launch_bounds__(kWindow) k_mesh_measure(MeshUpdate m, int4 *window_sums, int32_t whole)
 {
-    __shared__ int4 ws[32];
+    chained();
+    __shared__ int4 part[32];
     const int32_t i = blockIdx.x * kWindow + threadIdx.x;
     int4 v = make_int4(0, 0, 0, 0);
     if (i < m.n) v = sizes_of(whole ? mu::measure(m, i) : m.sizes[i] = mu::count_images(m, i, m.sizes[i]));
-    v = block_sum(v, ws);
-    if (threadIdx.x == kWindow - 1) window_sums[blockIdx.x] = v;
-}
-
-// window sums -> the sums before each window, and the totals; the mesh can be
-// written when no cell is listed for round `last` and it fits its arrays
-__global__ void __launch_bounds__(kWindow) k_mesh_totals(MeshUpdate m, int4 *window_sums, int32_t windows, int32_t last)
-{
-    __shared__ int4 ws[32];
-    __shared__ int4 carry;
-    if (threadIdx.x == 0) carry = make_int4(0, 0, 0, 0);
+    v = warp_total(v);
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = v;
     __syncthreads();
-    for (int32_t base = 0; base < windows; base += kWindow) {
-        const int32_t k = base + threadIdx.x;
-        const int4 own = k < windows ? window_sums[k] : make_int4(0, 0, 0, 0);
-        const int4 inc = block_sum(own, ws);
-        const int4 c = carry;
-        if (k < windows)
-            window_sums[k] = make_int4(c.x + inc.x - own.x, c.y + inc.y - own.y, c.z + inc.z - own.z, c.w + inc.w - own.w);
-        __syncthreads();
-        if (threadIdx.x == kWindow - 1) carry = plus(c, inc);
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-        m.count->slots = carry.x;
-        m.count->edges = carry.y;
-        m.count->tris = carry.z;
-        m.count->ghosts = carry.w;
-        const bool fits = carry.x >= 0 && carry.x <= m.max_slots && carry.y <= m.max_edges && carry.z <= m.max_tris &&
-                          carry.w <= m.max_ghosts;
-        m.count->ready = fits && m.count->listed[last] == 0 && !(m.n_inst == 1 && m.flags[0]) ? 1 : 0;
+    if (threadIdx.x < 32) {
+        v = warp_total(part[threadIdx.x]);
+        if (threadIdx.x == 0) window_sums[blockIdx.x] = v;
     }
 }
 
 // offsets per cell, the ghosts, and the processing order: within each window
 // cells by decreasing ring degree, stable (degree_order in mesh.cpp)
-__global__ void __launch_bounds__(kWindow) k_mesh_offsets(MeshUpdate m, const int4 *window_sums)
+// Every block adds up the windows before its own, and all of them: the mesh
+// can be written when no cell is listed for round `last` and it fits its
+// arrays.
+__global__ void __launch_bounds__(kWindow) k_mesh_offsets(MeshUpdate m, int4 *window_sums, int32_t last)
 {
-    if (!m.count->ready) return;
+    chained();
+    __shared__ int4 totals[2];
+    {
+        __shared__ int4 part[2][32];
+        const int w = threadIdx.x >> 5;
+        int4 before = make_int4(0, 0, 0, 0), all = before;
+        for (int32_t k = threadIdx.x; k < (int32_t)gridDim.x; k += kWindow) {
+            const int4 v = window_sums[k];
+            all = plus(all, v);
+            if (k < (int32_t)blockIdx.x) before = plus(before, v);
+        }
+        all = warp_total(all);
+        before = warp_total(before);
+        if ((threadIdx.x & 31) == 0) {
+            part[0][w] = before;
+            part[1][w] = all;
+        }
+        __syncthreads();
+        if (w < 2) {
+            const int4 t = warp_total(part[w][threadIdx.x & 31]);
+            if ((threadIdx.x & 31) == 0) totals[w] = t;
+        }
+        __syncthreads();
+        const int4 t = totals[1];
+        const bool fits = t.x >= 0 && t.x <= m.max_slots && t.y <= m.max_edges && t.z <= m.max_tris && t.w <= m.max_ghosts;
+        const bool ready = fits && m.count->listed[last] == 0 && !(m.n_inst == 1 && m.flags[0]);
+        if (blockIdx.x == 0 && threadIdx.x == 0) {
+            m.count->slots = t.x;
+            m.count->edges = t.y;
+            m.count->tris = t.z;
+            m.count->ghosts = t.w;
+            m.count->ready = ready ? 1 : 0;
+        }
+        if (!ready) return;
+    }
     __shared__ int4 ws[32];
+    __shared__ int32_t of_degree[65];
     __shared__ int32_t hist[32][65];  // cells of each degree in each warp, then their first places
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int32_t i = blockIdx.x * kWindow + threadIdx.x;
     const int4 own = i < m.n ? sizes_of(m.sizes[i]) : make_int4(0, 0, 0, 0);
-    const int4 inc = block_sum(own, ws), base = window_sums[blockIdx.x];
+    const int4 inc = block_sum(own, ws), base = totals[0];
     const int4 at = make_int4(base.x + inc.x - own.x, base.y + inc.y - own.y, base.z + inc.z - own.z,
                               base.w + inc.w - own.w);
     if (i < m.n) {
@@ -622,12 +656,30 @@ __global__ void __launch_bounds__(kWindow) k_mesh_offsets(MeshUpdate m, const in
             hist[w][threadIdx.x] = run;
             run += c;
         }
-        ((int *)ws)[threadIdx.x] = run;  // cells of this degree in the window (65 ints in 128)
+        of_degree[threadIdx.x] = run;  // cells of this degree in the window
+    }
+    __syncthreads();
+    if (wid == 0) {
+        // cells of larger degrees: sums from 64 down, two and then 64's own
+        int lo = of_degree[lane], hi = of_degree[32 + lane];
+        const int top = of_degree[64];
+        for (int o = 1; o < 32; o <<= 1) {
+            const int a = __shfl_down_sync(kAll, lo, o), b = __shfl_down_sync(kAll, hi, o);
+            if (lane + o < 32) {
+                lo += a;
+                hi += b;
+            }
+        }
+        const int all_hi = __shfl_sync(kAll, hi, 0);
+        __syncwarp();
+        // (exclusive: minus the degree's own)
+        of_degree[lane] = lo - of_degree[lane] + all_hi + top;
+        of_degree[32 + lane] = hi - of_degree[32 + lane] + top;
+        if (lane == 0) of_degree[64] = 0;
     }
     __syncthreads();
     if (deg >= 0) {
-        int place = hist[wid][deg] + before;
-        for (int d = deg + 1; d <= 64; d++) place += ((int *)ws)[d];
+        const int place = of_degree[deg] + hist[wid][deg] + before;
         m.cell_order[blockIdx.x * kWindow + place] = i;
     }
 }
@@ -638,6 +690,7 @@ __global__ void __launch_bounds__(kWindow) k_mesh_offsets(MeshUpdate m, const in
 // changed and that meets no image keeps its ids and their order.
 __global__ void __launch_bounds__(128) k_mesh_rings(MeshUpdate m)
 {
+    chained();
     if (!m.count->ready) return;
     using namespace mu;
     const int lane = threadIdx.x & 31, k = lane & 7, first = lane & 24;
@@ -865,6 +918,8 @@ __device__ __noinline__ bool lists_of_any(const MeshLists &l, int32_t i, bool li
 // per edge, and a check of both, 153 us at 1M cells.)
 __global__ void __launch_bounds__(128) k_mesh_lists(MeshLists l)
 {
+    chained();
+    if (l.next) clear_counters(l.next, l.next_words);
     if (l.ready && !*l.ready) return;
     const int lane = threadIdx.x & 31, k = lane & 7, first = lane & 24;
     const int32_t quads = (l.n + 3) >> 2, stride = gridDim.x * (blockDim.x >> 5);
@@ -980,8 +1035,8 @@ inline int pass_blocks(int64_t n)
 
 cudaError_t launch_lists(const MeshLists &l, cudaStream_t st)
 {
-    if (l.n > 0) k_mesh_lists<<<pass_blocks(l.n), 128, 0, st>>>(l);
-    return cudaGetLastError();
+    if (l.n > 0) return launch_chained(k_mesh_lists, pass_blocks(l.n), 128, st, l.n, l);
+    return cudaSuccess;
 }
 
 cudaError_t MeshStore::reserve(int32_t n, const MeshSizes &z)
@@ -1094,7 +1149,11 @@ cudaError_t MeshUpdater::reserve(int32_t n, int32_t n_inst, cudaStream_t st)
     MU_TRY(sums_.ensure((size_t)blocks(n, kWindow) * sizeof(int4)));
     // the counters, then the simulations' flags
     const size_t cb = sizeof(MeshUpdateCount) + (size_t)n_inst * i4;
-    MU_TRY(count_.ensure(cb));
+    for (DBuf &c : count_)
+        if (c.cap < cb) {
+            MU_TRY(c.ensure(cb));
+            MU_TRY(cudaMemsetAsync(c.p, 0, c.cap, st));
+        }
     MU_TRY(host_.ensure(cb));
     if (fresh || stamp_ > (1 << 28)) {
         MU_TRY(cudaMemsetAsync(mark_.p, 0, mark_.cap, st));
@@ -1130,7 +1189,7 @@ MeshUpdate MeshUpdater::params(const MeshArrays &a, const MeshOutput &o) const
     m.ring_ref = ring_ref_.as<int32_t>();
     m.extra_n = extra_n_.as<int32_t>();
     m.extra = extra_.as<int32_t>();
-    m.count = count_.as<MeshUpdateCount>();
+    m.count = count_[0].as<MeshUpdateCount>();
     m.flags = reinterpret_cast<int32_t *>(m.count + 1);
     m.sizes = sizes_.as<uint32_t>();
     m.images = images_.as<uint16_t>();
@@ -1162,15 +1221,14 @@ cudaError_t MeshUpdater::launch_rounds(const MeshArrays &a, const MeshOutput &o,
     // grids for the cells a step lists (a few per cent), looping beyond
     const int g = std::max(1, std::min(blocks(m.n, 16 * kListWarps), 152 * 8));
     for (int r = first; r < last; r++) {
-        if (r == 0) k_mesh_recompute_light<<<g, kListBlock, 0, st>>>(m);
-        k_mesh_recompute<<<g, kListBlock, 0, st>>>(m, r);
-        k_mesh_check<<<g, kListBlock, 0, st>>>(m, r);
+        if (r == 0) MU_TRY(launch_chained(k_mesh_recompute_light, g, kListBlock, st, m.n, m));
+        MU_TRY(launch_chained(k_mesh_recompute, g, kListBlock, st, m.n, m, r));
+        MU_TRY(launch_chained(k_mesh_check, g, kListBlock, st, m.n, m, r));
     }
     const int w = blocks(m.n, kWindow);
-    k_mesh_measure<<<w, kWindow, 0, st>>>(m, sums_.as<int4>(), whole_ ? 1 : 0);
-    k_mesh_totals<<<1, kWindow, 0, st>>>(m, sums_.as<int4>(), w, last);
-    k_mesh_offsets<<<w, kWindow, 0, st>>>(m, sums_.as<int4>());
-    k_mesh_rings<<<pass_blocks(m.n), 128, 0, st>>>(m);
+    MU_TRY(launch_chained(k_mesh_measure, w, kWindow, st, m.n, m, sums_.as<int4>(), (int32_t)(whole_ ? 1 : 0)));
+    MU_TRY(launch_chained(k_mesh_offsets, w, kWindow, st, m.n, m, sums_.as<int4>(), (int32_t)last));
+    MU_TRY(launch_chained(k_mesh_rings, pass_blocks(m.n), 128, st, m.n, m));
     MeshLists l = o.lists;
     l.n = a.n;
     l.cell_inst = a.cell_inst;
@@ -1185,8 +1243,10 @@ cudaError_t MeshUpdater::launch_rounds(const MeshArrays &a, const MeshOutput &o,
     l.tri_mask = m.tri_mask;
     l.ready = &m.count->ready;
     l.bad = &m.count->bad;
+    l.next = count_[1].as<int32_t>();
+    l.next_words = (int32_t)(sizeof(MeshUpdateCount) / sizeof(int32_t)) + a.n_inst;
     MU_TRY(launch_lists(l, st));
-    return cudaMemcpyAsync(host_.p, count_.p, sizeof(MeshUpdateCount) + (size_t)a.n_inst * sizeof(int32_t),
+    return cudaMemcpyAsync(host_.p, count_[0].p, sizeof(MeshUpdateCount) + (size_t)a.n_inst * sizeof(int32_t),
                            cudaMemcpyDeviceToHost, st);
 }
 
@@ -1198,10 +1258,13 @@ cudaError_t MeshUpdater::start(const MeshArrays &a, const MeshOutput &o, cudaStr
     MU_TRY(reserve(a.n, a.n_inst, st));
     stamp_ += 16;
     static_assert(kMaxRounds + 1 < 16, "one update's stamps");
+    // the counters cleared by the last update (or when they were allocated)
+    std::swap(count_[0].p, count_[1].p);
+    std::swap(count_[0].cap, count_[1].cap);
     const MeshUpdate m = params(a, o);
-    MU_TRY(cudaMemsetAsync(count_.p, 0, sizeof(MeshUpdateCount) + (size_t)a.n_inst * sizeof(int32_t), st));
-    k_mesh_verify<<<pass_blocks(a.n), kVerifyBlock, 0, st>>>(m);
-    k_mesh_verify_open<<<std::max(1, std::min(blocks(a.n, 16 * kListWarps), 152 * 8)), kListBlock, 0, st>>>(m);
+    MU_TRY(launch_chained(k_mesh_verify, pass_blocks(a.n), kVerifyBlock, st, m.n, m));
+    MU_TRY(launch_chained(k_mesh_verify_open, std::max(1, std::min(blocks(a.n, 16 * kListWarps), 152 * 8)), kListBlock, st,
+                          m.n, m));
     last_round_ = kFirstRounds;
     return launch_rounds(a, o, 0, kFirstRounds, st);
 }

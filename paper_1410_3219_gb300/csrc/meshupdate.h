@@ -321,7 +321,10 @@ RICH_HD inline int circle_pairs(const double x[4], const double y[4])
 RICH_MU_SLOW int circle_slow(int32_t *flags, double ax, double ay, double bx, double by, double cx, double cy,
                              double dx, double dy)
 {
-    {
+    // (the pairs first: at walls nearly every slow test is one)
+    const double px[4] = {ax, bx, cx, dx}, py[4] = {ay, by, cy, dy};
+    int s = circle_pairs(px, py);
+    if (s == 2) {
         const double adx = ax - dx, ady = ay - dy, bdx = bx - dx, bdy = by - dy, cdx = cx - dx, cdy = cy - dy;
         const double p1 = bdx * cdy, p2 = cdx * bdy, p3 = cdx * ady, p4 = adx * cdy, p5 = adx * bdy, p6 = bdx * ady;
         const double la = adx * adx + ady * ady, lb = bdx * bdx + bdy * bdy, lc = cdx * cdx + cdy * cdy;
@@ -331,10 +334,8 @@ RICH_MU_SLOW int circle_slow(int32_t *flags, double ax, double ay, double bx, do
         // (infinities and NaNs fail the comparisons)
         if (det > bound && det < 1e300) return 1;
         if (-det > bound && -det < 1e300) return -1;
+        s = exactint::incircle_sign(ax, ay, bx, by, cx, cy, dx, dy);
     }
-    const double px[4] = {ax, bx, cx, dx}, py[4] = {ay, by, cy, dy};
-    int s = circle_pairs(px, py);
-    if (s == 2) s = exactint::incircle_sign(ax, ay, bx, by, cx, cy, dx, dy);
     if (s == exactint::kUnknown) {
         a_or(flags, MU_EXACT);
         return 0;

@@ -3,6 +3,7 @@
 #pragma once
 
 #include "api_internal.h"
+#include "chain.cuh"
 #include "sweep.cuh"
 
 namespace rich {
@@ -47,6 +48,7 @@ struct MeshLists {
     const uint32_t *edge_mask, *tri_mask;  // slots whose edge / triangle the cell owns (rings of up to 32), or nullptr
     const int32_t *ready;       // nullptr, or 0 there: nothing is built
     int32_t *bad;
+    int32_t *next = nullptr, next_words = 0;  // words to clear (an update's next counters)
 };
 cudaError_t launch_lists(const MeshLists &l, cudaStream_t st);
 
@@ -129,7 +131,7 @@ private:
 
     int32_t stamp_ = 0, max_rings_ = 0, last_round_ = 0;
     bool whole_ = true;  // sizes_ does not describe the mesh to update
-    DBuf mark_, list_[2], heavy_, info_, at_, ring_deg_, ring_ref_, extra_n_, extra_, count_, sizes_, images_,
+    DBuf mark_, list_[2], heavy_, info_, at_, ring_deg_, ring_ref_, extra_n_, extra_, count_[2], sizes_, images_,
         ghost_off_, sums_, edge_mask_, tri_mask_;
     HBuf host_;
 };

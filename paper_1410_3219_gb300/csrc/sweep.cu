@@ -13,6 +13,7 @@
 #include <cfloat>
 #include <cmath>
 
+#include "chain.cuh"
 #include "fp64ops.cuh"
 #include "sweep.cuh"
 
@@ -187,6 +188,7 @@ template <class R> __device__ __forceinline__ void stage_circumcentre(const Swee
 // which the geometry stage's cells then lower)
 template <class R> __global__ void k_circumcentre(SweepParams<R> p)
 {
+    chained();
     int32_t t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t < p.n_inst) p.dtmin_bits[t] = 0x7f7f7f7f7f7f7f7full;
     if (t < p.T) stage_circumcentre(p, t);
@@ -390,6 +392,7 @@ __device__ __forceinline__ double stage_cell_geometry(const SweepParams<R> &p, c
 template <class R>
 __global__ void k_geometry(SweepParams<R> p, const double *__restrict__ init_W, int32_t edge_blocks)
 {
+    chained();
     if ((int32_t)blockIdx.x < edge_blocks) {
         int32_t e = blockIdx.x * blockDim.x + threadIdx.x;
         if (e < p.E) stage_edge_geometry(p, e);
@@ -849,6 +852,7 @@ __device__ __forceinline__ void cell_gradient(const SweepParams<float> &p, int32
 // neighbours share cache lines.
 template <class R> __global__ void __launch_bounds__(128, sizeof(R) == 4 ? 9 : 6) k_cell_gradient(SweepParams<R> p)
 {
+    chained();
     int32_t k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k < p.n) {
         const int32_t i = sizeof(R) == sizeof(double) ? cell_at(p, k) : k;
@@ -1094,6 +1098,7 @@ __device__ __forceinline__ void edge_flux(const SweepParams<float> &p, int32_t e
 // 64 warps: 0.069 -> 0.063 ms at 1M cells
 template <class R> __global__ void __launch_bounds__(128, sizeof(R) == 4 ? 16 : 10) k_edge_flux(SweepParams<R> p)
 {
+    chained();
     int32_t e = blockIdx.x * blockDim.x + threadIdx.x;
     if (e < p.E) edge_flux(p, e);
 }
@@ -1146,6 +1151,7 @@ template <class R> __device__ __forceinline__ void stage_advance(const SweepPara
 
 template <class R> __global__ void __launch_bounds__(kAdvanceBlock) k_advance_points(SweepParams<R> p)
 {
+    chained();
     int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < p.n) stage_advance(p, i);
 }
@@ -1200,6 +1206,7 @@ template <class R> __device__ __forceinline__ void stage_cell_update(const Sweep
 
 template <class R> __global__ void __launch_bounds__(kBlock) k_cell_update(SweepParams<R> p)
 {
+    chained();
     int32_t k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k < p.n) stage_cell_update(p, cell_at(p, k));
 }
@@ -1301,10 +1308,14 @@ inline int blocks(int64_t n) { return (int)((n + kBlock - 1) / kBlock); }
 // GB300 (Sedov, 262,144 cells): the gradient and flux stages, whose register
 // counts cap an SM at 16-21 warps, run best at 128, the others at 32.
 constexpr int kStageBlock[NUM_STAGES] = {32, 32, kAdvanceBlock, 128, 128, 32};
+static_assert(kStageBlock[K_GEOMETRY] == 32, "the geometry launch holds edge and cell blocks of one size");
 static_assert(kStageBlock[K_CELL_GRADIENT] == 128 && kStageBlock[K_EDGE_FLUX] == 128,
               "the gradient's and flux's launch bounds assume 128 threads");
-inline int stage_block(int k) { return kStageBlock[k]; }
-inline int nblk(int64_t n, int k) { return (int)((n + stage_block(k) - 1) / stage_block(k)); }
+// (below 2^16 units the gradient and flux take one warp per block as well: 32
+// blocks of 128 threads put the 4,096 cells of a small simulation on 32 of
+// the 152 SMs, four warps to an FP64 pipe)
+inline int stage_block(int k, int64_t units) { return units < (1 << 16) ? 32 : kStageBlock[k]; }
+inline int nblk(int64_t n, int k) { return (int)((n + stage_block(k, n) - 1) / stage_block(k, n)); }
 
 }  // namespace
 
@@ -1317,31 +1328,22 @@ const char *stage_name(int k)
 
 template <class R> void launch_stage(int k, const SweepParams<R> &p, const double *init_W, cudaStream_t st)
 {
+    auto run = [&](auto kernel, int64_t units, auto... args) {
+        if (units > 0) launch_chained(kernel, nblk(units, k), stage_block(k, units), st, p.n, args...);
+    };
     switch (k) {
-    case K_CIRCUMCENTRE: {
-        const int32_t m = p.T > p.n_inst ? p.T : p.n_inst;
-        if (m > 0) k_circumcentre<R><<<nblk(m, K_CIRCUMCENTRE), stage_block(K_CIRCUMCENTRE), 0, st>>>(p);
-        break;
-    }
+    case K_CIRCUMCENTRE: run(k_circumcentre<R>, p.T > p.n_inst ? p.T : p.n_inst, p); break;
     case K_GEOMETRY: {
+        // (32 threads at every size)
         const int eb = nblk(p.E, K_GEOMETRY), cb = nblk(p.n, K_GEOMETRY);
-        if (eb + cb > 0) k_geometry<R><<<eb + cb, stage_block(K_GEOMETRY), 0, st>>>(p, init_W, eb);
+        if (eb + cb > 0) launch_chained(k_geometry<R>, eb + cb, kStageBlock[K_GEOMETRY], st, p.n, p, init_W, (int32_t)eb);
         break;
     }
-    case K_ADVANCE:
-        if (p.n > 0) k_advance_points<R><<<nblk(p.n, K_ADVANCE), stage_block(K_ADVANCE), 0, st>>>(p);
-        break;
-    case K_CELL_GRADIENT:
-        if (p.n > 0) k_cell_gradient<R><<<nblk(p.n, K_CELL_GRADIENT), stage_block(K_CELL_GRADIENT), 0, st>>>(p);
-        break;
-    case K_EDGE_FLUX:
-        if (p.E > 0) k_edge_flux<R><<<nblk(p.E, K_EDGE_FLUX), stage_block(K_EDGE_FLUX), 0, st>>>(p);
-        break;
-    case K_CELL_UPDATE:
-        if (p.n > 0) k_cell_update<R><<<nblk(p.n, K_CELL_UPDATE), stage_block(K_CELL_UPDATE), 0, st>>>(p);
-        break;
-    default:
-        break;
+    case K_ADVANCE: run(k_advance_points<R>, p.n, p); break;
+    case K_CELL_GRADIENT: run(k_cell_gradient<R>, p.n, p); break;
+    case K_EDGE_FLUX: run(k_edge_flux<R>, p.E, p); break;
+    case K_CELL_UPDATE: run(k_cell_update<R>, p.n, p); break;
+    default: break;
     }
 }
 
