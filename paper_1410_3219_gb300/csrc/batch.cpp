@@ -957,7 +957,10 @@ int rich_batch_step(rich_batch *b, rich_step_info *info)
     //    the moved points (staged: beside the last stages; one wait for both)
     const std::vector<BatchSim *> ok = b->packed;
     const size_t N = (size_t)b->n_packed;
-    const bool update = (int64_t)N >= rich::kMeshUpdateMin && (int64_t)N <= rich::kMeshUpdateMax;
+    // (static meshes' points stay where they are, bit for bit: x + dt 0)
+    bool still = true;
+    for (const BatchSim *s : ok) still = still && s->cfg.motion == RICH_MESH_EULERIAN;
+    const bool update = !still && (int64_t)N >= rich::kMeshUpdateMin && (int64_t)N <= rich::kMeshUpdateMax;
     const LaunchShape shape = pick_shape(b);
     CUDA_TRY(cudaEventRecord(b->ev0, b->stream));
     if (shape.persistent) {
@@ -1031,6 +1034,10 @@ int rich_batch_step(rich_batch *b, rich_step_info *info)
     const double tf = now_ms();
     if (update && going > 0 && (rc = finish_update(b, nxt2))) return rc;
     if (update && going == 0) b->updater.forget();
+    if (still && going > 0) {
+        b->mesh_flag.assign(ok.size(), 0);
+        b->dev_mesh = b->dev_lists = true;
+    }
     const double t_fin = now_ms() - tf;
     if (info) {
         info->steps_done = (int64_t)ok.size();

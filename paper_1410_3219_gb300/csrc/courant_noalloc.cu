@@ -26,10 +26,10 @@
 namespace {
 
 constexpr int kBlock = 256;
-// cells a thread takes per pass of its block, and the largest grid: eight
-// blocks on each of 152 SMs
-constexpr int kCells = 4;
-constexpr int kMaxBlocks = 8 * 152;
+// cells a thread takes per pass, and the largest grid: six blocks on each of
+// 152 SMs (1,536 threads with ten to fourteen loads in flight each)
+constexpr int kCells = 2;
+constexpr int kMaxBlocks = 6 * 152;
 
 // scratch: per-block minima of the cell time step as bit patterns (the
 // integer order of non-negative doubles is their numeric order; kBad marks
@@ -88,13 +88,15 @@ __device__ __forceinline__ float inverse(float v)
 // in FP64 was bound by the FP64 pipe, which issues one warp instruction per
 // 16 clocks per SM: about 110 of them per cell step (three square roots and
 // two divides).  Each cell's time step is first estimated in FP32 within
-// 1e-6, and only cells whose estimate is within 4e-6 of the smallest so far
-// in their block, which the smallest time step's cell always is, are
-// evaluated in FP64 with the formula of the sweep: the result's bits are
-// those of evaluating every cell.  Cells outside the estimate's range
-// (gamma of 2^20 and above, density or pressure beyond 2^+-30, area beyond
-// 2^+-100, speeds above 2^60, and everything negative or not finite) always are.
-__global__ void __launch_bounds__(kBlock) k_courant_noalloc(
+// 1e-6, and only cells whose estimate is within 4e-6 of the smallest in their
+// block, which the smallest time step's cell always is, are evaluated in FP64
+// with the formula of the sweep: the result's bits are those of evaluating
+// every cell.  A thread keeps the latest such cell until the block's smallest
+// estimate is known, and evaluates a second one beside it (a tie) at once.
+// Cells outside the estimate's range (gamma of 2^20 and above, density or
+// pressure beyond 2^+-30, area beyond 2^+-100, speeds above 2^60, and
+// everything negative or not finite) are always evaluated.
+__global__ void __launch_bounds__(kBlock, 6) k_courant_noalloc(
     int32_t n, double gamma, float gamma_f, double cfl, int32_t motion_static, const double *__restrict__ area,
     const double *__restrict__ rho, const double *__restrict__ vx, const double *__restrict__ vy,
     const double *__restrict__ p, const double *__restrict__ wx, const double *__restrict__ wy,
@@ -108,6 +110,13 @@ __global__ void __launch_bounds__(kBlock) k_courant_noalloc(
     __shared__ unsigned smallest;
     if (threadIdx.x == 0) smallest = kNone;
     __syncthreads();
+    float kept = __uint_as_float(kNone);  // this thread's latest candidate
+    int32_t kept_cell = -1;
+    auto evaluate = [&](double area_i, double rho_i, double p_i, double ux_i, double uy_i) {
+        const double cs = sqrt(gamma * p_i / rho_i);
+        const double R = sqrt(area_i * (1.0 / M_PI));
+        k = key_min(k, step_key(R / (cs + sqrt(ux_i * ux_i + uy_i * uy_i)), bad));
+    };
     for (int32_t base = blockIdx.x * kBlock * kCells; base < n; base += gridDim.x * kBlock * kCells) {
         double A[kCells], r[kCells], P[kCells], ux[kCells], uy[kCells];
         float est[kCells];
@@ -144,20 +153,28 @@ __global__ void __launch_bounds__(kBlock) k_courant_noalloc(
             least = min(least, __float_as_uint(est[c]));
         }
         least = __reduce_min_sync(0xffffffffu, least);
-        if ((threadIdx.x & 31) == 0 && least < kNone) atomicMin(&smallest, least);
-        __syncthreads();
-        // (another warp may lower it meanwhile, from cells of its next pass:
-        // any of the values does)
-        const float limit = __uint_as_float(*(volatile unsigned *)&smallest) * 1.000004f;
+        // (the block's smallest so far, and this warp's; other warps may lower
+        // it meanwhile: any of its values does)
+        const unsigned before = *(volatile unsigned *)&smallest;
+        if ((threadIdx.x & 31) == 0 && least < before) atomicMin(&smallest, least);
+        const float limit = __uint_as_float(min(least, before)) * 1.000004f;
 #pragma unroll
         for (int c = 0; c < kCells; c++) {
             const int32_t i = base + c * kBlock + threadIdx.x;
-            if (i < n && est[c] <= limit) {
-                const double cs = sqrt(gamma * P[c] / r[c]);
-                const double R = sqrt(A[c] * (1.0 / M_PI));
-                k = key_min(k, step_key(R / (cs + sqrt(ux[c] * ux[c] + uy[c] * uy[c])), bad));
+            if (i >= n || !(est[c] <= limit)) continue;
+            if (est[c] == 0.0f || kept <= limit) {
+                evaluate(A[c], r[c], P[c], ux[c], uy[c]);
+            } else {
+                // (a kept cell above the limit cannot hold the minimum)
+                kept = est[c];
+                kept_cell = i;
             }
         }
+    }
+    __syncthreads();
+    if (kept_cell >= 0 && kept <= __uint_as_float(smallest) * 1.000004f) {
+        const int32_t i = kept_cell;
+        evaluate(area[i], rho[i], p[i], motion_static ? vx[i] : vx[i] - wx[i], motion_static ? vy[i] : vy[i] - wy[i]);
     }
     bad = __any_sync(0xffffffffu, bad);
     for (int o = 16; o > 0; o >>= 1) k = key_min(k, __shfl_down_sync(0xffffffffu, k, o));

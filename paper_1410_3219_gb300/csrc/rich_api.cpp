@@ -123,6 +123,7 @@ struct rich_sim {
     DBuf A, o, W, cs, g, gl, alpha, w, tess, initW, rounding, p64, psrc;
     bool diagnostics = true;
     DBuf perm_dev, unperm;  // caller index of each internal cell; reordered state for reads
+    rich::HBuf read_host;   // (small reads)
     DBuf ccx, ccy, eL, emlx, emly, emrx, emry, enx, eny, eqx, eqy, F, ePM;
     DBuf scal;   // dtmin bits, dt, status
     DBuf instp;  // one InstParams
@@ -718,11 +719,17 @@ int rich_sync(rich_sim *s, rich_step_info *info)
 static int step_sweep(rich_sim *s, double t_end, rich_step_info *info)
 {
     const int q = s->next_pts();
-    const bool update = can_update(s);
+    // (a static mesh's points stay where they are, bit for bit: x + dt 0)
+    const bool still = s->cfg.motion == RICH_MESH_EULERIAN;
+    const bool update = !still && can_update(s);
     int rc = launch_sweep(s, t_end, update);
     if (rc != RICH_OK) return rc;
     if (update && (rc = join_update(s)) != RICH_OK) return rc;
     rc = rich_sync(s, info);
+    if (still && rc == RICH_OK) {
+        s->tess_current = true;
+        report_sizes(s, info);
+    }
     if (!update) return rc;
     const double t0 = now_ms();
     const int urc = finish_update(s, q, rc == RICH_OK, info);
@@ -801,6 +808,28 @@ static int fetch_r(rich_sim *s, const void *dev, std::vector<double> &h, size_t 
     return RICH_OK;
 }
 
+// Fields of n doubles each, side by side on the device, to the caller's arrays
+// (null ones skipped): small ones in one copy through page-locked memory (each
+// copy to pageable memory costs about 8 us whatever its size), others
+// straight.  Waits.
+static int copy_out(rich_sim *s, const double *dev, double *const *outs, int fields)
+{
+    const size_t N = (size_t)s->n;
+    const bool staged = N * fields * 8 <= ((size_t)2 << 20);
+    if (staged) {
+        CUDA_TRY(s->read_host.ensure(N * fields * 8));
+        CUDA_TRY(cudaMemcpyAsync(s->read_host.p, dev, N * fields * 8, cudaMemcpyDeviceToHost, s->stream));
+    } else {
+        for (int f = 0; f < fields; f++)
+            if (outs[f]) CUDA_TRY(cudaMemcpyAsync(outs[f], dev + f * N, N * 8, cudaMemcpyDeviceToHost, s->stream));
+    }
+    CUDA_TRY(cudaStreamSynchronize(s->stream));
+    if (staged)
+        for (int f = 0; f < fields; f++)
+            if (outs[f]) std::memcpy(outs[f], s->read_host.as<double>() + f * N, N * 8);
+    return RICH_OK;
+}
+
 int rich_get_state(rich_sim *s, int64_t n, double *x, double *y, double *rho, double *vx, double *vy, double *p,
                    double *area)
 {
@@ -817,10 +846,7 @@ int rich_get_state(rich_sim *s, int64_t n, double *x, double *y, double *rho, do
     double *st = s->unperm.as<double>();
     CUDA_TRY(rich::launch_unpermute_state(s->n, s->perm_dev.as<int32_t>(), s->x[q].as<double>(), s->y[q].as<double>(),
                                           s->W.p, s->rsize() == sizeof(float), s->A.as<double>(), st, s->stream));
-    for (int f = 0; f < 7; f++)
-        if (outs[f]) CUDA_TRY(cudaMemcpyAsync(outs[f], st + (size_t)f * N, N * 8, cudaMemcpyDeviceToHost, s->stream));
-    CUDA_TRY(cudaStreamSynchronize(s->stream));
-    return RICH_OK;
+    return copy_out(s, st, outs, 7);
 }
 
 int rich_get_conserved(rich_sim *s, int64_t n, double *x, double *y, double *m, double *px, double *py, double *E)
@@ -839,10 +865,7 @@ int rich_get_conserved(rich_sim *s, int64_t n, double *x, double *y, double *m, 
     CUDA_TRY(s->unperm.ensure(6 * N * sizeof(double)));
     double *st = s->unperm.as<double>();
     CUDA_TRY(rich::launch_unpermute(s->n, s->perm_dev.as<int32_t>(), src, st, s->stream));
-    for (int f = 0; f < 6; f++)
-        if (outs[f]) CUDA_TRY(cudaMemcpyAsync(outs[f], st + (size_t)f * N, N * 8, cudaMemcpyDeviceToHost, s->stream));
-    CUDA_TRY(cudaStreamSynchronize(s->stream));
-    return RICH_OK;
+    return copy_out(s, st, outs, 6);
 }
 
 int rich_get_field(rich_sim *s, int32_t f, int64_t n, double *out)

@@ -284,8 +284,8 @@ def rich_kernel_name(k):
 def rich_courant_dt_noalloc(cfg, n, area, rho, vx, vy, p, wx, wy, dt_out, stream=0):
     """Device pointers (ints) in, device pointer out; see include/rich.h."""
     c = cfg if isinstance(cfg, rich_config) else rich_config.from_dict(cfg)
-    ptrs = [C.c_void_p(v) if v else None for v in (area, rho, vx, vy, p, wx, wy, dt_out)]
-    _check(_lib().rich_courant_dt_noalloc(C.byref(c), n, *ptrs, C.c_void_p(stream)))
+    _check(_lib().rich_courant_dt_noalloc(C.byref(c), n, area or None, rho or None, vx or None, vy or None, p or None,
+                                          wx or None, wy or None, dt_out or None, stream or None))
 
 
 def rich_probe_pipe_peaks():
