@@ -498,9 +498,8 @@ template <class R> __device__ __forceinline__ double step_dt(const SweepParams<R
 //    error go through every edge in FP64.
 // The prediction's cell terms come out folded: with the edge's midpoint m
 // (from the generator) and velocity w_f, Eq. 2 and the half-step prediction of
-// a side read C + g.(m + hdt w_f) with C = phi - g.(o + hdt v) - hdt S.  That
-// takes 12 FP64 instructions more per cell and 12 fewer per edge, and the flux
-// loads C in place of phi, o and S.
+// a side read C + g.(m + hdt w_f) with C = phi - g.(o + hdt v) - hdt S for
+// density and velocity.  (The pressure keeps its sum: see the flux.)
 // (Per cell of six slots: 204 FP64 instructions before, about 160 now.)
 template <class R, class Slots>
 __device__ __forceinline__ void stage_cell_gradient_fp64(const SweepParams<R> &p, int32_t i, int32_t lo, int32_t hi,
@@ -673,12 +672,12 @@ __device__ __forceinline__ void stage_cell_gradient_fp64(const SweepParams<R> &p
         // sweep)
         const double hdt = ip.phase == 0 ? halved(step_dt(p, inst)) : 0.0;
         const double sx = fma(hdt, Wi[1], (double)oi.x), sy = fma(hdt, Wi[2], (double)oi.y);
-        const double hd = hdt * (lg[2] + lg[5]), hr = hdt * recip(Wi[0]), gp = ip.gamma * Wi[3];
+        const double ldiv = lg[2] + lg[5], hd = hdt * ldiv, hr = hdt * recip(Wi[0]);
         const double C0 = fma(-Wi[0], hd, fma(-lg[1], sy, fma(-lg[0], sx, Wi[0])));
         const double C1 = fma(-hr, lg[6], fma(-lg[3], sy, fma(-lg[2], sx, Wi[1])));
         const double C2 = fma(-hr, lg[7], fma(-lg[5], sy, fma(-lg[4], sx, Wi[2])));
-        const double C3 = fma(-gp, hd, fma(-lg[7], sy, fma(-lg[6], sx, Wi[3])));
-        p.psrc[i] = Vec4<R>{C0, C1, C2, C3};
+        p.psrc[i] = Vec4<R>{C0, C1, C2, ip.gamma * Wi[3] * ldiv};
+        p.moved[i] = Vec2<R>{sx, sy};
     }
     if (p.diagnostics) {
         p.g[2 * i] = Vec4<R>{g[0], g[1], g[2], g[3]};
@@ -934,19 +933,23 @@ template <class R> __device__ __forceinline__ void hllc(R gam, R igm1, const R L
     F[2] = F[0] * tK;
 }
 
-// a7 in FP64: as stage_edge_flux below, with 98 FP64 instructions per edge
-// instead of 132.  The sides' states come from the cells' folded terms
-// (stage_cell_gradient_fp64); only the normal velocity is taken relative to
-// the edge, and only side K's tangential velocity is formed, in the lab frame.
-// With the contact (or, beyond the outer waves, side K's own) speed S relative
-// to the edge, density f, pressure P and internal energy density ei, and
-// V = S + w_n in the lab frame, the flux through the moving edge is
-//   mass f S, normal momentum f S V + P, tangential momentum f S T,
-//   energy S ei + P V + f S (V^2 + T^2)/2,
-// the edge-frame HLLC flux boosted back (the star state of Toro,
-// rho* = m_K/(S_K - S), p* = p_K + m_K (S - u_K), with the kinetic parts of
-// its energy put together: ei* = p_K (igm1 (S_K - u_K) + S - u_K)/(S_K - S) +
+// a7 in FP64: as stage_edge_flux below, with about 115 FP64 instructions per
+// edge instead of 132.  The sides' density and velocity come from the cells'
+// folded terms (stage_cell_gradient_fp64); only the normal velocity is taken
+// relative to the edge for both sides, the tangential one for the side K that
+// the flux comes from; the star state and the energy flux are put together:
+// with the contact (or, beyond the outer waves, side K's own) speed S relative
+// to the edge, density f, pressure P, internal energy density ei, and V, T the
+// normal and tangential velocity in the lab frame, the flux through the moving
+// edge is f S of mass and S ei + P V + f S (V^2 + T^2)/2 of energy (Toro's star
+// state: rho* = m_K/(S_K - S), p* = p_K + m_K (S - u_K), with the kinetic parts
+// of its energy summed: ei* = p_K (igm1 (S_K - u_K) + S - u_K)/(S_K - S) +
 // rho* (S - u_K)^2/2).
+// The pressure's way into the momentum flux (its prediction, the normal
+// momentum flux of side K and its correction, the rotation, the boost and the
+// edge length) keeps stage_edge_flux's order of additions: in a nearly uniform
+// pressure the momentum transverse to a flow is the rounding of these sums,
+// which cancel around each cell.
 template <class R> __device__ __forceinline__ void stage_edge_flux_fp64(const SweepParams<R> &p, int32_t e)
 {
     const int32_t l = p.edge_l[e];
@@ -969,20 +972,22 @@ template <class R> __device__ __forceinline__ void stage_edge_flux_fp64(const Sw
     {
         const double ax = fma(hdt, wfx, (double)p.emlx[e]), ay = fma(hdt, wfy, (double)p.emly[e]);
         const Vec4<R> C = p.psrc[l], g0 = p.gl[2 * l], g1 = p.gl[2 * l + 1];
+        const Vec2<R> o = p.moved[l];
         sL[0] = fma(g0.x, ax, fma(g0.y, ay, C.x));
         sL[1] = fma(g0.z, ax, fma(g0.w, ay, C.y));
         sL[2] = fma(g1.x, ax, fma(g1.y, ay, C.z));
-        sL[3] = fma(g1.z, ax, fma(g1.w, ay, C.w));
+        sL[3] = fma(-hdt, C.w, fma(g1.w, ay - o.y, fma(g1.z, ax - o.x, p.W[l].w)));
     }
     {
         // a mirrored source: each derivative takes the flip of its axis,
         // velocity components also the flip of their own axis
         const double ax = fma(hdt, wfx, (double)p.emrx[e]), ay = fma(hdt, wfy, (double)p.emry[e]);
         const Vec4<R> C = p.psrc[k], g0 = p.gl[2 * k], g1 = p.gl[2 * k + 1];
+        const Vec2<R> o = p.moved[k];
         sR[0] = fma(flip(g0.x, mx), ax, fma(flip(g0.y, my), ay, C.x));
         sR[1] = fma(g0.z, ax, fma(flip(g0.w, mxy), ay, flip(C.y, mx)));
         sR[2] = fma(flip(g1.x, mxy), ax, fma(g1.y, ay, flip(C.z, my)));
-        sR[3] = fma(flip(g1.z, mx), ax, fma(flip(g1.w, my), ay, C.w));
+        sR[3] = fma(-hdt, C.w, fma(flip(g1.w, my), ay - flip(o.y, my), fma(flip(g1.z, mx), ax - flip(o.x, mx), p.W[k].w)));
     }
     const double uL = fma(sL[1], nx, fma(sL[2], ny, -wn)), uR = fma(sR[1], nx, fma(sR[2], ny, -wn));
     const double rL = sL[0], rR = sR[0], pL = sL[3], pR = sR[3];
@@ -999,30 +1004,32 @@ template <class R> __device__ __forceinline__ void stage_edge_flux_fp64(const Sw
     const double num = fma(-uR, mR, fma(uL, mL, pR - pL)), den = mL - mR;
     const bool useL = supL || (sub && key_nonpos(num));
     const double rK = useL ? rL : rR, uK = useL ? uL : uR, pK = useL ? pL : pR;
-    const double T = fma(useL ? sL[2] : sR[2], nx, -((useL ? sL[1] : sR[1]) * ny));
-    const double igm1 = ip.igm1;
-    double S = uK, f = rK, P = pK, ei;
+    const double tK = fma((useL ? sL[2] : sR[2]) - wfy, nx, -(((useL ? sL[1] : sR[1]) - wfx) * ny));
+    const double igm1 = ip.igm1, ruK = rK * uK;
+    double S = uK, f = rK, P = pK, ei, F1 = fma(ruK, uK, pK);
     if (sub) {
-        const double dK = useL ? dL : dR, mK = useL ? mL : mR;
+        const double SK = useL ? SL : SR, dK = useL ? dL : dR, mK = useL ? mL : mR;
         S = quotient(num, den);
         const double dS = S - uK, inv = recip(dK - dS);
         f = mK * inv;
         P = fma(mK, dS, pK);
         ei = fma(pK * fma(igm1, dK, dS), inv, halved(f * dS) * dS);
+        F1 = fma(SK, fma(f, S, -ruK), F1);
     } else {
         ei = pK * igm1;
     }
-    const double L = p.eL[e], V = S + wn, LP = L * P;
+    const double L = p.eL[e];
     if (xf && k == l) {
         // a wall: the cell faces its own mirror image; only the normal
         // pressure flux remains (see stage_edge_flux)
-        const double Fn = fma(L * (f * S), S, LP);
-        p.F[e] = Vec4<R>{0.0, Fn * nx, Fn * ny, 0.0};
+        p.F[e] = Vec4<R>{0.0, L * F1 * nx, L * F1 * ny, 0.0};
         return;
     }
-    const double F0 = L * (f * S), Fn = fma(F0, V, LP), Ft = F0 * T;
-    const double E1 = fma(LP, V, (L * S) * ei);
-    p.F[e] = Vec4<R>{F0, fma(Fn, nx, -(Ft * ny)), fma(Fn, ny, Ft * nx), fma(halved(F0), fma(V, V, T * T), E1)};
+    const double F0 = f * S, F2 = F0 * tK;
+    const double Fx = fma(F0, wfx, fma(F1, nx, -(F2 * ny))), Fy = fma(F0, wfy, fma(F1, ny, F2 * nx));
+    const double V = S + wn, T = tK + fma(wfy, nx, -(wfx * ny));
+    const double E = fma(halved(F0), fma(V, V, T * T), fma(P, V, S * ei));
+    p.F[e] = Vec4<R>{L * F0, L * Fx, L * Fy, L * E};
 }
 
 // a7: one flux per edge in the frame of the moving edge
