@@ -104,12 +104,13 @@ class ThreadPool;
 int batch_create(int32_t precision, int64_t max_cells, int32_t host_threads, ThreadPool *shared, rich_batch **out);
 bool point_inside(const rich_config *c, double x, double y);
 
-// dst[f * n + perm[k]] = src[f][k] for the six fields (null sources skipped)
-cudaError_t launch_unpermute(int32_t n, const int32_t *perm, const double *const src[6], double *dst,
+// dst[f * n + u] = src[f][cell[u]] for the six fields (null sources skipped);
+// dst on the device or page-locked
+cudaError_t launch_unpermute(int32_t n, const int32_t *cell, const double *const src[6], double *dst,
                              cudaStream_t st);
-// x, y, rho, vx, vy, p, area into dst (7 n), cell k's at perm[k]; W holds the
+// x, y, rho, vx, vy, p, area into dst (7 n), that of cell[u] at u; W holds the
 // primitives of each cell side by side, in FP32 when `single`
-cudaError_t launch_unpermute_state(int32_t n, const int32_t *perm, const double *x, const double *y, const void *W,
+cudaError_t launch_unpermute_state(int32_t n, const int32_t *cell, const double *x, const double *y, const void *W,
                                    bool single, const double *area, double *dst, cudaStream_t st);
 
 }  // namespace rich

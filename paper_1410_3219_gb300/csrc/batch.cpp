@@ -116,9 +116,10 @@ struct rich_batch {
     int mcur = 0;
     bool dev_mesh = false, dev_lists = false;
     std::vector<int32_t> mesh_flag;
-    // reads: the caller's index of each packed cell (within its simulation),
-    // and a simulation's state in that order on the device and page-locked
-    DBuf perm_dev, read_dev;
+    // reads: the cell (within its simulation) of each caller index, packed,
+    // and the state in that order: page-locked, or for a large simulation on
+    // the device first
+    DBuf cell_of, read_dev;
     rich::HBuf read_host;
     rich::HBuf h_back;  // dt, status per simulation, then the list builder's flag
     cudaEvent_t ev2 = nullptr;
@@ -156,7 +157,7 @@ struct rich_batch {
     std::vector<int32_t> h_dptr, h_dnb, h_dgsrc, h_dgxf, h_dgshift, h_dgimg, h_dtoff, h_deoff;
     std::vector<int32_t> h_gsrc, h_gxf, h_cell_ptr, h_slot_nb, h_cell_inst;
     std::vector<int32_t> h_corder;
-    std::vector<int32_t> h_src, h_eoff, h_toff, h_gshift, h_gimg, h_perm;
+    std::vector<int32_t> h_src, h_eoff, h_toff, h_gshift, h_gimg, h_cell_of;
     std::vector<rich::InstParams> h_inst;
     int64_t nG = 0, nT = 0, nE = 0, nS = 0;
 
@@ -273,7 +274,7 @@ void pack_part(rich_batch *b, BatchSim &s, const PackTask &t)
         std::memcpy(&b->h_y[co + i0], s.hy.data() + i0, sizeof(double) * (i1 - i0));
         for (int64_t i = i0; i < i1; i++) {
             b->h_cell_inst[co + i] = t.k;
-            b->h_perm[co + i] = s.perm[i];
+            b->h_cell_of[co + s.perm[i]] = (int32_t)i;
             b->h_cell_ptr[co + i] = (int32_t)(so + m.cell_ptr[i]);
             b->h_corder[co + i] = (int32_t)(co + m.cell_order[i]);
             b->h_eoff[co + i] = (int32_t)(eo + m.edge_off[i]);
@@ -837,7 +838,7 @@ int pack_step(rich_batch *b, const std::vector<BatchSim *> &list, double &t1, do
     bool any_pending = false;
     for (BatchSim *s : ok) any_pending |= s->state == PENDING;
     b->h_x.resize(N); b->h_y.resize(N); b->h_cell_inst.resize(N); b->h_src.resize(N);
-    b->h_perm.resize(N);
+    b->h_cell_of.resize(N);
     b->h_gx.resize(go); b->h_gy.resize(go); b->h_gsrc.resize(go); b->h_gxf.resize(go);
     b->h_cell_ptr.resize(N + 1); b->h_corder.resize(N);
     b->h_slot_nb.resize(so);
@@ -875,7 +876,7 @@ int pack_step(rich_batch *b, const std::vector<BatchSim *> &list, double &t1, do
     CUDA_TRY(upload(b->x[b->cur], b->h_x, b->stream));
     CUDA_TRY(upload(b->y[b->cur], b->h_y, b->stream));
     CUDA_TRY(upload(b->cell_inst, b->h_cell_inst, b->stream));
-    CUDA_TRY(upload(b->perm_dev, b->h_perm, b->stream));
+    CUDA_TRY(upload(b->cell_of, b->h_cell_of, b->stream));
     rich::MeshStore &d = b->mesh[b->mcur];
     CUDA_TRY(upload(d.gx, b->h_gx, b->stream));
     CUDA_TRY(upload(d.gy, b->h_gy, b->stream));
@@ -1084,15 +1085,18 @@ int rich_batch_get_conserved(rich_batch *b, int32_t id, int64_t n, double *x, do
             for (int32_t k = 0; k < s->n; k++) outs[f][s->perm[k]] = src[(size_t)f * s->n + k];
         }
     } else if (s->state == RUNNING) {
-        // put in the caller's order on the device, one copy down
+        // put in the caller's order on the device, straight into page-locked
+        // memory or by one copy
         const size_t nn = (size_t)s->n, N = (size_t)b->n_packed, co = (size_t)s->cell_off;
         const double *U = b->U[b->cur].as<double>() + co;
         const double *src[6] = {b->x[b->cur].as<double>() + co, b->y[b->cur].as<double>() + co, U, U + N, U + 2 * N,
                                 U + 3 * N};
-        CUDA_TRY(b->read_dev.ensure(6 * nn * 8));
+        const bool direct = 6 * nn * 8 <= ((size_t)2 << 20);
         CUDA_TRY(b->read_host.ensure(6 * nn * 8));
-        CUDA_TRY(rich::launch_unpermute(s->n, b->perm_dev.as<int32_t>() + co, src, b->read_dev.as<double>(), b->stream));
-        CUDA_TRY(cudaMemcpyAsync(b->read_host.p, b->read_dev.p, 6 * nn * 8, cudaMemcpyDeviceToHost, b->stream));
+        if (!direct) CUDA_TRY(b->read_dev.ensure(6 * nn * 8));
+        double *to = direct ? b->read_host.as<double>() : b->read_dev.as<double>();
+        CUDA_TRY(rich::launch_unpermute(s->n, b->cell_of.as<int32_t>() + co, src, to, b->stream));
+        if (!direct) CUDA_TRY(cudaMemcpyAsync(b->read_host.p, to, 6 * nn * 8, cudaMemcpyDeviceToHost, b->stream));
         CUDA_TRY(cudaStreamSynchronize(b->stream));
         for (int f = 0; f < 6; f++)
             if (outs[f]) std::memcpy(outs[f], b->read_host.as<double>() + (size_t)f * nn, nn * 8);

@@ -122,8 +122,8 @@ struct rich_sim {
     DBuf x[3], y[3], U[3];
     DBuf A, o, W, cs, g, gl, alpha, w, tess, initW, rounding, p64, psrc, moved;
     bool diagnostics = true;
-    DBuf perm_dev, unperm;  // caller index of each internal cell; reordered state for reads
-    rich::HBuf read_host;   // (small reads)
+    DBuf cell_of, unperm;  // internal cell of each caller index; reordered state for reads
+    rich::HBuf read_host;  // (small reads)
     DBuf ccx, ccy, eL, emlx, emly, emrx, emry, enx, eny, eqx, eqy, F, ePM;
     DBuf scal;   // dtmin bits, dt, status
     DBuf instp;  // one InstParams
@@ -526,7 +526,9 @@ static int create_sim(const rich_config *cfg, int64_t n, const double *x, const 
         return bail(fail(RICH_ECUDA, "event creation failed"));
     if ((rc = alloc_cells(s)) != RICH_OK) return bail(rc);
     if (s->x[0].ensure(n * 8) != cudaSuccess) return bail(fail(RICH_ENOMEM, "device points"));
-    if (upload(s->perm_dev, s->perm, s->stream) != cudaSuccess) return bail(fail(RICH_ENOMEM, "device order"));
+    std::vector<int32_t> cell_of(n);
+    for (int32_t k = 0; k < s->n; k++) cell_of[s->perm[k]] = k;
+    if (upload(s->cell_of, cell_of, s->stream) != cudaSuccess) return bail(fail(RICH_ENOMEM, "device order"));
     cudaMemcpyAsync(s->x[0].p, hx, n * 8, cudaMemcpyHostToDevice, s->stream);
     cudaMemcpyAsync(s->y[0].p, hy, n * 8, cudaMemcpyHostToDevice, s->stream);
     if ((rc = tessellate(s, nullptr, false)) != RICH_OK) return bail(rc);
@@ -808,25 +810,28 @@ static int fetch_r(rich_sim *s, const void *dev, std::vector<double> &h, size_t 
     return RICH_OK;
 }
 
-// Fields of n doubles each, side by side on the device, to the caller's arrays
-// (null ones skipped): small ones in one copy through page-locked memory (each
-// copy to pageable memory costs about 8 us whatever its size), others
-// straight.  Waits.
-static int copy_out(rich_sim *s, const double *dev, double *const *outs, int fields)
+// Where a read of `fields` fields is gathered: page-locked memory for small
+// ones (each copy to pageable memory costs about 8 us whatever its size), else
+// the device.
+static int read_buffer(rich_sim *s, int fields, double **buf, bool *host)
+{
+    const size_t bytes = (size_t)s->n * fields * 8;
+    *host = bytes <= ((size_t)2 << 20);
+    if (*host) CUDA_TRY(s->read_host.ensure(bytes));
+    else CUDA_TRY(s->unperm.ensure(bytes));
+    *buf = *host ? s->read_host.as<double>() : s->unperm.as<double>();
+    return RICH_OK;
+}
+
+// From there to the caller's arrays (null ones skipped).  Waits.
+static int copy_out(rich_sim *s, const double *buf, bool host, double *const *outs, int fields)
 {
     const size_t N = (size_t)s->n;
-    const bool staged = N * fields * 8 <= ((size_t)2 << 20);
-    if (staged) {
-        CUDA_TRY(s->read_host.ensure(N * fields * 8));
-        CUDA_TRY(cudaMemcpyAsync(s->read_host.p, dev, N * fields * 8, cudaMemcpyDeviceToHost, s->stream));
-    } else {
-        for (int f = 0; f < fields; f++)
-            if (outs[f]) CUDA_TRY(cudaMemcpyAsync(outs[f], dev + f * N, N * 8, cudaMemcpyDeviceToHost, s->stream));
-    }
+    for (int f = 0; f < fields && !host; f++)
+        if (outs[f]) CUDA_TRY(cudaMemcpyAsync(outs[f], buf + f * N, N * 8, cudaMemcpyDeviceToHost, s->stream));
     CUDA_TRY(cudaStreamSynchronize(s->stream));
-    if (staged)
-        for (int f = 0; f < fields; f++)
-            if (outs[f]) std::memcpy(outs[f], s->read_host.as<double>() + f * N, N * 8);
+    for (int f = 0; f < fields && host; f++)
+        if (outs[f]) std::memcpy(outs[f], buf + f * N, N * 8);
     return RICH_OK;
 }
 
@@ -839,14 +844,14 @@ int rich_get_state(rich_sim *s, int64_t n, double *x, double *y, double *rho, do
     // put in the caller's order on the device, then copied straight into the
     // caller's arrays with one wait (on the host the reordering took 2.4 ms of
     // a 3.0 ms step and read at 262,144 cells)
-    const size_t N = (size_t)s->n;
     const int q = s->pts();
     double *outs[7] = {x, y, rho, vx, vy, p, area};
-    CUDA_TRY(s->unperm.ensure(7 * N * sizeof(double)));
-    double *st = s->unperm.as<double>();
-    CUDA_TRY(rich::launch_unpermute_state(s->n, s->perm_dev.as<int32_t>(), s->x[q].as<double>(), s->y[q].as<double>(),
+    double *st;
+    bool host;
+    if ((rc = read_buffer(s, 7, &st, &host))) return rc;
+    CUDA_TRY(rich::launch_unpermute_state(s->n, s->cell_of.as<int32_t>(), s->x[q].as<double>(), s->y[q].as<double>(),
                                           s->W.p, s->rsize() == sizeof(float), s->A.as<double>(), st, s->stream));
-    return copy_out(s, st, outs, 7);
+    return copy_out(s, st, host, outs, 7);
 }
 
 int rich_get_conserved(rich_sim *s, int64_t n, double *x, double *y, double *m, double *px, double *py, double *E)
@@ -862,10 +867,12 @@ int rich_get_conserved(rich_sim *s, int64_t n, double *x, double *y, double *m, 
                             s->U[q].as<double>() + N, s->U[q].as<double>() + 2 * N, s->U[q].as<double>() + 3 * N};
     for (int f = 0; f < 6; f++)
         if (!outs[f]) src[f] = nullptr;
-    CUDA_TRY(s->unperm.ensure(6 * N * sizeof(double)));
-    double *st = s->unperm.as<double>();
-    CUDA_TRY(rich::launch_unpermute(s->n, s->perm_dev.as<int32_t>(), src, st, s->stream));
-    return copy_out(s, st, outs, 6);
+    double *st;
+    bool host;
+    int rc = read_buffer(s, 6, &st, &host);
+    if (rc) return rc;
+    CUDA_TRY(rich::launch_unpermute(s->n, s->cell_of.as<int32_t>(), src, st, s->stream));
+    return copy_out(s, st, host, outs, 6);
 }
 
 int rich_get_field(rich_sim *s, int32_t f, int64_t n, double *out)

@@ -221,13 +221,13 @@ def rich_step(h, max_steps=1, t_end=float("inf")):
 
 
 def rich_get_state(h, n):
-    out = [np.zeros(n) for _ in range(7)]
+    out = [np.empty(n) for _ in range(7)]
     _check(_lib().rich_get_state(h, n, *[_p(a) for a in out]))
     return dict(zip(("x", "y", "rho", "vx", "vy", "p", "area"), out))
 
 
 def rich_get_conserved(h, n):
-    out = [np.zeros(n) for _ in range(6)]
+    out = [np.empty(n) for _ in range(6)]
     _check(_lib().rich_get_conserved(h, n, *[_p(a) for a in out]))
     return dict(zip(("x", "y", "m", "px", "py", "E"), out))
 
@@ -404,7 +404,7 @@ def rich_batch_query(b, sid):
 
 
 def rich_batch_get_conserved(b, sid, n):
-    out = [np.zeros(n) for _ in range(6)]
+    out = [np.empty(n) for _ in range(6)]
     _check(_lib().rich_batch_get_conserved(b, sid, n, *[_p(a) for a in out]))
     return dict(zip(("x", "y", "m", "px", "py", "E"), out))
 
