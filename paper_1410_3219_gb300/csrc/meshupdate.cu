@@ -30,7 +30,7 @@ __device__ __forceinline__ void clear_counters(int32_t *next, int32_t words)
 // cells, four at a time, and have the next four's ring slots in flight.
 __global__ void __launch_bounds__(kVerifyBlock) k_mesh_verify(MeshUpdate m)
 {
-    chained();
+    chained(m.n);
     using namespace mu;
     const int lane = threadIdx.x & 31, k = lane & 7, group = lane & 24;
     const unsigned byte = 0xffu << group;
@@ -120,7 +120,7 @@ __global__ void __launch_bounds__(kVerifyBlock) k_mesh_verify(MeshUpdate m)
 // (A thread per cell spent 127 us on the walls of 4,096 cells.)
 __global__ void __launch_bounds__(kListBlock) k_mesh_verify_open(MeshUpdate m)
 {
-    chained();
+    chained(m.n);
     using namespace mu;
     const int lane = threadIdx.x & 31;
     const int32_t count = m.count->open;
@@ -210,7 +210,7 @@ __device__ __forceinline__ bool commit_star(const MeshUpdate &m, const mu::Frame
 // 262,144: one cell's chain of steps.)
 __global__ void __launch_bounds__(kListBlock) k_mesh_recompute_light(MeshUpdate m)
 {
-    chained();
+    chained(m.n);
     using namespace mu;
     static_assert(kLight == 16, "a half warp per cell");
     const int lane = threadIdx.x & 31, c = lane & 15, first = lane & 16;
@@ -486,7 +486,7 @@ __device__ void warp_recompute(const MeshUpdate &m, int32_t i, int32_t round, St
 
 __global__ void __launch_bounds__(kListBlock) k_mesh_recompute(MeshUpdate m, int32_t round)
 {
-    chained();
+    chained(m.n);
     __shared__ StarWork work[kListWarps];
     const int32_t count = round ? m.count->listed[round] : m.count->heavy;
     const int32_t *list = round ? m.list[round & 1] : m.heavy;
@@ -499,7 +499,7 @@ __global__ void __launch_bounds__(kListBlock) k_mesh_recompute(MeshUpdate m, int
 // eight lanes per cell, one per triangle and per dropped neighbour
 __global__ void __launch_bounds__(kListBlock) k_mesh_check(MeshUpdate m, int32_t round)
 {
-    chained();
+    chained(m.n);
     const int t = threadIdx.x & 7;
     const int32_t count = m.count->listed[round], cells = kListBlock / 8;
     for (int32_t k = blockIdx.x * cells + (threadIdx.x >> 3); k < count; k += gridDim.x * cells) {
@@ -564,7 +564,7 @@ __device__ __forceinline__ int4 sizes_of(uint32_t s)
 // a mesh that the host built).
 __global__ void __launch_bounds__(kWindow) k_mesh_measure(MeshUpdate m, int4 *window_sums, int32_t whole)
 {
-    chained();
+    chained(m.n);
     __shared__ int4 part[32];
     const int32_t i = blockIdx.x * kWindow + threadIdx.x;
     int4 v = make_int4(0, 0, 0, 0);
@@ -585,7 +585,7 @@ __global__ void __launch_bounds__(kWindow) k_mesh_measure(MeshUpdate m, int4 *wi
 // arrays.
 __global__ void __launch_bounds__(kWindow) k_mesh_offsets(MeshUpdate m, int4 *window_sums, int32_t last)
 {
-    chained();
+    chained(m.n);
     __shared__ int4 totals[2];
     {
         __shared__ int4 part[2][32];
@@ -690,7 +690,7 @@ __global__ void __launch_bounds__(kWindow) k_mesh_offsets(MeshUpdate m, int4 *wi
 // changed and that meets no image keeps its ids and their order.
 __global__ void __launch_bounds__(128) k_mesh_rings(MeshUpdate m)
 {
-    chained();
+    chained(m.n);
     if (!m.count->ready) return;
     using namespace mu;
     const int lane = threadIdx.x & 31, k = lane & 7, first = lane & 24;
@@ -918,7 +918,7 @@ __device__ __noinline__ bool lists_of_any(const MeshLists &l, int32_t i, bool li
 // per edge, and a check of both, 153 us at 1M cells.)
 __global__ void __launch_bounds__(128) k_mesh_lists(MeshLists l)
 {
-    chained();
+    chained(l.n);
     if (l.next) clear_counters(l.next, l.next_words);
     if (l.ready && !*l.ready) return;
     const int lane = threadIdx.x & 31, k = lane & 7, first = lane & 24;

@@ -188,7 +188,7 @@ template <class R> __device__ __forceinline__ void stage_circumcentre(const Swee
 // which the geometry stage's cells then lower)
 template <class R> __global__ void k_circumcentre(SweepParams<R> p)
 {
-    chained();
+    chained(p.n);
     int32_t t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t < p.n_inst) p.dtmin_bits[t] = 0x7f7f7f7f7f7f7f7full;
     if (t < p.T) stage_circumcentre(p, t);
@@ -392,7 +392,7 @@ __device__ __forceinline__ double stage_cell_geometry(const SweepParams<R> &p, c
 template <class R>
 __global__ void k_geometry(SweepParams<R> p, const double *__restrict__ init_W, int32_t edge_blocks)
 {
-    chained();
+    chained(p.n);
     if ((int32_t)blockIdx.x < edge_blocks) {
         int32_t e = blockIdx.x * blockDim.x + threadIdx.x;
         if (e < p.E) stage_edge_geometry(p, e);
@@ -851,7 +851,7 @@ __device__ __forceinline__ void cell_gradient(const SweepParams<float> &p, int32
 // neighbours share cache lines.
 template <class R> __global__ void __launch_bounds__(128, sizeof(R) == 4 ? 9 : 6) k_cell_gradient(SweepParams<R> p)
 {
-    chained();
+    chained(p.n);
     int32_t k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k < p.n) {
         const int32_t i = sizeof(R) == sizeof(double) ? cell_at(p, k) : k;
@@ -1105,7 +1105,7 @@ __device__ __forceinline__ void edge_flux(const SweepParams<float> &p, int32_t e
 // 64 warps: 0.069 -> 0.063 ms at 1M cells
 template <class R> __global__ void __launch_bounds__(128, sizeof(R) == 4 ? 16 : 10) k_edge_flux(SweepParams<R> p)
 {
-    chained();
+    chained(p.n);
     int32_t e = blockIdx.x * blockDim.x + threadIdx.x;
     if (e < p.E) edge_flux(p, e);
 }
@@ -1158,7 +1158,7 @@ template <class R> __device__ __forceinline__ void stage_advance(const SweepPara
 
 template <class R> __global__ void __launch_bounds__(kAdvanceBlock) k_advance_points(SweepParams<R> p)
 {
-    chained();
+    chained(p.n);
     int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < p.n) stage_advance(p, i);
 }
@@ -1213,7 +1213,7 @@ template <class R> __device__ __forceinline__ void stage_cell_update(const Sweep
 
 template <class R> __global__ void __launch_bounds__(kBlock) k_cell_update(SweepParams<R> p)
 {
-    chained();
+    chained(p.n);
     int32_t k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k < p.n) stage_cell_update(p, cell_at(p, k));
 }
