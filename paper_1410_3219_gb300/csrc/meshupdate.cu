@@ -1250,8 +1250,11 @@ cudaError_t MeshUpdater::launch_rounds(const MeshArrays &a, const MeshOutput &o,
                            cudaMemcpyDeviceToHost, st);
 }
 
-// The rounds launched before the host looks: what nearly every step needs.
-constexpr int kFirstRounds = 2;
+// The rounds launched before the host looks.  Most steps are settled by one; a
+// second one's kernels are 5 us of empty launches in a step of 100 us (10,201
+// cells), but the host's look and another launch of what follows are 50 us.
+// So one round once kQuiet updates in a row needed no second.
+constexpr int kQuiet = 8;
 
 cudaError_t MeshUpdater::start(const MeshArrays &a, const MeshOutput &o, cudaStream_t st)
 {
@@ -1263,20 +1266,25 @@ cudaError_t MeshUpdater::start(const MeshArrays &a, const MeshOutput &o, cudaStr
     std::swap(count_[0].cap, count_[1].cap);
     const MeshUpdate m = params(a, o);
     MU_TRY(launch_chained(k_mesh_verify, pass_blocks(a.n), kVerifyBlock, st, m.n, m));
-    MU_TRY(launch_chained(k_mesh_verify_open, std::max(1, std::min(blocks(a.n, 16 * kListWarps), 152 * 8)), kListBlock, st,
-                          m.n, m));
-    last_round_ = kFirstRounds;
-    return launch_rounds(a, o, 0, kFirstRounds, st);
+    // (a warp per eight cells: steps of 10,201 cells took 105 us with one per
+    // sixteen, 98 with this.  With the list passes at eight as well their FP64
+    // tests slow the gradient of 4,096 cells, which runs beside them)
+    const int open = std::max(1, std::min(blocks(a.n, 8 * kListWarps), 152 * 8));
+    MU_TRY(launch_chained(k_mesh_verify_open, open, kListBlock, st, m.n, m));
+    last_round_ = quiet_ < kQuiet ? 2 : 1;
+    return launch_rounds(a, o, 0, last_round_, st);
 }
 
 cudaError_t MeshUpdater::settle(const MeshArrays &a, const MeshOutput &o, MeshResult &result, cudaStream_t st)
 {
     const MeshUpdateCount &c = *host_.as<MeshUpdateCount>();
     int r = last_round_;
-    static_assert((kMaxRounds - kFirstRounds) % 2 == 0, "further rounds come in pairs");
-    for (; c.listed[r] > 0 && r < kMaxRounds; r += 2) {
-        MU_TRY(launch_rounds(a, o, r, r + 2, st));
+    quiet_ = c.listed[1] > 0 ? 0 : std::min(quiet_ + 1, kQuiet);
+    while (c.listed[r] > 0 && r < kMaxRounds) {
+        const int to = std::min(r + 2, kMaxRounds);
+        MU_TRY(launch_rounds(a, o, r, to, st));
         MU_TRY(cudaStreamSynchronize(st));
+        r = to;
     }
     result.sizes = MeshSizes{c.ghosts, c.tris, c.edges, c.slots};
     result.flagged = false;

@@ -116,3 +116,25 @@ def test_batch_membership_changes_repack_updated_meshes(R):
             assert np.array_equal(got[f], want[f]), (sid, f)
         solo.close()
     b.close()
+
+
+def test_a_second_round_after_quiet_updates(R):
+    """After a run of updates that one round settled only one is launched at
+    first; a rough mesh that joins then needs a second, and every result
+    equals its solo run (whose first updates launch two) bit for bit."""
+    quiet, rough = W.gresho(n_side=24, seed=2), W.sod(n_side=225, seed=3, jitter=0.4)
+    b = R.Batch(max_cells=1 << 20)
+    ids = [b.add(quiet, max_steps=14)]
+    for k in range(14):
+        if k == 11:
+            ids.append(b.add(rough, max_steps=3))
+        b.step()
+    for w, sid, k in ((quiet, ids[0], 14), (rough, ids[1], 3)):
+        assert b.query(sid)["state"] == "done"
+        solo = R.Sim(w)
+        solo.step(k)
+        got, want = b.conserved(sid), solo.conserved()
+        for f in want:
+            assert np.array_equal(got[f], want[f]), (sid, f)
+        solo.close()
+    b.close()
