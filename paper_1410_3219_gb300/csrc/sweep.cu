@@ -838,9 +838,10 @@ __device__ __forceinline__ void cell_gradient(const SweepParams<float> &p, int32
     stage_cell_gradient(p, i, p.cell_ptr[i], p.cell_ptr[i + 1], GlobalSlots<float>{p});
 }
 
-// launched in blocks of 128 threads; six blocks per SM cap the FP64 build at
-// 80 registers (from 94, with a few spilled to L1), 24 warps instead of 20;
-// nine hold the FP32 build's 56 registers, 36 warps, which hide more of its
+// launched in blocks of 128 threads; five blocks per SM let the FP64 build have
+// 96 registers, with 68 bytes spilled to L1 (six, at 80 registers, spilled 250:
+// the same at 1M cells, 361 us, but two steps of 90,000 cells 369 us instead of
+// 348); nine hold the FP32 build's 56 registers, 36 warps, which hide more of its
 // gather latency than 28 did (0.102 -> 0.093 ms at 1M cells, when the cap
 // took it from 72 registers, before the mesh velocity and the time step
 // moved to the geometry stage; ten blocks spilled and lost it again).
@@ -849,7 +850,7 @@ __device__ __forceinline__ void cell_gradient(const SweepParams<float> &p, int32
 // build, bound by its gathers, visits them in the Hilbert order itself, so
 // that the rings of a warp's cells are adjacent in the slot arrays and their
 // neighbours share cache lines.
-template <class R> __global__ void __launch_bounds__(128, sizeof(R) == 4 ? 9 : 6) k_cell_gradient(SweepParams<R> p)
+template <class R> __global__ void __launch_bounds__(128, sizeof(R) == 4 ? 9 : 5) k_cell_gradient(SweepParams<R> p)
 {
     chained(p.n);
     int32_t k = blockIdx.x * blockDim.x + threadIdx.x;
@@ -1099,11 +1100,11 @@ template <class R> __device__ __forceinline__ void stage_edge_flux(const SweepPa
 __device__ __forceinline__ void edge_flux(const SweepParams<double> &p, int32_t e) { stage_edge_flux_fp64(p, e); }
 __device__ __forceinline__ void edge_flux(const SweepParams<float> &p, int32_t e) { stage_edge_flux(p, e); }
 
-// launched in blocks of 128 threads; ten blocks per SM cap the FP64 build
-// at 48 registers (a few spilled to L1): the FP64 flux times the same as
-// with 62 registers; sixteen cap the FP32 build at 32 (4 bytes spilled),
+// launched in blocks of 128 threads; eight blocks per SM let the FP64 build
+// have 64 registers, without a spill: 655 -> 643 us at 1M cells against ten
+// and 48 registers; sixteen cap the FP32 build at 32 (4 bytes spilled),
 // 64 warps: 0.069 -> 0.063 ms at 1M cells
-template <class R> __global__ void __launch_bounds__(128, sizeof(R) == 4 ? 16 : 10) k_edge_flux(SweepParams<R> p)
+template <class R> __global__ void __launch_bounds__(128, sizeof(R) == 4 ? 16 : 8) k_edge_flux(SweepParams<R> p)
 {
     chained(p.n);
     int32_t e = blockIdx.x * blockDim.x + threadIdx.x;
@@ -1313,14 +1314,15 @@ inline int blocks(int64_t n) { return (int)((n + kBlock - 1) / kBlock); }
 // to 17 % of the launch waiting for the last blocks (per-SM active cycles
 // from 0.77x to 1.17x of the mean).  Chosen by timing 32, 64, 128 and 256 on
 // GB300 (Sedov, 262,144 cells): the gradient and flux stages, whose register
-// counts cap an SM at 16-21 warps, run best at 128, the others at 32.
+// counts cap an SM at 20 and 32 warps, run best at 128, the others at 32.
 constexpr int kStageBlock[NUM_STAGES] = {32, 32, kAdvanceBlock, 128, 128, 32};
 static_assert(kStageBlock[K_GEOMETRY] == 32, "the geometry launch holds edge and cell blocks of one size");
 static_assert(kStageBlock[K_CELL_GRADIENT] == 128 && kStageBlock[K_EDGE_FLUX] == 128,
               "the gradient's and flux's launch bounds assume 128 threads");
 // (below 2^16 units the gradient and flux take one warp per block as well: 32
 // blocks of 128 threads put the 4,096 cells of a small simulation on 32 of
-// the 152 SMs, four warps to an FP64 pipe)
+// the 152 SMs, four warps to an FP64 pipe.  Two steps of 50,625 cells take
+// 430 us so, 440 with 128; of 90,000 cells the same, 349, with both)
 inline int stage_block(int k, int64_t units) { return units < (1 << 16) ? 32 : kStageBlock[k]; }
 inline int nblk(int64_t n, int k) { return (int)((n + stage_block(k, n) - 1) / stage_block(k, n)); }
 
