@@ -2,22 +2,27 @@
 // moving-mesh simulations of different sizes and parameters advanced
 // together, one device sweep per step over all of them.
 //
-// Every step:
-//   1. the generating points of all running simulations come back to the
-//      host in one copy;
-//   2. each simulation is tessellated on a host worker thread (a0), newly
-//      admitted ones included;
-//   3. the meshes are packed into one index space (cells of simulation k
-//      follow those of k-1; ghosts, triangles, edges and ring slots likewise)
-//      with a per-cell simulation id and a per-simulation parameter table;
-//      when membership changed, the FP64 conserved state is regathered on
+// The simulations are packed into one index space (cells of simulation k
+// follow those of k-1; ghosts, triangles, edges and ring slots likewise) with
+// a per-cell simulation id and a per-simulation parameter table.  A step with
+// the simulations of the last one, whose meshes the device updated, starts
+// with 6; else (pack_step):
+//   1. the meshes that the device updated come back to the host, and of the
+//      other running simulations the points;
+//   2. the simulations without a mesh, newly admitted ones included, are
+//      tessellated on the host's worker threads (a0);
+//   3. the meshes are packed, and the FP64 conserved state is regathered on
 //      the device;
-//   4. newly admitted simulations get their conserved variables from their
-//      initial primitives and first areas (geometry stage in init mode);
-//   5. one sweep (a1-a9) runs over all cells; each simulation keeps its own
-//      time step, remaining time and status flags;
-//   6. simulations that reached t_end or their step budget are copied out
-//      and leave the batch; a failed step rolls back that simulation only.
+//   4. the packed meshes are uploaded;
+//   5. newly admitted simulations get their conserved variables from their
+//      initial primitives and first areas (geometry stage in init mode).
+// Then, every step:
+//   6. one sweep (a1-a9) runs over all cells; each simulation keeps its own
+//      time step, remaining time and status flags; the meshes are updated for
+//      the moved points (a0) beside its last stages;
+//   7. simulations that reached t_end or their step budget are copied out
+//      and leave the batch; a failed step rolls back that simulation only;
+//   8. the updated meshes become the current ones.
 // The arithmetic of every cell depends only on its own simulation, so a
 // simulation's results do not depend on what else is in the batch.
 #include <algorithm>
@@ -472,6 +477,7 @@ rich::MeshArrays mesh_arrays(rich_batch *b, int q)
     a.slot_nb = m.slot_nb.as<int32_t>();
     a.ghost_src = m.ghost_src.as<int32_t>();
     a.ghost_img = m.ghost_img.as<int32_t>();
+    a.split = b->precision == RICH_FP32_SPLIT;
     return a;
 }
 
@@ -898,7 +904,7 @@ int pack_step(rich_batch *b, const std::vector<BatchSim *> &list, double &t1, do
         l.inst = b->instp.as<rich::InstParams>();
         l.bad = b->listbad.as<int32_t>();
         CUDA_TRY(cudaMemsetAsync(l.bad, 0, 4, b->stream));
-        CUDA_TRY(rich::launch_lists(l, b->stream));
+        CUDA_TRY(rich::launch_lists(l, true, b->stream));
         CUDA_TRY(cudaMemcpyAsync(b->list_flag(), l.bad, 4, cudaMemcpyDeviceToHost, b->stream));
         CUDA_TRY(cudaStreamSynchronize(b->stream));
         if (*b->list_flag()) return fail(RICH_ETESS, "the rings of a mesh do not close");

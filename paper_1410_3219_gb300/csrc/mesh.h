@@ -1,5 +1,7 @@
 // Host-side tessellation (paper Section 2.1) producing the connectivity the
-// device sweep consumes.
+// device sweep consumes: a simulation's first mesh, which the device then
+// updates from step to step (meshupdate.h), and the meshes that the update
+// leaves to the host.
 //
 //   1. ghost images of the real generating points inside a band of width w
 //      around the box: mirror images across reflecting walls (corners mirrored

@@ -25,7 +25,8 @@ __device__ __forceinline__ void clear_counters(int32_t *next, int32_t words)
 
 // mu::verify<true> with eight lanes per cell, a ring slot each: a thread per
 // cell walked its ring through a chain of dependent loads, slot after slot
-// (327 us at 1M cells; 24 us at 4,096).  Cells of more than eight neighbours
+// (327 us at 1M cells, 24 us at 4,096; now 170 to 330, by how many cells it
+// lists, and 9; bound by the latency of its gathers).  Cells of more than eight neighbours
 // (3 % of a random mesh) go to the undecided ones.  The warps loop over the
 // cells, four at a time, and have the next four's ring slots in flight.
 __global__ void __launch_bounds__(kVerifyBlock) k_mesh_verify(MeshUpdate m)
@@ -117,7 +118,8 @@ __global__ void __launch_bounds__(kVerifyBlock) k_mesh_verify(MeshUpdate m)
 
 // The cells FP32 left open, a warp each: a lane per ring slot, and for the
 // triangles of two images a lane per image that might lie in their circle.
-// (A thread per cell spent 127 us on the walls of 4,096 cells.)
+// (A thread per cell spent 127 us on the walls of 4,096 cells; now 18, one
+// cell's chain of FP64 and integer predicates.)
 __global__ void __launch_bounds__(kListBlock) k_mesh_verify_open(MeshUpdate m)
 {
     chained(m.n);
@@ -207,7 +209,8 @@ __device__ __forceinline__ bool commit_star(const MeshUpdate &m, const mu::Frame
 // mu::recompute_light for the first round's cells, a lane per candidate and
 // sixteen lanes per cell: the wrapping finds each next neighbour by a
 // tournament.  (A thread per cell took as long at 4,096 cells, 48 us, as at
-// 262,144: one cell's chain of steps.)
+// 262,144: one cell's chain of steps.  Now 11 us, and 32 to 50 with 7,500 to
+// 39,000 cells listed of 262,144, bound by instruction issue.)
 __global__ void __launch_bounds__(kListBlock) k_mesh_recompute_light(MeshUpdate m)
 {
     chained(m.n);
@@ -319,7 +322,8 @@ struct StarWork {
 // neighbour of the gift wrapping by a tournament of in-circle tests.  A step
 // lists a few hundred to a few per cent of the cells, so the pass is bound by
 // one cell's chain of dependent loads and tests: a thread per cell took 545 us
-// at 1M cells and 540 us for the wall cells of 4,096.
+// at 1M cells and 540 us for the wall cells of 4,096; now 13 us for 200 cells
+// at walls.
 __device__ void warp_recompute(const MeshUpdate &m, int32_t i, int32_t round, StarWork &w)
 {
     using namespace mu;
@@ -915,7 +919,8 @@ __device__ __noinline__ bool lists_of_any(const MeshLists &l, int32_t i, bool li
 // host built) number the edge and both triangles beside it, so every slot is
 // written once, by its own cell, and needs no clearing and no later check.
 // (Three kernels before: triangles and edges with a walk per triangle and
-// per edge, and a check of both, 153 us at 1M cells.)
+// per edge, and a check of both, 153 us at 1M cells with every block resident;
+// now 126 so, and 205 in the fewer blocks that run beside the FP64 stages.)
 __global__ void __launch_bounds__(128) k_mesh_lists(MeshLists l)
 {
     chained(l.n);
@@ -1024,18 +1029,21 @@ inline int blocks(int64_t n, int b) { return (int)((n + b - 1) / b); }
 // looping beyond `per SM` blocks on each of 152 SMs.  The update runs beside the
 // FP64 stages of a sweep, which keep their pace as long as they hold most of
 // the registers: at 1M cells a step and its read take 1.80 ms with 4 blocks
-// per SM, 1.87 with 8, 1.88 with 16 and 2.09 with 2; at 262,144 cells in split
-// precision, whose sweep is short, 1.10, 1.07, 1.08 and 1.19.
-inline int pass_blocks(int64_t n)
+// per SM, 1.87 with 8, 1.88 with 16 and 2.09 with 2.  A split-precision sweep is
+// over before the update, whose passes then count themselves: a step of 1M
+// cells takes 1.03 ms with 4, 0.83 with 8, 0.82 with 16 and 0.93 with every
+// block resident; of 640,000 cells 0.65, 0.55, 0.54 and 0.58; of 130,000 with 8
+// and 16 0.221 and 0.207.
+inline int pass_blocks(int64_t n, bool split)
 {
-    return std::max(1, std::min(blocks(8 * n, 128), 152 * (n >= (1 << 19) ? 4 : 8)));
+    return std::max(1, std::min(blocks(8 * n, 128), 152 * (split ? 16 : n >= (1 << 19) ? 4 : 8)));
 }
 
 }  // namespace
 
-cudaError_t launch_lists(const MeshLists &l, cudaStream_t st)
+cudaError_t launch_lists(const MeshLists &l, bool alone, cudaStream_t st)
 {
-    if (l.n > 0) return launch_chained(k_mesh_lists, pass_blocks(l.n), 128, st, l.n, l);
+    if (l.n > 0) return launch_chained(k_mesh_lists, pass_blocks(l.n, alone), 128, st, l.n, l);
     return cudaSuccess;
 }
 
@@ -1228,7 +1236,7 @@ cudaError_t MeshUpdater::launch_rounds(const MeshArrays &a, const MeshOutput &o,
     const int w = blocks(m.n, kWindow);
     MU_TRY(launch_chained(k_mesh_measure, w, kWindow, st, m.n, m, sums_.as<int4>(), (int32_t)(whole_ ? 1 : 0)));
     MU_TRY(launch_chained(k_mesh_offsets, w, kWindow, st, m.n, m, sums_.as<int4>(), (int32_t)last));
-    MU_TRY(launch_chained(k_mesh_rings, pass_blocks(m.n), 128, st, m.n, m));
+    MU_TRY(launch_chained(k_mesh_rings, pass_blocks(m.n, a.split), 128, st, m.n, m));
     MeshLists l = o.lists;
     l.n = a.n;
     l.cell_inst = a.cell_inst;
@@ -1245,7 +1253,7 @@ cudaError_t MeshUpdater::launch_rounds(const MeshArrays &a, const MeshOutput &o,
     l.bad = &m.count->bad;
     l.next = count_[1].as<int32_t>();
     l.next_words = (int32_t)(sizeof(MeshUpdateCount) / sizeof(int32_t)) + a.n_inst;
-    MU_TRY(launch_lists(l, st));
+    MU_TRY(launch_lists(l, a.split, st));
     return cudaMemcpyAsync(host_.p, count_[0].p, sizeof(MeshUpdateCount) + (size_t)a.n_inst * sizeof(int32_t),
                            cudaMemcpyDeviceToHost, st);
 }
@@ -1265,7 +1273,7 @@ cudaError_t MeshUpdater::start(const MeshArrays &a, const MeshOutput &o, cudaStr
     std::swap(count_[0].p, count_[1].p);
     std::swap(count_[0].cap, count_[1].cap);
     const MeshUpdate m = params(a, o);
-    MU_TRY(launch_chained(k_mesh_verify, pass_blocks(a.n), kVerifyBlock, st, m.n, m));
+    MU_TRY(launch_chained(k_mesh_verify, pass_blocks(a.n, a.split), kVerifyBlock, st, m.n, m));
     // (a warp per eight cells: steps of 10,201 cells took 105 us with one per
     // sixteen, 98 with this.  With the list passes at eight as well their FP64
     // tests slow the gradient of 4,096 cells, which runs beside them)

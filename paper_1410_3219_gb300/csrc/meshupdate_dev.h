@@ -21,6 +21,7 @@ struct MeshArrays {
     const int32_t *cell_inst;  // nullptr: one simulation
     const double *x, *y;
     const int32_t *cell_ptr, *slot_nb, *ghost_src, *ghost_img;
+    bool split;  // the sweep beside the update is a split-precision one
 };
 
 struct MeshSizes {
@@ -50,7 +51,8 @@ struct MeshLists {
     int32_t *bad;
     int32_t *next = nullptr, next_words = 0;  // words to clear (an update's next counters)
 };
-cudaError_t launch_lists(const MeshLists &l, cudaStream_t st);
+// (alone: no FP64 stages run beside)
+cudaError_t launch_lists(const MeshLists &l, bool alone, cudaStream_t st);
 
 // The updated mesh (cell_ptr, slot_nb, ghost_src and ghost_img apart from
 // the mesh being updated), the room its arrays have, and its lists' arrays.

@@ -1,7 +1,8 @@
 // C ABI of the library (include/rich.h): owns the device memory of a
-// simulation, runs the host tessellation (a0) and enqueues the device sweep
-// (a1-a9) on a CUDA stream.  There is no CPU fallback: without a CUDA device
-// rich_init_mesh fails with RICH_ENODEV.
+// simulation, builds its first mesh on the host (a0), and enqueues the device
+// sweep (a1-a9) and the mesh's update for the moved points (a0) on CUDA
+// streams.  There is no CPU fallback: without a CUDA device rich_init_mesh
+// fails with RICH_ENODEV.
 #include <array>
 #include <chrono>
 #include <climits>
@@ -81,8 +82,8 @@ struct rich_sim {
     rich_config cfg{};
     int32_t n = 0;
     std::vector<int32_t> perm;  // internal -> caller index
-    // host copy of the points (internal order), page-locked: x at [0, n),
-    // y at [n, 2n), then the dt of the sweep that moved them
+    // host copy of the points (internal order) for the host builder,
+    // page-locked: x at [0, n), y at [n, 2n)
     rich::HBuf hpts;
     double *hx() const { return hpts.as<double>(); }
     double *hy() const { return hpts.as<double>() + n; }
@@ -224,6 +225,7 @@ struct rich_sim {
         a.slot_nb = mesh[mcur].slot_nb.as<int32_t>();
         a.ghost_src = mesh[mcur].ghost_src.as<int32_t>();
         a.ghost_img = mesh[mcur].ghost_img.as<int32_t>();
+        a.split = cfg.precision == RICH_FP32_SPLIT;
         return a;
     }
     int32_t periodic() const { return cfg.boundary == RICH_BC_PERIODIC ? 1 : 0; }
@@ -319,7 +321,7 @@ int upload_mesh(rich_sim *s, rich_step_info *info)
     rich::MeshLists l = d.lists(s->n, s->periodic());
     l.bad = reinterpret_cast<int32_t *>(s->scal.as<char>() + 24);
     CUDA_TRY(cudaMemsetAsync(l.bad, 0, sizeof(int32_t), s->stream));
-    CUDA_TRY(rich::launch_lists(l, s->stream));
+    CUDA_TRY(rich::launch_lists(l, true, s->stream));
     CUDA_TRY(cudaMemcpyAsync(s->back.p, l.bad, sizeof(int32_t), cudaMemcpyDeviceToHost, s->stream));
     CUDA_TRY(cudaStreamSynchronize(s->stream));
     if (*s->back.as<int32_t>()) return fail(RICH_ETESS, "the rings of the mesh do not close");
@@ -336,8 +338,8 @@ bool can_update(const rich_sim *s)
 }
 
 // Enqueue the update of the mesh for the points in buffers q, on the mesh
-// stream after ev (recorded on the handle's stream once those points are
-// there); the handle's stream continues after it (join_update).
+// stream after what the handle's stream holds by now; join_update makes the
+// handle's stream continue after it.
 int start_update(rich_sim *s, int q)
 {
     rich::MeshStream &u = s->mesh_stream;
@@ -508,7 +510,7 @@ static int create_sim(const rich_config *cfg, int64_t n, const double *x, const 
     }
     int rc = RICH_OK;
     auto bail = [&](int code) { delete s; return code; };
-    if (s->hpts.ensure((2 * (size_t)n + 1) * sizeof(double)) != cudaSuccess)
+    if (s->hpts.ensure(2 * (size_t)n * sizeof(double)) != cudaSuccess)
         return bail(fail(RICH_ENOMEM, "page-locked host points"));
     std::vector<double> Fh(4 * (size_t)n);
     double *hx = s->hx(), *hy = s->hy();
@@ -1025,7 +1027,7 @@ int rich_edge_list_check(const rich_config *cfg, int64_t n, const double *x, con
         l.edge_l = el.as<int32_t>(); l.edge_r = er.as<int32_t>();
         l.edge_ta = eta.as<int32_t>(); l.edge_tb = etb.as<int32_t>();
         l.bad = bad.as<int32_t>();
-        e = rich::launch_lists(l, st);
+        e = rich::launch_lists(l, true, st);
     }
     auto down = [&](std::vector<int32_t> &h, DBuf &d) {
         if (e == cudaSuccess && !h.empty())

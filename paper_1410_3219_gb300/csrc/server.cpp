@@ -16,8 +16,8 @@
 //          its own batch (own CUDA stream) in a loop; the lanes share one
 //          pool of host workers task by task, the lanes of larger requests
 //          first.  Requests go to a lane by size, so a small request's step
-//          never waits for the whole host tessellation of a large one, and
-//          one lane's host work overlaps another lane's device sweep.
+//          never waits for the first host tessellation of a large one, and
+//          one lane's host work overlaps another lane's device work.
 //          Admission against the shared cell budget stays in arrival order
 //          within a lane.
 #include <algorithm>

@@ -1,4 +1,4 @@
-// A small persistent worker pool for the host side of the steps: the
+// A small persistent worker pool for the host's share of the work: the
 // tessellation (a0) tiles of one simulation, or the independent
 // simulations of a batch, run on all host cores.  parallel_for hands out
 // task indices dynamically (an atomic counter), so tasks of very different
