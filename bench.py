@@ -1,11 +1,11 @@
 """Benchmark of the moving-Voronoi-mesh sweep (cell-updates per second).
 
-One step = the host tessellation (a0, timed separately) followed by the
-device sweep a1-a9.  `value` is real cells x steps / summed device time of
+One step = the mesh update (a0, timed separately) followed by the device sweep
+a1-a9.  `value` is real cells x steps / summed device time of
 the sweeps (CUDA events on the launching stream, inputs resident in HBM, L2
 flushed before every timed sweep).  `e2e` is the same metric through the
-public C ABI call a user makes (rich_step with the host tessellation and all
-host<->device copies, plus a host read of the step's result).
+public C ABI call a user makes (rich_step, whose mesh update runs on the device
+beside the sweep, plus a host read of the step's result).
 
 Usage: python bench.py [--gpus N] [--steps K] [--warmup W] [--workload NAME]
        python bench.py --impl reference ...   (the CPU oracle, bounded sample)
@@ -42,20 +42,26 @@ HBM_PEAK_GBS_FALLBACK = 6800.0
 COMPULSORY_BYTES_PER_CELL = 124
 # kernels launched by one sweep
 NUM_KERNELS = 6
+# what a step copies beside the state that is read: the parameter record of
+# one simulation, and the mesh update's counters with one simulation's flag
+INST_PARAM_BYTES = 216
+MESH_COUNTER_BYTES = 92
 
 # Algorithmic floating-point operations of each kernel, counted from the
 # formulas as the kernels evaluate them: add, subtract, multiply = 1, fused
 # multiply-add = 2, divide, square root and reciprocal square root = 1 (the
 # extra FMAs that refine a reciprocal are not counted); compares, min/max,
 # sign flips and the FP64 <-> FP32 conversions run on the integer pipe and
-# are not counted.  Per unit kind (triangle, edge, cell, ring slot) and pipe.
+# are not counted, nor what FP32 estimates decide and how many FP64 values
+# those decisions still ask for (Courant candidates, limiter differences).  Per
+# unit kind (triangle, edge, cell, ring slot) and pipe.
 FLOPS = {
     "fp64": {
         "k_circumcentre": {"tri": {"fp64": 25}},
-        "k_geometry": {"edge": {"fp64": 32}, "cell": {"fp64": 52}, "slot": {"fp64": 11}},
+        "k_geometry": {"edge": {"fp64": 32}, "cell": {"fp64": 40}, "slot": {"fp64": 11}},
         "k_advance_points": {"cell": {"fp64": 5}},
-        "k_cell_gradient": {"cell": {"fp64": 67}, "slot": {"fp64": 33}},
-        "k_edge_flux": {"edge": {"fp64": 177}},
+        "k_cell_gradient": {"cell": {"fp64": 77}, "slot": {"fp64": 18}},
+        "k_edge_flux": {"edge": {"fp64": 147}},
         "k_cell_update": {"cell": {"fp64": 17}, "slot": {"fp64": 4}},
     },
     "split": {
@@ -338,9 +344,8 @@ def run_ours(args):
             return ms, dict(info, tess_ms=tms), kt
 
         # W warm-up steps; before the first timed run, also warmup_seconds
-        # of steps of throwaway copies of the run (the steps are mostly host
-        # tessellation; on a fresh box the first seconds of FP64 kernels ran
-        # ~4 % slow)
+        # of steps of throwaway copies of the run (on a fresh box the first
+        # seconds of FP64 kernels ran ~4 % slow)
         if not warm_state["done"] and args.warmup_seconds > 0:
             t_warm = time.perf_counter()
             while time.perf_counter() - t_warm < args.warmup_seconds:
@@ -409,8 +414,8 @@ def run_ours(args):
     value = head["value"]
     head_prec = "split" if precs[0] == "split" else "fp64"
 
-    # end to end through the public API: rich_step (host tessellation, copies,
-    # sweep) plus a host read of the step's result
+    # end to end through the public API: rich_step (mesh update and sweep)
+    # plus a host read of the step's result
     # (the same K timed steps after the same W warm-up steps as the device
     # measurement, each a whole step with its copies)
     e2e_steps = max(2, args.steps)
@@ -437,15 +442,12 @@ def run_ours(args):
             phases[k] = phases.get(k, 0.0) + v / e2e_steps
         rc = L.rich_get_conserved(sim2.h, n, *[b.ctypes.data_as(Dp) for b in bufs])
         assert rc == 0
-        # what rich_tessellate uploads: ghost positions, sources, mirror
-        # flags and shifts; ring offsets, processing order, first owned
-        # edge and first owned triangle per cell; ring neighbours (the
-        # triangle and edge lists themselves are built on the device)
-        h2d = (28 * info["n_ghost"] + 4 * (n + 1) + 4 * n + 4 * (n + 1) + 4 * (n + 1)
-               + 4 * info["n_slots"])
-        # down: the moved points and dt read early, the mesh builds' two
-        # check flags, the step's dt and status, the conserved state read
-        d2h = (16 * n + 8) + 8 + 12 + 48 * n
+        # up: the simulation's parameters with the step's remaining time (the
+        # state and the mesh stay on the device)
+        h2d = INST_PARAM_BYTES
+        # down: the step's dt and status, the mesh update's counters, the
+        # conserved state read
+        d2h = 12 + MESH_COUNTER_BYTES + 48 * n
     e2e_s = time.perf_counter() - t0
     e2e_s = max_over_ranks(e2e_s, ws)
     e2e_val = job_value(ws, n * e2e_steps, e2e_s)
@@ -530,9 +532,7 @@ def run_batched(rich, precision, n_inst, steps, seed=4):
         wl["cfg"]["precision"] = precision
         b.add(wl, max_steps=1 << 40)
     cells = sum(len(wl["x"]) for wl in wls)
-    # the autotuner's 8 trial steps, then 2 steps in the chosen shape (the
-    # first of them tessellates twice: its own points, which the persistent
-    # trials left unmeshed, and the next step's during its sweep)
+    # the autotuner's 8 trial steps, then 2 steps in the chosen shape
     for _ in range(8 + 2):
         b.step()
     sweep_ms, tess_ms, copy_ms, wall = [], [], [], []
@@ -558,9 +558,7 @@ def run_batched(rich, precision, n_inst, steps, seed=4):
             "host_other_ms_per_step": float(np.mean(copy_ms)),
             "e2e": {"value": cells * steps / (sum(wall) / 1e3), "unit": UNIT,
                     "wall_ms_per_step": float(np.mean(wall))},
-            # (host tessellation + other host work + device sweep) / wall: above
-            # 1 where the host's tessellation of the next step runs beside the
-            # sweep's last stages
+            # (mesh time beyond the sweep + other host work + device sweep) / wall
             "host_device_overlap": float((np.mean(tess_ms) + np.mean(copy_ms) + np.mean(sweep_ms)) / np.mean(wall)),
             "launch": {"persistent": li["persistent"], "block": li["block"], "grid": li["grid"],
                        "graph_replay": li["graph"]},

@@ -104,8 +104,8 @@ typedef struct {
     double t;           /* simulation time after the call */
     double dt_last;     /* last time step */
     double sweep_ms;    /* device time of steps a1-a9 summed over the call (CUDA events) */
-    double tess_ms;     /* time of a0 summed over the call: host builds (wall), updates on the device (their checks
-                           by CUDA events, and the host's time to enqueue the rest) */
+    double tess_ms;     /* time of a0 summed over the call: host builds (wall), updates on the device (what they
+                           take beyond the end of the sweep they run beside, and the host's time for them) */
     double copy_ms;     /* host time spent in host<->device copies and waits */
     int64_t n_ghost, n_tri, n_edges, n_slots; /* size of the last tessellation */
 } rich_step_info;
@@ -127,12 +127,10 @@ int rich_init_mesh(const rich_config *cfg, int64_t n, const double *x, const dou
 
 /* Advance up to max_steps steps, stopping early once the time reaches t_end
    (the last step is shortened to land on t_end).  Each step: a1-a9 on the
-   device for the current points and mesh, then a0 for the moved points
-   (twice, with a0 for the half-step points in between, in the time-centred
-   scheme).  A step that does not land on t_end thus leaves the mesh of its
-   points updated, and the next step or call starts with the sweep; the device
-   may still be writing that mesh when the call returns, and later calls wait
-   for it.  A mesh left to the host (see rich_tessellate) is built by the next
+   device for the current points and mesh, and a0 for the moved points beside
+   the stages after the point motion (twice, the first time for the half-step
+   points, in the time-centred scheme).  A step thus leaves the mesh of its
+   points updated, and the next step or call starts with the sweep.  A mesh left to the host (see rich_tessellate) is built by the next
    step or call.  Results equal those of rich_tessellate / rich_sweep / rich_sync in
    turn, bit for bit.  info may be NULL.
    Errors: RICH_ENEGATIVE / RICH_ENAN (state left at the last good step),
@@ -241,10 +239,11 @@ int64_t rich_num_cells(const rich_sim *s);
 
 /* A batch advances many independent simulations (different sizes, problems
    and scheme parameters, one precision) with ONE device sweep per step over
-   all their cells: each step tessellates every simulation on a pool of host
-   threads, packs the meshes into one index space with a per-cell simulation
-   id, and runs steps a1-a9 once; every simulation keeps its own time step,
-   end time, step budget and status.  A cell's arithmetic depends only on its
+   all their cells: newly admitted simulations are tessellated on a pool of
+   host threads and packed with the others into one index space with a per-cell
+   simulation id, steps a1-a9 run once, and the meshes of the moved points are
+   updated on the device; every simulation keeps its own time step, end time,
+   step budget and status.  A cell's arithmetic depends only on its
    own simulation, so results are identical alone and in any mix.  The batch
    owns its device memory and stream. */
 typedef struct rich_batch rich_batch;
@@ -268,13 +267,14 @@ int rich_batch_add(rich_batch *b, const rich_config *cfg, int64_t n, const doubl
                    int64_t max_steps, int32_t *id);
 
 /* One step of every pending or running simulation.  The meshes of the moved
-   points are updated on the device after the sweep; a step with the same
+   points are updated on the device beside the sweep; a step with the same
    simulations as the last then starts with the sweep, and one with others
    reads those meshes back and packs them with the host-built ones of the
    newly admitted simulations.
    info (nullable): steps_done = simulations stepped, sweep_ms = device time
-   of the sweep, tess_ms = time of the host tessellations and of the mesh
-   updates, copy_ms = other host time outside the sweep. */
+   of the sweep (with what the mesh update beside it slows it down), tess_ms =
+   time of the host tessellations and of the mesh update beyond the sweep's
+   end, copy_ms = other host time outside the sweep. */
 int rich_batch_step(rich_batch *b, rich_step_info *info);
 
 /* State (RICH_SIM_*), error code of a failed simulation, its time and steps
@@ -376,8 +376,8 @@ int rich_server_fetch(rich_server *s, int64_t req, int64_t n, double *x, double 
    the server's host threads task by task, the lanes of larger requests
    first.  A request goes to lane k when its cell count is at
    least split_cells * 8^(k-1) (lane 0 below split_cells), so small requests
-   never wait on the host tessellation of large ones, and one lane's host
-   tessellation overlaps another's device sweep.  Admission takes each
+   never wait on the first host tessellation of large ones, and one lane's host
+   work overlaps another's device work.  Admission takes each
    lane's queue in arrival order against the shared cell budget; the lane of
    the largest requests also holds at most top_lane_cells cells at once (a
    larger request alone; 0: no limit but the budget), so that its requests
@@ -389,10 +389,9 @@ int rich_server_fetch(rich_server *s, int64_t req, int64_t n, double *x, double 
 int rich_server_start(rich_server *s, int32_t lanes, int64_t split_cells, int64_t top_lane_cells);
 
 /* Totals over the server's steps (each output may be NULL): batched steps
-   taken by all lanes, summed device sweep time, host tessellation time and
-   other host time (ms), and the wall time since rich_server_start (ms; 0 in
-   tick mode).  (sweep + tessellation) / wall above one shows host and
-   device work overlapping. */
+   taken by all lanes, summed device sweep time, tessellation time (tess_ms of
+   rich_batch_step) and other host time (ms), and the wall time since
+   rich_server_start (ms; 0 in tick mode). */
 int rich_server_stats(rich_server *s, int64_t *steps, double *sweep_ms, double *tess_ms, double *other_ms,
                       double *wall_ms);
 
