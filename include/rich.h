@@ -254,7 +254,7 @@ typedef struct rich_batch rich_batch;
 #define RICH_SIM_FAILED 3   /* a step or a tessellation failed; last good state kept */
 
 /* max_cells: admission budget (cells of pending + running simulations);
-   device memory grows to about 1 KiB per admitted cell.  host_threads <= 0:
+   device memory grows to about 1.3 KiB per admitted cell.  host_threads <= 0:
    one per hardware thread.  Errors: RICH_EINVAL, RICH_ENODEV, RICH_ECUDA. */
 int rich_batch_create(int32_t precision, int64_t max_cells, int32_t host_threads, rich_batch **out);
 
