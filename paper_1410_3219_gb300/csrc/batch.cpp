@@ -994,10 +994,11 @@ int rich_batch_step(rich_batch *b, rich_step_info *info)
         }
     }
     if (update && shape.persistent && (rc = start_update(b, 1 - b->cur))) return rc;
-    if (update && (rc = join_update(b))) return rc;
-    CUDA_TRY(cudaEventRecord(b->ev2, b->stream));
+    // (copied while the update still runs)
     CUDA_TRY(cudaMemcpyAsync(b->dt_back(), b->dtout.p, ok.size() * 8, cudaMemcpyDeviceToHost, b->stream));
     CUDA_TRY(cudaMemcpyAsync(b->status_back(), b->status.p, ok.size() * 4, cudaMemcpyDeviceToHost, b->stream));
+    if (update && (rc = join_update(b))) return rc;
+    CUDA_TRY(cudaEventRecord(b->ev2, b->stream));
     CUDA_TRY(cudaStreamSynchronize(b->stream));
     float ms = 0.0f;
     cudaEventElapsedTime(&ms, b->ev0, b->ev1);

@@ -655,17 +655,20 @@ static int launch_sweep(rich_sim *s, double t_end, bool update)
 
 int rich_sweep(rich_sim *s, double t_end) { return launch_sweep(s, t_end, false); }
 
-int rich_sync(rich_sim *s, rich_step_info *info)
+// The sweep's dt and status, into page-locked memory (dt, then the status)
+static int fetch_result(rich_sim *s)
 {
-    rich::Range range("rich sync");
-    if (!s) return fail(RICH_EINVAL, "NULL handle");
-    if (!s->pending) return fail(RICH_ESTATE, "no sweep pending");
+    CUDA_TRY(cudaMemcpyAsync(s->back.as<double>() + 1, s->scal.as<char>() + 8, 12, cudaMemcpyDeviceToHost, s->stream));
+    return RICH_OK;
+}
+
+// rich_sync after fetch_result
+static int wait_sweep(rich_sim *s, rich_step_info *info)
+{
     double t0 = now_ms();
     char *sc = s->scal.as<char>();
-    // (into page-locked memory: dt, then the status)
-    double *dt_host = s->back.as<double>() + 1;
-    int32_t *status_host = reinterpret_cast<int32_t *>(dt_host + 1);
-    CUDA_TRY(cudaMemcpyAsync(dt_host, sc + 8, 12, cudaMemcpyDeviceToHost, s->stream));
+    const double *dt_host = s->back.as<double>() + 1;
+    const int32_t *status_host = reinterpret_cast<const int32_t *>(dt_host + 1);
     CUDA_TRY(cudaStreamSynchronize(s->stream));
     const double dt = *dt_host;
     const int32_t status = *status_host;
@@ -714,6 +717,15 @@ int rich_sync(rich_sim *s, rich_step_info *info)
     return RICH_OK;
 }
 
+int rich_sync(rich_sim *s, rich_step_info *info)
+{
+    rich::Range range("rich sync");
+    if (!s) return fail(RICH_EINVAL, "NULL handle");
+    if (!s->pending) return fail(RICH_ESTATE, "no sweep pending");
+    const int rc = fetch_result(s);
+    return rc != RICH_OK ? rc : wait_sweep(s, info);
+}
+
 // One sweep of rich_step: the update of the mesh for the moved points runs on
 // the mesh stream beside the gradients, fluxes and update, from when the
 // points are there (those stages leave the memory pipes and the FP32 and
@@ -728,8 +740,10 @@ static int step_sweep(rich_sim *s, double t_end, rich_step_info *info)
     const bool update = !still && can_update(s);
     int rc = launch_sweep(s, t_end, update);
     if (rc != RICH_OK) return rc;
+    // (the sweep's result is copied while the update still runs)
+    if ((rc = fetch_result(s)) != RICH_OK) return rc;
     if (update && (rc = join_update(s)) != RICH_OK) return rc;
-    rc = rich_sync(s, info);
+    rc = wait_sweep(s, info);
     if (still && rc == RICH_OK) {
         s->tess_current = true;
         report_sizes(s, info);
