@@ -45,7 +45,7 @@ NUM_KERNELS = 6
 # what a step copies beside the state that is read: the parameter record of
 # one simulation, and the mesh update's counters with one simulation's flag
 INST_PARAM_BYTES = 216
-MESH_COUNTER_BYTES = 92
+MESH_COUNTER_BYTES = 96
 
 # Algorithmic floating-point operations of each kernel, counted from the
 # formulas as the kernels evaluate them: add, subtract, multiply = 1, fused

@@ -73,6 +73,7 @@ struct MeshUpdateCount {
     int32_t slots, edges, tris, ghosts;
     int32_t ready;                   // the rounds are done and the new mesh fits its arrays
     int32_t bad;                     // the lists of the new mesh do not close
+    int32_t done;                    // blocks that have written their lists
 };
 
 struct MeshUpdate {

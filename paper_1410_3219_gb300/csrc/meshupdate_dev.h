@@ -50,6 +50,11 @@ struct MeshLists {
     const int32_t *ready;       // nullptr, or 0 there: nothing is built
     int32_t *bad;
     int32_t *next = nullptr, next_words = 0;  // words to clear (an update's next counters)
+    // the update's counters, which the last block copies to page-locked memory
+    // (`done` counts the blocks and is left at zero)
+    int32_t *report = nullptr, *done = nullptr;
+    const int32_t *counters = nullptr;
+    int32_t words = 0;
 };
 // (alone: no FP64 stages run beside)
 cudaError_t launch_lists(const MeshLists &l, bool alone, cudaStream_t st);
