@@ -43,6 +43,19 @@ RICH_HD inline uint64_t bits_of(double v)
 #endif
 }
 
+// 2^k for |k| <= 1022
+RICH_HD inline double pow2(int k)
+{
+    const uint64_t b = (uint64_t)(1023 + k) << 52;
+#ifdef __CUDA_ARCH__
+    return __longlong_as_double((long long)b);
+#else
+    double v;
+    std::memcpy(&v, &b, 8);
+    return v;
+#endif
+}
+
 RICH_HD inline uint64_t mul_hi(uint64_t a, uint64_t b)
 {
 #ifdef __CUDA_ARCH__

@@ -74,10 +74,9 @@ __global__ void __launch_bounds__(kVerifyBlock) k_mesh_verify(MeshUpdate m)
         const float p = b.fx * d.fy, q = b.fy * d.fx, cbd = p - q;
         const float p3 = a.fx * d.fy, p4 = a.fy * d.fx, p5 = a.fx * b.fy, p6 = a.fy * b.fx;
         const float det = a.l * cbd - b.l * (p3 - p4) + d.l * (p5 - p6);
-        const float bound = kCircleBound * (a.l * (fabsf(p) + fabsf(q)) + b.l * (fabsf(p3) + fabsf(p4)) +
-                                            d.l * (fabsf(p5) + fabsf(p6)));
+        const float bound = circle_error(a.l, p, q, b.l, p3, p4, d.l, p5, p6);
         bool bad = -det > bound;
-        bool open = !small || !(cbd > kCrossBound * (fabsf(p) + fabsf(q))) || !(det > bound || bad);
+        bool open = !small || !(cbd > cross_error(p, q)) || !(det > bound || bad);
         if (!f.periodic) open = open || ((b.ref & 15) != 4 && (d.ref & 15) != 4);
         open = live && open && (mine || !small);
         bad = bad && mine;
@@ -148,7 +147,7 @@ __global__ void __launch_bounds__(kListBlock) k_mesh_verify_open(MeshUpdate m)
                     list_bad(m, f.periodic, a.ref, b.ref, d.ref);
                     self = true;
                 }
-                if (d.ref != ref || !disk_ok(f, b, d)) self = true;
+                if (d.ref != ref || !disk_ok_any(f, b, d)) self = true;
                 turns += (b.fy < 0.0f && d.fy >= 0.0f) ? 1 : 0;
                 pair = !f.periodic && (b.ref & 15) != 4 && (d.ref & 15) != 4;
             }
@@ -260,7 +259,7 @@ __global__ void __launch_bounds__(kListBlock) k_mesh_recompute_light(MeshUpdate 
             a.fx = __shfl_sync(kAll, d.fx, first + last);
             a.fy = __shfl_sync(kAll, d.fy, first + last);
             a.l = a.fx * a.fx + a.fy * a.fy;
-            const float p = a.fx * d.fy, q = a.fy * d.fx, cr = p - q, cb = kCrossBound * (fabsf(p) + fabsf(q));
+            const float p = a.fx * d.fy, q = a.fy * d.fx, cr = p - q, cb = cross_error(p, q);
             const bool cand = mine && c != last;
             bool unsure = cand && !(cr > cb) && !(-cr > cb);
             int best = cand && cr > cb ? c : -1;
@@ -282,8 +281,7 @@ __global__ void __launch_bounds__(kListBlock) k_mesh_recompute_light(MeshUpdate 
                 const float p1 = b.fx * e.fy, p2 = b.fy * e.fx, p3 = a.fx * e.fy, p4 = a.fy * e.fx, p5 = a.fx * b.fy,
                             p6 = a.fy * b.fx;
                 const float det = a.l * (p1 - p2) - b.l * (p3 - p4) + e.l * (p5 - p6);
-                const float bound = kCircleBound * (a.l * (fabsf(p1) + fabsf(p2)) + b.l * (fabsf(p3) + fabsf(p4)) +
-                                                    e.l * (fabsf(p5) + fabsf(p6)));
+                const float bound = circle_error(a.l, p1, p2, b.l, p3, p4, e.l, p5, p6);
                 if (-det > bound) best = other;
                 else if (!(det > bound)) unsure = true;
             }
@@ -440,8 +438,7 @@ __device__ void warp_recompute(const MeshUpdate &m, int32_t i, int32_t round, St
         const float p1 = pb.fx * pd.fy, p2 = pb.fy * pd.fx, p3 = a.fx * pd.fy, p4 = a.fy * pd.fx, p5 = a.fx * pb.fy,
                     p6 = a.fy * pb.fx;
         const float det = a.l * (p1 - p2) - pb.l * (p3 - p4) + pd.l * (p5 - p6);
-        const float bound = kCircleBound * (a.l * (fabsf(p1) + fabsf(p2)) + pb.l * (fabsf(p3) + fabsf(p4)) +
-                                            pd.l * (fabsf(p5) + fabsf(p6)));
+        const float bound = circle_error(a.l, p1, p2, pb.l, p3, p4, pd.l, p5, p6);
         if (det > bound) return false;
         if (-det > bound) return true;
         return circle_slow(f, point_of(f, a.ref), point_of(f, pb.ref), point_of(f, pd.ref)) > 0;
@@ -460,7 +457,7 @@ __device__ void warp_recompute(const MeshUpdate &m, int32_t i, int32_t round, St
         for (int c = lane; c < nc; c += 32) {
             if (c == last || w.ref[c] < 0) continue;
             const float p = a.fx * w.fy[c], q = a.fy * w.fx[c], cr = p - q;
-            const float cb = kCrossBound * (fabsf(p) + fabsf(q));
+            const float cb = cross_error(p, q);
             bool left = cr > cb;
             if (!left && !(-cr > cb)) left = orient_slow(f, point_of(f, a.ref), point_of(f, w.ref[c])) > 0;
             if (left && (best < 0 || inside(a, best, c))) best = c;
@@ -476,7 +473,7 @@ __device__ void warp_recompute(const MeshUpdate &m, int32_t i, int32_t round, St
             break;
         }
         const Point b = at_of(best);
-        if (lane == 0 && !disk_ok(f, a, b)) a_or(f.flags, MU_FAR);
+        if (lane == 0 && !disk_ok_any(f, a, b)) a_or(f.flags, MU_FAR);
         turns += (a.fy < 0.0f && b.fy >= 0.0f) ? 1 : 0;
         last = best;
     } while (last != near);

@@ -55,6 +55,7 @@ constexpr int kMaxCand = 96;    // candidates of a recomputed cell
 constexpr int kMaxSources = 256;  // cells of its neighbours' rings, repeats included (device)
 constexpr int kMaxExtra = 8;    // vertices another cell can tell it of per round
 constexpr int kMaxRounds = 12;  // rounds before the host takes over
+constexpr int kMaxShift = 800;  // exponents to_float scales by
 
 enum : int32_t {
     MU_FAR = 1,       // a circumdisk near or beyond the ghost band
@@ -150,8 +151,9 @@ RICH_HD inline double image_coord(double v, double lo, double hi, int a, bool pe
     return a > 0 ? v + (hi - lo) : v - (hi - lo);
 }
 
-// One cell's frame: its position, its simulation's box, and a length scale
-// that keeps FP32 products of neighbour offsets in range.
+// One cell's frame: its position, its simulation's box, and the power of two
+// by which neighbour offsets are scaled for FP32 (a mean spacing becomes one
+// to two).
 struct Frame {
     const MeshUpdate *m;
     int32_t i;
@@ -159,7 +161,8 @@ struct Frame {
     double xi, yi;
     double x0, x1, y0, y1;  // box
     float half_x, half_y;   // half its sides (scaled)
-    float scale, rlim2, rper2, reach;
+    int32_t shift;
+    float rlim2, rper2, reach;
     bool periodic;
 };
 
@@ -177,7 +180,7 @@ RICH_HD inline Frame frame_of(const MeshUpdate &m, int32_t i)
     f.yi = m.y[i];
     f.x0 = ip.x0; f.x1 = ip.x1; f.y0 = ip.y0; f.y1 = ip.y1;
     f.half_x = ip.half_x; f.half_y = ip.half_y;
-    f.scale = ip.mesh_scale;
+    f.shift = ip.mesh_shift;
     f.rlim2 = ip.mesh_rlim2;
     f.rper2 = ip.mesh_rper2;
     f.reach = ip.mesh_reach;
@@ -191,22 +194,24 @@ struct Point {
     int32_t ref;
 };
 
-// v in FP32 with its mantissa cut to 24 bits, on the integer pipe (FP64 to
-// FP32 conversions issue on the FP64 pipe); below FP32's normal range zero,
-// above it infinite
-RICH_HD inline float to_float(double v)
+// v 2^k (|k| <= kMaxShift) in FP32 with its mantissa cut to 24 bits, on the
+// integer pipe (FP64 to FP32 conversions issue on the FP64 pipe); below FP32's
+// normal range zero, above it infinite.  The scaling comes first, so that the
+// range is about the point spacing whatever the box's units.
+RICH_HD inline float to_float(double v, int32_t k)
 {
 #ifdef __CUDA_ARCH__
     const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
-    const unsigned e = (hi >> 20) & 0x7ffu;
-    unsigned u = __funnelshift_l(lo, hi, 3) - 0xc0000000u;
-    u = e < 897u ? 0u : (e > 1150u ? 0x7f800000u : u);
+    const int e = (int)((hi >> 20) & 0x7ffu) + k;
+    unsigned u = __funnelshift_l(lo, hi, 3) + ((unsigned)k << 23) - 0xc0000000u;
+    u = e < 897 ? 0u : (e > 1150 ? 0x7f800000u : u);
     return __uint_as_float((u & 0x7fffffffu) | (hi & 0x80000000u));
 #else
     const uint64_t b = exactint::bits_of(v);
-    const unsigned hi = (unsigned)(b >> 32), lo = (unsigned)b, e = (hi >> 20) & 0x7ffu;
-    unsigned u = ((hi << 3) | (lo >> 29)) - 0xc0000000u;
-    u = e < 897u ? 0u : (e > 1150u ? 0x7f800000u : u);
+    const unsigned hi = (unsigned)(b >> 32), lo = (unsigned)b;
+    const int e = (int)((hi >> 20) & 0x7ffu) + k;
+    unsigned u = ((hi << 3) | (lo >> 29)) + ((unsigned)k << 23) - 0xc0000000u;
+    u = e < 897 ? 0u : (e > 1150 ? 0x7f800000u : u);
     u = (u & 0x7fffffffu) | (hi & 0x80000000u);
     float f;
     std::memcpy(&f, &u, 4);
@@ -231,19 +236,19 @@ RICH_HD inline Point point_of(const Frame &f, int32_t ref)
             p.y = image_coord(p.y, f.y0, f.y1, img / 3 - 1, false);
         }
     }
-    p.fx = to_float(p.x - f.xi) * f.scale;
-    p.fy = to_float(p.y - f.yi) * f.scale;
+    p.fx = to_float(p.x - f.xi, f.shift);
+    p.fy = to_float(p.y - f.yi, f.shift);
     if (f.periodic) {
         int a = 0, b = 0;
         if (fabsf(p.fx) > f.half_x) {
             a = p.fx > 0.0f ? -1 : 1;
             p.x = image_coord(p.x, f.x0, f.x1, a, true);
-            p.fx = to_float(p.x - f.xi) * f.scale;
+            p.fx = to_float(p.x - f.xi, f.shift);
         }
         if (fabsf(p.fy) > f.half_y) {
             b = p.fy > 0.0f ? -1 : 1;
             p.y = image_coord(p.y, f.y0, f.y1, b, true);
-            p.fy = to_float(p.y - f.yi) * f.scale;
+            p.fy = to_float(p.y - f.yi, f.shift);
         }
         p.ref = src * 16 + (a + 1) + 3 * (b + 1);
     }
@@ -251,12 +256,25 @@ RICH_HD inline Point point_of(const Frame &f, int32_t ref)
     return p;
 }
 
-// FP32 determinants of offsets, each offset within 3 2^-24 of its value (cut,
-// then scaled): a product of two is within 7 2^-24 and the cross product's
-// error below 9 2^-24 = 5.4e-7 of its permanent; |a|^2 is within 9 2^-24, and
-// the in-circle sum within 22 2^-24 = 1.3e-6 of its permanent.
-constexpr float kCrossBound = 1e-6f;
-constexpr float kCircleBound = 3e-6f;
+// FP32 determinants of offsets, each offset within 2^-23 of its value (cut): a
+// product of two is within 5 2^-24 and the cross product's error below 7 2^-24
+// = 4.2e-7 of its permanent; |a|^2 is within 7 2^-24, and the in-circle sum
+// within 18 2^-24 = 1.1e-6 of its permanent.  Below FP32's normal range errors
+// are absolute instead: an offset is cut to zero from 2^-126, and products lose
+// up to 2^-150 each.  With offsets up to r the two determinants are off by at
+// most 4 r 2^-126 + 2^-149 and 24 r^3 2^-126 + 24 r^2 2^-150, below the floors
+// for r up to 600 spacings; points 1e-11 spacings apart, whose in-circle sums
+// are such numbers, are so left to FP64.
+constexpr float kCrossBound = 1e-6f, kCrossFloor = 1e-30f;
+constexpr float kCircleBound = 3e-6f, kCircleFloor = 1e-28f;
+constexpr float kTinyTriangle = 1e-30f;  // 4 (twice its area)^2
+RICH_HD inline float cross_error(float p, float q) { return kCrossBound * (fabsf(p) + fabsf(q)) + kCrossFloor; }
+RICH_HD inline float circle_error(float al, float p1, float p2, float bl, float p3, float p4, float dl, float p5,
+                                  float p6)
+{
+    return kCircleBound * (al * (fabsf(p1) + fabsf(p2)) + bl * (fabsf(p3) + fabsf(p4)) + dl * (fabsf(p5) + fabsf(p6))) +
+           kCircleFloor;
+}
 
 #ifdef __CUDA_ARCH__
 #define RICH_MU_SLOW __device__ __noinline__
@@ -408,31 +426,68 @@ RICH_HD inline int incircle(const Frame &f, const Point &a, const Point &b, cons
     const float p1 = b.fx * d.fy, p2 = b.fy * d.fx, p3 = a.fx * d.fy, p4 = a.fy * d.fx, p5 = a.fx * b.fy,
                 p6 = a.fy * b.fx;
     const float det = a.l * (p1 - p2) - b.l * (p3 - p4) + d.l * (p5 - p6);
-    const float bound = kCircleBound * (a.l * (fabsf(p1) + fabsf(p2)) + b.l * (fabsf(p3) + fabsf(p4)) +
-                                        d.l * (fabsf(p5) + fabsf(p6)));
+    const float bound = circle_error(a.l, p1, p2, b.l, p3, p4, d.l, p5, p6);
     if (det > bound) return -1;
     if (-det > bound) return 1;
     return circle_slow(f, a, b, d);
+}
+
+// Whether a circumdisk of radius R about (ux, uy), from the cell, is inside the
+// ghost band (all scaled).
+RICH_HD inline bool disk_inside(const Frame &f, float ux, float uy, float R)
+{
+    const float lx = to_float(f.xi - f.x0, f.shift), rx = to_float(f.x1 - f.xi, f.shift);
+    const float ly = to_float(f.yi - f.y0, f.shift), ry = to_float(f.y1 - f.yi, f.shift);
+    return R - ux - lx <= f.reach && R + ux - rx <= f.reach && R - uy - ly <= f.reach && R + uy - ry <= f.reach;
 }
 
 // Whether the circumdisk of (cell, a, b) is certainly inside the ghost band
 // (and, in a periodic box, smaller than a quarter of it).  A disk through
 // the cell reaches past a wall by less than its diameter, so a radius below
 // 0.48 bands is enough; larger disks are placed.  In FP32, with margins of
-// 2 %.
+// 2 %; false for triangles of less than 2.5e-16 squared spacings, which the
+// products underflow for (disk_ok_any takes them).
 RICH_HD inline bool disk_ok(const Frame &f, const Point &a, const Point &b)
 {
     const float cr = a.fx * b.fy - a.fy * b.fx;
     const float ex = a.fx - b.fx, ey = a.fy - b.fy;
     const float q = a.l * b.l * (ex * ex + ey * ey), c4 = 4.0f * cr * cr;
+    if (!(c4 >= kTinyTriangle)) return false;
     if (q <= c4 * f.rlim2) return true;
     if (!(q <= c4 * f.rper2)) return false;
     const float i2 = 0.5f / cr;
     const float ux = (b.fy * a.l - a.fy * b.l) * i2, uy = (a.fx * b.l - b.fx * a.l) * i2;
-    const float R = sqrtf(ux * ux + uy * uy) * 1.001f;
-    const float lx = to_float(f.xi - f.x0) * f.scale, rx = to_float(f.x1 - f.xi) * f.scale;
-    const float ly = to_float(f.yi - f.y0) * f.scale, ry = to_float(f.y1 - f.yi) * f.scale;
-    return R - ux - lx <= f.reach && R + ux - rx <= f.reach && R - uy - ly <= f.reach && R + uy - ry <= f.reach;
+    return disk_inside(f, ux, uy, sqrtf(ux * ux + uy * uy) * 1.001f);
+}
+
+// Circumcentre of (0, a, b) in FP64, all scaled (NaN where the cross product
+// is of the size of its rounding).
+RICH_MU_SLOW float2 centre_slow(double ax, double ay, double bx, double by, int32_t shift)
+{
+    const double s = exactint::pow2(shift);
+    ax *= s;
+    ay *= s;
+    bx *= s;
+    by *= s;
+    const double l = ax * by, r = ay * bx, cr = l - r;
+    float2 u = {NAN, NAN};
+    if (fabs(cr) > 1e-12 * (fabs(l) + fabs(r))) {
+        const double al = ax * ax + ay * ay, bl = bx * bx + by * by;
+        u.x = to_float((by * al - ay * bl) / (cr + cr), 0);
+        u.y = to_float((ax * bl - bx * al) / (cr + cr), 0);
+    }
+    return u;
+}
+
+// disk_ok for triangles of any size, in FP64 where FP32 has not the range.
+RICH_HD inline bool disk_ok_any(const Frame &f, const Point &a, const Point &b)
+{
+    const float cr = a.fx * b.fy - a.fy * b.fx;
+    if (4.0f * cr * cr >= kTinyTriangle) return disk_ok(f, a, b);
+    const Point p = point_of(f, a.ref), q = point_of(f, b.ref);
+    const float2 u = centre_slow(p.x - f.xi, p.y - f.yi, q.x - f.xi, q.y - f.yi, f.shift);
+    const float R2 = u.x * u.x + u.y * u.y;
+    return R2 <= f.rlim2 || (R2 <= f.rper2 && disk_inside(f, u.x, u.y, sqrtf(R2) * 1.001f));
 }
 
 // List a cell for the round of `stamp` (once).
@@ -542,14 +597,13 @@ template <bool kFast> RICH_HD inline bool verify(const MeshUpdate &m, int32_t i)
         const Point d = point_of(f, ref);
         const float p = b.fx * d.fy, q = b.fy * d.fx, cbd = p - q;
         bool bad = false;
-        if (!(cbd > kCrossBound * (fabsf(p) + fabsf(q)))) {
+        if (!(cbd > cross_error(p, q))) {
             if (kFast) open = true;
             else bad = orient_slow(f, b, d) <= 0;
         }
         const float p3 = a.fx * d.fy, p4 = a.fy * d.fx, p5 = a.fx * b.fy, p6 = a.fy * b.fx;
         const float det = a.l * cbd - b.l * (p3 - p4) + d.l * cab;
-        const float bound = kCircleBound * (a.l * (fabsf(p) + fabsf(q)) + b.l * (fabsf(p3) + fabsf(p4)) +
-                                            d.l * (fabsf(p5) + fabsf(p6)));
+        const float bound = circle_error(a.l, p, q, b.l, p3, p4, d.l, p5, p6);
         if (!(det > bound)) {
             if (-det > bound) bad = true;
             else if (kFast) open = true;
@@ -568,7 +622,7 @@ template <bool kFast> RICH_HD inline bool verify(const MeshUpdate &m, int32_t i)
         }
         // another image than the mesh had, or a disk near the band's edge:
         // this cell alone
-        if (d.ref != ref || !disk_ok(f, b, d)) self = true;
+        if (d.ref != ref || !(kFast ? disk_ok(f, b, d) : disk_ok_any(f, b, d))) self = true;
         turns += (b.fy < 0.0f && d.fy >= 0.0f) ? 1 : 0;
         a = b;
         b = d;
@@ -632,15 +686,14 @@ inline bool recompute_light(const MeshUpdate &m, int32_t i, int32_t round)
             Point d;
             d.fx = fx[k];
             d.fy = fy[k];
-            const float p3 = a.fx * d.fy, p4 = a.fy * d.fx, c = p3 - p4, cb = kCrossBound * (fabsf(p3) + fabsf(p4));
+            const float p3 = a.fx * d.fy, p4 = a.fy * d.fx, c = p3 - p4, cb = cross_error(p3, p4);
             if (-c > cb) continue;
             if (!(c > cb)) return false;
             d.l = d.fx * d.fx + d.fy * d.fy;
             if (best >= 0) {
                 const float p1 = b.fx * d.fy, p2 = b.fy * d.fx, p5 = a.fx * b.fy, p6 = a.fy * b.fx;
                 const float det = a.l * (p1 - p2) - b.l * c + d.l * (p5 - p6);
-                const float bound = kCircleBound * (a.l * (fabsf(p1) + fabsf(p2)) + b.l * (fabsf(p3) + fabsf(p4)) +
-                                                    d.l * (fabsf(p5) + fabsf(p6)));
+                const float bound = circle_error(a.l, p1, p2, b.l, p3, p4, d.l, p5, p6);
                 if (det > bound) continue;
                 if (!(-det > bound)) return false;
             }
@@ -777,7 +830,7 @@ RICH_HD inline void recompute(const MeshUpdate &m, int32_t i, int32_t round)
         for (int k = 0; k < nc; k++) {
             if (k == last) continue;
             const float p = a.fx * fy[k], q = a.fy * fx[k], c = p - q;
-            const float cb = kCrossBound * (fabsf(p) + fabsf(q));
+            const float cb = cross_error(p, q);
             bool left = c > cb;
             if (!left && !(-c > cb)) left = orient_slow(f, whole(last), whole(k)) > 0;
             if (!left) continue;
@@ -788,8 +841,7 @@ RICH_HD inline void recompute(const MeshUpdate &m, int32_t i, int32_t round)
             const Point b = point(best);
             const float p1 = b.fx * fy[k], p2 = b.fy * fx[k], p5 = a.fx * b.fy, p6 = a.fy * b.fx;
             const float det = a.l * (p1 - p2) - b.l * c + fl[k] * (p5 - p6);
-            const float bound = kCircleBound * (a.l * (fabsf(p1) + fabsf(p2)) + b.l * (fabsf(p) + fabsf(q)) +
-                                                fl[k] * (fabsf(p5) + fabsf(p6)));
+            const float bound = circle_error(a.l, p1, p2, b.l, p, q, fl[k], p5, p6);
             if (det > bound) continue;
             if (-det > bound || circle_slow(f, whole(last), whole(best), whole(k)) > 0) best = k;
         }
@@ -797,7 +849,7 @@ RICH_HD inline void recompute(const MeshUpdate &m, int32_t i, int32_t round)
             bad = true;
             break;
         }
-        if (!disk_ok(f, a, point(best))) a_or(f.flags, MU_FAR);
+        if (!disk_ok_any(f, a, point(best))) a_or(f.flags, MU_FAR);
         turns += (a.fy < 0.0f && fy[best] >= 0.0f) ? 1 : 0;
         last = best;
     } while (last != near);

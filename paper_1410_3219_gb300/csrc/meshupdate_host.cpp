@@ -15,18 +15,20 @@ void mesh_params(const BoxConfig &box, int32_t n, InstParams &ip)
     const double h = std::sqrt(Lx * Ly / std::max(n, 1));
     const double w = std::min(5.0 * h, lmin);
     const double margin = 1e-9 * (std::fabs(box.x0) + std::fabs(box.x1) + std::fabs(box.y0) + std::fabs(box.y1) + w);
-    ip.half_x = (float)(0.5 * Lx / h);
-    ip.half_y = (float)(0.5 * Ly / h);
+    // the power of two that scales a mean spacing to [1, 2)
+    ip.mesh_shift = h > 0.0 && std::isfinite(h) ? std::max(-kMaxShift, std::min(kMaxShift, -std::ilogb(h))) : 0;
+    const double scale = exactint::pow2(ip.mesh_shift);
+    ip.half_x = (float)(0.5 * Lx * scale);
+    ip.half_y = (float)(0.5 * Ly * scale);
     ip.band = w;
     ip.in_x0 = box.x0 + w + margin;
     ip.in_x1 = box.x1 - w - margin;
     ip.in_y0 = box.y0 + w + margin;
     ip.in_y1 = box.y1 - w - margin;
-    ip.mesh_scale = (float)(1.0 / h);
-    const double rl = 0.48 * w / h, rp = box.boundary == 1 ? 0.24 * lmin / h : 1e18;
+    const double rl = 0.48 * w * scale, rp = box.boundary == 1 ? 0.24 * lmin * scale : 1e18;
     ip.mesh_rlim2 = (float)(std::min(rl, rp) * std::min(rl, rp));
     ip.mesh_rper2 = (float)(rp * rp);
-    ip.mesh_reach = (float)(0.98 * w / h);
+    ip.mesh_reach = (float)(0.98 * w * scale);
 }
 
 int mesh_update_serial(const BoxConfig &box, int32_t n, const double *x, const double *y, HostMesh &mesh, int32_t &flags,

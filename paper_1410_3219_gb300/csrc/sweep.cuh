@@ -72,11 +72,13 @@ struct InstParams {
     int32_t pad;
     // constants of the device mesh update (mesh_params in meshupdate.h):
     // the ghost band and the box inside which no point has an image in it,
-    // and in FP32, in mean point spacings (lengths times mesh_scale), half the
-    // box's sides, the squared circumradii that need no placing and that a
-    // periodic box allows, and how far a disk may reach past a wall
+    // the power of two that scales a mean point spacing to [1, 2), and so
+    // scaled, in FP32, half the box's sides, the squared circumradii that need
+    // no placing and that a periodic box allows, and how far a disk may reach
+    // past a wall
     double band, in_x0, in_x1, in_y0, in_y1;
-    float half_x, half_y, mesh_scale, mesh_rlim2, mesh_rper2, mesh_reach;
+    int32_t mesh_shift;
+    float half_x, half_y, mesh_rlim2, mesh_rper2, mesh_reach;
 };
 
 template <class R> struct SweepParams {

@@ -104,3 +104,37 @@ def test_coincident_points_are_left_to_the_host_builder():
     x2[17], y2[17] = x[18], y[18]
     with pytest.raises(R.RichError, match="EDUPLICATE"):
         R.rich_device_update_check(W.default_cfg(), np.array([x, x2]), np.array([y, y2]))
+
+
+@pytest.mark.parametrize("boundary", [W.BC_PERIODIC, W.BC_REFLECTIVE])
+@pytest.mark.parametrize("points,radius,noise,seed", [(4, 4e-12, 1e-5, 76), (5, 2e-12, 1e-5, 110), (8, 2e-12, 1e-5, 71),
+                                                       (25, 7e-12, 1e-4, 3), (6, 1e-10, 1e-5, 5), (6, 1e-8, 1e-6, 6)])
+def test_clusters_far_below_the_spacing(points, radius, noise, seed, boundary):
+    """Points on a circle of 1e-11 to 1e-7 mean spacings among 200 others: the
+    products of FP32 in-circle sums fall below its normal range, and their
+    signs must not be taken."""
+    rng = np.random.default_rng(seed)
+    x, y = W.jittered_lattice(15, 15, 0.0, 1.0, 0.0, 1.0, 0.3, rng)
+    c = rng.uniform(0.3, 0.7, 2)
+    far = np.hypot(x - c[0], y - c[1]) > 0.03
+    x, y = x[far], y[far]
+    angle = 2 * np.pi * (np.arange(points) + rng.uniform(-0.3, 0.3, points)) / points
+    sets = []
+    for _ in range(2):
+        r = radius * (1 + rng.uniform(-noise, noise, points))
+        sets.append((np.concatenate([x, c[0] + r * np.cos(angle)]), np.concatenate([y, c[1] + r * np.sin(angle)])))
+    mismatched, updated, _ = R.rich_device_update_check(W.default_cfg(boundary=boundary),
+                                                        np.array([s[0] for s in sets]), np.array([s[1] for s in sets]))
+    assert (mismatched, updated) == (0, 1)
+
+
+@pytest.mark.parametrize("boundary", [W.BC_PERIODIC, W.BC_REFLECTIVE])
+@pytest.mark.parametrize("side", [1e-60, 1e-38, 1e-35, 1e-34, 1e-30, 1e38, 1e60])
+def test_boxes_of_any_unit(side, boundary):
+    """Offsets are scaled by the point spacing before FP32 holds them, so a
+    box's unit does not cut them to zero or infinity."""
+    for seed in range(4):
+        xs, ys = _walk((0.0, side, 0.0, side), boundary, 20, 20, 0.05 * (1 + seed), 0.02, 6, seed=seed)
+        cfg = W.default_cfg(boundary=boundary, x0=0.0, x1=side, y0=0.0, y1=side)
+        mismatched, updated, _ = R.rich_device_update_check(cfg, xs, ys)
+        assert (mismatched, updated) == (0, 5)
