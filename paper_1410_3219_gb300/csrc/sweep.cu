@@ -603,10 +603,13 @@ __device__ __forceinline__ void stage_cell_gradient_fp64(const SweepParams<R> &p
             const float gx = fabsf(gf[2 * v]), gy = fabsf(gf[2 * v + 1]), err = 1e-6f * (gx + gy) * reach;
             const double n1 = ext[v].max() - Wi[v], n2 = Wi[v] - ext[v].min();
             const float f1 = estimate(n1), f2 = estimate(n2);
-            // (products far from FP32's smallest numbers; a gradient of
-            // exactly zero is exact)
+            // (products far from FP32's smallest numbers, where a gradient of
+            // exactly zero is exact, and everything below its largest: an
+            // estimate of 2^128 and above is infinite, and would clear any
+            // difference as large)
             const bool known = reach > 1e-12f && (gx > 1e-22f || dkey0(g[2 * v]) == 0) &&
-                               (gy > 1e-22f || dkey0(g[2 * v + 1]) == 0);
+                               (gy > 1e-22f || dkey0(g[2 * v + 1]) == 0) &&
+                               fmaxf(fmaxf(f1, f2), fmaxf(up[v] - dn[v], err)) < 1e37f;
             // a side is free when its numerator clears its largest difference
             const bool free1 = f1 >= (up[v] + err) * 1.000001f, free2 = f2 >= (err - dn[v]) * 1.000001f;
             if (known && free1 && free2) continue;
@@ -620,8 +623,8 @@ __device__ __forceinline__ void stage_cell_gradient_fp64(const SweepParams<R> &p
             const float c1 = f1 * (-dn[v]), c2 = f2 * up[v], ce = 1e-5f * (fabsf(c1) + fabsf(c2)) + err * (f1 + f2);
             const bool one = known && up[v] > err && (free2 || (dn[v] < -err && c1 < c2 - ce));
             const bool two = known && dn[v] < -err && (free1 || (up[v] > err && c2 < c1 - ce));
-            // (an infinite or NaN estimate fails these; a tie between edges or
-            // sides, or a difference of the size of its error, goes on)
+            // (a product beyond FP32 fails these; a tie between edges or sides,
+            // or a difference of the size of its error, goes on)
             if ((one && up2[v] < up[v] - 2.0f * err) || (two && dn2[v] > dn[v] + 2.0f * err)) {
                 double mx, my;
                 sl.midpoint(one ? su[v] : sd[v], mx, my);

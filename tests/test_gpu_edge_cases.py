@@ -109,3 +109,27 @@ def test_device_edge_list_equals_host_list(R, name):
         wl = W.uniform(n_side=12, jitter=0.0, seed=35)
     edges, bad = R.rich_edge_list_check(wl["cfg"], wl["x"], wl["y"])
     assert edges > 0 and bad == 0, (name, edges, bad)
+
+
+@pytest.mark.parametrize("limiter", [W.LIM_SWITCHED, W.LIM_AREPO, W.LIM_TESS])
+@pytest.mark.parametrize("power", [-300, -130, 120, 127, 128, 140, 200, 300])
+def test_units_of_mass_scale_out(R, power, limiter):
+    """Density and pressure times a power of two: every FP64 operation of a
+    step scales exactly, so the points and velocities stay the same bits and
+    the conserved state is the unscaled one times that power.  The FP32
+    estimates behind the limiter's decisions do not scale (they end at 2^128),
+    and must leave such values to FP64."""
+    wl = W.random_mixed(n=400, seed=8)
+    wl["cfg"]["limiter"] = limiter
+    big = dict(wl, rho=np.ldexp(wl["rho"], power), p=np.ldexp(wl["p"], power))
+    a, b = R.Sim(wl), R.Sim(big)
+    for _ in range(3):
+        ia, ib = a.step(1), b.step(1)
+        assert ia["dt_last"] == ib["dt_last"]
+    ca, cb = a.conserved(), b.conserved()
+    for k in ("x", "y"):
+        assert np.array_equal(ca[k], cb[k]), k
+    for k in ("m", "px", "py", "E"):
+        assert np.array_equal(np.ldexp(ca[k], power), cb[k]), k
+    a.close()
+    b.close()
