@@ -525,7 +525,8 @@ __device__ __forceinline__ void stage_cell_gradient_fp64(const SweepParams<R> &p
     // point contacts: edges of at most 1e-9 sqrt(A)
     const double Lmin = 1.7724538509055160273e-9 * Rad;
     const float pif = magnitude(Wi[3]);
-    const bool pi_ok = estimable(Wi[3]);
+    // (a delta_p below FP32's normal range has no estimate; 0 is exact)
+    const bool pi_ok = estimable(Wi[3]) && (dpf > 1e-37f || dkey0(dp) == 0);
     float reach = 0.0f;  // the farthest midpoint (largest coordinate)
     for (int32_t s = lo; s < hi; s++) {
         const double L = sl.L(s);

@@ -133,3 +133,24 @@ def test_units_of_mass_scale_out(R, power, limiter):
         assert np.array_equal(np.ldexp(ca[k], power), cb[k]), k
     a.close()
     b.close()
+
+
+@pytest.mark.parametrize("delta_p,drop,fires", [(1e-50, 1e-53, True), (1e-50, 1e-47, False), (1e-43, 1e-45, True),
+                                                 (1e-37, 1e-39, True), (0.0, 1e-53, False), (0.7, 0.5, True),
+                                                 (0.7, 0.9, False)])
+def test_pressure_switch_at_any_threshold(R, delta_p, drop, fires):
+    """min(p_i, p_j) < delta_p max(p_i, p_j) over the edges of a disc of low
+    pressure in a gas at rest: the switch fires in the cells beside its rim or
+    nowhere, for thresholds that FP32 cannot hold too."""
+    wl = W.uniform(n_side=20, vx=0.0, vy=0.0)
+    wl["cfg"]["delta_p"], wl["cfg"]["delta_v"] = delta_p, 1e300
+    inside = np.hypot(wl["x"] - 0.5, wl["y"] - 0.5) < 0.25
+    wl["p"] = np.where(inside, 1e25 * drop, 1e25)
+    sim = R.Sim(wl)
+    try:
+        sim.step(1)
+    except R.RichError:
+        pass  # (cells of such a jump may empty; the switch describes the attempt)
+    tess = sim.field("tess")
+    assert (tess.sum() > 20) == fires and (fires or tess.sum() == 0)
+    sim.close()
