@@ -1163,7 +1163,7 @@ cudaError_t MeshUpdater::reserve(int32_t n, int32_t n_inst, cudaStream_t st)
     const size_t N = (size_t)n, i4 = sizeof(int32_t);
     max_rings_ = std::max(std::min(n, 4096), n / 2);
     const size_t R = (size_t)max_rings_;
-    // stamps and counts that only ever grow must start at zero
+    // stamps, which only ever grow, must start at zero
     const bool fresh = !(mark_.p && mark_.cap >= N * i4);
     MU_TRY(mark_.ensure(N * i4)); MU_TRY(info_.ensure(N * i4)); MU_TRY(extra_n_.ensure(N * i4));
     MU_TRY(list_[0].ensure(N * i4)); MU_TRY(list_[1].ensure(N * i4)); MU_TRY(heavy_.ensure(N * i4));
@@ -1185,8 +1185,8 @@ cudaError_t MeshUpdater::reserve(int32_t n, int32_t n_inst, cudaStream_t st)
     if (fresh || stamp_ > (1 << 28)) {
         MU_TRY(cudaMemsetAsync(mark_.p, 0, mark_.cap, st));
         MU_TRY(cudaMemsetAsync(info_.p, 0, info_.cap, st));
-        MU_TRY(cudaMemsetAsync(extra_n_.p, 0, extra_n_.cap, st));
         stamp_ = 0;
+        told_ = true;
     }
     return cudaSuccess;
 }
@@ -1293,6 +1293,10 @@ cudaError_t MeshUpdater::start(const MeshArrays &a, const MeshOutput &o, cudaStr
     // the counters cleared by the last update (or when they were allocated)
     std::swap(count_[0].p, count_[1].p);
     std::swap(count_[0].cap, count_[1].cap);
+    // what an update that did not settle every cell it told of others left
+    // behind: references in the numbering of the mesh it was started for
+    if (told_) MU_TRY(cudaMemsetAsync(extra_n_.p, 0, extra_n_.cap, st));
+    told_ = true;
     const MeshUpdate m = params(a, o);
     MU_TRY(launch_chained(k_mesh_verify, pass_blocks(a.n, a.split), kVerifyBlock, st, m.n, m));
     // (a warp per eight cells: steps of 10,201 cells took 105 us with one per
@@ -1323,10 +1327,9 @@ cudaError_t MeshUpdater::settle(const MeshArrays &a, const MeshOutput &o, MeshRe
     result.state = !settled ? MeshResult::kHost : c.ready ? MeshResult::kDone : MeshResult::kGrow;
     if (result.state == MeshResult::kGrow && a.n_inst == 1 && result.flagged) result.state = MeshResult::kHost;
     result.bad = c.bad != 0;
-    // (what was reported to cells that no round recomputed is dropped, and
-    // sizes of rings that were not kept are measured again)
+    // (sizes of rings that were not kept are measured again)
     whole_ = result.state == MeshResult::kHost || result.flagged;
-    if (whole_) MU_TRY(cudaMemsetAsync(extra_n_.p, 0, extra_n_.cap, st));
+    told_ = whole_ || result.state == MeshResult::kGrow;
     last_round_ = r;
     return cudaSuccess;
 }

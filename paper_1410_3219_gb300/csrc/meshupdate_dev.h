@@ -139,6 +139,7 @@ private:
     int32_t stamp_ = 0, max_rings_ = 0, last_round_ = 0;
     int quiet_ = 0;      // updates in a row that needed one round (at most kQuiet)
     bool whole_ = true;  // sizes_ does not describe the mesh to update
+    bool told_ = true;   // extra_n_ may hold counts (else it is zero)
     DBuf mark_, list_[2], heavy_, info_, at_, ring_deg_, ring_ref_, extra_n_, extra_, count_[2], sizes_, images_,
         ghost_off_, sums_, edge_mask_, tri_mask_;
     HBuf host_;

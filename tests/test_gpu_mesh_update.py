@@ -166,3 +166,32 @@ def test_clusters_far_below_the_spacing(R, points, radius, boundary):
         assert mismatched == 0
         assert updates >= 1
     sim.close()
+
+
+@pytest.mark.parametrize("seed", [3, 4, 5])
+def test_refill_after_members_ended_together(R, seed):
+    """Every member of a batch ends in a step whose mesh update needed another
+    round than the one launched (after quiet updates, a rough mesh's first
+    step): what that update had told cells of others must not reach the
+    smaller simulations that fill the batch next, whose results equal their
+    solo runs bit for bit."""
+    b = R.Batch(max_cells=1 << 20)
+    b.add(W.gresho(n_side=24, seed=2), max_steps=12)
+    for k in range(12):
+        if k == 11:
+            b.add(W.sod(n_side=225, seed=seed, jitter=0.4), max_steps=1)
+        b.step()
+    wls = [W.sod(n_side=40, seed=seed, jitter=0.4), W.kelvin_helmholtz(n_side=50, seed=seed, amp=0.2),
+           W.sod(n_side=33, seed=seed + 10, jitter=0.3)]
+    ids = [b.add(w, max_steps=6) for w in wls]
+    for _ in range(6):
+        b.step()
+    for w, sid in zip(wls, ids):
+        assert b.query(sid)["state"] == "done"
+        solo = R.Sim(w)
+        solo.step(6)
+        got, want = b.conserved(sid), solo.conserved()
+        for f in want:
+            assert np.array_equal(got[f], want[f]), (sid, f)
+        solo.close()
+    b.close()
