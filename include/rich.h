@@ -328,6 +328,11 @@ int rich_batch_launch_info(const rich_batch *b, int32_t *persistent, int32_t *bl
    Errors: RICH_EINVAL. */
 int rich_batch_inject_barrier_timeout(rich_batch *b, int32_t spin_limit, int64_t *timeouts_seen);
 
+/* How many meshes of its simulations the batch has had from the device's
+   update and from the host builder so far (a simulation's first mesh is the
+   host's, and a static simulation keeps its mesh).  Errors: RICH_EINVAL. */
+int rich_batch_mesh_counts(const rich_batch *b, int64_t *updated, int64_t *built);
+
 void rich_batch_destroy(rich_batch *b);
 
 /* ---- continuous-batching server -------------------------------------------- */

@@ -128,6 +128,7 @@ struct rich_batch {
     rich::HBuf read_host;
     rich::HBuf h_back;  // dt, status per simulation, then the list builder's flag
     cudaEvent_t ev2 = nullptr;
+    int64_t meshes_updated = 0, meshes_built = 0;  // members' meshes made on the device, and on the host
     bool diagnostics = false;
     int cur = 0;
     // device
@@ -543,6 +544,8 @@ int finish_update(rich_batch *b, int q)
     b->nS = r.sizes.slots;
     b->dev_mesh = true;
     b->dev_lists = !r.flagged;
+    for (size_t k = 0; k < b->packed.size(); k++)
+        b->meshes_updated += b->packed[k]->state == RUNNING && !b->mesh_flag[k];
     CUDA_TRY(b->mesh[1 - b->mcur].reserve(a.n, r.sizes));
     return reserve_geometry(b, r.sizes);
 }
@@ -743,6 +746,7 @@ namespace {
 void tessellate_members(rich_batch *b, const std::vector<BatchSim *> &sims)
 {
     rich::Range range("rich batch tessellate (a0)");
+    b->meshes_built += (int64_t)sims.size();
     std::vector<BatchSim *> by_size(sims);
     std::stable_sort(by_size.begin(), by_size.end(), [](const BatchSim *a, const BatchSim *c) { return a->n > c->n; });
     size_t n_large = 0;
@@ -1150,6 +1154,14 @@ int rich_batch_set_launch(rich_batch *b, int32_t mode, int32_t block)
     b->tuned = false;
     b->cands.clear();
     b->cand_next = 0;
+    return RICH_OK;
+}
+
+int rich_batch_mesh_counts(const rich_batch *b, int64_t *updated, int64_t *built)
+{
+    if (!b || !updated || !built) return fail(RICH_EINVAL, "bad arguments");
+    *updated = b->meshes_updated;
+    *built = b->meshes_built;
     return RICH_OK;
 }
 

@@ -1271,11 +1271,12 @@ cudaError_t MeshUpdater::launch_rounds(const MeshArrays &a, const MeshOutput &o,
     l.ready = &m.count->ready;
     l.bad = &m.count->bad;
     l.next = count_[1].as<int32_t>();
-    l.next_words = (int32_t)(sizeof(MeshUpdateCount) / sizeof(int32_t)) + a.n_inst;
+    // (all of it: an update before the last may have had more simulations)
+    l.next_words = (int32_t)(count_[1].cap / sizeof(int32_t));
     l.report = host_.as<int32_t>();
     l.done = &m.count->done;
     l.counters = count_[0].as<int32_t>();
-    l.words = l.next_words;
+    l.words = (int32_t)(sizeof(MeshUpdateCount) / sizeof(int32_t)) + a.n_inst;
     return launch_lists(l, a.split, st);
 }
 

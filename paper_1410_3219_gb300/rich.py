@@ -37,7 +37,7 @@ EXPORTS = ["rich_default_config", "rich_init_mesh", "rich_step", "rich_get_state
            "rich_init_conserved", "rich_get_order", "rich_time", "rich_mesh_update_check",
            "rich_probe_pipe_peaks", "rich_batch_inject_barrier_timeout", "rich_server_start",
            "rich_server_stats", "rich_edge_list_check", "rich_tess_phases", "rich_device_update_check",
-           "rich_mesh_check"]
+           "rich_mesh_check", "rich_batch_mesh_counts"]
 
 REQ_STATES = {0: "queued", 1: "running", 2: "done", 3: "failed"}
 
@@ -146,6 +146,7 @@ def _lib():
         L.rich_time.restype = d
         L.rich_probe_pipe_peaks.argtypes = [_D, _D]
         L.rich_batch_inject_barrier_timeout.argtypes = [P, I32, C.POINTER(I64)]
+        L.rich_batch_mesh_counts.argtypes = [P, C.POINTER(I64), C.POINTER(I64)]
         L.rich_server_start.argtypes = [P, I32, I64, I64]
         L.rich_tess_phases.argtypes = [P, _D]
         L.rich_edge_list_check.argtypes = [C.POINTER(rich_config), I64, _D, _D, C.POINTER(I64), C.POINTER(I64)]
@@ -468,6 +469,12 @@ class Batch:
 
     def launch_info(self):
         return rich_batch_launch_info(self.h)
+
+    def mesh_counts(self):
+        """(meshes updated on the device, meshes built on the host) so far."""
+        a, b = C.c_int64(), C.c_int64()
+        _check(_lib().rich_batch_mesh_counts(self.h, C.byref(a), C.byref(b)))
+        return a.value, b.value
 
     def inject_barrier_timeout(self, spin_limit=0):
         """Arm (spin_limit > 0) a barrier timeout in the next persistent

@@ -195,3 +195,24 @@ def test_refill_after_members_ended_together(R, seed):
             assert np.array_equal(got[f], want[f]), (sid, f)
         solo.close()
     b.close()
+
+
+def test_flags_of_a_larger_packing_are_cleared(R):
+    """A batch of three, two and three simulations: the first packing's third
+    one (a box too small for the update) leaves its flag in one of the two
+    counter buffers, which the second packing's update does not reach; the
+    third packing's third simulation must be updated on the device."""
+    b = R.Batch(max_cells=1 << 20)
+    for k, steps in ((24, 8), (28, 8)):
+        b.add(W.gresho(n_side=k, seed=k), max_steps=steps)
+    b.add(W.uniform(n_side=2, jitter=0.2, seed=34), max_steps=1)
+    b.step()
+    b.step()
+    late = b.add(W.gresho(n_side=32, seed=6), max_steps=4)
+    for _ in range(4):
+        b.step()
+    assert b.query(late)["state"] == "done"
+    # the four first meshes only; two members' updates after each of six
+    # steps, and the late one's after its first three
+    assert b.mesh_counts() == (2 * 6 + 3, 4)
+    b.close()
