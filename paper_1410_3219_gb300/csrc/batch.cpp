@@ -532,7 +532,7 @@ int finish_update(rich_batch *b, int q)
         CUDA_TRY(to.reserve(a.n, r.sizes));
         CUDA_TRY(b->updater.again(a, to.output(0), r, st));
     }
-    if (r.state != rich::MeshResult::kDone || (r.bad && !r.flagged)) {
+    if (r.state != rich::MeshResult::kDone) {
         b->updater.forget();
         return RICH_OK;
     }

@@ -513,6 +513,15 @@ __global__ void __launch_bounds__(kListBlock) k_mesh_check(MeshUpdate m, int32_t
     }
 }
 
+// The simulations of cells still listed for `round`: theirs are left to the
+// host, and the others' meshes can be written.
+__global__ void k_mesh_give_up(MeshUpdate m, int32_t round)
+{
+    const int32_t count = m.count->listed[round];
+    for (int32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < count; k += gridDim.x * blockDim.x)
+        mu::a_or(m.flags + mu::inst_at(m, m.list[round & 1][k]), MU_ROUNDS);
+}
+
 __device__ __forceinline__ int4 plus(int4 a, int4 b) { return make_int4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w); }
 
 __device__ __forceinline__ int4 warp_total(int4 v)
@@ -946,15 +955,20 @@ __global__ void __launch_bounds__(128) k_mesh_lists(MeshLists l)
     }
     const int lane = threadIdx.x & 31, k = lane & 7, first = lane & 24;
     const int32_t quads = (l.n + 3) >> 2, stride = gridDim.x * (blockDim.x >> 5);
-    bool bad = false;
+    // (a cell's lists are its simulation's: another's are good all the same)
+    auto report_bad = [&](int32_t i) {
+        *l.bad = 1;
+        if (l.flags) atomicOr(l.flags + (l.cell_inst ? l.cell_inst[i] : 0), (int32_t)MU_LISTS);
+    };
     for (int32_t quad = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); quad < quads; quad += stride) {
+        bool bad = false;
         const int32_t cell = 4 * quad + (first >> 3);
         const bool live = cell < l.n;
         const int32_t i = live ? cell : l.n - 1;
         const bool periodic = l.cell_inst ? l.inst[l.cell_inst[i]].boundary == 1 : l.periodic != 0;
         const int32_t lo = l.cell_ptr[i], deg = l.cell_ptr[i + 1] - lo;
         if (!__all_sync(kAll, l.edge_mask && deg <= 8)) {
-            bad |= lists_of_any(l, i, live, periodic);
+            if (lists_of_any(l, i, live, periodic)) report_bad(i);
             continue;
         }
         const int q = k < deg ? k : 0;
@@ -1037,8 +1051,8 @@ __global__ void __launch_bounds__(128) k_mesh_lists(MeshLists l)
             l.edge_tb[num] = tri;
             l.slot_edge[lo + q] = 2 * num;
         }
+        if (bad) report_bad(i);
     }
-    if (bad) *l.bad = 1;
     report_counters(l);
 }
 
@@ -1270,6 +1284,7 @@ cudaError_t MeshUpdater::launch_rounds(const MeshArrays &a, const MeshOutput &o,
     l.tri_mask = m.tri_mask;
     l.ready = &m.count->ready;
     l.bad = &m.count->bad;
+    l.flags = m.flags;
     l.next = count_[1].as<int32_t>();
     // (all of it: an update before the last may have had more simulations)
     l.next_words = (int32_t)(count_[1].cap / sizeof(int32_t));
@@ -1320,6 +1335,14 @@ cudaError_t MeshUpdater::settle(const MeshArrays &a, const MeshOutput &o, MeshRe
         MU_TRY(cudaStreamSynchronize(st));
         r = to;
     }
+    if (c.listed[r] > 0 && a.n_inst > 1) {
+        const MeshUpdate m = params(a, o);
+        k_mesh_give_up<<<64, 256, 0, st>>>(m, r);
+        MU_TRY(cudaGetLastError());
+        MU_TRY(cudaMemsetAsync(&m.count->listed[r], 0, sizeof(int32_t), st));
+        MU_TRY(launch_rounds(a, o, r, r, st));
+        MU_TRY(cudaStreamSynchronize(st));
+    }
     result.sizes = MeshSizes{c.ghosts, c.tris, c.edges, c.slots};
     result.flagged = false;
     const int32_t *f = flags();
@@ -1327,7 +1350,6 @@ cudaError_t MeshUpdater::settle(const MeshArrays &a, const MeshOutput &o, MeshRe
     const bool settled = c.listed[r] == 0 && c.slots >= 0 && c.slots <= INT32_MAX / 2;
     result.state = !settled ? MeshResult::kHost : c.ready ? MeshResult::kDone : MeshResult::kGrow;
     if (result.state == MeshResult::kGrow && a.n_inst == 1 && result.flagged) result.state = MeshResult::kHost;
-    result.bad = c.bad != 0;
     // (sizes of rings that were not kept are measured again)
     whole_ = result.state == MeshResult::kHost || result.flagged;
     told_ = whole_ || result.state == MeshResult::kGrow;

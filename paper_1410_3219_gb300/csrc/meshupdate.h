@@ -63,6 +63,8 @@ enum : int32_t {
     MU_STAR = 4,      // a star did not close (coincident points)
     MU_EXACT = 8,     // coordinates beyond the exact predicates' grid
     MU_IMAGE = 16,    // a neighbour image outside the ghost band
+    MU_LISTS = 32,    // its rings do not agree with each other
+    MU_ROUNDS = 64,   // stars that still disagreed after the last round
 };
 
 // Counters of one update (device memory, cleared at its start).

@@ -38,8 +38,8 @@ struct MeshSizes {
 // in ring order from edge_off[i] (edge_off[n] = E).  Writes slot_edge (2 e, or
 // 2 e + 1 on the partner's slot) and edge_l / edge_r / edge_ta / edge_tb
 // (Voronoi edge from circumcentre ta to tb, counter-clockwise about the left
-// cell), and sets *bad where the rings do not agree with each other or with
-// the offsets.
+// cell), and sets *bad (and the simulation's MU_LISTS) where the rings do not
+// agree with each other or with the offsets.
 struct MeshLists {
     int32_t n, periodic;        // box type where cell_inst is null
     const int32_t *cell_inst;   // else each cell's box type from its simulation
@@ -49,6 +49,7 @@ struct MeshLists {
     const uint32_t *edge_mask, *tri_mask;  // slots whose edge / triangle the cell owns (rings of up to 32), or nullptr
     const int32_t *ready;       // nullptr, or 0 there: nothing is built
     int32_t *bad;
+    int32_t *flags = nullptr;   // MU_* of each simulation (an update)
     int32_t *next = nullptr, next_words = 0;  // words to clear (an update's next counters)
     // the update's counters, which the last block copies to page-locked memory
     // (`done` counts the blocks and is left at zero)
@@ -109,11 +110,11 @@ struct MeshStream {
 struct MeshResult {
     // kDone: the mesh and its lists are written (but for the meshes of
     // simulations with flags()); kGrow: an array is too small for `sizes`;
-    // kHost: the rounds did not converge or the only simulation is flagged
+    // kHost: no mesh is written (the only simulation is flagged, or the sizes
+    // do not fit)
     enum { kDone, kGrow, kHost } state;
     MeshSizes sizes;
     bool flagged;  // some simulation's mesh is left to the host
-    bool bad;      // the lists do not close
 };
 
 class MeshUpdater {

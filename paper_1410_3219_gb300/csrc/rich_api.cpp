@@ -374,7 +374,7 @@ int finish_update(rich_sim *s, int q, bool keep, rich_step_info *info)
         CUDA_TRY(to.reserve(s->n, r.sizes));
         CUDA_TRY(s->updater.again(a, to.output(s->periodic()), r, st));
     }
-    if (r.state != rich::MeshResult::kDone || r.flagged || r.bad) {
+    if (r.state != rich::MeshResult::kDone || r.flagged) {
         s->updater.forget();
         return RICH_OK;
     }

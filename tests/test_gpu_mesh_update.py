@@ -216,3 +216,40 @@ def test_flags_of_a_larger_packing_are_cleared(R):
     # steps, and the late one's after its first three
     assert b.mesh_counts() == (2 * 6 + 3, 4)
     b.close()
+
+
+def _hub(spokes=40, n_side=20):
+    """A gas at rest with one cell of `spokes` neighbours."""
+    wl = W.uniform(n_side=n_side, vx=0.0, vy=0.0, jitter=0.2)
+    far = np.hypot(wl["x"] - 0.5, wl["y"] - 0.5) > 0.2
+    angle = 2 * np.pi * (np.arange(spokes) + 0.5) / spokes
+    wl["x"] = np.concatenate([[0.5], wl["x"][far], 0.5 + 0.16 * np.cos(angle)])
+    wl["y"] = np.concatenate([[0.5], wl["y"][far], 0.5 + 0.16 * np.sin(angle)])
+    for k, v in (("rho", 1.0), ("vx", 0.0), ("vy", 0.0), ("p", 1.0)):
+        wl[k] = np.full(wl["x"].size, v)
+    wl["cfg"]["chi"] = 0.0  # (no rounding: the ring stays)
+    return wl
+
+
+@pytest.mark.parametrize("place", [0, 1, 2])
+def test_a_member_left_to_the_host_leaves_the_others_on_the_device(R, place):
+    """A cell of more than 32 neighbours beside small ones is more than the
+    update's lists take: that simulation's meshes are built on the host, and
+    only its."""
+    wls = [W.gresho(n_side=24, seed=2), W.sod(n_side=30, seed=3)]
+    wls.insert(place, _hub())
+    b = R.Batch(max_cells=1 << 20)
+    ids = [b.add(w, max_steps=6) for w in wls]
+    for _ in range(6):
+        b.step()
+    updated, built = b.mesh_counts()
+    assert (updated, built) == (2 * 5, 3 + 5)
+    for w, sid in zip(wls, ids):
+        assert b.query(sid)["state"] == "done"
+        solo = R.Sim(w)
+        solo.step(6)
+        got, want = b.conserved(sid), solo.conserved()
+        for f in want:
+            assert np.array_equal(got[f], want[f]), (sid, f)
+        solo.close()
+    b.close()
