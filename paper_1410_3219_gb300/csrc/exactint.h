@@ -26,6 +26,7 @@ namespace exactint {
 
 constexpr int kUnknown = 2;  // the coordinates do not fit the integer grid
 constexpr int kSpan = 72;    // exponents a grid covers beyond a mantissa
+constexpr int kImageSpan = 68;  // with multiples of a box's sides
 
 template <int N> struct Big {  // s * sum_k w[k] 2^(64 k), s in {-1, 0, 1}
     uint64_t w[N];
@@ -76,7 +77,7 @@ RICH_HD inline int low_exp(double v)
 
 // The common grid of k values: its exponent, or false when they are not
 // finite or spread too far.
-RICH_HD inline bool grid_of(const double *v, int k, int &E)
+RICH_HD inline bool grid_of(const double *v, int k, int &E, int span = kSpan)
 {
     int lo = 1 << 20, hi = -(1 << 20);
     for (int i = 0; i < k; i++) {
@@ -87,25 +88,26 @@ RICH_HD inline bool grid_of(const double *v, int k, int &E)
         if (e > hi) hi = e;
     }
     E = lo == 1 << 20 ? 0 : lo;
-    return hi < lo || hi - lo <= kSpan;
+    return hi < lo || hi - lo <= span;
 }
 
-// a - b on the grid 2^E
-RICH_HD inline Big<2> diff(double a, double b, int E)
+// a - b + k c on the grid 2^E (|k| <= 8; c counts only where k does)
+RICH_HD inline Big<2> diff(double a, double b, int E, int k = 0, double c = 0.0)
 {
     uint64_t lo = 0, hi = 0;
-    for (int t = 0; t < 2; t++) {
-        const double v = t ? b : a;
+    for (int t = 0; t < (k ? 3 : 2); t++) {
+        const double v = t == 0 ? a : (t == 1 ? b : c);
         const uint64_t u = bits_of(v);
         if ((u << 1) == 0) continue;
         uint64_t m = u & 0xfffffffffffffull;
         if ((u >> 52) & 0x7ff) m |= 1ull << 52;
-        const int sh = low_exp(v) - E;  // 0 .. kSpan
+        if (t == 2) m *= (uint64_t)(k < 0 ? -k : k);
+        const int sh = low_exp(v) - E;  // 0 .. the span
         uint64_t l, h;
         if (sh == 0) { l = m; h = 0; }
         else if (sh < 64) { l = m << sh; h = m >> (64 - sh); }
         else { l = 0; h = m << (sh - 64); }
-        const bool neg = ((u >> 63) != 0) != (t == 1);
+        const bool neg = ((u >> 63) != 0) != (t == 1 || (t == 2 && k < 0));
         if (neg) {  // two's complement
             l = ~l + 1;
             h = ~h + (l == 0 ? 1 : 0);
@@ -196,16 +198,9 @@ RICH_HD inline int orient_sign(double ax, double ay, double bx, double by, doubl
     return add(mul(diff(bx, ax, E), diff(cy, ay, E)), mul(diff(by, ay, E), diff(cx, ax, E)), -1).s;
 }
 
-// Sign of the in-circle determinant of counter-clockwise a, b, c against d
-// (> 0: d strictly inside), or kUnknown.
-RICH_HD inline int incircle_sign(double ax, double ay, double bx, double by, double cx, double cy, double dx,
-                                 double dy)
+// the in-circle determinant of differences from the fourth point
+RICH_HD inline int incircle_of(const Big<2> p[3], const Big<2> q[3])
 {
-    const double v[8] = {ax, ay, bx, by, cx, cy, dx, dy};
-    int E;
-    if (!grid_of(v, 8, E)) return kUnknown;
-    const Big<2> p[3] = {diff(ax, dx, E), diff(bx, dx, E), diff(cx, dx, E)};
-    const Big<2> q[3] = {diff(ay, dy, E), diff(by, dy, E), diff(cy, dy, E)};
     Big<12> sum;
     for (int i = 0; i < 12; i++) sum.w[i] = 0;
     sum.s = 0;
@@ -223,6 +218,76 @@ RICH_HD inline int incircle_sign(double ax, double ay, double bx, double by, dou
         sum.s = s.s;
     }
     return sum.s;
+}
+
+// Sign of the in-circle determinant of counter-clockwise a, b, c against d
+// (> 0: d strictly inside), or kUnknown.
+RICH_HD inline int incircle_sign(double ax, double ay, double bx, double by, double cx, double cy, double dx,
+                                 double dy)
+{
+    const double v[8] = {ax, ay, bx, by, cx, cy, dx, dy};
+    int E;
+    if (!grid_of(v, 8, E)) return kUnknown;
+    const Big<2> p[3] = {diff(ax, dx, E), diff(bx, dx, E), diff(cx, dx, E)};
+    const Big<2> q[3] = {diff(ay, dy, E), diff(by, dy, E), diff(cy, dy, E)};
+    return incircle_of(p, q);
+}
+
+// Points of a periodic plane: cell positions x, y and shifts by kx, ky box
+// sides Lx, Ly, taken exactly.  (The coordinates of an image in floating point
+// are rounded, differently in each copy of the same four points.)
+struct Images {
+    double x[4], y[4], Lx, Ly;
+    int8_t kx[4], ky[4];  // -2 .. 2
+    RICH_HD bool grid(int &E) const
+    {
+        double v[10];
+        for (int k = 0; k < 4; k++) {
+            v[2 * k] = x[k];
+            v[2 * k + 1] = y[k];
+        }
+        v[8] = Lx;
+        v[9] = Ly;
+        return grid_of(v, 10, E, kImageSpan);
+    }
+    RICH_HD Big<2> dx(int a, int b, int E) const { return diff(x[a], x[b], E, kx[a] - kx[b], Lx); }
+    RICH_HD Big<2> dy(int a, int b, int E) const { return diff(y[a], y[b], E, ky[a] - ky[b], Ly); }
+    RICH_HD int orient(int a, int b, int c, int E) const
+    {
+        return add(mul(dx(b, a, E), dy(c, a, E)), mul(dy(b, a, E), dx(c, a, E)), -1).s;
+    }
+};
+
+// Orientation of its first three points, or kUnknown.
+RICH_HD inline int orient_images(const Images &m)
+{
+    int E;
+    return m.grid(E) ? m.orient(0, 1, 2, E) : kUnknown;
+}
+
+// In-circle of its counter-clockwise first three points against the fourth
+// (> 0: inside) with the symbolic tie-break of predicates.h, or kUnknown.
+RICH_HD inline int incircle_images(const Images &m)
+{
+    int E;
+    if (!m.grid(E)) return kUnknown;
+    {
+        const Big<2> p[3] = {m.dx(0, 3, E), m.dx(1, 3, E), m.dx(2, 3, E)};
+        const Big<2> q[3] = {m.dy(0, 3, E), m.dy(1, 3, E), m.dy(2, 3, E)};
+        const int s = incircle_of(p, q);
+        if (s) return s;
+    }
+    int k = 0;  // the lexicographically smallest
+    for (int c = 1; c < 4; c++) {
+        const int sx = m.dx(c, k, E).s;
+        if (sx < 0 || (sx == 0 && m.dy(c, k, E).s < 0)) k = c;
+    }
+    switch (k) {
+    case 0: return m.orient(1, 2, 3, E);
+    case 1: return -m.orient(0, 2, 3, E);
+    case 2: return m.orient(0, 1, 3, E);
+    default: return -m.orient(0, 1, 2, E);
+    }
 }
 
 }  // namespace exactint

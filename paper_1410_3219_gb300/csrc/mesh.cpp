@@ -10,6 +10,7 @@
 #include <cmath>
 #include <cstring>
 
+#include "exactint.h"
 #include "predicates.h"
 #include "threadpool.h"
 
@@ -91,11 +92,61 @@ void hilbert_order(int32_t n, const double *x, const double *y, std::vector<int3
 // ---------------------------------------------------------------------------
 // Delaunay by point insertion + Lawson flips
 
-int Delaunay::incircle(int32_t t, int32_t d) const
+Frames::Frames(const BoxConfig &b, const double *px, const double *py) : box(b), x(px), y(py)
 {
-    const Tri &T = tris[t];
-    return incircle_sos(px_[T.v[0]], py_[T.v[0]], px_[T.v[1]], py_[T.v[1]], px_[T.v[2]], py_[T.v[2]], px_[d],
-                        py_[d]);
+    // An image's coordinate is off by at most 2^-53 M, M the largest one, so a
+    // difference of two by two of those; the determinant's derivative by each
+    // of its six differences is at most 8 r^3, with r the largest of them:
+    // 96 2^-53 M r^3.
+    const double M = std::max(std::max(std::fabs(b.x0), std::fabs(b.x1)), std::max(std::fabs(b.y0), std::fabs(b.y1))) +
+                     2.0 * std::max(b.x1 - b.x0, b.y1 - b.y0);
+    widen = 128.0 * 0x1p-53 * M;
+}
+
+// In-circle of counter-clockwise a, b, c against d with the tie-break (> 0:
+// inside), as incircle_sos, and with frames where the images' rounding matters.
+inline int Delaunay::incircle(int32_t a, int32_t b, int32_t c, int32_t d) const
+{
+    if (!framed_) return incircle_sos(px_[a], py_[a], px_[b], py_[b], px_[c], py_[c], px_[d], py_[d]);
+    const double adx = px_[a] - px_[d], ady = py_[a] - py_[d], bdx = px_[b] - px_[d], bdy = py_[b] - py_[d];
+    const double cdx = px_[c] - px_[d], cdy = py_[c] - py_[d];
+    const double p1 = bdx * cdy, p2 = cdx * bdy, p3 = cdx * ady, p4 = adx * cdy, p5 = adx * bdy, p6 = bdx * ady;
+    const double la = adx * adx + ady * ady, lb = bdx * bdx + bdy * bdy, lc = cdx * cdx + cdy * cdy;
+    const double det = la * (p1 - p2) + lb * (p3 - p4) + lc * (p5 - p6);
+    const double sides = std::fabs(adx) + std::fabs(ady) + std::fabs(bdx) + std::fabs(bdy) + std::fabs(cdx) +
+                         std::fabs(cdy);
+    const double bound = kIncircleBound * (la * (std::fabs(p1) + std::fabs(p2)) + lb * (std::fabs(p3) + std::fabs(p4)) +
+                                           lc * (std::fabs(p5) + std::fabs(p6))) +
+                         frames_.widen * sides * (la + lb + lc);
+    // (an infinite bound, or a NaN, goes on)
+    if (det > bound) return 1;
+    if (-det > bound) return -1;
+    return incircle_near(a, b, c, d);
+}
+
+int Delaunay::incircle_near(int32_t a, int32_t b, int32_t c, int32_t d) const
+{
+    const int32_t v[4] = {a, b, c, d};
+    auto plain = [&] { return incircle_sos(px_[a], py_[a], px_[b], py_[b], px_[c], py_[c], px_[d], py_[d]); };
+    exactint::Images m{};
+    m.Lx = frames_.box.x1 - frames_.box.x0;
+    m.Ly = frames_.box.y1 - frames_.box.y0;
+    int64_t images = 0;
+    for (int k = 0; k < 4; k++) {
+        const int32_t q = v[k];
+        // (a corner; or a vertex that move_all holds at its old position)
+        if (ref_[q] < 0 || ((size_t)q < back_.size() && back_[q])) return plain();
+        const int64_t src = ref_[q] >> 4;
+        const int img = (int)(ref_[q] & 15);
+        images |= img ^ 4;
+        m.x[k] = frames_.x[src];
+        m.y[k] = frames_.y[src];
+        m.kx[k] = (int8_t)(img % 3);
+        m.ky[k] = (int8_t)(img / 3);
+    }
+    if (!images) return plain();
+    const int s = exactint::incircle_images(m);
+    return s == exactint::kUnknown ? plain() : s;
 }
 
 void Delaunay::set_nb(int32_t t, int32_t old_nb, int32_t new_nb)
@@ -230,7 +281,11 @@ void Delaunay::legalize(int32_t p)
         while (m < 3 && U.nb[m] != t) m++;
         if (m == 3) continue;
         int32_t d = U.v[m];
-        if (incircle(t, d) <= 0) continue;
+        if (incircle(T.v[0], T.v[1], T.v[2], d) <= 0) continue;
+        if (!spend()) {
+            stack_.clear();
+            return;
+        }
         // flip edge (b, c) of T = (p, b, c) and U = (d, c, b) into (b, d)
         int32_t b = T.v[1], c = T.v[2];
         int32_t T_cp = T.nb[1], T_pb = T.nb[2];
@@ -246,8 +301,19 @@ void Delaunay::legalize(int32_t p)
     }
 }
 
-int Delaunay::build(const double *x, const double *y, int32_t np)
+int Delaunay::build(const double *x, const double *y, int32_t np, const Frames *frames, const int64_t *refs)
 {
+    framed_ = frames != nullptr;
+    flips_left_ = INT64_MAX;
+    back_.clear();
+    ref_.clear();
+    if (framed_) {
+        frames_ = *frames;
+        ref_.assign(refs, refs + np);
+        ref_.resize((size_t)np + 3, -1);
+        // (an insertion takes three flips in the mean)
+        flips_left_ = 64 * (int64_t)np + 65536;
+    }
     log_.clear();
     log_all_ = true;
     tris.clear();
@@ -282,6 +348,7 @@ int Delaunay::build(const double *x, const double *y, int32_t np)
         if (r < 0) return -3;
         if (r == 0) insert_inside(t, p);
         else insert_on_edge(t, edge, p);
+        if (flips_left_ < 0) return -5;
     }
     return 0;
 }
@@ -401,6 +468,7 @@ int Delaunay::insert_at(int32_t v)
 bool Delaunay::move_all(const std::vector<double> &nx, const std::vector<double> &ny, int32_t max_back)
 {
     const int32_t NV = size();
+    if (framed_) flips_left_ = 64 * (int64_t)NV + 65536;
     old_x_.assign(px_.begin(), px_.end());
     old_y_.assign(py_.begin(), py_.end());
     const std::vector<double> &ox = old_x_, &oy = old_y_;
@@ -459,6 +527,7 @@ bool Delaunay::move_all(const std::vector<double> &nx, const std::vector<double>
     if ((int32_t)S.size() > max_back) return false;
     const size_t mark = log_.size();
     make_delaunay();
+    if (flips_left_ < 0) return false;
     if (S.empty()) return true;
     // out with them.  A triangle of each: the one it was put back from,
     // unless the flips rewrote it (then the vertex is in a rewritten slot,
@@ -497,9 +566,10 @@ bool Delaunay::move_all(const std::vector<double> &nx, const std::vector<double>
     for (int32_t v : S) {
         px_[v] = nx[v];
         py_[v] = ny[v];
+        back[v] = 0;
         const int32_t h = where[v];
         if (h >= 0 && h < (int32_t)tris.size() && tris[h].v[0] >= 0) hint_ = h;
-        if (insert_at(v) != 0) return false;
+        if (insert_at(v) != 0 || flips_left_ < 0) return false;
     }
     reinserted += (int64_t)S.size();
     return true;
@@ -551,7 +621,7 @@ void Delaunay::make_delaunay(const std::vector<int32_t> *seed)
                 const Tri &U = tris[T.nb[k]];
                 const int32_t a = T.v[k], b = T.v[(k + 1) % 3], c = T.v[(k + 2) % 3];
                 const int32_t d = U.v[0] ^ U.v[1] ^ U.v[2] ^ b ^ c;
-                if (incircle_sos(px_[a], py_[a], px_[b], py_[b], px_[c], py_[c], px_[d], py_[d]) > 0)
+                if (incircle(a, b, c, d) > 0)
                     edges_.push_back(((int64_t)t << 2) | k);
             }
         }
@@ -567,7 +637,11 @@ void Delaunay::make_delaunay(const std::vector<int32_t> *seed)
         const Tri &U = tris[u];
         const int32_t a = T.v[k], b = T.v[(k + 1) % 3], c = T.v[(k + 2) % 3];
         const int32_t d = U.v[0] ^ U.v[1] ^ U.v[2] ^ b ^ c;
-        if (incircle_sos(px_[a], py_[a], px_[b], py_[b], px_[c], py_[c], px_[d], py_[d]) <= 0) continue;
+        if (incircle(a, b, c, d) <= 0) continue;
+        if (!spend()) {
+            edges_.clear();
+            return;
+        }
         // flip edge (b, c) of (a, b, c) and (d, c, b) into (a, d)
         flip(t, k);
         edges_.push_back(((int64_t)t << 2) | 0);
@@ -577,11 +651,12 @@ void Delaunay::make_delaunay(const std::vector<int32_t> *seed)
     }
 }
 
-int32_t Delaunay::insert_point(double x, double y)
+int32_t Delaunay::insert_point(double x, double y, int64_t ref)
 {
     const int32_t p = (int32_t)px_.size();
     px_.push_back(x);
     py_.push_back(y);
+    if (framed_) ref_.push_back(ref);
     int32_t t = -1;
     int edge = -1;
     const int r = locate(p, t, edge);
@@ -589,6 +664,7 @@ int32_t Delaunay::insert_point(double x, double y)
     if (r < 0) return -3;
     if (r == 0) insert_inside(t, p);
     else insert_on_edge(t, edge, p);
+    if (flips_left_ < 0) return -3;
     return p;
 }
 
@@ -827,6 +903,7 @@ struct SlabCtx {
     const PointGrid *ggrid = nullptr;  // ghosts of this build
     const double *band = nullptr;
     double pad = 0.0;
+    const Frames *frames = nullptr;           // a periodic box
     const MeshWork *work = nullptr;           // ghost key lookup of this build
 };
 
@@ -839,6 +916,11 @@ inline int64_t point_key(const SlabCtx &c, int32_t q)
     if (q < c.n) return q;
     const int32_t g = q - c.n;
     return (int64_t)c.n + 9 * (int64_t)c.m->ghost_src[g] + c.m->ghost_img[g];
+}
+
+inline int64_t ref_of_key(const SlabCtx &c, int64_t k)
+{
+    return k < c.n ? vertex_ref(k, 4) : vertex_ref((k - c.n) / 9, (int32_t)((k - c.n) % 9));
 }
 
 // The tile's rectangle with its halo (a halo that covers every point makes
@@ -889,7 +971,8 @@ bool update_slab(const SlabCtx &c, const Rect &R, Delaunay &dt, std::vector<int3
                  std::vector<double> &ny)
 {
     const int32_t NL = dt.size();
-    if ((int32_t)keys.size() != NL || NL < 3) return false;
+    if ((int32_t)keys.size() != NL || NL < 3 || dt.framed() != (c.frames != nullptr)) return false;
+    if (c.frames) dt.set_frames(*c.frames);
     const MeshWork &w = *c.work;
     if ((int32_t)stamp.size() < c.np) stamp.resize(c.np, 0u);
     loc.resize(NL);
@@ -940,13 +1023,14 @@ bool update_slab(const SlabCtx &c, const Rect &R, Delaunay &dt, std::vector<int3
     bool ok = true;
     for_rect_points(c, R, [&](int32_t q) {
         if (!ok || stamp[q] == w.gen) return;
-        const int32_t v = dt.insert_point(c.X[q], c.Y[q]);
+        const int64_t key = point_key(c, q);
+        const int32_t v = dt.insert_point(c.X[q], c.Y[q], ref_of_key(c, key));
         if (v < 0) {
             ok = false;
             return;
         }
         loc.push_back(q);
-        keys.push_back(point_key(c, q));
+        keys.push_back(key);
         stamp[q] = w.gen;
     });
     return ok;
@@ -1240,11 +1324,19 @@ void build_slab(const SlabCtx &c, const Tile &tile, double H, bool update, Delau
     }
     const int32_t nl = (int32_t)loc.size();
     if (nl == 0) return;
-    r.rc = dt.build(LX.data(), LY.data(), nl);
+    keys.resize(nl);
+    for (int32_t v = 0; v < nl; v++) keys[v] = point_key(c, loc[v]);
+    r.rc = -5;
+    if (c.frames) {
+        std::vector<int64_t> refs(nl);
+        for (int32_t v = 0; v < nl; v++) refs[v] = ref_of_key(c, keys[v]);
+        r.rc = dt.build(LX.data(), LY.data(), nl, c.frames, refs.data());
+    }
+    // (walls; or flips that do not end: every test in the tile's own frame)
+    if (r.rc == -5) r.rc = dt.build(LX.data(), LY.data(), nl);
     if (r.rc) return;
     loc.resize(nl + 3, -2);
     keys.resize(nl + 3, -2);
-    for (int32_t v = 0; v < nl; v++) keys[v] = point_key(c, loc[v]);
     read_stars(c, tile, R, dt, loc, r);
     if (r.rc == kRedo) r.rc = -3;  // (a fresh build has no stale images)
 }
@@ -1411,6 +1503,8 @@ int build_host_mesh(const BoxConfig &box, int32_t n, const double *x, const doub
         ctx.band = band;
         ctx.pad = pad;
         ctx.work = &work;
+        const Frames frames(box, X.data(), Y.data());
+        ctx.frames = box.boundary == 1 ? &frames : nullptr;
         // column cuts at x-quantiles of (a sample of) the real + ghost
         // points, then row cuts at y-quantiles within each column (or the
         // last build's tiles, to update them in place)

@@ -65,6 +65,26 @@ struct HostMesh {
     int attempts = 0;
 };
 
+// The periodic box whose images a triangulation holds.  An image's coordinates
+// are rounded, so four nearly co-circular points can come out on one side of a
+// circle near one boundary and on the other near the opposite one, where the
+// same four are other images: their cells would disagree about the edge
+// between them.  In-circle tests that the rounding of the images can decide
+// therefore take the images exactly (exactint.h), as the device's mesh update
+// does, so that all copies of four points come to the same answer, that of one
+// point set.
+struct Frames {
+    BoxConfig box;
+    const double *x = nullptr, *y = nullptr;  // the real points
+    // what the images' rounding can change an in-circle determinant by, per
+    // (sum of coordinate differences) (sum of their squares)
+    double widen = 0.0;
+    Frames() = default;
+    Frames(const BoxConfig &b, const double *px, const double *py);
+};
+// a vertex's point: real point src's image img ((a+1) + 3*(b+1), 4: itself)
+inline int64_t vertex_ref(int64_t src, int32_t img) { return src * 16 + img; }
+
 struct Tri {
     int32_t v[3];   // counter-clockwise
     int32_t nb[3];  // nb[k]: triangle across the edge opposite v[k], -1 if none
@@ -74,8 +94,15 @@ class Delaunay {
 public:
     // Triangulate np distinct points.  Returns 0, or -2 for coincident points,
     // -3 if the construction failed.  Vertices np..np+2 are the corners of an
-    // enclosing triangle.
-    int build(const double *x, const double *y, int32_t np);
+    // enclosing triangle.  With frames, refs holds each point's vertex_ref;
+    // -5 if the flips do not end (a test that exactint.h cannot hold is taken
+    // with rounded images, and five and more nearly co-circular points then
+    // need not be those of any one point set).
+    int build(const double *x, const double *y, int32_t np, const Frames *frames = nullptr,
+              const int64_t *refs = nullptr);
+    // the real points' new positions, before move_all
+    void set_frames(const Frames &f) { frames_ = f; }
+    bool framed() const { return framed_; }
     std::vector<Tri> tris;
 
     // Vertices, corners included (corner() .. corner() + 2), and positions.
@@ -112,10 +139,10 @@ public:
     // edges of those triangles only (valid when every other edge is locally
     // Delaunay already).  insert_point adds a point after
     // the corners (returns the new vertex, -2 for a point that coincides
-    // with one, -3 if location fails).
+    // with one, -3 if location fails or the flips do not end).
     bool move_all(const std::vector<double> &nx, const std::vector<double> &ny, int32_t max_back);
     void make_delaunay(const std::vector<int32_t> *seed = nullptr);
-    int32_t insert_point(double x, double y);
+    int32_t insert_point(double x, double y, int64_t ref = -1);
     // vertices taken out and inserted again by move_all, over the object's life
     int64_t reinserted = 0;
 
@@ -124,7 +151,9 @@ private:
     void insert_inside(int32_t t, int32_t p);
     void insert_on_edge(int32_t t, int k, int32_t p);
     void legalize(int32_t p);
-    int incircle(int32_t t, int32_t d) const;
+    int incircle(int32_t a, int32_t b, int32_t c, int32_t d) const;
+    int incircle_near(int32_t a, int32_t b, int32_t c, int32_t d) const;
+    bool spend() { return --flips_left_ >= 0; }
     void set_nb(int32_t t, int32_t old_nb, int32_t new_nb);
     void alloc2(int32_t &a, int32_t &b);
     bool flip_ok(int32_t t, int k) const;
@@ -133,6 +162,12 @@ private:
     int insert_at(int32_t v);
 
     std::vector<double> px_, py_;
+    bool framed_ = false;
+    Frames frames_;
+    std::vector<int64_t> ref_;  // framed: each vertex's point (-1: a corner)
+    // flips the present build or update may still take (framed), and whether
+    // it ran out of them
+    int64_t flips_left_ = INT64_MAX;
     std::vector<int32_t> order_;
     std::vector<int32_t> stack_;
     std::vector<int64_t> edges_;

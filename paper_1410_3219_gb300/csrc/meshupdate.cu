@@ -119,7 +119,7 @@ __global__ void __launch_bounds__(kVerifyBlock) k_mesh_verify(MeshUpdate m)
 // triangles of two images a lane per image that might lie in their circle.
 // (A thread per cell spent 127 us on the walls of 4,096 cells; now 18, one
 // cell's chain of FP64 and integer predicates.)
-__global__ void __launch_bounds__(kListBlock) k_mesh_verify_open(MeshUpdate m)
+__global__ void __launch_bounds__(kListBlock, 2) k_mesh_verify_open(MeshUpdate m)
 {
     chained(m.n);
     using namespace mu;
@@ -441,7 +441,7 @@ __device__ void warp_recompute(const MeshUpdate &m, int32_t i, int32_t round, St
         const float bound = circle_error(a.l, p1, p2, pb.l, p3, p4, pd.l, p5, p6);
         if (det > bound) return false;
         if (-det > bound) return true;
-        return circle_slow(f, point_of(f, a.ref), point_of(f, pb.ref), point_of(f, pd.ref)) > 0;
+        return circle_slow(f, a.ref, pb.ref, pd.ref) > 0;
     };
     int deg = 0, last = near, turns = 0;
     bool bad = false;
@@ -459,7 +459,7 @@ __device__ void warp_recompute(const MeshUpdate &m, int32_t i, int32_t round, St
             const float p = a.fx * w.fy[c], q = a.fy * w.fx[c], cr = p - q;
             const float cb = cross_error(p, q);
             bool left = cr > cb;
-            if (!left && !(-cr > cb)) left = orient_slow(f, point_of(f, a.ref), point_of(f, w.ref[c])) > 0;
+            if (!left && !(-cr > cb)) left = orient_slow(f, a.ref, w.ref[c]) > 0;
             if (left && (best < 0 || inside(a, best, c))) best = c;
         }
         __syncwarp();
@@ -485,7 +485,7 @@ __device__ void warp_recompute(const MeshUpdate &m, int32_t i, int32_t round, St
     commit_star(m, f, round, lane < deg ? w.out[lane] : 0, deg, 0, 32, true);
 }
 
-__global__ void __launch_bounds__(kListBlock) k_mesh_recompute(MeshUpdate m, int32_t round)
+__global__ void __launch_bounds__(kListBlock, 2) k_mesh_recompute(MeshUpdate m, int32_t round)
 {
     chained(m.n);
     __shared__ StarWork work[kListWarps];
@@ -945,7 +945,7 @@ __device__ __forceinline__ void report_counters(const MeshLists &l)
 // (Three kernels before: triangles and edges with a walk per triangle and
 // per edge, and a check of both, 153 us at 1M cells with every block resident;
 // now 126 so, and 205 in the fewer blocks that run beside the FP64 stages.)
-__global__ void __launch_bounds__(128) k_mesh_lists(MeshLists l)
+__global__ void __launch_bounds__(128, 8) k_mesh_lists(MeshLists l)
 {
     chained(l.n);
     if (l.next) clear_counters(l.next, l.next_words);

@@ -160,6 +160,7 @@ struct Frame {
     const MeshUpdate *m;
     int32_t i;
     int32_t *flags;
+    const InstParams *ip;
     double xi, yi;
     double x0, x1, y0, y1;  // box
     float half_x, half_y;   // half its sides (scaled)
@@ -178,6 +179,7 @@ RICH_HD inline Frame frame_of(const MeshUpdate &m, int32_t i)
     f.flags = m.flags + k;
     f.m = &m;
     f.i = i;
+    f.ip = &ip;
     f.xi = m.x[i];
     f.yi = m.y[i];
     f.x0 = ip.x0; f.x1 = ip.x1; f.y0 = ip.y0; f.y1 = ip.y1;
@@ -286,7 +288,7 @@ RICH_HD inline float circle_error(float al, float p1, float p2, float bl, float 
 
 // orientation of a, b, c from FP64 with the host's bound, else exact
 // (0 with MU_EXACT set when the integers cannot hold it)
-RICH_MU_SLOW int orient_slow(int32_t *flags, double ax, double ay, double bx, double by, double cx, double cy)
+RICH_MU_SLOW int orient_points(int32_t *flags, double ax, double ay, double bx, double by, double cx, double cy)
 {
     const double l = (bx - ax) * (cy - ay), r = (by - ay) * (cx - ax);
     const double det = l - r, bound = kOrientBound * (fabs(l) + fabs(r));
@@ -339,8 +341,8 @@ RICH_HD inline int circle_pairs(const double x[4], const double y[4])
 
 // in-circle of counter-clockwise a, b, c and d, likewise, with the symbolic
 // tie-break of predicates.h: > 0 when d is inside
-RICH_MU_SLOW int circle_slow(int32_t *flags, double ax, double ay, double bx, double by, double cx, double cy,
-                             double dx, double dy)
+RICH_MU_SLOW int circle_points(int32_t *flags, double ax, double ay, double bx, double by, double cx, double cy,
+                                 double dx, double dy)
 {
     // (the pairs first: at walls nearly every slow test is one)
     const double px[4] = {ax, bx, cx, dx}, py[4] = {ay, by, cy, dy};
@@ -368,56 +370,85 @@ RICH_MU_SLOW int circle_slow(int32_t *flags, double ax, double ay, double bx, do
     if (lex_less(cx, cy, mx, my)) { k = 2; mx = cx; my = cy; }
     if (lex_less(dx, dy, mx, my)) { k = 3; }
     switch (k) {
-    case 0: return orient_slow(flags, bx, by, cx, cy, dx, dy);
-    case 1: return -orient_slow(flags, ax, ay, cx, cy, dx, dy);
-    case 2: return orient_slow(flags, ax, ay, bx, by, dx, dy);
-    default: return -orient_slow(flags, ax, ay, bx, by, cx, cy);
+    case 0: return orient_points(flags, bx, by, cx, cy, dx, dy);
+    case 1: return -orient_points(flags, ax, ay, cx, cy, dx, dy);
+    case 2: return orient_points(flags, ax, ay, bx, by, dx, dy);
+    default: return -orient_points(flags, ax, ay, bx, by, cx, cy);
     }
 }
 
-// Positions for the slow predicates.  In a periodic box every cell of a
-// triangle or quadrilateral has to come to the same answer, but an image's
-// coordinates are rounded, differently from each cell's own frame: near-ties
-// (a drifting lattice is made of them) would then be decided differently on
-// the two sides of the boundary.  So the points are taken in the frame of the
-// smallest cell among them, one of the frames the host builder tests them in.
-RICH_HD inline double shifted(double v, double lo, double hi, int k)
+// The slow predicates of images in a periodic box.  Every cell of a triangle
+// or quadrilateral has to come to the same answer, but an image's coordinates
+// are rounded, differently from each cell's own frame: near-ties (a drifting
+// lattice is made of them) would then be decided differently on the two sides
+// of the boundary.  So the images are taken exactly, as the host builder takes
+// them: a cell's position and whole box sides.  (X, Y: the cells' positions;
+// ref: the cell, a, b and for the in-circle test d.)
+RICH_MU_SLOW int images_slow(int32_t *flags, const double *X, const double *Y, int32_t i, int32_t a, int32_t b,
+                             int32_t d, double Lx, double Ly, bool circle)
 {
-    const double L = hi - lo;
-    return k == 0 ? v : (k > 0 ? v + (k > 1 ? L + L : L) : v - (k < -1 ? L + L : L));
-}
-
-RICH_HD inline void common_frame(const Frame &f, const int32_t *ref, int n, double *x, double *y)
-{
-    int32_t least = ref[0];
-    for (int k = 1; k < n; k++) least = (ref[k] >> 4) < (least >> 4) ? ref[k] : least;
-    const int a0 = (least & 15) % 3, b0 = (least & 15) / 3;
-    for (int k = 0; k < n; k++) {
-        x[k] = shifted(f.m->x[ref[k] >> 4], f.x0, f.x1, (ref[k] & 15) % 3 - a0);
-        y[k] = shifted(f.m->y[ref[k] >> 4], f.y0, f.y1, (ref[k] & 15) / 3 - b0);
+    exactint::Images m;
+    m.Lx = Lx;
+    m.Ly = Ly;
+    const int32_t ref[4] = {i * 16 + 4, a, b, d};
+    for (int k = 0; k < 4; k++) {
+        m.x[k] = X[ref[k] >> 4];
+        m.y[k] = Y[ref[k] >> 4];
+        m.kx[k] = (int8_t)((ref[k] & 15) % 3);
+        m.ky[k] = (int8_t)((ref[k] & 15) / 3);
     }
+    const int s = circle ? exactint::incircle_images(m) : exactint::orient_images(m);
+    if (s != exactint::kUnknown) return s;
+    a_or(flags, MU_EXACT);
+    return 0;
 }
 
 // orientation of (cell, a, b)
 RICH_HD inline int orient_slow(const Frame &f, const Point &a, const Point &b)
 {
-    double x[3] = {f.xi, a.x, b.x}, y[3] = {f.yi, a.y, b.y};
-    if (f.periodic) {
-        const int32_t ref[3] = {f.i * 16 + 4, a.ref, b.ref};
-        common_frame(f, ref, 3, x, y);
-    }
-    return orient_slow(f.flags, x[0], y[0], x[1], y[1], x[2], y[2]);
+    if (f.periodic && ((a.ref & 15) != 4 || (b.ref & 15) != 4))
+        return images_slow(f.flags, f.m->x, f.m->y, f.i, a.ref, b.ref, b.ref, f.x1 - f.x0, f.y1 - f.y0, false);
+    return orient_points(f.flags, f.xi, f.yi, a.x, a.y, b.x, b.y);
 }
 
 // d against the circle of the counter-clockwise (cell, a, b)
 RICH_HD inline int circle_slow(const Frame &f, const Point &a, const Point &b, const Point &d)
 {
-    double x[4] = {f.xi, a.x, b.x, d.x}, y[4] = {f.yi, a.y, b.y, d.y};
-    if (f.periodic) {
-        const int32_t ref[4] = {f.i * 16 + 4, a.ref, b.ref, d.ref};
-        common_frame(f, ref, 4, x, y);
+    if (f.periodic && ((a.ref & 15) != 4 || (b.ref & 15) != 4 || (d.ref & 15) != 4))
+        return images_slow(f.flags, f.m->x, f.m->y, f.i, a.ref, b.ref, d.ref, f.x1 - f.x0, f.y1 - f.y0, true);
+    return circle_points(f.flags, f.xi, f.yi, a.x, a.y, b.x, b.y, d.x, d.y);
+}
+
+// The same from references, for code that keeps no absolute positions: what is
+// read again here costs it less than holding them (k_mesh_recompute of 50,625
+// cells 22 us so, 25 with them; k_mesh_verify_open, which has them at hand, 24
+// with them and 28 so).
+RICH_MU_SLOW int refs_slow(int32_t *flags, const double *X, const double *Y, const InstParams *ip, int32_t i,
+                           int32_t a, int32_t b, int32_t d, bool circle)
+{
+    const bool periodic = ip->boundary == 1;
+    const int32_t ref[4] = {i * 16 + 4, a, b, d};
+    if (periodic && ((a & 15) != 4 || (b & 15) != 4 || (d & 15) != 4))
+        return images_slow(flags, X, Y, i, a, b, d, ip->x1 - ip->x0, ip->y1 - ip->y0, circle);
+    double x[4], y[4];
+    for (int k = 0; k < 4; k++) {
+        const int img = ref[k] & 15;
+        x[k] = X[ref[k] >> 4];
+        y[k] = Y[ref[k] >> 4];
+        if (img == 4) continue;
+        x[k] = image_coord(x[k], ip->x0, ip->x1, img % 3 - 1, false);
+        y[k] = image_coord(y[k], ip->y0, ip->y1, img / 3 - 1, false);
     }
-    return circle_slow(f.flags, x[0], y[0], x[1], y[1], x[2], y[2], x[3], y[3]);
+    return circle ? circle_points(flags, x[0], y[0], x[1], y[1], x[2], y[2], x[3], y[3])
+                  : orient_points(flags, x[0], y[0], x[1], y[1], x[2], y[2]);
+}
+RICH_HD inline int orient_slow(const Frame &f, int32_t a, int32_t b)
+{
+    return refs_slow(f.flags, f.m->x, f.m->y, f.ip, f.i, a, b, b, false);
+}
+RICH_HD inline int circle_slow(const Frame &f, int32_t a, int32_t b, int32_t d)
+{
+    return refs_slow(f.flags, f.m->x, f.m->y, f.ip, f.i, a, b, d, true);
 }
 
 // > 0 when d is inside the circumcircle of the counter-clockwise (cell, a, b).
@@ -813,8 +844,6 @@ RICH_HD inline void recompute(const MeshUpdate &m, int32_t i, int32_t round)
     // (FP32 in-circle: with offsets from the cell, d is inside the circle of
     // the counter-clockwise (cell, a, b) when |a|^2 (b x d) - |b|^2 (a x d) +
     // |d|^2 (a x b) < 0)
-    // the absolute coordinates, wanted only by the slow predicates
-    auto whole = [&](int k) { return point_of(f, ref[k]); };
     // gift wrapping from the nearest candidate (always a neighbour): the next
     // one is the point to the left of the last whose circle with the cell and
     // the last is empty
@@ -834,7 +863,7 @@ RICH_HD inline void recompute(const MeshUpdate &m, int32_t i, int32_t round)
             const float p = a.fx * fy[k], q = a.fy * fx[k], c = p - q;
             const float cb = cross_error(p, q);
             bool left = c > cb;
-            if (!left && !(-c > cb)) left = orient_slow(f, whole(last), whole(k)) > 0;
+            if (!left && !(-c > cb)) left = orient_slow(f, ref[last], ref[k]) > 0;
             if (!left) continue;
             if (best < 0) {
                 best = k;
@@ -845,7 +874,7 @@ RICH_HD inline void recompute(const MeshUpdate &m, int32_t i, int32_t round)
             const float det = a.l * (p1 - p2) - b.l * c + fl[k] * (p5 - p6);
             const float bound = circle_error(a.l, p1, p2, b.l, p, q, fl[k], p5, p6);
             if (det > bound) continue;
-            if (-det > bound || circle_slow(f, whole(last), whole(best), whole(k)) > 0) best = k;
+            if (-det > bound || circle_slow(f, ref[last], ref[best], ref[k]) > 0) best = k;
         }
         if (best < 0) {
             bad = true;

@@ -253,3 +253,22 @@ def test_a_member_left_to_the_host_leaves_the_others_on_the_device(R, place):
             assert np.array_equal(got[f], want[f]), (sid, f)
         solo.close()
     b.close()
+
+
+@pytest.mark.parametrize("n_side", [32, 33])
+def test_drifting_lattice_equals_fresh_builds_and_restarts(R, n_side):
+    """Near-ties across the periodic boundary: the device's mesh is the host's
+    entry by entry at every step, and a restart from a checkpoint, whose
+    first mesh is the host's, continues bit for bit."""
+    sim = R.Sim(W.advection(n_side=n_side))
+    for k in range(40):
+        sim.step(3)
+        assert R.rich_mesh_check(sim.h) == (0, 3 * (k + 1))
+        if k == 20:
+            other = R.Sim.restart(W.advection(n_side=n_side)["cfg"], sim.checkpoint())
+    other.step(3 * 19)
+    got, want = other.conserved(), sim.conserved()
+    for f in want:
+        assert np.array_equal(got[f], want[f]), f
+    sim.close()
+    other.close()

@@ -138,3 +138,38 @@ def test_boxes_of_any_unit(side, boundary):
         cfg = W.default_cfg(boundary=boundary, x0=0.0, x1=side, y0=0.0, y1=side)
         mismatched, updated, _ = R.rich_device_update_check(cfg, xs, ys)
         assert (mismatched, updated) == (0, 5)
+
+
+def _drifting(n_side, noise, steps, holes, seed=0):
+    """A square lattice (with holes of 2 x 2 points: eight co-circular points
+    around each) that drifts through a periodic box, its positions off the
+    lattice by their rounding and by `noise`."""
+    wl = W.advection(n_side=n_side)
+    x, y = wl["x"], wl["y"]
+    if holes:
+        i, j = np.arange(n_side * n_side) % n_side, np.arange(n_side * n_side) // n_side
+        keep = ~(((i % 8) // 2 == 0) & ((j % 8) // 2 == 0))
+        x, y = x[keep], y[keep]
+    rng = np.random.default_rng(seed)
+    xs, ys = [], []
+    for _ in range(steps):
+        x, y = -0.5 + np.mod(x + 0.5, 1.0), -0.5 + np.mod(y + 0.5, 1.0)
+        x, y = np.where(x >= 0.5, -0.5, x), np.where(y >= 0.5, -0.5, y)
+        xs.append(x)
+        ys.append(y)
+        x = x + 0.231 / n_side + rng.uniform(-noise, noise, x.size)
+        y = y + 0.231 / n_side + rng.uniform(-noise, noise, y.size)
+    return np.array(xs), np.array(ys), wl["cfg"]
+
+
+@pytest.mark.parametrize("holes", [False, True])
+@pytest.mark.parametrize("n_side", [24, 33])
+@pytest.mark.parametrize("noise", [0.0, 1e-16, 1e-15, 1e-14])
+def test_near_ties_across_the_periodic_boundary(n_side, noise, holes):
+    """In-circle tests that the rounding of periodic images decides: every copy
+    of the four points must come to the same answer, in the update and in the
+    host builder (fresh and in place, whose lists must close)."""
+    xs, ys, cfg = _drifting(n_side, noise, 40, holes)
+    mismatched, updated, _ = R.rich_device_update_check(cfg, xs, ys)
+    assert (mismatched, updated) == (0, 39)
+    assert R.rich_mesh_update_check(cfg, xs, ys)[0] == 0
