@@ -133,7 +133,7 @@ struct rich_batch {
     int cur = 0;
     // device
     DBuf x[2], y[2], U[2], A, o, W, cs, g, gl, alpha, w, tess, rounding, p64, cell_inst, initW, src;
-    DBuf psrc, moved, ccx, ccy, eL, emlx, emly, emrx, emry, enx, eny, eqx, eqy, F, ePM;
+    DBuf psrc, ccx, ccy, eL, emlx, emly, emrx, emry, enx, eny, eqx, eqy, F, ePM;
     DBuf instp, dtmin, dtout, status, dsizes, gsync, listbad;
     // launch shape: autotuned over the first steps unless fixed by the caller
     int launch_mode = 0;  // 0 autotune, 1 staged, 2 persistent
@@ -210,7 +210,7 @@ struct rich_batch {
         p.g = g.as<rich::Vec4<R>>(); p.gl = gl.as<rich::Vec4<R>>(); p.alpha = alpha.as<rich::Vec4<R>>();
         p.w = w.as<rich::Vec2<R>>();
         p.rounding = rounding.as<uint8_t>(); p.p64 = p64.as<double>();
-        p.tess = tess.as<int32_t>(); p.F = F.as<rich::Vec4<R>>(); p.psrc = psrc.as<rich::Vec4<R>>(); p.moved = moved.as<rich::Vec2<R>>();
+        p.tess = tess.as<int32_t>(); p.F = F.as<rich::Vec4<R>>(); p.psrc = psrc.as<rich::Vec4<R>>();
         p.dtmin_bits = dtmin.as<unsigned long long>();
         p.dt_out = dtout.as<double>();
         p.status = status.as<int32_t>();
@@ -339,7 +339,7 @@ int ensure_device(rich_batch *b)
     CUDA_TRY(b->g.ensure(8 * N * r + 64)); CUDA_TRY(b->gl.ensure(8 * N * r + 64));
     CUDA_TRY(b->alpha.ensure(4 * N * r + 32)); CUDA_TRY(b->w.ensure(2 * N * r + 16));
     CUDA_TRY(b->tess.ensure(N * 4 + 4)); CUDA_TRY(b->rounding.ensure(N + 8)); CUDA_TRY(b->p64.ensure(N * d + 8));
-    CUDA_TRY(b->psrc.ensure(4 * N * r + 32)); CUDA_TRY(b->moved.ensure(2 * N * r + 16));
+    CUDA_TRY(b->psrc.ensure(4 * N * r + 32));
     CUDA_TRY(b->instp.ensure(K * sizeof(rich::InstParams) + 8));
     CUDA_TRY(b->dtmin.ensure(K * 8 + 8)); CUDA_TRY(b->dtout.ensure(K * 8 + 8)); CUDA_TRY(b->status.ensure(K * 4 + 8));
     CUDA_TRY(b->h_back.ensure(K * 12 + 64));

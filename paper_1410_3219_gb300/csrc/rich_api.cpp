@@ -121,7 +121,7 @@ struct rich_sim {
     double last_dt = 0.0;
     // device buffers
     DBuf x[3], y[3], U[3];
-    DBuf A, o, W, cs, g, gl, alpha, w, tess, initW, rounding, p64, psrc, moved;
+    DBuf A, o, W, cs, g, gl, alpha, w, tess, initW, rounding, p64, psrc;
     bool diagnostics = true;
     DBuf cell_of, unperm;  // internal cell of each caller index; reordered state for reads
     rich::HBuf read_host;  // (small reads)
@@ -166,7 +166,7 @@ struct rich_sim {
         p.g = g.as<rich::Vec4<R>>(); p.gl = gl.as<rich::Vec4<R>>(); p.alpha = alpha.as<rich::Vec4<R>>();
         p.w = w.as<rich::Vec2<R>>();
         p.rounding = rounding.as<uint8_t>(); p.p64 = p64.as<double>();
-        p.tess = tess.as<int32_t>(); p.F = F.as<rich::Vec4<R>>(); p.psrc = psrc.as<rich::Vec4<R>>(); p.moved = moved.as<rich::Vec2<R>>();
+        p.tess = tess.as<int32_t>(); p.F = F.as<rich::Vec4<R>>(); p.psrc = psrc.as<rich::Vec4<R>>();
         char *sc = scal.as<char>();
         p.dtmin_bits = reinterpret_cast<unsigned long long *>(sc);
         p.dt_out = reinterpret_cast<double *>(sc + 8);
@@ -244,7 +244,7 @@ int alloc_cells(rich_sim *s)
     CUDA_TRY(s->A.ensure(n * d)); CUDA_TRY(s->o.ensure(2 * n * r));
     CUDA_TRY(s->W.ensure(4 * n * r)); CUDA_TRY(s->cs.ensure(n * r));
     CUDA_TRY(s->g.ensure(8 * n * r)); CUDA_TRY(s->gl.ensure(8 * n * r)); CUDA_TRY(s->alpha.ensure(4 * n * r));
-    CUDA_TRY(s->w.ensure(2 * n * r)); CUDA_TRY(s->tess.ensure(n * 4)); CUDA_TRY(s->psrc.ensure(4 * n * r)); CUDA_TRY(s->moved.ensure(2 * n * r));
+    CUDA_TRY(s->w.ensure(2 * n * r)); CUDA_TRY(s->tess.ensure(n * 4)); CUDA_TRY(s->psrc.ensure(4 * n * r));
     CUDA_TRY(s->rounding.ensure(n)); CUDA_TRY(s->p64.ensure(n * d));
     CUDA_TRY(s->scal.ensure(64));
     CUDA_TRY(cudaMemsetAsync(s->scal.p, 0, 64, s->stream));

@@ -496,10 +496,9 @@ template <class R> __device__ __forceinline__ double step_dt(const SweepParams<R
 //    evaluates one extrapolated difference per limited variable (and none for
 //    an unlimited one) instead of four per edge; ties within the estimates'
 //    error go through every edge in FP64.
-// The prediction's cell terms come out folded: with the edge's midpoint m
-// (from the generator) and velocity w_f, Eq. 2 and the half-step prediction of
-// a side read C + g.(m + hdt w_f) with C = phi - g.(o + hdt v) - hdt S for
-// density and velocity.  (The pressure keeps its sum: see the flux.)
+// The prediction's cell terms come out with their time step: phi - hdt S for the
+// density, -hdt S for the velocity, which the flux adds to the velocity relative
+// to the edge.  (The pressure keeps its sum: see the flux.)
 // (Per cell of six slots: 204 FP64 instructions before, about 160 now.)
 template <class R, class Slots>
 __device__ __forceinline__ void stage_cell_gradient_fp64(const SweepParams<R> &p, int32_t i, int32_t lo, int32_t hi,
@@ -675,13 +674,8 @@ __device__ __forceinline__ void stage_cell_gradient_fp64(const SweepParams<R> &p
         // motion, which records dt, runs beside this stage in the persistent
         // sweep)
         const double hdt = ip.phase == 0 ? halved(step_dt(p, inst)) : 0.0;
-        const double sx = fma(hdt, Wi[1], (double)oi.x), sy = fma(hdt, Wi[2], (double)oi.y);
-        const double ldiv = lg[2] + lg[5], hd = hdt * ldiv, hr = hdt * recip(Wi[0]);
-        const double C0 = fma(-Wi[0], hd, fma(-lg[1], sy, fma(-lg[0], sx, Wi[0])));
-        const double C1 = fma(-hr, lg[6], fma(-lg[3], sy, fma(-lg[2], sx, Wi[1])));
-        const double C2 = fma(-hr, lg[7], fma(-lg[5], sy, fma(-lg[4], sx, Wi[2])));
-        p.psrc[i] = Vec4<R>{C0, C1, C2, ip.gamma * Wi[3] * ldiv};
-        p.moved[i] = Vec2<R>{sx, sy};
+        const double ldiv = lg[2] + lg[5], hr = hdt * recip(Wi[0]);
+        p.psrc[i] = Vec4<R>{fma(-Wi[0], hdt * ldiv, Wi[0]), -(hr * lg[6]), -(hr * lg[7]), ip.gamma * Wi[3] * ldiv};
     }
     if (p.diagnostics) {
         p.g[2 * i] = Vec4<R>{g[0], g[1], g[2], g[3]};
@@ -939,10 +933,14 @@ template <class R> __device__ __forceinline__ void hllc(R gam, R igm1, const R L
 }
 
 // a7 in FP64: as stage_edge_flux below, with about 115 FP64 instructions per
-// edge instead of 132.  The sides' density and velocity come from the cells'
-// folded terms (stage_cell_gradient_fp64); only the normal velocity is taken
-// relative to the edge for both sides, the tangential one for the side K that
-// the flux comes from; the star state and the energy flux are put together:
+// edge instead of 132.  The sides' states come from the cells' terms
+// (stage_cell_gradient_fp64) and the velocities relative to the edge, which are
+// formed first: v and the edge's own velocity are each as large as the flow
+// through the box, and what follows must not round at that size (folding
+// hdt v into the cells' terms and hdt w_f into the edge's point, eight
+// instructions fewer, multiplied the prediction's rounding by 6 at 100 sound
+// speeds and by 60 at 1,000).  Only side K's tangential velocity is formed; the
+// star state and the energy flux are put together:
 // with the contact (or, beyond the outer waves, side K's own) speed S relative
 // to the edge, density f, pressure P, internal energy density ei, and V, T the
 // normal and tangential velocity in the lab frame, the flux through the moving
@@ -973,28 +971,32 @@ template <class R> __device__ __forceinline__ void stage_edge_flux_fp64(const Sw
     const double dwc = fma(wrx - wl.x, (double)p.eqx[e], (wry - wl.y) * p.eqy[e]);
     const double wfx = fma(-dwc, nx, halved(wl.x + wrx)), wfy = fma(-dwc, ny, halved(wl.y + wry));
     const double wn = fma(wfx, nx, wfy * ny);
+    // rho, v - w_f, p of each side at the edge's midpoint, half a step on:
+    // phi + g.(m - o - hdt u) - hdt S, u = v - w_f
     double sL[4], sR[4];
     {
-        const double ax = fma(hdt, wfx, (double)p.emlx[e]), ay = fma(hdt, wfy, (double)p.emly[e]);
-        const Vec4<R> C = p.psrc[l], g0 = p.gl[2 * l], g1 = p.gl[2 * l + 1];
-        const Vec2<R> o = p.moved[l];
+        const Vec4<R> W = p.W[l], C = p.psrc[l], g0 = p.gl[2 * l], g1 = p.gl[2 * l + 1];
+        const Vec2<R> o = p.o[l];
+        const double ux = W.y - wfx, uy = W.z - wfy;
+        const double ax = fma(-hdt, ux, p.emlx[e] - o.x), ay = fma(-hdt, uy, p.emly[e] - o.y);
         sL[0] = fma(g0.x, ax, fma(g0.y, ay, C.x));
-        sL[1] = fma(g0.z, ax, fma(g0.w, ay, C.y));
-        sL[2] = fma(g1.x, ax, fma(g1.y, ay, C.z));
-        sL[3] = fma(-hdt, C.w, fma(g1.w, ay - o.y, fma(g1.z, ax - o.x, p.W[l].w)));
+        sL[1] = fma(g0.z, ax, fma(g0.w, ay, ux + C.y));
+        sL[2] = fma(g1.x, ax, fma(g1.y, ay, uy + C.z));
+        sL[3] = fma(-hdt, C.w, fma(g1.w, ay, fma(g1.z, ax, W.w)));
     }
     {
         // a mirrored source: each derivative takes the flip of its axis,
         // velocity components also the flip of their own axis
-        const double ax = fma(hdt, wfx, (double)p.emrx[e]), ay = fma(hdt, wfy, (double)p.emry[e]);
-        const Vec4<R> C = p.psrc[k], g0 = p.gl[2 * k], g1 = p.gl[2 * k + 1];
-        const Vec2<R> o = p.moved[k];
+        const Vec4<R> W = p.W[k], C = p.psrc[k], g0 = p.gl[2 * k], g1 = p.gl[2 * k + 1];
+        const Vec2<R> o = p.o[k];
+        const double ux = flip(W.y, mx) - wfx, uy = flip(W.z, my) - wfy;
+        const double ax = fma(-hdt, ux, p.emrx[e] - flip(o.x, mx)), ay = fma(-hdt, uy, p.emry[e] - flip(o.y, my));
         sR[0] = fma(flip(g0.x, mx), ax, fma(flip(g0.y, my), ay, C.x));
-        sR[1] = fma(g0.z, ax, fma(flip(g0.w, mxy), ay, flip(C.y, mx)));
-        sR[2] = fma(flip(g1.x, mxy), ax, fma(g1.y, ay, flip(C.z, my)));
-        sR[3] = fma(-hdt, C.w, fma(flip(g1.w, my), ay - flip(o.y, my), fma(flip(g1.z, mx), ax - flip(o.x, mx), p.W[k].w)));
+        sR[1] = fma(g0.z, ax, fma(flip(g0.w, mxy), ay, ux + flip(C.y, mx)));
+        sR[2] = fma(flip(g1.x, mxy), ax, fma(g1.y, ay, uy + flip(C.z, my)));
+        sR[3] = fma(-hdt, C.w, fma(flip(g1.w, my), ay, fma(flip(g1.z, mx), ax, W.w)));
     }
-    const double uL = fma(sL[1], nx, fma(sL[2], ny, -wn)), uR = fma(sR[1], nx, fma(sR[2], ny, -wn));
+    const double uL = fma(sL[1], nx, sL[2] * ny), uR = fma(sR[1], nx, sR[2] * ny);
     const double rL = sL[0], rR = sR[0], pL = sL[3], pR = sR[3];
     // c = sqrt(gamma p / rho) = gamma p / sqrt(gamma p rho)
     const double gam = ip.gamma, gpL = gam * pL, gpR = gam * pR;
@@ -1009,7 +1011,7 @@ template <class R> __device__ __forceinline__ void stage_edge_flux_fp64(const Sw
     const double num = fma(-uR, mR, fma(uL, mL, pR - pL)), den = mL - mR;
     const bool useL = supL || (sub && key_nonpos(num));
     const double rK = useL ? rL : rR, uK = useL ? uL : uR, pK = useL ? pL : pR;
-    const double tK = fma((useL ? sL[2] : sR[2]) - wfy, nx, -(((useL ? sL[1] : sR[1]) - wfx) * ny));
+    const double tK = fma(useL ? sL[2] : sR[2], nx, -((useL ? sL[1] : sR[1]) * ny));
     const double igm1 = ip.igm1, ruK = rK * uK;
     double S = uK, f = rK, P = pK, ei, F1 = fma(ruK, uK, pK);
     if (sub) {

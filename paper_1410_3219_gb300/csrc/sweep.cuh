@@ -122,11 +122,9 @@ template <class R> struct SweepParams {
     Vec4<R> *gl, *g, *alpha;
     // per cell, from the limited gradient: the cell-only terms of the
     // half-step prediction.  Split: {rho div v, (dp/dx)/rho, (dp/dy)/rho,
-    // gamma p div v}.  FP64: the first three folded into the extrapolation,
-    // {C_rho, C_vx, C_vy, gamma p div v} with C = phi - g.s - hdt S about
-    // s = o + hdt v (moved)
+    // gamma p div v}.  FP64, with half the time step: {rho - hdt rho div v,
+    // -hdt (dp/dx)/rho, -hdt (dp/dy)/rho, gamma p div v}
     Vec4<R> *psrc;
-    Vec2<R> *moved;  // (see psrc; FP64 only)
     Vec2<R> *w;
     int32_t *tess;
     Vec4<R> *F;  // L_ij F_ij in the reconstruction precision (see the flux layout)
