@@ -83,7 +83,8 @@ struct rich_sim {
     int32_t n = 0;
     std::vector<int32_t> perm;  // internal -> caller index
     // host copy of the points (internal order) for the host builder,
-    // page-locked: x at [0, n), y at [n, 2n)
+    // page-locked: x at [0, n), y at [n, 2n), then the dt of the sweep that
+    // moved them
     rich::HBuf hpts;
     double *hx() const { return hpts.as<double>(); }
     double *hy() const { return hpts.as<double>() + n; }
@@ -98,6 +99,8 @@ struct rich_sim {
     bool mesh_on_device = false;
     rich::MeshUpdater updater;
     int64_t updates = 0;   // meshes made by it
+    int missed = 0;        // updates in a row that left the mesh to the host
+    int host_sweeps = 0;   // sweeps whose next mesh the host builds before another is tried
     rich::HBuf back;       // the step's dt and status, and the list builder's flag
     DBuf mesh_inst;        // the box and mesh_params
     rich::MeshStream mesh_stream;
@@ -356,9 +359,14 @@ int join_update(rich_sim *s)
     return RICH_OK;
 }
 
+// Sweeps between two tries of an update that keeps leaving the mesh to the host:
+// what such a try costs (an update, and a host build that no sweep hides) is
+// then little beside the host builds of the sweeps between.
+constexpr int kMostHostSweeps = 32;
+
 // After the handle's stream was waited for: the updated mesh made the current
-// one (keep), or dropped.  Where it could not be made the present mesh stays
-// on the device, and the host has to build the points' own.
+// one (keep), or dropped.  Where it could not be made the host has to build
+// the points' own.
 int finish_update(rich_sim *s, int q, bool keep, rich_step_info *info)
 {
     if (!keep) {
@@ -376,8 +384,13 @@ int finish_update(rich_sim *s, int q, bool keep, rich_step_info *info)
     }
     if (r.state != rich::MeshResult::kDone || r.flagged) {
         s->updater.forget();
+        // (the same points would fail again)
+        s->mesh_on_device = false;
+        s->missed++;
+        s->host_sweeps = s->missed < 2 ? 0 : std::min(1 << std::min(s->missed - 2, 5), kMostHostSweeps);
         return RICH_OK;
     }
+    s->missed = 0;
     s->mcur = 1 - s->mcur;
     s->msz = r.sizes;
     s->updates++;
@@ -510,7 +523,7 @@ static int create_sim(const rich_config *cfg, int64_t n, const double *x, const 
     }
     int rc = RICH_OK;
     auto bail = [&](int code) { delete s; return code; };
-    if (s->hpts.ensure(2 * (size_t)n * sizeof(double)) != cudaSuccess)
+    if (s->hpts.ensure((2 * (size_t)n + 1) * sizeof(double)) != cudaSuccess)
         return bail(fail(RICH_ENOMEM, "page-locked host points"));
     std::vector<double> Fh(4 * (size_t)n);
     double *hx = s->hx(), *hy = s->hy();
@@ -628,7 +641,25 @@ int rich_tessellate(rich_sim *s, rich_step_info *info)
     return tessellate(s, info, true);
 }
 
-static int launch_sweep(rich_sim *s, double t_end, bool update)
+// What a sweep starts once the points are moved: nothing, the update of the
+// mesh for them, or their copy (and the dt's) to the host, which builds it.
+enum class NextMesh { none, update, host };
+
+// The moved points in buffers q and the dt to the host, on the mesh stream.
+static int start_read(rich_sim *s, int q)
+{
+    rich::MeshStream &u = s->mesh_stream;
+    const size_t bytes = (size_t)s->n * sizeof(double);
+    CUDA_TRY(cudaEventRecord(u.moved, s->stream));
+    CUDA_TRY(cudaStreamWaitEvent(u.stream, u.moved, 0));
+    CUDA_TRY(cudaMemcpyAsync(s->hx(), s->x[q].p, bytes, cudaMemcpyDeviceToHost, u.stream));
+    CUDA_TRY(cudaMemcpyAsync(s->hy(), s->y[q].p, bytes, cudaMemcpyDeviceToHost, u.stream));
+    CUDA_TRY(cudaMemcpyAsync(s->hy() + s->n, s->scal.as<char>() + 8, 8, cudaMemcpyDeviceToHost, u.stream));
+    CUDA_TRY(cudaEventRecord(u.done, u.stream));
+    return RICH_OK;
+}
+
+static int launch_sweep(rich_sim *s, double t_end, NextMesh next)
 {
     rich::Range range("rich sweep launch (a1-a9)");
     if (!s) return fail(RICH_EINVAL, "NULL handle");
@@ -641,8 +672,8 @@ static int launch_sweep(rich_sim *s, double t_end, bool update)
     for (int k = 0; k < rich::NUM_STAGES; k++) {
         if (s->profiling) CUDA_TRY(cudaEventRecord(s->kev[k], s->stream));
         s->launch(k, nullptr);
-        if (update && k == rich::K_ADVANCE) {
-            int rc = start_update(s, s->next_pts());
+        if (next != NextMesh::none && k == rich::K_ADVANCE) {
+            const int q = s->next_pts(), rc = next == NextMesh::update ? start_update(s, q) : start_read(s, q);
             if (rc != RICH_OK) return rc;
         }
     }
@@ -653,7 +684,7 @@ static int launch_sweep(rich_sim *s, double t_end, bool update)
     return RICH_OK;
 }
 
-int rich_sweep(rich_sim *s, double t_end) { return launch_sweep(s, t_end, false); }
+int rich_sweep(rich_sim *s, double t_end) { return launch_sweep(s, t_end, NextMesh::none); }
 
 // The sweep's dt and status, into page-locked memory (dt, then the status)
 static int fetch_result(rich_sim *s)
@@ -731,24 +762,48 @@ int rich_sync(rich_sim *s, rich_step_info *info)
 // points are there (those stages leave the memory pipes and the FP32 and
 // integer units idle, which the update lives on), and one wait serves both.
 // A failed sweep drops the updated mesh; one that the update cannot make is
-// left to the next tessellation.
+// left to the next tessellation.  Where updates keep failing, and for sizes
+// that they do not take, the host builds the mesh beside those stages instead,
+// unless the sweep ends the run at t_end.
 static int step_sweep(rich_sim *s, double t_end, rich_step_info *info)
 {
     const int q = s->next_pts();
     // (a static mesh's points stay where they are, bit for bit: x + dt 0)
     const bool still = s->cfg.motion == RICH_MESH_EULERIAN;
-    const bool update = !still && can_update(s);
-    int rc = launch_sweep(s, t_end, update);
+    const NextMesh next = still                                   ? NextMesh::none
+                          : can_update(s) && s->host_sweeps == 0 ? NextMesh::update
+                                                                  : NextMesh::host;
+    if (next == NextMesh::host && s->host_sweeps > 0) s->host_sweeps--;
+    int rc = launch_sweep(s, t_end, next);
     if (rc != RICH_OK) return rc;
     // (the sweep's result is copied while the update still runs)
     if ((rc = fetch_result(s)) != RICH_OK) return rc;
-    if (update && (rc = join_update(s)) != RICH_OK) return rc;
+    if (next == NextMesh::update && (rc = join_update(s)) != RICH_OK) return rc;
+    bool built = false;
+    if (next == NextMesh::host) {
+        const double t0 = now_ms();
+        CUDA_TRY(cudaEventSynchronize(s->mesh_stream.done));
+        if (info) info->copy_ms += now_ms() - t0;
+        // the half-step points always get a mesh; after a full step, the
+        // points get one unless the step lands on t_end
+        if ((s->time_centred() && s->tc_phase == 0) || s->hy()[s->n] < t_end - s->t) {
+            s->tess_current = false;
+            // (a mesh that cannot be built is reported by the next
+            // tessellation of the same points)
+            built = build_mesh(s, info) == RICH_OK;
+        }
+    }
     rc = wait_sweep(s, info);
     if (still && rc == RICH_OK) {
         s->tess_current = true;
         report_sizes(s, info);
     }
-    if (!update) return rc;
+    if (next == NextMesh::host) {
+        // (after a failed sweep the host's mesh is not that of the points)
+        if (rc != RICH_OK || !built) return rc;
+        return upload_mesh(s, info);
+    }
+    if (next != NextMesh::update) return rc;
     const double t0 = now_ms();
     const int urc = finish_update(s, q, rc == RICH_OK, info);
     // (what the update takes beyond the end of the sweep)

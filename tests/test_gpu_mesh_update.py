@@ -272,3 +272,50 @@ def test_drifting_lattice_equals_fresh_builds_and_restarts(R, n_side):
         assert np.array_equal(got[f], want[f]), f
     sim.close()
     other.close()
+
+
+def _mesh_is_current(R, sim):
+    try:
+        assert R.rich_mesh_check(sim.h)[0] == 0
+        return True
+    except R.RichError as e:
+        assert e.code == R.RICH_ESTATE
+        return False
+
+
+@pytest.mark.parametrize("scheme", [W.SCHEME_EXTRAPOLATED, W.SCHEME_TIME_CENTRED])
+@pytest.mark.parametrize("name", ["hub", "small"])
+def test_meshes_left_to_the_host_are_built_beside_the_sweep(R, name, scheme):
+    """Where the update keeps failing (a cell of 40 neighbours) or is not tried
+    (49 cells), the host builds the next mesh while the sweep ends, so a step
+    leaves the mesh of its points; now and then the update is tried again.
+    Results equal those of the pieces API, which builds every mesh anew."""
+    wl = _hub() if name == "hub" else W.gresho(n_side=7)
+    wl["cfg"]["scheme"] = scheme
+    sim = R.Sim(wl)
+    current = 0
+    for _ in range(20):
+        sim.step(1)
+        current += _mesh_is_current(R, sim)
+    assert current >= (20 if name == "small" else 12)
+    if name == "small":
+        sim.step(1, R.rich_time(sim.h) + 1e-9)  # lands on t_end: no mesh is built
+        assert not _mesh_is_current(R, sim)
+    pieces = R.Sim(wl)
+    for _ in range(20 * (2 if scheme == W.SCHEME_TIME_CENTRED else 1)):
+        pieces.tessellate()
+        pieces.sweep()
+        pieces.sync()
+    if name == "small":
+        pieces.tessellate()
+        pieces.sweep(R.rich_time(pieces.h) + 1e-9)
+        pieces.sync()
+        if scheme == W.SCHEME_TIME_CENTRED:
+            pieces.tessellate()
+            pieces.sweep(R.rich_time(pieces.h) + 1e-9)
+            pieces.sync()
+    got, want = sim.conserved(), pieces.conserved()
+    for f in want:
+        assert np.array_equal(got[f], want[f]), f
+    sim.close()
+    pieces.close()
