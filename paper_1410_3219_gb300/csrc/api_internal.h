@@ -98,6 +98,15 @@ inline double now_ms()
 
 bool valid_config(const rich_config *c);
 
+// Sweeps whose next mesh the host builds, beside the sweep, before the device's
+// update is tried again: after `missed` updates in a row that left the mesh to
+// the host.  What a try costs (an update, and a host build that no sweep hides)
+// is little beside 32 host builds.
+inline int host_sweeps_after(int missed)
+{
+    return missed < 2 ? 0 : 1 << (missed < 7 ? missed - 2 : 5);
+}
+
 class ThreadPool;
 // rich_batch_create whose host work runs on a pool shared with other
 // batches (nullptr: its own pool of host_threads threads)

@@ -19,7 +19,8 @@
 // Then, every step:
 //   6. one sweep (a1-a9) runs over all cells; each simulation keeps its own
 //      time step, remaining time and status flags; the meshes are updated for
-//      the moved points (a0) beside its last stages;
+//      the moved points (a0) beside its last stages (those of simulations
+//      whose updates keep failing are built by the host meanwhile);
 //   7. simulations that reached t_end or their step budget are copied out
 //      and leave the batch; a failed step rolls back that simulation only;
 //   8. the updated meshes become the current ones.
@@ -63,8 +64,10 @@ struct BatchSim {
     rich::MeshWork mw;           // (edge lists built on the device, packed)
     rich::HostMesh hm;
     int mesh_rc = 0;
-    // hm is the mesh of its current points (read back from the device)
+    // hm is the mesh of its current points (read back from the device, or
+    // built beside the last sweep)
     bool prebuilt = false;
+    int missed = 0;  // updates in a row that left its mesh to the host
     double t = 0.0, t_end = 0.0, last_dt = 0.0;
     int64_t steps = 0, max_steps = 0;
     int state = PENDING;
@@ -127,7 +130,9 @@ struct rich_batch {
     DBuf cell_of, read_dev;
     rich::HBuf read_host;
     rich::HBuf h_back;  // dt, status per simulation, then the list builder's flag
-    cudaEvent_t ev2 = nullptr;
+    cudaEvent_t ev2 = nullptr, ev_read = nullptr;
+    rich::HBuf h_moved;  // moved points read during a sweep: x, y (packed), then dt per simulation
+    int missed = 0, host_sweeps = 0;  // as rich_sim's, of updates that failed for every simulation
     int64_t meshes_updated = 0, meshes_built = 0;  // members' meshes made on the device, and on the host
     bool diagnostics = false;
     int cur = 0;
@@ -176,7 +181,7 @@ struct rich_batch {
             if (gexec[k]) cudaGraphExecDestroy(gexec[k]);
             if (graph[k]) cudaGraphDestroy(graph[k]);
         }
-        for (cudaEvent_t e : {ev0, ev1, ev2})
+        for (cudaEvent_t e : {ev0, ev1, ev2, ev_read})
             if (e) cudaEventDestroy(e);
         if (stream) cudaStreamDestroy(stream);
     }
@@ -501,17 +506,37 @@ int join_update(rich_batch *b)
     return RICH_OK;
 }
 
+// The moved points (in buffers q) of some simulations and the time steps to the
+// host, on the mesh stream from where the batch's stream is now.
+int start_read(rich_batch *b, int q, const std::vector<BatchSim *> &sims)
+{
+    rich::MeshStream &u = b->mesh_stream;
+    const size_t N = (size_t)b->n_packed, K = b->packed.size();
+    double *h = b->h_moved.as<double>();
+    CUDA_TRY(cudaEventRecord(u.moved, b->stream));
+    CUDA_TRY(cudaStreamWaitEvent(u.stream, u.moved, 0));
+    for (const BatchSim *s : sims) {
+        const size_t co = (size_t)s->cell_off, bytes = (size_t)s->n * sizeof(double);
+        CUDA_TRY(cudaMemcpyAsync(h + co, b->x[q].as<double>() + co, bytes, cudaMemcpyDeviceToHost, u.stream));
+        CUDA_TRY(cudaMemcpyAsync(h + N + co, b->y[q].as<double>() + co, bytes, cudaMemcpyDeviceToHost, u.stream));
+    }
+    CUDA_TRY(cudaMemcpyAsync(h + 2 * N, b->dtout.p, K * sizeof(double), cudaMemcpyDeviceToHost, u.stream));
+    CUDA_TRY(cudaEventRecord(b->ev_read, u.stream));
+    return RICH_OK;
+}
+
 // The sweep stage by stage; with `update` the mesh update for the moved points
-// runs on the mesh stream beside the stages after the point motion.
-int run_staged(rich_batch *b, bool update)
+// runs on the mesh stream beside the stages after the point motion, and the
+// points of `early` are read there.
+int run_staged(rich_batch *b, bool update, const std::vector<BatchSim *> &early)
 {
     CUDA_TRY(cudaMemsetAsync(b->status.p, 0, b->status.cap, b->stream));
     for (int k = 0; k < rich::NUM_STAGES; k++) {
         b->launch(k, nullptr);
-        if (update && k == rich::K_ADVANCE) {
-            const int rc = start_update(b, 1 - b->cur);
-            if (rc) return rc;
-        }
+        if (k != rich::K_ADVANCE) continue;
+        int rc;
+        if (!early.empty() && (rc = start_read(b, 1 - b->cur, early))) return rc;
+        if (update && (rc = start_update(b, 1 - b->cur))) return rc;
     }
     CUDA_TRY(cudaGetLastError());
     b->staged_launches++;
@@ -523,6 +548,13 @@ int run_staged(rich_batch *b, bool update)
 int finish_update(rich_batch *b, int q)
 {
     b->dev_mesh = b->dev_lists = false;
+    bool all_missed = true;
+    // (a mesh made here takes the place of one that the host built meanwhile)
+    auto note = [&](BatchSim *s, bool made) {
+        s->missed = made ? 0 : s->missed + 1;
+        if (made) s->prebuilt = false;
+        if (s->state == RUNNING && made) all_missed = false;
+    };
     const rich::MeshArrays a = mesh_arrays(b, q);
     rich::MeshStore &to = b->mesh[1 - b->mcur];
     cudaStream_t st = b->mesh_stream.stream;
@@ -532,7 +564,11 @@ int finish_update(rich_batch *b, int q)
         CUDA_TRY(to.reserve(a.n, r.sizes));
         CUDA_TRY(b->updater.again(a, to.output(0), r, st));
     }
-    if (r.state != rich::MeshResult::kDone) {
+    const bool done = r.state == rich::MeshResult::kDone;
+    for (size_t k = 0; k < b->packed.size(); k++) note(b->packed[k], done && !b->updater.flags()[k]);
+    b->missed = all_missed ? b->missed + 1 : 0;
+    b->host_sweeps = rich::host_sweeps_after(b->missed);
+    if (!done || all_missed) {
         b->updater.forget();
         return RICH_OK;
     }
@@ -666,7 +702,8 @@ int batch_create(int32_t precision, int64_t max_cells, int32_t host_threads, Thr
     b->max_cells = max_cells;
     if (cudaStreamCreateWithFlags(&b->stream, cudaStreamNonBlocking) != cudaSuccess ||
         cudaEventCreate(&b->ev0) != cudaSuccess || cudaEventCreate(&b->ev1) != cudaSuccess ||
-        cudaEventCreate(&b->ev2) != cudaSuccess || b->mesh_stream.create() != cudaSuccess) {
+        cudaEventCreate(&b->ev2) != cudaSuccess || cudaEventCreate(&b->ev_read) != cudaSuccess ||
+        b->mesh_stream.create() != cudaSuccess) {
         delete b;
         return fail(RICH_ECUDA, "stream or event creation failed");
     }
@@ -971,13 +1008,26 @@ int rich_batch_step(rich_batch *b, rich_step_info *info)
     // (static meshes' points stay where they are, bit for bit: x + dt 0)
     bool still = true;
     for (const BatchSim *s : ok) still = still && s->cfg.motion == RICH_MESH_EULERIAN;
-    const bool update = !still && (int64_t)N >= rich::kMeshUpdateMin && (int64_t)N <= rich::kMeshUpdateMax;
+    const bool fits = (int64_t)N >= rich::kMeshUpdateMin && (int64_t)N <= rich::kMeshUpdateMax;
     const LaunchShape shape = pick_shape(b);
+    // simulations whose meshes the host builds while a staged sweep ends: those
+    // that the last two updates could not make (they are tried again with the
+    // others', or now and then where there are no others)
+    std::vector<BatchSim *> early;
+    bool hopeful = false;
+    for (BatchSim *s : ok) {
+        const bool wait = s->missed >= 2;
+        hopeful = hopeful || !wait;
+        if (!still && !shape.persistent && (wait || !fits)) early.push_back(s);
+    }
+    const bool update = !still && fits && (hopeful || b->host_sweeps == 0);
+    if (!still && fits && !update) b->host_sweeps--;
+    if (!early.empty()) CUDA_TRY(b->h_moved.ensure((2 * N + ok.size()) * sizeof(double)));
     CUDA_TRY(cudaEventRecord(b->ev0, b->stream));
     if (shape.persistent) {
         rc = b->precision == RICH_FP32_SPLIT ? run_persistent<float>(b, shape.block) : run_persistent<double>(b, shape.block);
     } else {
-        rc = run_staged(b, update);
+        rc = run_staged(b, update, early);
     }
     if (rc) return rc;
     CUDA_TRY(cudaEventRecord(b->ev1, b->stream));
@@ -993,7 +1043,7 @@ int rich_batch_step(rich_batch *b, rich_step_info *info)
             b->barrier_timeouts++;
             b->graph_note = "persistent sweep barrier timed out; staged launches used";
             CUDA_TRY(cudaEventRecord(b->ev0, b->stream));
-            if ((rc = run_staged(b, false))) return rc;
+            if ((rc = run_staged(b, false, {}))) return rc;
             CUDA_TRY(cudaEventRecord(b->ev1, b->stream));
         }
     }
@@ -1003,6 +1053,31 @@ int rich_batch_step(rich_batch *b, rich_step_info *info)
     CUDA_TRY(cudaMemcpyAsync(b->status_back(), b->status.p, ok.size() * 4, cudaMemcpyDeviceToHost, b->stream));
     if (update && (rc = join_update(b))) return rc;
     CUDA_TRY(cudaEventRecord(b->ev2, b->stream));
+    double t_pre = 0.0;
+    if (!early.empty()) {
+        CUDA_TRY(cudaEventSynchronize(b->ev_read));
+        const double tp = now_ms();
+        const double *h = b->h_moved.as<double>();
+        // those that go on after this step (the bookkeeping below takes the
+        // same decision), unless the step fails
+        std::vector<BatchSim *> next;
+        for (size_t k = 0; k < ok.size(); k++) {
+            BatchSim *s = ok[k];
+            if (fits && s->missed < 2) continue;
+            const double dt = h[2 * N + k], rem = s->t_end - s->t;
+            const double tn = dt >= rem ? s->t_end : s->t + dt;
+            if (tn >= s->t_end || s->steps + 1 >= s->max_steps) continue;
+            next.push_back(s);
+        }
+        b->pool->parallel_for((int64_t)next.size(), [&](int64_t k) {
+            BatchSim *s = next[k];
+            std::memcpy(s->hx.data(), h + s->cell_off, sizeof(double) * s->n);
+            std::memcpy(s->hy.data(), h + N + s->cell_off, sizeof(double) * s->n);
+        });
+        tessellate_members(b, next);
+        for (BatchSim *s : next) s->prebuilt = true;
+        t_pre = now_ms() - tp;
+    }
     CUDA_TRY(cudaStreamSynchronize(b->stream));
     float ms = 0.0f;
     cudaEventElapsedTime(&ms, b->ev0, b->ev1);
@@ -1019,6 +1094,7 @@ int rich_batch_step(rich_batch *b, rich_step_info *info)
     for (size_t k = 0; k < ok.size(); k++) {
         BatchSim *s = ok[k];
         if (status[k]) {
+            s->prebuilt = false;
             s->err = (status[k] & rich::ST_NAN) ? RICH_ENAN : RICH_ENEGATIVE;
             s->err_msg = "step rejected (non-finite, non-positive mass or thermal energy, or a point left the box)";
             finish_copy_out(b, *s, b->cur);
@@ -1054,7 +1130,7 @@ int rich_batch_step(rich_batch *b, rich_step_info *info)
     if (info) {
         info->steps_done = (int64_t)ok.size();
         info->sweep_ms = ms;
-        info->tess_ms = (t2 - t1) + up_ms + t_fin;
+        info->tess_ms = (t2 - t1) + t_pre + up_ms + t_fin;
         info->copy_ms = (t1 - t0) + (t3 - t2) + (now_ms() - tnow) - t_fin;
         info->n_ghost = b->nG;
         info->n_tri = b->nT;

@@ -359,11 +359,6 @@ int join_update(rich_sim *s)
     return RICH_OK;
 }
 
-// Sweeps between two tries of an update that keeps leaving the mesh to the host:
-// what such a try costs (an update, and a host build that no sweep hides) is
-// then little beside the host builds of the sweeps between.
-constexpr int kMostHostSweeps = 32;
-
 // After the handle's stream was waited for: the updated mesh made the current
 // one (keep), or dropped.  Where it could not be made the host has to build
 // the points' own.
@@ -387,7 +382,7 @@ int finish_update(rich_sim *s, int q, bool keep, rich_step_info *info)
         // (the same points would fail again)
         s->mesh_on_device = false;
         s->missed++;
-        s->host_sweeps = s->missed < 2 ? 0 : std::min(1 << std::min(s->missed - 2, 5), kMostHostSweeps);
+        s->host_sweeps = rich::host_sweeps_after(s->missed);
         return RICH_OK;
     }
     s->missed = 0;

@@ -319,3 +319,38 @@ def test_meshes_left_to_the_host_are_built_beside_the_sweep(R, name, scheme):
         assert np.array_equal(got[f], want[f]), f
     sim.close()
     pieces.close()
+
+
+@pytest.mark.parametrize("mode", [1, 2])
+@pytest.mark.parametrize("others", [False, True])
+def test_members_that_keep_failing_are_built_beside_the_sweep(R, mode, others):
+    """Simulations whose every update fails, alone and beside others: their
+    meshes come from the host (in a staged sweep while it ends), each once, and
+    results equal the solo runs bit for bit, also when members end or fail."""
+    wls = [_hub(), _hub(36, 24), _hub(50, 30)]
+    budget = [20, 13, 17]
+    if others:
+        wls += [W.gresho(n_side=24, seed=2), W.sod(n_side=30, seed=3)]
+        budget += [20, 9]
+    bad = W.random_mixed(n=400, seed=8)
+    bad["p"] = np.where(np.arange(400) == 7, 1e12, bad["p"])
+    b = R.Batch(max_cells=1 << 20)
+    b.set_launch(mode, 256)
+    ids = [b.add(w, max_steps=k) for w, k in zip(wls, budget)]
+    if others:
+        b.add(bad, max_steps=20)
+    for _ in range(20):
+        b.step()
+    updated, built = b.mesh_counts()
+    if not others:
+        assert (updated, built) == (0, sum(budget))
+    for w, sid, k in zip(wls, ids, budget):
+        q = b.query(sid)
+        assert q["state"] == "done" and q["steps"] == k
+        solo = R.Sim(w)
+        solo.step(k)
+        got, want = b.conserved(sid), solo.conserved()
+        for f in want:
+            assert np.array_equal(got[f], want[f]), (sid, f)
+        solo.close()
+    b.close()
