@@ -43,6 +43,7 @@ struct DBuf {
         size_t want = bytes + bytes / 4 + 256;
         cudaError_t e = cudaMalloc(&p, want);
         if (e == cudaSuccess) cap = want;
+        else cudaGetLastError();  // (reported here, not by the next launch's check)
         return e;
     }
     template <class T> T *as() const { return static_cast<T *>(p); }
@@ -68,6 +69,7 @@ struct HBuf {
         cap = 0;
         cudaError_t e = cudaMallocHost(&p, bytes);
         if (e == cudaSuccess) cap = bytes;
+        else cudaGetLastError();
         return e;
     }
     template <class T> T *as() const { return static_cast<T *>(p); }
