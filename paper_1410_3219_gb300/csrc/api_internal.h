@@ -23,6 +23,15 @@ int set_error(int code, const std::string &msg);
                                      std::string(#expr) + ": " + cudaGetErrorString(err_));       \
     } while (0)
 
+// An error other than that device memory ran out (which is cleared), for room
+// that a mesh update can do without: the host then builds the mesh.
+inline cudaError_t unless_no_room(cudaError_t e)
+{
+    if (e != cudaErrorMemoryAllocation) return e;
+    cudaGetLastError();
+    return cudaSuccess;
+}
+
 // Device allocation that only grows (25% headroom), freed with the owner.
 struct DBuf {
     void *p = nullptr;
@@ -45,6 +54,12 @@ struct DBuf {
         if (e == cudaSuccess) cap = want;
         else cudaGetLastError();  // (reported here, not by the next launch's check)
         return e;
+    }
+    void release()
+    {
+        if (p) cudaFree(p);
+        p = nullptr;
+        cap = 0;
     }
     template <class T> T *as() const { return static_cast<T *>(p); }
 };

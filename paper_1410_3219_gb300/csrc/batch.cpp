@@ -469,6 +469,12 @@ int reserve_geometry(rich_batch *b, const rich::MeshSizes &z)
     return RICH_OK;
 }
 
+// Whether the packed cells are as many as the device's update takes.
+bool fits_update(const rich_batch *b)
+{
+    return b->n_packed >= rich::kMeshUpdateMin && b->n_packed <= rich::kMeshUpdateMax;
+}
+
 rich::MeshArrays mesh_arrays(rich_batch *b, int q)
 {
     rich::MeshArrays a{};
@@ -489,13 +495,24 @@ rich::MeshArrays mesh_arrays(rich_batch *b, int q)
 
 // Enqueue the update of the packed meshes for the points in buffers q, on the
 // mesh stream from where the batch's stream is now; join_update makes the
-// batch's stream continue after it.
-int start_update(rich_batch *b, int q)
+// batch's stream continue after it.  Without memory for it nothing is enqueued,
+// `update` becomes false, and the room that updates hold is given back: the
+// host builds the meshes, as if every simulation's had failed before.
+int start_update(rich_batch *b, int q, bool &update)
 {
     rich::MeshStream &u = b->mesh_stream;
     CUDA_TRY(cudaEventRecord(u.moved, b->stream));
     CUDA_TRY(cudaStreamWaitEvent(u.stream, u.moved, 0));
-    CUDA_TRY(b->updater.start(mesh_arrays(b, q), b->mesh[1 - b->mcur].output(0), u.stream));
+    const cudaError_t e = b->updater.start(mesh_arrays(b, q), b->mesh[1 - b->mcur].output(0), u.stream);
+    CUDA_TRY(rich::unless_no_room(e));
+    if (e != cudaSuccess) {
+        update = false;
+        b->mesh[1 - b->mcur].release();
+        for (BatchSim *s : b->packed) s->missed = std::max(s->missed, 2);
+        b->missed = std::max(b->missed + 1, 2);
+        b->host_sweeps = rich::host_sweeps_after(b->missed);
+        return RICH_OK;
+    }
     CUDA_TRY(cudaEventRecord(u.done, u.stream));
     return RICH_OK;
 }
@@ -528,7 +545,7 @@ int start_read(rich_batch *b, int q, const std::vector<BatchSim *> &sims)
 // The sweep stage by stage; with `update` the mesh update for the moved points
 // runs on the mesh stream beside the stages after the point motion, and the
 // points of `early` are read there.
-int run_staged(rich_batch *b, bool update, const std::vector<BatchSim *> &early)
+int run_staged(rich_batch *b, bool &update, const std::vector<BatchSim *> &early)
 {
     CUDA_TRY(cudaMemsetAsync(b->status.p, 0, b->status.cap, b->stream));
     for (int k = 0; k < rich::NUM_STAGES; k++) {
@@ -536,7 +553,7 @@ int run_staged(rich_batch *b, bool update, const std::vector<BatchSim *> &early)
         if (k != rich::K_ADVANCE) continue;
         int rc;
         if (!early.empty() && (rc = start_read(b, 1 - b->cur, early))) return rc;
-        if (update && (rc = start_update(b, 1 - b->cur))) return rc;
+        if (update && (rc = start_update(b, 1 - b->cur, update))) return rc;
     }
     CUDA_TRY(cudaGetLastError());
     b->staged_launches++;
@@ -561,8 +578,9 @@ int finish_update(rich_batch *b, int q)
     rich::MeshResult r;
     CUDA_TRY(b->updater.settle(a, to.output(0), r, st));
     if (r.state == rich::MeshResult::kGrow) {
-        CUDA_TRY(to.reserve(a.n, r.sizes));
-        CUDA_TRY(b->updater.again(a, to.output(0), r, st));
+        const cudaError_t e = to.reserve(a.n, r.sizes);
+        CUDA_TRY(rich::unless_no_room(e));
+        if (e == cudaSuccess) CUDA_TRY(b->updater.again(a, to.output(0), r, st));
     }
     const bool done = r.state == rich::MeshResult::kDone;
     for (size_t k = 0; k < b->packed.size(); k++) note(b->packed[k], done && !b->updater.flags()[k]);
@@ -582,7 +600,7 @@ int finish_update(rich_batch *b, int q)
     b->dev_lists = !r.flagged;
     for (size_t k = 0; k < b->packed.size(); k++)
         b->meshes_updated += b->packed[k]->state == RUNNING && !b->mesh_flag[k];
-    CUDA_TRY(b->mesh[1 - b->mcur].reserve(a.n, r.sizes));
+    CUDA_TRY(rich::unless_no_room(b->mesh[1 - b->mcur].reserve(a.n, r.sizes)));
     return reserve_geometry(b, r.sizes);
 }
 
@@ -902,8 +920,11 @@ int pack_step(rich_batch *b, const std::vector<BatchSim *> &list, double &t1, do
     if ((rc = ensure_device(b))) return rc;
     const rich::MeshSizes z{(int32_t)go, (int32_t)to, (int32_t)eo, (int32_t)so};
     b->updater.forget();
-    for (rich::MeshStore &m : b->mesh) CUDA_TRY(m.reserve((int32_t)N, z));
+    CUDA_TRY(b->mesh[b->mcur].reserve((int32_t)N, z));
     if ((rc = reserve_geometry(b, z))) return rc;
+    // (the other store too where an update follows, as far as there is memory)
+    if (fits_update(b) && b->host_sweeps == 0)
+        CUDA_TRY(rich::unless_no_room(b->mesh[1 - b->mcur].reserve((int32_t)N, z)));
     const int nxt = 1 - b->cur;
     if (!same_layout && n_old > 0) {
         // regather the conserved state of continuing simulations into the other
@@ -1008,7 +1029,7 @@ int rich_batch_step(rich_batch *b, rich_step_info *info)
     // (static meshes' points stay where they are, bit for bit: x + dt 0)
     bool still = true;
     for (const BatchSim *s : ok) still = still && s->cfg.motion == RICH_MESH_EULERIAN;
-    const bool fits = (int64_t)N >= rich::kMeshUpdateMin && (int64_t)N <= rich::kMeshUpdateMax;
+    const bool fits = fits_update(b);
     const LaunchShape shape = pick_shape(b);
     // simulations whose meshes the host builds while a staged sweep ends: those
     // that the last two updates could not make (they are tried again with the
@@ -1020,7 +1041,7 @@ int rich_batch_step(rich_batch *b, rich_step_info *info)
         hopeful = hopeful || !wait;
         if (!still && !shape.persistent && (wait || !fits)) early.push_back(s);
     }
-    const bool update = !still && fits && (hopeful || b->host_sweeps == 0);
+    bool update = !still && fits && (hopeful || b->host_sweeps == 0);
     if (!still && fits && !update) b->host_sweeps--;
     if (!early.empty()) CUDA_TRY(b->h_moved.ensure((2 * N + ok.size()) * sizeof(double)));
     CUDA_TRY(cudaEventRecord(b->ev0, b->stream));
@@ -1043,11 +1064,12 @@ int rich_batch_step(rich_batch *b, rich_step_info *info)
             b->barrier_timeouts++;
             b->graph_note = "persistent sweep barrier timed out; staged launches used";
             CUDA_TRY(cudaEventRecord(b->ev0, b->stream));
-            if ((rc = run_staged(b, false, {}))) return rc;
+            bool none = false;
+            if ((rc = run_staged(b, none, {}))) return rc;
             CUDA_TRY(cudaEventRecord(b->ev1, b->stream));
         }
     }
-    if (update && shape.persistent && (rc = start_update(b, 1 - b->cur))) return rc;
+    if (update && shape.persistent && (rc = start_update(b, 1 - b->cur, update))) return rc;
     // (copied while the update still runs)
     CUDA_TRY(cudaMemcpyAsync(b->dt_back(), b->dtout.p, ok.size() * 8, cudaMemcpyDeviceToHost, b->stream));
     CUDA_TRY(cudaMemcpyAsync(b->status_back(), b->status.p, ok.size() * 4, cudaMemcpyDeviceToHost, b->stream));
@@ -1061,9 +1083,10 @@ int rich_batch_step(rich_batch *b, rich_step_info *info)
         // those that go on after this step (the bookkeeping below takes the
         // same decision), unless the step fails
         std::vector<BatchSim *> next;
-        for (size_t k = 0; k < ok.size(); k++) {
+        for (size_t k = 0, e = 0; k < ok.size() && e < early.size(); k++) {
             BatchSim *s = ok[k];
-            if (fits && s->missed < 2) continue;
+            if (s != early[e]) continue;
+            e++;
             const double dt = h[2 * N + k], rem = s->t_end - s->t;
             const double tn = dt >= rem ? s->t_end : s->t + dt;
             if (tn >= s->t_end || s->steps + 1 >= s->max_steps) continue;

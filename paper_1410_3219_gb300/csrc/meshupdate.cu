@@ -1097,7 +1097,15 @@ cudaError_t MeshStore::reserve(int32_t n, const MeshSizes &z)
     for (DBuf *b : {&edge_l, &edge_r, &edge_ta, &edge_tb}) need(*b, E * i4);
     for (DBuf *b : {&gx, &gy}) need(*b, G * sizeof(double));
     for (DBuf *b : {&ghost_src, &ghost_xf, &ghost_shift, &ghost_img}) need(*b, G * i4);
+    if (e != cudaSuccess) release();
     return e;
+}
+
+void MeshStore::release()
+{
+    for (DBuf *b : {&cell_ptr, &slot_nb, &slot_tri, &slot_edge, &tri, &tri_off, &edge_off, &cell_order, &edge_l, &edge_r,
+                    &edge_ta, &edge_tb, &gx, &gy, &ghost_src, &ghost_xf, &ghost_shift, &ghost_img})
+        b->release();
 }
 
 MeshLists MeshStore::lists(int32_t n, int32_t periodic) const
@@ -1205,6 +1213,14 @@ cudaError_t MeshUpdater::reserve(int32_t n, int32_t n_inst, cudaStream_t st)
     return cudaSuccess;
 }
 
+void MeshUpdater::release()
+{
+    for (DBuf *b : {&mark_, &list_[0], &list_[1], &heavy_, &info_, &at_, &ring_deg_, &ring_ref_, &extra_n_, &extra_,
+                    &count_[0], &count_[1], &sizes_, &images_, &ghost_off_, &sums_, &edge_mask_, &tri_mask_})
+        b->release();
+    whole_ = told_ = true;
+}
+
 MeshUpdate MeshUpdater::params(const MeshArrays &a, const MeshOutput &o) const
 {
     MeshUpdate m{};
@@ -1303,7 +1319,11 @@ constexpr int kQuiet = 8;
 
 cudaError_t MeshUpdater::start(const MeshArrays &a, const MeshOutput &o, cudaStream_t st)
 {
-    MU_TRY(reserve(a.n, a.n_inst, st));
+    const cudaError_t room = reserve(a.n, a.n_inst, st);
+    if (room != cudaSuccess) {
+        release();
+        return room;
+    }
     stamp_ += 16;
     static_assert(kMaxRounds + 1 < 16, "one update's stamps");
     // the counters cleared by the last update (or when they were allocated)

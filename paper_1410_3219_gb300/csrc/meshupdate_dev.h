@@ -76,8 +76,10 @@ struct MeshStore {
     DBuf cell_ptr, slot_nb, slot_tri, slot_edge, tri, tri_off, edge_off, cell_order;
     DBuf edge_l, edge_r, edge_ta, edge_tb, gx, gy, ghost_src, ghost_xf, ghost_shift, ghost_img;
     // Room for a mesh of these sizes.  Nothing enqueued may still use the
-    // arrays: those that grow are reallocated.
+    // arrays: those that grow are reallocated.  All are released when one fails
+    // (no array has more room than another then).
     cudaError_t reserve(int32_t n, const MeshSizes &z);
+    void release();
     // where an update writes, with the room there is
     MeshOutput output(int32_t periodic) const;
     // the list builder's arguments for the mesh held (its lists from its rings)
@@ -119,7 +121,8 @@ struct MeshResult {
 
 class MeshUpdater {
 public:
-    // Enqueue the whole update, with the counters' copy to the host.
+    // Enqueue the whole update, with the counters' copy to the host.  Nothing
+    // is enqueued, and nothing held, when its memory cannot be had.
     cudaError_t start(const MeshArrays &a, const MeshOutput &o, cudaStream_t st);
     // After the stream was waited for: what came of it (after more rounds, if
     // the cells did not agree yet).
@@ -131,6 +134,8 @@ public:
     // The next mesh to update is not the last update's (the host built it, or
     // the update's was not kept).
     void forget() { whole_ = true; }
+    // its device memory given back (nothing enqueued may use it)
+    void release();
 
 private:
     cudaError_t reserve(int32_t n, int32_t n_inst, cudaStream_t st);

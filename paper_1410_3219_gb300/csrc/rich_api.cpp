@@ -295,6 +295,9 @@ void report_sizes(const rich_sim *s, rich_step_info *info)
     info->n_slots = s->msz.slots;
 }
 
+// Sizes that the device's update takes.
+bool updatable(const rich_sim *s) { return s->n >= rich::kMeshUpdateMin && s->n <= rich::kMeshUpdateMax; }
+
 // upload of the host mesh; the triangle and edge lists are built on the
 // device from the rings (the host sends each cell's first owned triangle
 // and edge, and the ghosts' images)
@@ -305,11 +308,14 @@ int upload_mesh(rich_sim *s, rich_step_info *info)
     s->mesh_on_device = false;
     s->updater.forget();
     s->msz = rich::MeshSizes{m.g, m.n_tris, m.n_edges, (int32_t)m.slot_nb.size()};
-    // (the other buffers too: the first update then has room)
-    for (rich::MeshStore &k : s->mesh) CUDA_TRY(k.reserve(s->n, s->msz));
+    rich::MeshStore &d = s->mesh[s->mcur];
+    CUDA_TRY(d.reserve(s->n, s->msz));
     int rc = reserve_geometry(s, s->msz);
     if (rc != RICH_OK) return rc;
-    rich::MeshStore &d = s->mesh[s->mcur];
+    // (the other store too where updates follow, as far as there is memory: the
+    // first one then has room)
+    if (updatable(s) && s->cfg.motion != RICH_MESH_EULERIAN && s->host_sweeps == 0)
+        CUDA_TRY(rich::unless_no_room(s->mesh[1 - s->mcur].reserve(s->n, s->msz)));
     CUDA_TRY(upload(d.gx, m.gx, s->stream));
     CUDA_TRY(upload(d.gy, m.gy, s->stream));
     CUDA_TRY(upload(d.ghost_src, m.ghost_src, s->stream));
@@ -337,18 +343,38 @@ int upload_mesh(rich_sim *s, rich_step_info *info)
 // Whether the mesh of new points can be an update of the one on the device.
 bool can_update(const rich_sim *s)
 {
-    return s->mesh_on_device && s->n >= rich::kMeshUpdateMin && s->n <= rich::kMeshUpdateMax;
+    return s->mesh_on_device && updatable(s);
+}
+
+// An update left the mesh to the host.
+void missed_update(rich_sim *s)
+{
+    s->updater.forget();
+    // (the same points would fail again)
+    s->mesh_on_device = false;
+    s->missed++;
+    s->host_sweeps = rich::host_sweeps_after(s->missed);
 }
 
 // Enqueue the update of the mesh for the points in buffers q, on the mesh
 // stream after what the handle's stream holds by now; join_update makes the
-// handle's stream continue after it.
-int start_update(rich_sim *s, int q)
+// handle's stream continue after it.  Without memory for it nothing is
+// enqueued, and `started` is false: the mesh is the host's, and the room that
+// updates hold is given back.
+int start_update(rich_sim *s, int q, bool &started)
 {
     rich::MeshStream &u = s->mesh_stream;
     CUDA_TRY(cudaEventRecord(u.moved, s->stream));
     CUDA_TRY(cudaStreamWaitEvent(u.stream, u.moved, 0));
-    CUDA_TRY(s->updater.start(s->mesh_arrays(q), s->mesh[1 - s->mcur].output(s->periodic()), u.stream));
+    const cudaError_t e = s->updater.start(s->mesh_arrays(q), s->mesh[1 - s->mcur].output(s->periodic()), u.stream);
+    started = e == cudaSuccess;
+    CUDA_TRY(rich::unless_no_room(e));
+    if (!started) {
+        s->mesh[1 - s->mcur].release();
+        s->missed = std::max(s->missed, 1);
+        missed_update(s);
+        return RICH_OK;
+    }
     CUDA_TRY(cudaEventRecord(u.done, u.stream));
     return RICH_OK;
 }
@@ -374,15 +400,12 @@ int finish_update(rich_sim *s, int q, bool keep, rich_step_info *info)
     rich::MeshResult r;
     CUDA_TRY(s->updater.settle(a, to.output(s->periodic()), r, st));
     if (r.state == rich::MeshResult::kGrow) {
-        CUDA_TRY(to.reserve(s->n, r.sizes));
-        CUDA_TRY(s->updater.again(a, to.output(s->periodic()), r, st));
+        const cudaError_t e = to.reserve(s->n, r.sizes);
+        CUDA_TRY(rich::unless_no_room(e));
+        if (e == cudaSuccess) CUDA_TRY(s->updater.again(a, to.output(s->periodic()), r, st));
     }
     if (r.state != rich::MeshResult::kDone || r.flagged) {
-        s->updater.forget();
-        // (the same points would fail again)
-        s->mesh_on_device = false;
-        s->missed++;
-        s->host_sweeps = rich::host_sweeps_after(s->missed);
+        missed_update(s);
         return RICH_OK;
     }
     s->missed = 0;
@@ -392,7 +415,7 @@ int finish_update(rich_sim *s, int q, bool keep, rich_step_info *info)
     s->tess_current = true;
     report_sizes(s, info);
     // (the next update's buffers have as much room as these)
-    CUDA_TRY(s->mesh[1 - s->mcur].reserve(s->n, r.sizes));
+    CUDA_TRY(rich::unless_no_room(s->mesh[1 - s->mcur].reserve(s->n, r.sizes)));
     return reserve_geometry(s, r.sizes);
 }
 
@@ -404,11 +427,13 @@ int tessellate(rich_sim *s, rich_step_info *info, bool fetch_points)
     if (fetch_points && can_update(s)) {
         const double t0 = now_ms();
         const int q = s->pts();
-        int rc;
-        if ((rc = start_update(s, q)) != RICH_OK || (rc = join_update(s)) != RICH_OK) return rc;
+        bool started = false;
+        int rc = start_update(s, q, started);
+        if (rc == RICH_OK && started) rc = join_update(s);
+        if (rc != RICH_OK) return rc;
         s->tess_current = false;
         CUDA_TRY(cudaStreamSynchronize(s->stream));
-        if ((rc = finish_update(s, q, true, info)) != RICH_OK) return rc;
+        if (started && (rc = finish_update(s, q, true, info)) != RICH_OK) return rc;
         if (info) info->tess_ms += now_ms() - t0;
         if (s->tess_current) return RICH_OK;
     }
@@ -654,7 +679,8 @@ static int start_read(rich_sim *s, int q)
     return RICH_OK;
 }
 
-static int launch_sweep(rich_sim *s, double t_end, NextMesh next)
+// (next: what was started)
+static int launch_sweep(rich_sim *s, double t_end, NextMesh &next)
 {
     rich::Range range("rich sweep launch (a1-a9)");
     if (!s) return fail(RICH_EINVAL, "NULL handle");
@@ -667,10 +693,15 @@ static int launch_sweep(rich_sim *s, double t_end, NextMesh next)
     for (int k = 0; k < rich::NUM_STAGES; k++) {
         if (s->profiling) CUDA_TRY(cudaEventRecord(s->kev[k], s->stream));
         s->launch(k, nullptr);
-        if (next != NextMesh::none && k == rich::K_ADVANCE) {
-            const int q = s->next_pts(), rc = next == NextMesh::update ? start_update(s, q) : start_read(s, q);
-            if (rc != RICH_OK) return rc;
+        if (k != rich::K_ADVANCE) continue;
+        int rc = RICH_OK;
+        if (next == NextMesh::update) {
+            bool started = false;
+            rc = start_update(s, s->next_pts(), started);
+            if (!started) next = NextMesh::host;
         }
+        if (rc == RICH_OK && next == NextMesh::host) rc = start_read(s, s->next_pts());
+        if (rc != RICH_OK) return rc;
     }
     if (s->profiling) CUDA_TRY(cudaEventRecord(s->kev[rich::NUM_STAGES], s->stream));
     CUDA_TRY(cudaGetLastError());
@@ -679,7 +710,11 @@ static int launch_sweep(rich_sim *s, double t_end, NextMesh next)
     return RICH_OK;
 }
 
-int rich_sweep(rich_sim *s, double t_end) { return launch_sweep(s, t_end, NextMesh::none); }
+int rich_sweep(rich_sim *s, double t_end)
+{
+    NextMesh next = NextMesh::none;
+    return launch_sweep(s, t_end, next);
+}
 
 // The sweep's dt and status, into page-locked memory (dt, then the status)
 static int fetch_result(rich_sim *s)
@@ -765,9 +800,9 @@ static int step_sweep(rich_sim *s, double t_end, rich_step_info *info)
     const int q = s->next_pts();
     // (a static mesh's points stay where they are, bit for bit: x + dt 0)
     const bool still = s->cfg.motion == RICH_MESH_EULERIAN;
-    const NextMesh next = still                                   ? NextMesh::none
-                          : can_update(s) && s->host_sweeps == 0 ? NextMesh::update
-                                                                  : NextMesh::host;
+    NextMesh next = still                                  ? NextMesh::none
+                    : can_update(s) && s->host_sweeps == 0 ? NextMesh::update
+                                                            : NextMesh::host;
     if (next == NextMesh::host && s->host_sweeps > 0) s->host_sweeps--;
     int rc = launch_sweep(s, t_end, next);
     if (rc != RICH_OK) return rc;
