@@ -426,12 +426,13 @@ void rich_server_destroy(rich_server *s);
    FP32).  Cells whose time step is +inf are skipped, as the sweep skips
    them; a cell whose time step is NaN, negative or -0.0 (a negative or NaN
    pressure or density) makes *dt_out a NaN instead of being skipped.
-   It allocates nothing: its scratch (one partial minimum per block and a
-   completion counter, 10 KB) is a fixed array in the library's device image,
-   which every GPU that loads the library holds until the process exits.  The first call on each device looks up that array's
-   address (cudaGetSymbolAddress), so make it before any stream capture.
-   Every call shares the array: calls that overlap on
-   the GPU (other streams, other host threads) race and must not be issued.
+   It allocates nothing: its scratch (one partial minimum per block and 64
+   completion counters, 8 KB) is a fixed array in the library's device image,
+   which every GPU that loads the library holds until the process exits.  The
+   first call on each device looks up that array's address
+   (cudaGetSymbolAddress), so make it before any stream capture.
+   Every call shares the array: calls that overlap on the GPU (other streams,
+   other host threads) race and must not be issued.
    Returns RICH_EINVAL for a configuration that rich_init_mesh rejects, a
    NULL array, or n outside [1, RICH_NOALLOC_MAX_CELLS], RICH_ECUDA if the
    set-up or launch fails (rich_last_error gives the reason). */

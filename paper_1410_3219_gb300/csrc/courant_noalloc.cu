@@ -4,8 +4,8 @@
 // time step: code running inside a memory pool or arena that owns the whole
 // device, and code that must not synchronise the device (cudaMalloc/cudaFree
 // can).  This entry point gives them the time step of the sweep without any
-// allocation: its scratch (one partial minimum per thread block and a
-// completion counter) lives in a file-scope __device__ array that every
+// allocation: its scratch (one partial minimum per thread block and completion
+// counters) lives in a file-scope __device__ array that every
 // process loading the library holds on every GPU it uses, until exit.
 //
 // Set-up: the first call on each device looks up the array's device address
@@ -14,6 +14,7 @@
 // Calls share the array: calls that overlap on the GPU (different streams,
 // or different host threads) race and must not be issued.
 #include <algorithm>
+#include <atomic>
 #include <cfloat>
 #include <cmath>
 #include <mutex>
@@ -34,9 +35,14 @@ constexpr int kMaxBlocks = 6 * 152;
 // scratch: per-block minima of the cell time step as bit patterns (the
 // integer order of non-negative doubles is their numeric order; kBad marks
 // a block that met a cell whose time step is not a finite non-negative
-// number), then the number of blocks that have finished, which wraps back to
-// zero with the last one
-static __device__ __align__(256) unsigned long long g_courant_scratch[kMaxBlocks + 1];
+// number), then counters of the blocks that have finished.  Calls take the
+// counters in turn; a call leaves its own at zero, and clears the one that comes
+// kCounters / 2 calls later, so that calls that overlapped against the rule, or
+// a kernel that did not finish, spoil no later one.  (One counter that a memset
+// cleared before each call: 1 us more of a small call's 8.  A captured call
+// keeps its counter in every replay.)
+constexpr int kCounters = 64;
+static __device__ __align__(256) unsigned long long g_courant_scratch[kMaxBlocks + kCounters];
 
 constexpr unsigned long long kBad = ~0ull;
 
@@ -100,8 +106,9 @@ __global__ void __launch_bounds__(kBlock, 6) k_courant_noalloc(
     int32_t n, double gamma, float gamma_f, double cfl, int32_t motion_static, const double *__restrict__ area,
     const double *__restrict__ rho, const double *__restrict__ vx, const double *__restrict__ vy,
     const double *__restrict__ p, const double *__restrict__ wx, const double *__restrict__ wy,
-    unsigned long long *scratch, double *dt_out)
+    unsigned long long *scratch, int32_t counter, double *dt_out)
 {
+    if (blockIdx.x == 0 && threadIdx.x == 0) scratch[kMaxBlocks + (counter + kCounters / 2) % kCounters] = 0;
     // kMax: the bits of +inf, above every finite non-negative time step
     const unsigned long long kMax = 0x7ff0000000000000ull;
     constexpr unsigned kNone = 0x7f800000u;  // estimate of no cell
@@ -194,12 +201,13 @@ __global__ void __launch_bounds__(kBlock, 6) k_courant_noalloc(
         for (int q = 1; q < kBlock / 32; q++) m = key_min(m, red[q]);
         scratch[blockIdx.x] = bad_block ? kBad : m;
         __threadfence();
-        last = atomicInc(reinterpret_cast<unsigned *>(&scratch[kMaxBlocks]), gridDim.x - 1) == gridDim.x - 1;
+        last = atomicAdd(&scratch[kMaxBlocks + counter], 1ull) == gridDim.x - 1;
     }
     __syncthreads();
     if (!last) return;
     // the last block to finish reduces the per-block minima
     __threadfence();
+    if (threadIdx.x == 0) scratch[kMaxBlocks + counter] = 0;
     unsigned long long m = kMax;
     bool any_bad = false;
     for (int32_t b = threadIdx.x; b < (int32_t)gridDim.x; b += blockDim.x) {
@@ -224,6 +232,7 @@ __global__ void __launch_bounds__(kBlock, 6) k_courant_noalloc(
     }
 }
 
+std::atomic<uint32_t> g_calls{0};
 std::mutex g_setup_mutex;
 unsigned long long *g_scratch_addr[64] = {};
 
@@ -238,8 +247,7 @@ extern "C" int rich_courant_dt_noalloc(const rich_config *cfg, int64_t n, const 
     if (cfg->motion != RICH_MESH_EULERIAN && (!wx || !wy))
         return rich::set_error(RICH_EINVAL, "wx, wy are needed with a moving mesh");
     if (n < 1 || n > RICH_NOALLOC_MAX_CELLS)
-        return rich::set_error(RICH_EINVAL, "n must be in [1, RICH_NOALLOC_MAX_CELLS]: the fixed scratch holds one "
-                                            "partial minimum per 256 cells");
+        return rich::set_error(RICH_EINVAL, "n must be in [1, RICH_NOALLOC_MAX_CELLS]");
     int dev = -1;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return rich::set_error(RICH_ECUDA, "no device");
     unsigned long long *scratch;
@@ -254,10 +262,11 @@ extern "C" int rich_courant_dt_noalloc(const rich_config *cfg, int64_t n, const 
         scratch = g_scratch_addr[dev];
     }
     cudaStream_t st = static_cast<cudaStream_t>(stream);
+    const int32_t counter = (int32_t)(g_calls.fetch_add(1, std::memory_order_relaxed) % kCounters);
     const int64_t tile = (int64_t)kBlock * kCells;
     const int blocks = (int)std::min<int64_t>((n + tile - 1) / tile, kMaxBlocks);
     k_courant_noalloc<<<blocks, kBlock, 0, st>>>((int32_t)n, cfg->gamma, (float)cfg->gamma, cfg->cfl,
                                                  cfg->motion == RICH_MESH_EULERIAN ? 1 : 0, area, rho, vx, vy, p,
-                                                 wx, wy, scratch, dt_out);
+                                                 wx, wy, scratch, counter, dt_out);
     return cudaGetLastError() == cudaSuccess ? RICH_OK : rich::set_error(RICH_ECUDA, "launch failed");
 }

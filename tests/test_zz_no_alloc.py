@@ -144,3 +144,52 @@ def test_noalloc_minimum_over_all_cells(n, case):
     dt = dt[torch.isfinite(dt)]
     want = cfg["cfl"] * float(dt.min())
     assert abs(float(out.item()) - want) <= 4 * 2.0 ** -52 * want
+
+
+def test_noalloc_calls_after_overlapping_ones():
+    """Calls that overlap on the GPU race for the shared scratch (their own
+    results are not looked at), but must not spoil the calls after them; and
+    captured calls of different sizes, replayed, count their own blocks."""
+    import torch
+    rich = _lib()
+    g = torch.Generator(device="cuda").manual_seed(3)
+    n_max = 2000001
+    a = {k: torch.empty(n_max, dtype=torch.float64, device="cuda").uniform_(0.5, 2.0, generator=g) for k in FIELDS}
+    cfg = W.default_cfg()
+
+    def call(n, out, stream):
+        rich.rich_courant_dt_noalloc(cfg, n, *[a[k].data_ptr() for k in FIELDS], out.data_ptr(), stream.cuda_stream)
+
+    def want(n):
+        q = {k: a[k][:n] for k in FIELDS}
+        ux, uy = q["vx"] - q["wx"], q["vy"] - q["wy"]
+        dt = torch.sqrt(q["area"] * (1.0 / math.pi)) / (torch.sqrt(cfg["gamma"] * q["p"] / q["rho"]) +
+                                                        torch.sqrt(ux * ux + uy * uy))
+        return cfg["cfl"] * float(dt.min())
+
+    sizes = [1, 700, 4097, 60001, 467000, n_max]
+    wants = [want(n) for n in sizes]
+    s1, s2 = torch.cuda.Stream(), torch.cuda.Stream()
+    o1, o2 = (torch.zeros(1, dtype=torch.float64, device="cuda") for _ in range(2))
+    call(1, o1, s1)
+    torch.cuda.synchronize()
+    graphs, outs = [], []
+    for n in sizes:
+        outs.append(torch.zeros(1, dtype=torch.float64, device="cuda"))
+        graphs.append(torch.cuda.CUDAGraph())
+        with torch.cuda.graph(graphs[-1]):
+            call(n, outs[-1], torch.cuda.current_stream())
+    for rep in range(3):
+        for k in range(40):
+            call(sizes[(k + rep) % 6], o1, s1)
+            call(sizes[(3 * k + 1) % 6], o2, s2)
+        torch.cuda.synchronize()
+        for n, w in zip(sizes, wants):
+            call(n, o1, s1)
+            s1.synchronize()
+            assert abs(float(o1.item()) - w) <= 4 * 2.0 ** -52 * w, n
+        for graph, out, w in zip(graphs, outs, wants):
+            out.zero_()
+            graph.replay()
+            torch.cuda.synchronize()
+            assert abs(float(out.item()) - w) <= 4 * 2.0 ** -52 * w
