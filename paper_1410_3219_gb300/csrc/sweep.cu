@@ -242,10 +242,11 @@ template <class R> __device__ __forceinline__ void stage_edge_geometry(const Swe
 // a1 + a2: area and centre of mass (shoelace about the generator, FP64),
 // then the primitive variables; in a sweep also a5 (mesh velocity) and a6:
 // returns the cell's Courant time step R_i / (c_s + |v - w|) (DBL_MAX
-// outside a sweep).  With init_W the conserved variables are set.
+// outside a sweep).  With init_W the conserved variables are set.  lanes: those
+// of the warp that call it.
 template <class R>
 __device__ __forceinline__ double stage_cell_geometry(const SweepParams<R> &p, const double *__restrict__ init_W,
-                                                      int32_t i, int32_t &my_inst)
+                                                      int32_t i, unsigned lanes, int32_t &my_inst)
 {
     const int32_t lo = p.cell_ptr[i], hi = p.cell_ptr[i + 1];
     const double xi = p.x[i], yi = p.y[i];
@@ -366,12 +367,11 @@ __device__ __forceinline__ double stage_cell_geometry(const SweepParams<R> &p, c
         // (beyond 2^60 a square would overflow, and chi is the caller's)
         known = known && speed < 1.15e18f;
         const float est = sqrtf(magnitude(A) * 0.318309886f) / (magnitude((double)cs) + speed);
-        const unsigned act = __activemask();
         unsigned least = known ? __float_as_uint(est) : 0x7f800000u;
         // (lanes of one simulation share the warp's smallest; in a mixed warp
         // each lane stands alone)
-        const int32_t lead = __shfl_sync(act, my_inst, __ffs(act) - 1);
-        if (__all_sync(act, my_inst == lead)) least = __reduce_min_sync(act, least);
+        const int32_t lead = __shfl_sync(lanes, my_inst, __ffs(lanes) - 1);
+        if (__all_sync(lanes, my_inst == lead)) least = __reduce_min_sync(lanes, least);
         const float far = estimate(__longlong_as_double((long long)__ldcg(p.dtmin_bits + my_inst)));
         const float limit = fminf(__uint_as_float(least), far) * 1.000004f;
         if (known && est > limit) return DBL_MAX;
@@ -400,7 +400,8 @@ __global__ void k_geometry(SweepParams<R> p, const double *__restrict__ init_W, 
         int32_t k = (blockIdx.x - edge_blocks) * blockDim.x + threadIdx.x;
         double dt_cell = DBL_MAX;
         int32_t my_inst = 0;
-        if (k < p.n) dt_cell = stage_cell_geometry(p, init_W, cell_at(p, k), my_inst);
+        const unsigned lanes = __ballot_sync(0xffffffffu, k < p.n);
+        if (k < p.n) dt_cell = stage_cell_geometry(p, init_W, cell_at(p, k), lanes, my_inst);
         // (init_W and motion are the same for the whole grid)
         if (!init_W && p.motion) warp_min_to(dt_cell, my_inst, p.dtmin_bits);
     }
@@ -1287,7 +1288,8 @@ __global__ void __launch_bounds__(512) k_sweep_persistent(SweepParams<R> p, cons
         const int32_t k = base + threadIdx.x;
         double v = DBL_MAX;
         int32_t inst = 0;
-        if (k < p.n) v = stage_cell_geometry(p, (const double *)nullptr, cell_at(p, k), inst);
+        const unsigned lanes = __ballot_sync(0xffffffffu, k < p.n);
+        if (k < p.n) v = stage_cell_geometry(p, (const double *)nullptr, cell_at(p, k), lanes, inst);
         warp_min_to(v, inst, p.dtmin_bits);
     }
     if (!grid_sync(gs, nb, lim)) return;
