@@ -179,3 +179,23 @@ def test_mass_fluxes_do_not_depend_on_the_frame(R, bulk):
     assert out[0][0] == out[1][0]
     assert np.array_equal(out[0][1], out[1][1])
     assert np.abs(out[0][1] / 2.0 ** -10 - wl["rho"]).max() > 1e-3
+
+
+@pytest.mark.parametrize("n_side", [127, 128, 129, 138, 139])
+def test_reads_on_both_sides_of_the_page_locked_size(R, n_side):
+    """Reads through page-locked memory (up to 7/8 MB: 19,114 cells of six
+    fields, 16,384 of seven) and through the device's memory give the caller's
+    cells in the caller's order, null outputs left out."""
+    wl = W.kelvin_helmholtz(n_side=n_side, seed=n_side)
+    sim = R.Sim(wl)
+    c, s = sim.conserved(), sim.state()
+    for k in ("x", "y"):
+        assert np.array_equal(c[k], wl[k]) and np.array_equal(s[k], wl[k])
+    assert np.array_equal(np.rint(s["rho"]), np.rint(wl["rho"]))
+    assert np.allclose(c["m"], s["rho"] * s["area"], rtol=1e-12)
+    import ctypes as C
+    m = np.zeros(sim.n)
+    assert R.lib().rich_get_conserved(sim.h, sim.n, None, None, m.ctypes.data_as(C.POINTER(C.c_double)), None, None,
+                                      None) == 0
+    assert np.array_equal(m, c["m"])
+    sim.close()
