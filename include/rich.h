@@ -130,9 +130,12 @@ int rich_init_mesh(const rich_config *cfg, int64_t n, const double *x, const dou
    device for the current points and mesh, and a0 for the moved points beside
    the stages after the point motion (twice, the first time for the half-step
    points, in the time-centred scheme).  A step thus leaves the mesh of its
-   points updated, and the next step or call starts with the sweep.  A mesh left to the host (see rich_tessellate) is built by the next
-   step or call.  Results equal those of rich_tessellate / rich_sweep / rich_sync in
-   turn, bit for bit.  info may be NULL.
+   points updated, and the next step or call starts with the sweep.  A mesh
+   left to the host (see rich_tessellate) is built by the next step or call;
+   where that happens again and again, and for sizes that are not updated, the
+   host builds it beside the stages after the point motion, and the update is
+   tried again every 2 to 33 sweeps.  Results equal those of rich_tessellate /
+   rich_sweep / rich_sync in turn, bit for bit.  info may be NULL.
    Errors: RICH_ENEGATIVE / RICH_ENAN (state left at the last good step),
    RICH_ETESS, RICH_EDUPLICATE, RICH_ECUDA. */
 int rich_step(rich_sim *s, int32_t max_steps, double t_end, rich_step_info *info);
@@ -182,11 +185,17 @@ int rich_set_stream(rich_sim *s, void *cuda_stream);
 /* a0 for the current points: the mesh on the device, of whichever points it
    is, updated for them, with its triangle and edge lists.  The update leaves
    a mesh to the host (the points are copied there, tessellated, and the rings
-   uploaded) for fewer than 64 cells, when a Voronoi circumdisk of a real cell
-   reaches 0.98 of the ghost band or, in a periodic box, a quarter of it, when
-   a cell has more than 32 neighbours, when points coincide, and when
+   uploaded) for fewer than 64 cells (in a batch: of all its simulations) and
+   for more than 2^26; when a Voronoi circumdisk of a real cell reaches 0.98 of
+   the ghost band or, in a periodic box, a quarter of it; when a cell of more
+   than 32 neighbours has one of up to eight; when a cell whose neighbours
+   change has more than 32 (or 96 candidates for them, or 256 cells in its
+   neighbours' rings); when the neighbours of more than half the cells change;
+   when the cells do not agree in twelve rounds; when points coincide; when
    coordinates that decide an exact predicate spread over more than 72 binary
-   orders of magnitude.  Synchronous.  RICH_ETESS if the lists do not close. */
+   orders of magnitude (68 where periodic images are among them); and when the
+   device has no memory for it.  Synchronous.  RICH_ETESS if the lists do not
+   close. */
 int rich_tessellate(rich_sim *s, rich_step_info *info);
 
 /* Enqueue a1-a9 for one step on the current connectivity (asynchronous; no
@@ -270,7 +279,9 @@ int rich_batch_add(rich_batch *b, const rich_config *cfg, int64_t n, const doubl
    points are updated on the device beside the sweep; a step with the same
    simulations as the last then starts with the sweep, and one with others
    reads those meshes back and packs them with the host-built ones of the
-   newly admitted simulations.
+   newly admitted simulations and of those that the update cannot make (see
+   rich_tessellate; beside a staged sweep once that has happened twice in a
+   row).
    info (nullable): steps_done = simulations stepped, sweep_ms = device time
    of the sweep (with what the mesh update beside it slows it down), tess_ms =
    time of the host tessellations and of the mesh update beyond the sweep's
@@ -501,8 +512,9 @@ int rich_mesh_update_check(const rich_config *cfg, int64_t n, int32_t steps, con
 /* The device's mesh update against the host builder (host only; no GPU
    needed): from the mesh of each of `steps` successive point sets (xs, ys:
    steps x n, row-major, the same cells in each) the next set's mesh is made
-   by the update's per-cell code, run serially, and compared with a fresh
-   host build.  *mismatched counts entries that differ (rings, offsets,
+   by the update's steps in serial form (with the predicates of the kernels,
+   which take a cell with several lanes), and compared with a fresh host
+   build.  *mismatched counts entries that differ (rings, offsets,
    processing order, ghosts), *updated the meshes made by the update (the
    others it leaves to the host builder), *recomputed the stars built again.
    Errors: RICH_EINVAL, tessellation errors. */

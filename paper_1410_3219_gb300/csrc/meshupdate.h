@@ -1,6 +1,10 @@
-// Update of a tessellation for moved points (a0), per-cell bodies shared by
-// the device kernels (meshupdate.cu) and a serial host run that checks them
-// (meshupdate_host.cpp).
+// Update of a tessellation for moved points (a0): the predicates, frames,
+// checks, sizes and ghosts of a cell, which the device kernels (meshupdate.cu)
+// call, and the serial forms of verify, recompute_light, recompute and
+// place_ring, which meshupdate_host.cpp runs.  Of those four the kernels are
+// versions of their own, with lanes per ring slot or candidate; both are
+// compared with the host builder (rich_device_update_check on the CPU,
+// rich_mesh_check on the device).
 //
 // The mesh is the set of stars: every real cell's ring of Delaunay
 // neighbours in counter-clockwise order.  Between steps the points move a
@@ -21,10 +25,13 @@
 // repairing Delaunay triangulations and convex hulls", 2005): stars that
 // are all locally Delaunay and agree with each other form the Delaunay
 // triangulation, which the symbolic tie-break makes unique, so the result is
-// the host builder's mesh, ring for ring.  What the bodies do not handle (a
-// circumdisk beyond the ghost band, more than kMaxDeg neighbours, rounds that
-// do not converge, coordinates the exact predicates cannot hold) sets a flag,
-// and the caller builds that mesh on the host.
+// the host builder's mesh, ring for ring.  What the update does not handle (a
+// circumdisk beyond the ghost band or a quarter of a periodic box; a listed cell
+// of more than kMaxDeg neighbours, told vertices included, kMaxCand candidates
+// or kMaxSources two-ring members; a cell of more than 32 neighbours beside one
+// of up to eight; more than half the cells recomputed; rounds that do not
+// converge; coordinates the exact predicates cannot hold) sets a flag of its
+// simulation, and the caller builds that mesh on the host.
 //
 // Neighbours are references src * 16 + img: the image img = (a + 1) +
 // 3 (b + 1), a, b in {-1, 0, 1}, of real cell src (4: the cell itself).  In a
@@ -35,8 +42,8 @@
 // Predicates: the sign of a determinant is taken from FP32 when it exceeds
 // its error bound (FP64 runs at 1/64 of the FP32 rate on GB300; fewer than
 // one edge in 10^4 goes on), else from FP64 with the host's bounds, else from
-// exact integers.  This file must be compiled without floating-point
-// contraction.
+// exact integers (at once where periodic images are among the points).  This
+// file must be compiled without floating-point contraction.
 #pragma once
 
 #include <cmath>
@@ -1100,7 +1107,7 @@ RICH_HD inline void place_ring(const MeshUpdate &m, int32_t i)
 void mesh_params(const BoxConfig &box, int32_t n, InstParams &ip);
 
 // The update of `mesh` (a build_host_mesh result, or this function's) for
-// new points by the device bodies, run serially on the host.  Returns 1, or
+// new points by the serial forms above, on the host.  Returns 1, or
 // 0 with `flags` set when the host builder has to take the mesh.
 int mesh_update_serial(const BoxConfig &box, int32_t n, const double *x, const double *y, HostMesh &mesh,
                        int32_t &flags, int32_t &rounds, int32_t &recomputed);

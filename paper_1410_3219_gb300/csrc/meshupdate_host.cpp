@@ -1,5 +1,5 @@
-// Host side of the mesh update of meshupdate.h: its constants, and a serial
-// run of the device bodies that the tests compare with the host builder.
+// Host side of the mesh update of meshupdate.h: its constants, and a run of its
+// serial forms that the tests compare with the host builder.
 #include "meshupdate.h"
 
 #include <algorithm>

@@ -356,8 +356,8 @@ def rich_mesh_update_check(cfg, xs, ys, threads=4):
 
 
 def rich_device_update_check(cfg, xs, ys):
-    """Meshes of successive point sets made by the device update's per-cell
-    code (run on the host) against fresh host builds: (entries that differ,
+    """Meshes of successive point sets made by the device update's steps in
+    serial form (on the host) against fresh host builds: (entries that differ,
     meshes updated, stars built again)."""
     c = cfg if isinstance(cfg, rich_config) else rich_config.from_dict(cfg)
     xs, ys = np.atleast_2d(xs), np.atleast_2d(ys)
