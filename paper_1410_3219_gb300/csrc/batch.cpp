@@ -1199,14 +1199,25 @@ int rich_batch_get_conserved(rich_batch *b, int32_t id, int64_t n, double *x, do
         // memory (24 us for 4,096 cells, 28 by one copy; 111 and 118 for 32,761)
         // or, where a gather at the link's pace would hold the SMs that other
         // batches' sweeps use for long, by one copy (65,536 cells: 242 us, 215
-        // straight; 160,000: 570 and 530)
+        // straight; 160,000: 570 and 530).  Without memory for that the host
+        // reorders.
         const size_t nn = (size_t)s->n, N = (size_t)b->n_packed, co = (size_t)s->cell_off;
         const double *U = b->U[b->cur].as<double>() + co;
         const double *src[6] = {b->x[b->cur].as<double>() + co, b->y[b->cur].as<double>() + co, U, U + N, U + 2 * N,
                                 U + 3 * N};
         const bool direct = 6 * nn * 8 <= ((size_t)2 << 20);
-        CUDA_TRY(b->read_host.ensure(6 * nn * 8));
-        if (!direct) CUDA_TRY(b->read_dev.ensure(6 * nn * 8));
+        CUDA_TRY(rich::unless_no_room(b->read_host.ensure(6 * nn * 8)));
+        if (!direct) CUDA_TRY(rich::unless_no_room(b->read_dev.ensure(6 * nn * 8)));
+        if (!b->read_host.p || (!direct && !b->read_dev.p)) {
+            std::vector<double> h(nn);
+            for (int f = 0; f < 6; f++) {
+                if (!outs[f]) continue;
+                CUDA_TRY(cudaMemcpyAsync(h.data(), src[f], nn * 8, cudaMemcpyDeviceToHost, b->stream));
+                CUDA_TRY(cudaStreamSynchronize(b->stream));
+                for (size_t k = 0; k < nn; k++) outs[f][s->perm[k]] = h[k];
+            }
+            return RICH_OK;
+        }
         double *to = direct ? b->read_host.as<double>() : b->read_dev.as<double>();
         CUDA_TRY(rich::launch_unpermute(s->n, b->cell_of.as<int32_t>() + co, src, to, b->stream));
         if (!direct) CUDA_TRY(cudaMemcpyAsync(b->read_host.p, to, 6 * nn * 8, cudaMemcpyDeviceToHost, b->stream));

@@ -916,14 +916,27 @@ static int fetch_r(rich_sim *s, const void *dev, std::vector<double> &h, size_t 
 // the device (the host then copies nothing itself).  Reads of the conserved state
 // take 24 and 63 us for 4,096 cells, 60 and 68 for 16,384, 69 and 68 for 19,600
 // (0.90 MB), 110 and 72 for 32,761; of the state (seven fields) 83 and 88 us for
-// 16,384, 96 and 92 for 19,600 (1.05 MB).
+// 16,384, 96 and 92 for 19,600 (1.05 MB).  (Null without memory for it: the host
+// reorders then.)
 static int read_buffer(rich_sim *s, int fields, double **buf, bool *host)
 {
     const size_t bytes = (size_t)s->n * fields * 8;
     *host = bytes <= ((size_t)7 << 17);
-    if (*host) CUDA_TRY(s->read_host.ensure(bytes));
-    else CUDA_TRY(s->unperm.ensure(bytes));
+    CUDA_TRY(rich::unless_no_room(*host ? s->read_host.ensure(bytes) : s->unperm.ensure(bytes)));
     *buf = *host ? s->read_host.as<double>() : s->unperm.as<double>();
+    return RICH_OK;
+}
+
+// Fields (null ones skipped) through host memory, field by field.
+static int read_fields(rich_sim *s, const double *const *src, double *const *outs, int fields)
+{
+    std::vector<double> h;
+    for (int f = 0; f < fields; f++) {
+        if (!outs[f]) continue;
+        const int rc = fetch(s, src[f], h, (size_t)s->n);
+        if (rc) return rc;
+        unpermute(s, h.data(), outs[f]);
+    }
     return RICH_OK;
 }
 
@@ -953,6 +966,20 @@ int rich_get_state(rich_sim *s, int64_t n, double *x, double *y, double *rho, do
     double *st;
     bool host;
     if ((rc = read_buffer(s, 7, &st, &host))) return rc;
+    if (!st) {
+        const double *src[3] = {s->x[q].as<double>(), s->y[q].as<double>(), s->A.as<double>()};
+        double *const to[3] = {x, y, area};
+        if ((rc = read_fields(s, src, to, 3))) return rc;
+        std::vector<double> h, W;
+        if ((rc = fetch_r(s, s->W.p, W, 4 * (size_t)n))) return rc;
+        h.resize((size_t)n);
+        for (int c = 0; c < 4; c++) {
+            if (!outs[2 + c]) continue;
+            for (size_t k = 0; k < (size_t)n; k++) h[k] = W[4 * k + c];
+            unpermute(s, h.data(), outs[2 + c]);
+        }
+        return RICH_OK;
+    }
     CUDA_TRY(rich::launch_unpermute_state(s->n, s->cell_of.as<int32_t>(), s->x[q].as<double>(), s->y[q].as<double>(),
                                           s->W.p, s->rsize() == sizeof(float), s->A.as<double>(), st, s->stream));
     return copy_out(s, st, host, outs, 7);
@@ -975,6 +1002,7 @@ int rich_get_conserved(rich_sim *s, int64_t n, double *x, double *y, double *m, 
     bool host;
     int rc = read_buffer(s, 6, &st, &host);
     if (rc) return rc;
+    if (!st) return read_fields(s, src, outs, 6);
     CUDA_TRY(rich::launch_unpermute(s->n, s->cell_of.as<int32_t>(), src, st, s->stream));
     return copy_out(s, st, host, outs, 6);
 }

@@ -124,3 +124,25 @@ def test_a_batch_without_room_for_the_update(R, mode):
     for sid, want in zip(ids, solo):
         _same(b.conserved(sid), want)
     b.close()
+
+
+@pytest.mark.parametrize("precision", [W.FP64, W.FP32_SPLIT])
+def test_reads_without_room_on_the_device(R, precision):
+    """A read that finds no device memory to reorder in is reordered by the host."""
+    wl = W.kelvin_helmholtz(n_side=512)
+    wl["cfg"]["precision"] = precision
+    ref, sim = R.Sim(wl), R.Sim(wl)
+    b = R.Batch(precision=precision, max_cells=1 << 20)
+    sid = b.add(wl)
+    b.step()
+    ref.step(1)
+    sim.step(1)
+    want = ref.conserved(), ref.state()
+    sim.tessellate()
+    with _filled(4 << 20):
+        got, state, member = sim.conserved(), sim.state(), b.conserved(sid)
+    _same(got, want[0])
+    _same(state, want[1])
+    _same(member, want[0])
+    for h in (ref, sim, b):
+        h.close()
