@@ -60,8 +60,8 @@ FLOPS = {
         "k_circumcentre": {"tri": {"fp64": 25}},
         "k_geometry": {"edge": {"fp64": 32}, "cell": {"fp64": 40}, "slot": {"fp64": 11}},
         "k_advance_points": {"cell": {"fp64": 5}},
-        "k_cell_gradient": {"cell": {"fp64": 77}, "slot": {"fp64": 18}},
-        "k_edge_flux": {"edge": {"fp64": 147}},
+        "k_cell_gradient": {"cell": {"fp64": 59}, "slot": {"fp64": 18}},
+        "k_edge_flux": {"edge": {"fp64": 151}},
         "k_cell_update": {"cell": {"fp64": 17}, "slot": {"fp64": 4}},
     },
     "split": {

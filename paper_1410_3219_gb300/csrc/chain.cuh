@@ -13,6 +13,8 @@
 
 namespace rich {
 
+constexpr int kSMs = 152;  // of a GB300
+
 // From this many cells on kernels are launched plainly: the next one's
 // waiting blocks would take the room of the running one's.  A step (with the
 // mesh update) takes in dependent and in plain launches, FP64: 96 and 108 us for

@@ -23,6 +23,7 @@
 
 #include "../../include/rich.h"
 #include "api_internal.h"
+#include "chain.cuh"
 
 namespace {
 
@@ -30,7 +31,7 @@ constexpr int kBlock = 256;
 // cells a thread takes per pass, and the largest grid: six blocks on each of
 // 152 SMs (1,536 threads with ten to fourteen loads in flight each)
 constexpr int kCells = 2;
-constexpr int kMaxBlocks = 6 * 152;
+constexpr int kMaxBlocks = 6 * rich::kSMs;
 
 // scratch: per-block minima of the cell time step as bit patterns (the
 // integer order of non-negative doubles is their numeric order; kBad marks

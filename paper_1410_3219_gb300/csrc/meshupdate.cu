@@ -1076,7 +1076,7 @@ inline int blocks(int64_t n, int b) { return (int)((n + b - 1) / b); }
 // and 16 0.221 and 0.207.
 inline int pass_blocks(int64_t n, bool split)
 {
-    return std::max(1, std::min(blocks(8 * n, 128), 152 * (split ? 16 : n >= (1 << 19) ? 4 : 8)));
+    return std::max(1, std::min(blocks(8 * n, 128), kSMs * (split ? 16 : n >= (1 << 19) ? 4 : 8)));
 }
 
 }  // namespace
@@ -1283,7 +1283,7 @@ cudaError_t MeshUpdater::launch_rounds(const MeshArrays &a, const MeshOutput &o,
 {
     const MeshUpdate m = params(a, o);
     // grids for the cells a step lists (a few per cent), looping beyond
-    const int g = std::max(1, std::min(blocks(m.n, 16 * kListWarps), 152 * 8));
+    const int g = std::max(1, std::min(blocks(m.n, 16 * kListWarps), kSMs * 8));
     for (int r = first; r < last; r++) {
         if (r == 0) MU_TRY(launch_chained(k_mesh_recompute_light, g, kListBlock, st, m.n, m));
         MU_TRY(launch_chained(k_mesh_recompute, g, kListBlock, st, m.n, m, r));
@@ -1345,7 +1345,7 @@ cudaError_t MeshUpdater::start(const MeshArrays &a, const MeshOutput &o, cudaStr
     // (a warp per eight cells: steps of 10,201 cells took 105 us with one per
     // sixteen, 98 with this.  With the list passes at eight as well their FP64
     // tests slow the gradient of 4,096 cells, which runs beside them)
-    const int open = std::max(1, std::min(blocks(a.n, 8 * kListWarps), 152 * 8));
+    const int open = std::max(1, std::min(blocks(a.n, 8 * kListWarps), kSMs * 8));
     MU_TRY(launch_chained(k_mesh_verify_open, open, kListBlock, st, m.n, m));
     last_round_ = quiet_ < kQuiet ? 2 : 1;
     return launch_rounds(a, o, 0, last_round_, st);

@@ -500,7 +500,7 @@ template <class R> __device__ __forceinline__ double step_dt(const SweepParams<R
 // The prediction's cell terms come out with their time step: phi - hdt S for the
 // density, -hdt S for the velocity, which the flux adds to the velocity relative
 // to the edge.  (The pressure keeps its sum: see the flux.)
-// (Per cell of six slots: 204 FP64 instructions before, about 160 now.)
+// (Per cell of six slots: 204 FP64 instructions before, about 152 now.)
 template <class R, class Slots>
 __device__ __forceinline__ void stage_cell_gradient_fp64(const SweepParams<R> &p, int32_t i, int32_t lo, int32_t hi,
                                                          const Slots &sl)
@@ -933,12 +933,12 @@ template <class R> __device__ __forceinline__ void hllc(R gam, R igm1, const R L
     F[2] = F[0] * tK;
 }
 
-// a7 in FP64: as stage_edge_flux below, with about 115 FP64 instructions per
+// a7 in FP64: as stage_edge_flux below, with about 121 FP64 instructions per
 // edge instead of 132.  The sides' states come from the cells' terms
 // (stage_cell_gradient_fp64) and the velocities relative to the edge, which are
 // formed first: v and the edge's own velocity are each as large as the flow
 // through the box, and what follows must not round at that size (folding
-// hdt v into the cells' terms and hdt w_f into the edge's point, eight
+// hdt v into the cells' terms and hdt w_f into the edge's point, six
 // instructions fewer, multiplied the prediction's rounding by 6 at 100 sound
 // speeds and by 60 at 1,000).  Only side K's tangential velocity is formed; the
 // star state and the energy flux are put together:
