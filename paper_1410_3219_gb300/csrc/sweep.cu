@@ -838,9 +838,9 @@ __device__ __forceinline__ void cell_gradient(const SweepParams<float> &p, int32
 }
 
 // launched in blocks of 128 threads; five blocks per SM let the FP64 build have
-// 96 registers, with 68 bytes spilled to L1 (six, at 80 registers, spilled 250:
-// the same at 1M cells, 361 us, but two steps of 90,000 cells 369 us instead of
-// 348); nine hold the FP32 build's 56 registers, 36 warps, which hide more of its
+// 96 registers, with 68 bytes spilled to L1 (six, at 80 registers, spill 200:
+// the same at 1M cells, 353 us, but two steps of 90,000 cells and their read 479
+// us instead of 471); nine hold the FP32 build's 56 registers, 36 warps, which hide more of its
 // gather latency than 28 did (0.102 -> 0.093 ms at 1M cells, when the cap
 // took it from 72 registers, before the mesh velocity and the time step
 // moved to the geometry stage; ten blocks spilled and lost it again).
@@ -1108,7 +1108,7 @@ __device__ __forceinline__ void edge_flux(const SweepParams<double> &p, int32_t 
 __device__ __forceinline__ void edge_flux(const SweepParams<float> &p, int32_t e) { stage_edge_flux(p, e); }
 
 // launched in blocks of 128 threads; eight blocks per SM let the FP64 build
-// have 64 registers, without a spill: 655 -> 643 us at 1M cells against ten
+// have 64 registers, without a spill: 703 -> 680 us at 1M cells against ten
 // and 48 registers; sixteen cap the FP32 build at 32 (4 bytes spilled),
 // 64 warps: 0.069 -> 0.063 ms at 1M cells
 template <class R> __global__ void __launch_bounds__(128, sizeof(R) == 4 ? 16 : 8) k_edge_flux(SweepParams<R> p)
@@ -1329,8 +1329,8 @@ static_assert(kStageBlock[K_CELL_GRADIENT] == 128 && kStageBlock[K_EDGE_FLUX] ==
               "the gradient's and flux's launch bounds assume 128 threads");
 // (below 2^16 units the gradient and flux take one warp per block as well: 32
 // blocks of 128 threads put the 4,096 cells of a small simulation on 32 of
-// the 152 SMs, four warps to an FP64 pipe.  Two steps of 50,625 cells take
-// 430 us so, 440 with 128; of 90,000 cells the same, 349, with both)
+// the 152 SMs, four warps to an FP64 pipe.  Two steps of 50,625 cells took
+// 430 us so, 440 with 128; of 90,000 cells the same with both)
 inline int stage_block(int k, int64_t units) { return units < (1 << 16) ? 32 : kStageBlock[k]; }
 inline int nblk(int64_t n, int k) { return (int)((n + stage_block(k, n) - 1) / stage_block(k, n)); }
 
